@@ -15,7 +15,7 @@ import math
 
 import torch
 
-from paper_2312_05693_b200 import binding, inputs
+from paper_2312_05693_b200 import binding
 
 # Case fields (kind "layers"): m token rows; hidden, ffn: the model's widths; part: which layers (see _shapes);
 # group: 0 = one weight scale per output channel, 128 = one per 128 inputs; bits: activation codes; mode:
