@@ -133,7 +133,8 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     cudaError_t e = cudaSuccess;
     // a single row on the few-row kernel: that kernel finds the scale and makes the codes itself
     const bool fuse = !w_offsets && !alpha && kernel_for(h, M) == AQ_KERNEL_DECODE &&
-                      decode_can_fuse_quantize(M, K, N, group, h->dev.sm_count);
+                      decode_can_fuse_quantize(M, K, N, group, acc_dump != nullptr, h->dev.sm_count) &&
+                      (!group || aligned(w_scales, 16));
     if (fuse) {
     } else if (w_offsets) {
         // zero-point variant: min / max, then e, zp and codes; then the per-channel term -(zp - 2^(b-1)) * r[n]

@@ -3,10 +3,10 @@
 // Sec. 4.4 / Algorithm 1 and the floating-point output.
 //
 // Two kernels:
-//  * a general one (per-group scales, or any M when forced): a CTA owns 32 output channels
+//  * a general one (dumps of per-group sums, scales that are not 16-byte aligned, or any M when forced): a CTA owns 32 output channels
 //    (one lane each), its 8 warps split K by 128-k block, products use dp4a on weights
 //    widened to 16*code, warps meet in shared memory;
-//  * a streaming one for one scale per channel and M <= 16: a thread-block cluster shares a
+//  * a streaming one for M <= 16: a thread-block cluster shares a
 //    128-channel tile and splits K; in each CTA a producer thread streams 8 KB packed blocks
 //    and their activation codes into a shared-memory ring with TMA, eight consumer warps
 //    multiply (dp4a for one row, the warp-level int8 MMA above). Every CTA keeps the sums over
@@ -179,7 +179,7 @@ gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
 }
 
 // ---------------------------------------------------------------------------------------
-// Streaming kernel (one scale per channel, M <= 16)
+// Streaming kernel (M <= 16)
 // ---------------------------------------------------------------------------------------
 constexpr unsigned long long kStrWaitCycles = 4000000000ull;
 constexpr int kFuseMaxBlocks = 64;        // k blocks per CTA up to which a single row is quantized inside the product kernel
@@ -238,13 +238,14 @@ template <int MB> struct StreamCfg {
     static constexpr int kThreads = (1 + kConsumerWarps) * 32;
 };
 
-template <int MB, bool WIDE = false>
+template <int MB, bool WIDE = false, bool GROUPED = false>
 struct StreamSmem {
     static constexpr int kRows = StreamCfg<MB>::kRows;
     static constexpr int kStages = StreamCfg<MB>::kStages;
     alignas(1024) int8_t x[kStages][kRows * kTileK];       // activation codes of the unit's k block
     alignas(128) uint8_t w[kStages][kBlockBytes];          // packed weight block of the unit
-    // this CTA's sums over its k range; rows padded by 8 words so that the MMA route's fragment owners (eight
+    alignas(16) __half sc[GROUPED ? kStages : 1][kTileN];  // per-group scales: those of the unit's k block (= its group)
+    // this CTA's sums (per-group scales: the bits of fp32 sums) over its k range; rows padded by 8 words so that the MMA route's fragment owners (eight
     // rows at the same columns) spread over the banks
     static constexpr int kSumStride = kTileN + 8;
     alignas(16) int sum[kRows][kSumStride];
@@ -288,13 +289,26 @@ struct StreamParams {
 // tile and take consecutive k ranges; CTA r adds up and writes its slice of the tile's channels:
 // [r, r+1) * 128 / split for split 1, 2, 4; WIDE (split 5 to 8, 16-row route only) the groups of four
 // channels [32 r / split, 32 (r + 1) / split).
-template <int MB, bool FUSEQ = false, bool WIDE = false>
+//
+// GROUPED (one scale per 128 k): a k block is one group, so a block's integer sums are scaled and added in fp32 as
+// soon as the block is done, by the warp that made them; what the warps, and the CTAs of the cluster, then add up
+// are fp32 sums (in an order that does not depend on timing). The block's 128 scales ride along in the ring. The
+// per-block cost is one conversion and one FMA per accumulator and a half-word read per channel, on top of a kernel
+// whose consumers wait for memory most of the time; the kernel it replaced here (32 channels per CTA,
+// every lane reading every activation byte) took 9.5 us at M = 1 and 30 us at M = 6 on K = N = 4096. The seven layers of
+// a 4096 / 11008 block, quantization included, in graph replay: 116 -> 42 us at M = 1, 283 -> 65 us at M = 6.
+template <bool GROUPED>
+__device__ __forceinline__ int add_sums(int a, int b) {
+    return GROUPED ? __float_as_int(__int_as_float(a) + __int_as_float(b)) : a + b;
+}
+
+template <int MB, bool FUSEQ = false, bool WIDE = false, bool GROUPED = false>
 __global__ void __launch_bounds__(StreamCfg<MB>::kThreads, 2)
 gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const StreamParams p) {
     static_assert(!FUSEQ || MB == 1, "only a single row is quantized inside the product kernel");
     static_assert(!WIDE || MB == 16, "clusters of 5 to 8 are for the 16-row route");
     extern __shared__ uint8_t smem_raw[];
-    using Smem = StreamSmem<MB, WIDE>;
+    using Smem = StreamSmem<MB, WIDE, GROUPED>;
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr bool kUseMma = StreamCfg<MB>::kUseMma;
     constexpr int kRows = StreamCfg<MB>::kRows;
@@ -337,10 +351,14 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     };
     auto issue_w = [&](int kb, int s) {
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                     ::"r"(s_u32(&sm.full[s])), "r"((uint32_t)kBlockBytes + x_bytes(kb)) : "memory");
+                     ::"r"(s_u32(&sm.full[s])), "r"((uint32_t)kBlockBytes + (GROUPED ? kTileN * 2u : 0u) + x_bytes(kb)) : "memory");
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(s_u32(sm.w[s])), "l"(wsrc + (size_t)kb * kBlockBytes), "r"((uint32_t)kBlockBytes),
                        "r"(s_u32(&sm.full[s])) : "memory");
+        if constexpr (GROUPED)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(s_u32(sm.sc[s])), "l"(p.w_scales + (size_t)kb * p.Npad + tile * kTileN),
+                           "r"((uint32_t)(kTileN * 2)), "r"(s_u32(&sm.full[s])) : "memory");
     };
     auto issue_x = [&](int kb, int s) {
         if constexpr (FUSEQ) {
@@ -478,7 +496,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             // lane reading every activation byte, took twelve. The sum over k does not care which lane adds
             // which k; the lanes' partial sums meet once, after the k range.
             const int g = lane & 7, t = lane >> 3;
-            int acc[MB][4];
+            int acc[MB][4];                                          // per-group scales: the bits of fp32 sums
 #pragma unroll
             for (int m = 0; m < MB; ++m)
 #pragma unroll
@@ -500,7 +518,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                     for (int i = 0; i < 4; ++i) {
                         // word u of a unit: k 8u..8u+3 of the chunk in its low nibbles, k 8u+4..8u+7 in its high ones
                         const uint32_t w[4] = {wv[i].x, wv[i].y, wv[i].z, wv[i].w};
-                        int a = acc[m][i];
+                        int a = GROUPED ? 0 : acc[m][i];
                         a = __dp4a((int)((w[0] << 4) & 0xF0F0F0F0u), (int)x0.x, a);      // 16*code
                         a = __dp4a((int)(w[0] & 0xF0F0F0F0u), (int)x0.y, a);
                         a = __dp4a((int)((w[1] << 4) & 0xF0F0F0F0u), (int)x0.z, a);
@@ -509,7 +527,11 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                         a = __dp4a((int)(w[2] & 0xF0F0F0F0u), (int)x1.y, a);
                         a = __dp4a((int)((w[3] << 4) & 0xF0F0F0F0u), (int)x1.z, a);
                         a = __dp4a((int)(w[3] & 0xF0F0F0F0u), (int)x1.w, a);
-                        acc[m][i] = a;
+                        if constexpr (GROUPED)
+                            acc[m][i] = __float_as_int(fmaf((float)a, __half2float(sm.sc[s][quarter * 32 + 8 * i + g]),
+                                                            __int_as_float(acc[m][i])));
+                        else
+                            acc[m][i] = a;
                     }
                 }
                 __syncwarp();
@@ -523,8 +545,8 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             for (int m = 0; m < MB; ++m) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    acc[m][i] += __shfl_xor_sync(0xFFFFFFFFu, acc[m][i], 8);
-                    acc[m][i] += __shfl_xor_sync(0xFFFFFFFFu, acc[m][i], 16);
+                    acc[m][i] = add_sums<GROUPED>(acc[m][i], __shfl_xor_sync(0xFFFFFFFFu, acc[m][i], 8));
+                    acc[m][i] = add_sums<GROUPED>(acc[m][i], __shfl_xor_sync(0xFFFFFFFFu, acc[m][i], 16));
                 }
                 mine[m] = t == 0 ? acc[m][0] : t == 1 ? acc[m][1] : t == 2 ? acc[m][2] : acc[m][3];
             }
@@ -536,7 +558,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
 #pragma unroll
                     for (int m = 0; m < MB; ++m) {
                         if (ph == 0) sm.sum[m][r] = mine[m];
-                        else sm.sum[m][r] += mine[m];
+                        else sm.sum[m][r] = add_sums<GROUPED>(sm.sum[m][r], mine[m]);
                     }
                 }
             }
@@ -554,6 +576,13 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) acc[i][c] = 0;
+            [[maybe_unused]] float fsum[4][4];
+            if constexpr (GROUPED) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) fsum[i][c] = 0.0f;
+            }
             for (int kb = kb0 + phase; kb < kb1; kb += kPhases) {
                 const uint32_t it = (uint32_t)(kb - kb0);
                 const int s = (int)(it % kStrStages);
@@ -589,6 +618,17 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                             : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
                     }
                 }
+                if constexpr (GROUPED) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 sg = __half22float2(*reinterpret_cast<const __half2*>(&sm.sc[s][quarter * 32 + 8 * i + 2 * t]));
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            fsum[i][c] = fmaf((float)acc[i][c], (c & 1) ? sg.y : sg.x, fsum[i][c]);
+                            acc[i][c] = 0;
+                        }
+                    }
+                }
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_u32(&sm.empty[s])) : "memory");
             }
@@ -604,8 +644,9 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             int& dst = sm.sum[g + 8 * (c >> 1)][quarter * 32 + 8 * i + 2 * t + (c & 1)];
-                            if (ph == 0) dst = acc[i][c];
-                            else dst += acc[i][c];
+                            const int own = GROUPED ? __float_as_int(fsum[i][c]) : acc[i][c];
+                            if (ph == 0) dst = own;
+                            else dst = add_sums<GROUPED>(dst, own);
                         }
                 }
             }
@@ -632,13 +673,13 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     const int g_first = (32 * rank) / split, g_count = (32 * (rank + 1)) / split - g_first;   // this CTA's groups (wide)
     const int ft = (int)threadIdx.x - 32;                     // the consumer threads finish (a multiple of 128 = 4 cw at most)
     const int rc = ft & (cw - 1);                             // channel inside the slice (only used when ft >= 0)
-    const int out_r = wide ? 4 * g_first + rc : rank * cw + rc;
+    const int out_r = wide ? min(4 * g_first + rc, kTileN - 1) : rank * cw + rc;   // wide: lanes behind the slice only keep their warp whole
     const int out_n = tile * kTileN + out_r;
     const bool mine = ft >= 0 && out_n < p.N && (!wide || rc < 4 * g_count);
     float sc = 0.0f, off = 0.0f;
     if (mine) {
         const float pe = __int_as_float((127 + (FUSEQ ? fused_exp : *p.scale_exp)) << 23);
-        sc = __half2float(p.w_scales[out_n]) * pe;
+        sc = GROUPED ? 0.0625f * pe : __half2float(p.w_scales[out_n]) * pe;     // the fp32 sums carry a factor 16
         if (p.chan_offset) off = p.chan_offset[out_n] * pe;
     }
     const int rows = p.M < kRows ? p.M : kRows;
@@ -661,7 +702,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     } else {
         __syncthreads();
     }
-    if (mine) {
+    if (mine || (wide && ft >= 0)) {
         // All shared-memory reads of this thread's outputs are issued before the first is used and without
         // branches around them (rows that do not exist read the last row of the buffer and are dropped):
         // taken one after the other, each behind its own test, they were the longest part of the finish at
@@ -679,30 +720,30 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 const int col = c * cw + rc;
 #pragma unroll
                 for (int i = 0; i < kIt; ++i)
-                    if (i * stride < kRows) av[i] += sm.recv[min(m0 + i * stride, kRows - 1)][col];   // the same test in every thread
+                    if (i * stride < kRows)                               // the same test in every thread
+                        av[i] = add_sums<GROUPED>(av[i], sm.recv[min(m0 + i * stride, kRows - 1)][col]);
             }
         }
+        auto value = [&](int a) { return GROUPED ? __int_as_float(a) : (float)(a >> 4); };     // integer sums carry a factor 16
         if (!p.acc_dump && !p.q_next) {
 #pragma unroll
             for (int i = 0; i < kIt; ++i) {
                 const int m = m0 + i * stride;
-                const __half hv = __float2half_rn(fmaf((float)(av[i] >> 4), sc, off));     // sums carry a factor 16
-                if (m < rows) p.y[(size_t)m * p.N + out_n] = hv;
+                const __half hv = __float2half_rn(fmaf(value(av[i]), sc, off));
+                if (mine && m < rows) p.y[(size_t)m * p.N + out_n] = hv;
             }
         } else {
 #pragma unroll
             for (int i = 0; i < kIt; ++i) {
                 const int m = m0 + i * stride;
                 if (m < rows) {
-                    const int a = av[i] >> 4;
-                    if (p.acc_dump) p.acc_dump[(size_t)m * p.N + out_n] = a;
-                    const __half hv = __float2half_rn(fmaf((float)a, sc, off));
-                    // (a warp's lanes hold consecutive channels and run this loop together: slices of 32 and
-                    // more channels; clusters of 5 to 8 are not used with chained outputs)
+                    if (!GROUPED && p.acc_dump && mine) p.acc_dump[(size_t)m * p.N + out_n] = av[i] >> 4;
+                    const __half hv = __float2half_rn(fmaf(value(av[i]), sc, off));
+                    // (a warp's lanes hold consecutive channels, even lanes even channels, and run this loop together)
                     if (p.q_next)
                         store_next_code(p.q_next, (size_t)m * p.N + out_n, next_code(hv, p.next_inv, p.next_lo, p.next_hi),
-                                        p.next_packed, true, lane);
-                    else p.y[(size_t)m * p.N + out_n] = hv;
+                                        p.next_packed, mine, lane);
+                    else if (mine) p.y[(size_t)m * p.N + out_n] = hv;
                 }
             }
         }
@@ -725,12 +766,12 @@ inline int decode_split(int tiles, int KB, int sm_count) {
     return split;
 }
 
-template <int MB, bool FUSEQ = false, bool WIDE = false>
+template <int MB, bool FUSEQ, bool WIDE, bool GROUPED>
 cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int wide_split = 0) {
-    using Smem = StreamSmem<MB, WIDE>;
+    using Smem = StreamSmem<MB, WIDE, GROUPED>;
     const size_t smem_bytes = sizeof(Smem) + 1024;
     static SmemOptIn opt_in;
-    if (const cudaError_t e = opt_in.ensure(gemm_decode_stream_kernel<MB, FUSEQ, WIDE>, dev.device, smem_bytes); e != cudaSuccess)
+    if (const cudaError_t e = opt_in.ensure(gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED>, dev.device, smem_bytes); e != cudaSuccess)
         return e;
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
@@ -778,18 +819,19 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;       // the kernel reads and writes nothing before the kernel ahead of it has completed
-    return cudaLaunchKernelEx(&cfg, gemm_decode_stream_kernel<MB, FUSEQ, WIDE>, map, p);
+    return cudaLaunchKernelEx(&cfg, gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED>, map, p);
 }
 
 // 16-row route: its consumers, not the memory, set a CTA's pace, so more CTAs per tile pay as long as each
 // keeps five k blocks and all clusters still run at once (a GPC holds only so many clusters of a size: the
 // occupancy query says how many the device does). Measured on the 13B shapes with N = 5120 (clusters of 7):
 // K = 13824 12.5 / 13.2 -> 9.8 / 10.4 us at M = 4 / 16, K = 5120 6.9 / 7.3 -> 6.0 / 6.5 us; a single row
-// loses with clusters of 8 (N = 4096, K = 5120: 5.1 -> 6.2 us). Chained outputs keep slices of at least 32
-// channels. Returns the cluster size (5 to 8), or 0 for the usual 1, 2 or 4.
+// loses with clusters of 8 (N = 4096, K = 5120: 5.1 -> 6.2 us). Plain and chained calls take the same cluster
+// (with per-group scales its size sets the order of the fp32 sums). Returns the cluster size (5 to 8), or 0 for the usual 1, 2 or 4.
+template <bool GROUPED>
 int wide_split_for(const GemmArgs& a, const DeviceInfo& dev) {
     const int tiles = round_up(a.N, kTileN) / kTileN, KB = k_blocks(a.K);
-    if (a.q_next || decode_split(tiles, KB, dev.sm_count) != 4) return 0;
+    if (decode_split(tiles, KB, dev.sm_count) != 4) return 0;
     static std::atomic<int> fits[kMaxDevices][9];               // clusters of s that run at once, + 1 (0: not asked yet)
     int s = (2 * dev.sm_count) / tiles;
     if (s > 8) s = 8;
@@ -797,11 +839,11 @@ int wide_split_for(const GemmArgs& a, const DeviceInfo& dev) {
         if (KB / s < 5) continue;
         int known = fits[dev.device][s].load(std::memory_order_relaxed);
         if (known == 0) {
-            using Smem = StreamSmem<16, true>;
+            using Smem = StreamSmem<16, true, GROUPED>;
             const size_t smem_bytes = sizeof(Smem) + 1024;
             static SmemOptIn opt_in;
             int n = 0;
-            if (opt_in.ensure(gemm_decode_stream_kernel<16, false, true>, dev.device, smem_bytes) == cudaSuccess) {
+            if (opt_in.ensure(gemm_decode_stream_kernel<16, false, true, GROUPED>, dev.device, smem_bytes) == cudaSuccess) {
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(s, tiles, 1);
                 cfg.blockDim = dim3(StreamCfg<16>::kThreads);
@@ -813,7 +855,7 @@ int wide_split_for(const GemmArgs& a, const DeviceInfo& dev) {
                 attr[0].val.clusterDim.z = 1;
                 cfg.attrs = attr;
                 cfg.numAttrs = 1;
-                if (cudaOccupancyMaxActiveClusters(&n, gemm_decode_stream_kernel<16, false, true>, &cfg) != cudaSuccess) {
+                if (cudaOccupancyMaxActiveClusters(&n, gemm_decode_stream_kernel<16, false, true, GROUPED>, &cfg) != cudaSuccess) {
                     (void)cudaGetLastError();
                     n = 0;
                 }
@@ -845,25 +887,34 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
 
 }  // namespace
 
-// One row, one scale per channel, and a k range per CTA that fits the kernel's code buffer: the product
-// kernel can quantize the row itself (one launch for the layer).
-bool decode_can_fuse_quantize(int M, int K, int N, int group, int sm_count) {
-    if (M != 1 || group) return false;
+// One row and a k range per CTA that fits the kernel's code buffer: the product kernel can quantize the row itself
+// (one launch for the layer). Dumps of per-group sums are left to the general kernel.
+bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, int sm_count) {
+    if (M != 1 || (group && dump)) return false;
     const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
     const int split = decode_split(tiles, KB, sm_count);
     return (KB + split - 1) / split + 1 <= kFuseMaxBlocks;
 }
 
+namespace {
+template <bool GROUPED>
+cudaError_t launch_stream_rows(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+    // one row: dp4a; 2..16 rows: the warp MMA on a 16-row tile (fewer instructions per weight
+    // chunk than dp4a from two rows on; measured faster at M = 4: 7.5 / 11.1 / 13.3 us against
+    // 8.1 / 12.8 / 15.2 us on the three 13B shapes)
+    if (a.M <= 1 && a.fuse_x) return launch_stream<1, true, false, GROUPED>(a, dev, stream);
+    if (a.M <= 1) return launch_stream<1, false, false, GROUPED>(a, dev, stream);
+    if (const int ws = wide_split_for<GROUPED>(a, dev)) return launch_stream<16, false, true, GROUPED>(a, dev, stream, ws);
+    return launch_stream<16, false, false, GROUPED>(a, dev, stream);
+}
+}  // namespace
+
 cudaError_t launch_gemm_decode(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    if (!a.group && a.M <= 16) {
-        // one row: dp4a; 2..16 rows: the warp MMA on a 16-row tile (fewer instructions per weight
-        // chunk than dp4a from two rows on; measured faster at M = 4: 7.5 / 11.1 / 13.3 us against
-        // 8.1 / 12.8 / 15.2 us on the three 13B shapes)
-        if (a.M <= 1 && a.fuse_x) return launch_stream<1, true>(a, dev, stream);
-        if (a.M <= 1) return launch_stream<1>(a, dev, stream);
-        if (const int ws = wide_split_for(a, dev)) return launch_stream<16, false, true>(a, dev, stream, ws);
-        return launch_stream<16>(a, dev, stream);
-    }
+    if (a.M <= 16 && !a.group) return launch_stream_rows<false>(a, dev, stream);
+    // The streaming kernel never holds a group's whole integer sum in one place (a single row's lanes scale their
+    // parts of it), so the dump of per-group sums takes the general kernel. Its scales ride in 16-byte copies.
+    if (a.M <= 16 && !a.acc_dump && (reinterpret_cast<uintptr_t>(a.w_scales) & 15u) == 0)
+        return launch_stream_rows<true>(a, dev, stream);
     if (a.M <= 1) return launch_mb<1>(a, stream);
     if (a.M <= 2) return launch_mb<2>(a, stream);
     if (a.M <= 4) return launch_mb<4>(a, stream);

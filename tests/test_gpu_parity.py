@@ -241,6 +241,38 @@ def test_decode_clusters_of_five_to_eight(M, K, N):
         assert np.array_equal(q_next.cpu().numpy(), oracle.quantize_act(gpu["y"], 8, e_next))
 
 
+@pytest.mark.parametrize("M,K,N", [(1, 128, 1), (1, 1280, 392), (1, 11008, 520), (2, 128, 128), (5, 5120, 136), (8, 4096, 4096),
+                                   (9, 384, 200), (16, 11008, 4000), (16, 9216, 5760), (1, 65536, 40)])
+def test_few_rows_with_per_group_scales(M, K, N):
+    """M <= 16 with one scale per 128 inputs and no dump of the sums (the streaming kernel; a single row in one launch
+    while its k range fits, clusters of one to eight CTAs): codes exact, outputs within tolerance of the checker,
+    integer products scaled in fp32 (at most K / 128 + 16 additions: below 1e-4 of the largest term), and plain and
+    chained calls in agreement."""
+    x = inputs.activations(M, K, seed=M + K, outlier_frac=0.01, outlier_mult=20.0)
+    w = inputs.weights(N, K, seed=N + K)
+    gpu, ref = run_layer_both(x, w, 8, 128, binding.AQ_KERNEL_AUTO, want_acc=False)
+    assert gpu["e"] == ref["e"] and np.array_equal(gpu["q"], ref["q"])
+    assert_y_close(gpu["y"], ref["y"])
+    rows = np.arange(M, dtype=np.int32)[::-1].copy()
+    gpu, ref = run_layer_both(x, w, 4, 128, binding.AQ_KERNEL_AUTO, clip=2, row_idx=rows, want_acc=False)
+    assert np.array_equal(gpu["q"], ref["q"])
+    assert_y_close(gpu["y"], ref["y"])
+    h = handle()
+    packed, scales = h.aq_pack_w4(dev(w), 128)
+    y = h.aq_linear_w4a8(dev(x), packed, scales, N, 128).cpu().numpy()
+    e_next = oracle.layer_exponent(y, 4) - 1
+    ref_next = oracle.quantize_act(y, 4, e_next)
+    assert np.array_equal(h.aq_linear_chain(8, dev(x), packed, scales, N, 128, 4, e_next).cpu().numpy(), ref_next)
+    if N % 32 == 0:
+        q4 = h.aq_linear_chain_act4(8, dev(x), packed, scales, N, 128, e_next)
+        assert np.array_equal(q4.cpu().numpy(), oracle.pack_act4(ref_next))
+    r = h.aq_weight_offsets(packed, scales, N, K, 128)
+    ya = h.aq_linear_asym(8, dev(x), packed, scales, r, N, 128).cpu().numpy()
+    codes, sc = oracle.quantize_weights(w, 128)
+    e, zp = oracle.asym_params(x, 8)
+    assert_y_close(ya, oracle.linear_asym(oracle.quantize_act_asym(x, 8, e, zp), zp, codes, sc, e, 128)[1])
+
+
 @pytest.mark.parametrize("kernel", KERNELS)
 @pytest.mark.parametrize("M,K,N,group", [(16, 768, 768, 0), (129, 384, 200, 128), (260, 1152, 520, 128)])
 def test_linear_w4a4_matches_checker(kernel, M, K, N, group):
