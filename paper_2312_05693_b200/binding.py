@@ -1,4 +1,5 @@
-"""ctypes binding for libagileq.so: same names as the C ABI, argument marshalling only.
+"""Binding for libagileq.so: same names as the C ABI, argument marshalling only. The calls a program makes per
+layer are marshalled by the native module beside this file (csrc/aq_host.cpp), the rest through ctypes.
 
 Tensors are torch CUDA tensors used purely as device memory; every step of the layer runs
 in the library's kernels. Nothing here computes, and nothing falls back to another path:
@@ -26,6 +27,7 @@ AQ_SCALE_DYNAMIC, AQ_SCALE_STATIC = 0, 1
 AQ_KERNEL_AUTO, AQ_KERNEL_TENSOR, AQ_KERNEL_DECODE = 0, 1, 2
 
 _lib = None
+_native = None
 
 
 class AgileqError(RuntimeError):
@@ -118,6 +120,17 @@ def load():
     return L
 
 
+def _host():
+    """The native half of the binding (loads the library first, so that a missing build is reported as such)."""
+    global _native
+    if _native is None:
+        load()
+        from . import _aq_host
+        _aq_host.set_error(AgileqError)
+        _native = _aq_host
+    return _native
+
+
 def status_string(status: int) -> str:
     return load().aq_status_string(status).decode()
 
@@ -132,7 +145,7 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _stream() -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def aq_packed_w4_bytes(N: int, K: int) -> int:
@@ -175,6 +188,7 @@ class Handle:
     def __init__(self, device: int = 0):
         self._h = C.c_void_p()
         self.device = device
+        self._native = _host()
         _check(load().aq_create(C.byref(self._h), device), "aq_create")
 
     def close(self):
@@ -228,38 +242,17 @@ class Handle:
     def aq_quantize_act(self, x: torch.Tensor, bits: int, scale_mode: int = AQ_SCALE_DYNAMIC,
                         clip_shift_or_exp: int = 0, row_idx: Optional[torch.Tensor] = None,
                         workspace: Optional[torch.Tensor] = None) -> Tuple[torch.Tensor, torch.Tensor]:
-        M_in, K = x.shape
-        M = M_in if row_idx is None else row_idx.shape[0]
-        q = torch.empty((M, K), dtype=torch.int8, device=x.device)
-        e = torch.empty(1, dtype=torch.int32, device=x.device)
-        ws = workspace if workspace is not None else torch.empty(256, dtype=torch.uint8, device=x.device)
-        _check(load().aq_quantize_act(self._h, _ptr(x), M, K, bits, scale_mode, clip_shift_or_exp,
-                                      _ptr(row_idx), _ptr(q), _ptr(e), _ptr(ws), ws.numel(), _stream()),
-               "aq_quantize_act")
-        return q, e
-
-    def _linear(self, fn, name, x, packed, scales, N, group_size, scale_mode, clip_shift_or_exp, row_idx,
-                y, acc_dump, workspace):
-        M_in, K = x.shape
-        M = M_in if row_idx is None else row_idx.shape[0]
-        if y is None:
-            y = torch.empty((M, N), dtype=torch.float16, device=x.device)
-        if workspace is None:
-            workspace = self.alloc_workspace(M, K, N, group_size)
-        _check(fn(self._h, _ptr(x), M, K, _ptr(packed), _ptr(scales), N, group_size, scale_mode,
-                  clip_shift_or_exp, _ptr(row_idx), _ptr(y), _ptr(acc_dump), _ptr(workspace),
-                  workspace.numel(), _stream()), name)
-        return y
+        return self._native.quantize_act(self._h.value, x, bits, scale_mode, clip_shift_or_exp, row_idx, workspace)
 
     def aq_linear_w4a8(self, x, packed, scales, N, group_size, scale_mode=AQ_SCALE_DYNAMIC,
                        clip_shift_or_exp=0, row_idx=None, y=None, acc_dump=None, workspace=None):
-        return self._linear(load().aq_linear_w4a8, "aq_linear_w4a8", x, packed, scales, N, group_size,
-                            scale_mode, clip_shift_or_exp, row_idx, y, acc_dump, workspace)
+        return self._native.linear(self._h.value, 8, x, packed, scales, N, group_size, scale_mode, clip_shift_or_exp,
+                                   row_idx, y, acc_dump, workspace, 0, None, 0)
 
     def aq_linear_w4a4(self, x, packed, scales, N, group_size, scale_mode=AQ_SCALE_DYNAMIC,
                        clip_shift_or_exp=0, row_idx=None, y=None, acc_dump=None, workspace=None):
-        return self._linear(load().aq_linear_w4a4, "aq_linear_w4a4", x, packed, scales, N, group_size,
-                            scale_mode, clip_shift_or_exp, row_idx, y, acc_dump, workspace)
+        return self._native.linear(self._h.value, 4, x, packed, scales, N, group_size, scale_mode, clip_shift_or_exp,
+                                   row_idx, y, acc_dump, workspace, 0, None, 0)
 
     # ---- log2 codes of the softmax output and attention x value (Eq. 3)
     def aq_log2_quantize(self, x: torch.Tensor, bits: int) -> Tuple[torch.Tensor, torch.Tensor]:
@@ -281,66 +274,25 @@ class Handle:
         return y
 
     def aq_attn_v_log2_tc(self, p_codes, p_max_bits, v_codes, v_scale_exp, y=None, workspace=None):
-        H, M, J = p_codes.shape
-        D = v_codes.shape[2]
-        if y is None:
-            y = torch.empty((H, M, D), dtype=torch.float16, device=p_codes.device)
-        if workspace is None:
-            workspace = torch.empty(load().aq_attn_workspace_bytes(H, M, J, D), dtype=torch.uint8, device=p_codes.device)
-        _check(load().aq_attn_v_log2_tc(self._h, _ptr(p_codes), _ptr(p_max_bits), _ptr(v_codes), _ptr(v_scale_exp), H, M,
-                                        J, D, _ptr(y), _ptr(workspace), workspace.numel(), _stream()),
-               "aq_attn_v_log2_tc")
-        return y, workspace
+        return self._native.attn_v(self._h.value, 0, p_codes, p_max_bits, v_codes, v_scale_exp, y, workspace)
 
     def aq_log2_quantize_factors(self, x: torch.Tensor, factors: Optional[torch.Tensor] = None,
                                  workspace: Optional[torch.Tensor] = None):
         """(uint8 byte factors 128 >> k of x's shape, uint32[1] holding the fp16 bits of max|x|, workspace)."""
-        if factors is None:
-            factors = torch.empty(x.shape, dtype=torch.uint8, device=x.device)
-        mx = torch.zeros(1, dtype=torch.int32, device=x.device)
-        ws = workspace if workspace is not None else torch.empty(256, dtype=torch.uint8, device=x.device)
-        _check(load().aq_log2_quantize_factors(self._h, _ptr(x), x.numel(), _ptr(factors), _ptr(mx), _ptr(ws), ws.numel(),
-                                               _stream()), "aq_log2_quantize_factors")
-        return factors, mx, ws
+        return self._native.log2_factors(self._h.value, x, factors, workspace)
 
     def aq_attn_v_factors_tc(self, p_factors, p_max_bits, v_codes, v_scale_exp, y=None, workspace=None):
-        H, M, J = p_factors.shape
-        D = v_codes.shape[2]
-        if y is None:
-            y = torch.empty((H, M, D), dtype=torch.float16, device=p_factors.device)
-        if workspace is None:
-            workspace = torch.empty(load().aq_attn_workspace_bytes(H, M, J, D), dtype=torch.uint8, device=p_factors.device)
-        _check(load().aq_attn_v_factors_tc(self._h, _ptr(p_factors), _ptr(p_max_bits), _ptr(v_codes), _ptr(v_scale_exp), H,
-                                           M, J, D, _ptr(y), _ptr(workspace), workspace.numel(), _stream()),
-               "aq_attn_v_factors_tc")
-        return y, workspace
+        return self._native.attn_v(self._h.value, 1, p_factors, p_max_bits, v_codes, v_scale_exp, y, workspace)
 
     def aq_attn_qk_tc(self, q_codes, q_exp, k_codes, k_exp, s=None, workspace=None):
-        H, M, D = q_codes.shape
-        J = k_codes.shape[1]
-        if s is None:
-            s = torch.empty((H, M, J), dtype=torch.float16, device=q_codes.device)
-        if workspace is None:
-            workspace = torch.empty(256, dtype=torch.uint8, device=q_codes.device)
-        _check(load().aq_attn_qk_tc(self._h, _ptr(q_codes), _ptr(q_exp), _ptr(k_codes), _ptr(k_exp), H, M, J, D, _ptr(s),
-                                    _ptr(workspace), workspace.numel(), _stream()), "aq_attn_qk_tc")
-        return s, workspace
+        return self._native.attn_qk(self._h.value, q_codes, q_exp, k_codes, k_exp, s, workspace)
 
     # ---- chaining: the next layer's codes instead of fp16 outputs (Sec. 4.4)
     def aq_linear_chain(self, bits, x, packed, scales, N, group_size, next_bits, next_exp,
                         scale_mode=AQ_SCALE_DYNAMIC, clip_shift_or_exp=0, row_idx=None, q_next=None, acc_dump=None,
                         workspace=None):
-        M_in, K = x.shape
-        M = M_in if row_idx is None else row_idx.shape[0]
-        if q_next is None:
-            q_next = torch.empty((M, N), dtype=torch.int8, device=x.device)
-        if workspace is None:
-            workspace = self.alloc_workspace(M, K, N, group_size)
-        fn = load().aq_linear_w4a8_chain if bits == 8 else load().aq_linear_w4a4_chain
-        _check(fn(self._h, _ptr(x), M, K, _ptr(packed), _ptr(scales), N, group_size, scale_mode, clip_shift_or_exp,
-                  _ptr(row_idx), _ptr(q_next), next_bits, next_exp, _ptr(acc_dump), _ptr(workspace),
-                  workspace.numel(), _stream()), "aq_linear_chain")
-        return q_next
+        return self._native.linear_chain(self._h.value, bits, 0, x, packed, scales, N, group_size, next_bits, next_exp,
+                                         scale_mode, clip_shift_or_exp, row_idx, q_next, acc_dump, workspace)
 
     # ---- activations with a zero point (Eq. 2, Eq. 5-7)
     def aq_weight_offsets(self, packed: torch.Tensor, scales: torch.Tensor, N: int, K: int, group_size: int
@@ -364,16 +316,8 @@ class Handle:
 
     def aq_linear_asym(self, bits, x, packed, scales, w_offsets, N, group_size, row_idx=None, y=None, acc_dump=None,
                        workspace=None):
-        M_in, K = x.shape
-        M = M_in if row_idx is None else row_idx.shape[0]
-        if y is None:
-            y = torch.empty((M, N), dtype=torch.float16, device=x.device)
-        if workspace is None:
-            workspace = self.alloc_workspace(M, K, N, group_size)
-        fn = load().aq_linear_w4a8_asym if bits == 8 else load().aq_linear_w4a4_asym
-        _check(fn(self._h, _ptr(x), M, K, _ptr(packed), _ptr(scales), _ptr(w_offsets), N, group_size, _ptr(row_idx),
-                  _ptr(y), _ptr(acc_dump), _ptr(workspace), workspace.numel(), _stream()), "aq_linear_asym")
-        return y
+        return self._native.linear_asym(self._h.value, bits, x, packed, scales, w_offsets, N, group_size, row_idx, y,
+                                        acc_dump, workspace)
 
     # ---- per-channel TRIP factors (Eq. 5-8)
     def aq_trip_calibrate(self, x: torch.Tensor, k_max: int, row_idx: Optional[torch.Tensor] = None
@@ -402,42 +346,16 @@ class Handle:
 
     def aq_linear_w4a4_trip(self, x, packed, scales, N, group_size, alpha, k_max, scale_mode=AQ_SCALE_DYNAMIC,
                             clip_shift_or_exp=0, row_idx=None, y=None, acc_dump=None, workspace=None):
-        M_in, K = x.shape
-        M = M_in if row_idx is None else row_idx.shape[0]
-        if y is None:
-            y = torch.empty((M, N), dtype=torch.float16, device=x.device)
-        if workspace is None:
-            workspace = self.alloc_workspace(M, K, N, group_size)
-        _check(load().aq_linear_w4a4_trip(self._h, _ptr(x), M, K, _ptr(packed), _ptr(scales), N, group_size,
-                                          _ptr(alpha), k_max, scale_mode, clip_shift_or_exp, _ptr(row_idx),
-                                          _ptr(y), _ptr(acc_dump), _ptr(workspace), workspace.numel(), _stream()),
-               "aq_linear_w4a4_trip")
-        return y
+        return self._native.linear(self._h.value, 4, x, packed, scales, N, group_size, scale_mode, clip_shift_or_exp,
+                                   row_idx, y, acc_dump, workspace, 1, alpha, k_max)
 
     def aq_gemm_w4(self, q, packed, scales, N, group_size, scale_exp, y=None, acc_dump=None, workspace=None):
-        M, K = q.shape
-        if y is None:
-            y = torch.empty((M, N), dtype=torch.float16, device=q.device)
-        if workspace is None:
-            workspace = self.alloc_workspace(M, K, N, group_size)
-        _check(load().aq_gemm_w4(self._h, _ptr(q), M, K, _ptr(packed), _ptr(scales), N, group_size,
-                                 _ptr(scale_exp), _ptr(y), _ptr(acc_dump), _ptr(workspace),
-                                 workspace.numel(), _stream()), "aq_gemm_w4")
-        return y
+        return self._native.gemm(self._h.value, 0, q, packed, scales, N, group_size, scale_exp, y, acc_dump, workspace)
 
     def aq_linear_chain_act4(self, bits, x, packed, scales, N, group_size, next_exp, scale_mode=AQ_SCALE_DYNAMIC,
                              clip_shift_or_exp=0, row_idx=None, q4_next=None, acc_dump=None, workspace=None):
-        M_in, K = x.shape
-        M = M_in if row_idx is None else row_idx.shape[0]
-        if q4_next is None:
-            q4_next = torch.empty((M, N // 2), dtype=torch.uint8, device=x.device)
-        if workspace is None:
-            workspace = self.alloc_workspace(M, K, N, group_size)
-        fn = load().aq_linear_w4a8_chain_act4 if bits == 8 else load().aq_linear_w4a4_chain_act4
-        _check(fn(self._h, _ptr(x), M, K, _ptr(packed), _ptr(scales), N, group_size, scale_mode, clip_shift_or_exp,
-                  _ptr(row_idx), _ptr(q4_next), next_exp, _ptr(acc_dump), _ptr(workspace), workspace.numel(),
-                  _stream()), "aq_linear_chain_act4")
-        return q4_next
+        return self._native.linear_chain(self._h.value, bits, 1, x, packed, scales, N, group_size, 4, next_exp, scale_mode,
+                                         clip_shift_or_exp, row_idx, q4_next, acc_dump, workspace)
 
     def aq_act4_pack(self, q: torch.Tensor, q4: Optional[torch.Tensor] = None) -> torch.Tensor:
         M, K = q.shape
@@ -466,25 +384,10 @@ class Handle:
         return q4, e
 
     def aq_gemm_w4_act4(self, q4, packed, scales, N, group_size, scale_exp, y=None, acc_dump=None, workspace=None):
-        M, K2 = q4.shape
-        K = 2 * K2
-        if y is None:
-            y = torch.empty((M, N), dtype=torch.float16, device=q4.device)
-        if workspace is None:
-            workspace = self.alloc_workspace(M, K, N, group_size)
-        _check(load().aq_gemm_w4_act4(self._h, _ptr(q4), M, K, _ptr(packed), _ptr(scales), N, group_size,
-                                      _ptr(scale_exp), _ptr(y), _ptr(acc_dump), _ptr(workspace),
-                                      workspace.numel(), _stream()), "aq_gemm_w4_act4")
-        return y
+        return self._native.gemm(self._h.value, 1, q4, packed, scales, N, group_size, scale_exp, y, acc_dump, workspace)
 
     def aq_token_select(self, scores: torch.Tensor, n_keep: int, workspace=None) -> torch.Tensor:
-        M = scores.shape[0]
-        idx = torch.empty(max(n_keep, 1), dtype=torch.int32, device=scores.device)[:n_keep]
-        if workspace is None:
-            workspace = torch.empty(256 + ((M + 255) // 256) * 256, dtype=torch.uint8, device=scores.device)
-        _check(load().aq_token_select(self._h, _ptr(scores), M, n_keep, _ptr(idx), _ptr(workspace),
-                                      workspace.numel(), _stream()), "aq_token_select")
-        return idx
+        return self._native.token_select(self._h.value, scores, n_keep, workspace)
 
     def aq_token_compact(self, x: torch.Tensor, idx: torch.Tensor, out=None) -> torch.Tensor:
         M, K = x.shape

@@ -1,14 +1,18 @@
-"""Builds libagileq.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libagileq.so (nvcc, sm_100a; cross-compiles without a GPU) and the binding's native half in-tree."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_DIR, "csrc")
 LIB = os.path.join(_DIR, "libagileq.so")
+# native half of the binding: a CPython module against this interpreter's torch, linked to the library beside it
+HOST_SRC = os.path.join(CSRC, "aq_host.cpp")
+HOST_LIB = os.path.join(_DIR, "_aq_host.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
@@ -29,7 +33,33 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _host_stale() -> bool:
+    header = os.path.join(os.path.dirname(_DIR), "include", "agileq.h")
+    return not os.path.exists(HOST_LIB) or os.path.getmtime(HOST_LIB) < max(os.path.getmtime(HOST_SRC), os.path.getmtime(header))
+
+
+def _build_host() -> None:
+    import torch
+    root = os.path.dirname(torch.__file__)
+    tmp = HOST_LIB + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", HOST_SRC, "-o", tmp,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(root, "include"),
+           "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"), "-I/usr/local/cuda/include",
+           "-L" + os.path.join(root, "lib"), "-Wl,-rpath," + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
+           "-ltorch_python", "-L" + _DIR, "-l:libagileq.so", "-Wl,-rpath,$ORIGIN"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, HOST_LIB)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    lib = _build_lib(force, verbose)
+    if force or _host_stale():
+        _build_host()
+    return lib
+
+
+def _build_lib(force: bool, verbose: bool) -> str:
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
