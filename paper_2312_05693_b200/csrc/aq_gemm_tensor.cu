@@ -104,6 +104,21 @@ struct TensorParams {
     int y_tma;                     // outputs leave through y_map (needs N % 8 == 0 and a 16-byte aligned y)
 };
 
+// One column of this thread's row, waited for.
+__device__ __forceinline__ int tc_ld1(uint32_t taddr) {
+    uint32_t v;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;" : "=r"(v) : "r"(taddr) : "memory");
+    return (int)v;
+}
+// Two fp32 FMAs with the same factor in one instruction: no more of them a clock than single ones, but half the issue slots.
+__device__ __forceinline__ void fma_pair(float& a0, float& a1, float x0, float x1, float s) {
+    asm("{\n\t.reg .b64 a, x, s;\n\t"
+        "mov.b64 a, {%0, %1};\n\tmov.b64 x, {%2, %3};\n\tmov.b64 s, {%4, %4};\n\t"
+        "fma.rn.f32x2 a, x, s, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(x0), "f"(x1), "f"(s));
+}
+
 // The code the next layer's quantizer gives the fp16 output value (static exponent; NaN -> 0).
 __device__ __forceinline__ int chain_code(__half hv, float inv, float lo, float hi) {
     const float t = __half2float(hv) * inv;                 // exact: inv is a power of two
@@ -235,23 +250,33 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
             constexpr uint32_t idesc = idesc_i8(128, BM);
             const uint32_t total_iters = (uint32_t)my_tiles * (uint32_t)(kb_last - kb_first);
             if (GROUPED) {
-                // every k block is one accumulation into its own accumulator stage
+                // Every k block is one accumulation into its own accumulator stage. Ring positions and phases are
+                // carried in counters (steps of kNumMmaThreads): the divisions that gave them from the block's number
+                // were most of this loop, one thread whose every instruction waits for the one before.
+                uint32_t a = (uint32_t)mma_id % kNumAcc, st = (uint32_t)mma_id, ai = (uint32_t)mma_id;
+                uint32_t acc_ph = 1u, a_ph = 0u;
+                const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm.x[0]));
                 for (uint32_t it = mma_id; it < total_iters; it += kNumMmaThreads) {
-                    const int a = (int)(it % kNumAcc);
-                    const int s = (int)(it % kNumStages);
-                    const int ai = (int)(it % kNumASlices);
-                    if (!mbar_wait(&sm.acc_empty[a], ((it / kNumAcc) & 1u) ^ 1u, abort_flag, 2u)) goto role_done;
-                    if (!mbar_wait(&sm.a_full[ai], (it / kNumASlices) & 1u, abort_flag, 3u)) goto role_done;
+                    const bool got_a = mbar_try_wait(&sm.a_full[ai], a_ph);       // both asked before either answer is used
+                    const bool got_acc = mbar_try_wait(&sm.acc_empty[a], acc_ph);
+                    if (!got_acc && !mbar_wait(&sm.acc_empty[a], acc_ph, abort_flag, 2u)) goto role_done;
+                    if (!got_a && !mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 3u)) goto role_done;
                     tc_fence_after();
-                    const uint32_t d_addr = tmem_acc + (uint32_t)(a * kAccStride);
-                    const uint32_t a_addr = tmem_a + (uint32_t)(ai * kAColsPerStage);
-                    const uint64_t bdesc = smem_desc_sw128(smem_u32(sm.x[s]));
+                    const uint32_t d_addr = tmem_acc + a * (uint32_t)kAccStride;
+                    const uint32_t a_addr = tmem_a + ai * (uint32_t)kAColsPerStage;
+                    const uint64_t bdesc = bdesc0 + (uint64_t)(st * (uint32_t)(BM * 128 / 16));
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
                         tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc, j > 0 ? 1u : 0u);
-                    tc_commit(&sm.a_empty[ai]);
-                    tc_commit(&sm.smem_empty[s]);
                     tc_commit(&sm.acc_full[a]);
+                    tc_commit(&sm.a_empty[ai]);
+                    tc_commit(&sm.smem_empty[st]);
+                    a += kNumMmaThreads;
+                    if (a >= (uint32_t)kNumAcc) { a -= kNumAcc; acc_ph ^= 1u; }
+                    st += kNumMmaThreads;
+                    if (st >= (uint32_t)kNumStages) st -= kNumStages;
+                    ai += kNumMmaThreads;
+                    if (ai >= (uint32_t)kNumASlices) { ai -= kNumASlices; a_ph ^= 1u; }
                 }
             } else {
                 uint32_t it = 0;
@@ -428,6 +453,15 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                     if (++g_slot == (uint32_t)Smem::kNumScaleSlots) g_slot = 0;
                     static_assert(kColsPerEpiWarp == 32 || kColsPerEpiWarp == 64, "epilogue register plan");
                     const uint32_t taddr = tmem_acc + lane_addr + (uint32_t)(a * kAccStride + col0);
+                    if (p.acc_dump) {
+                        // a rolled loop of its own: unrolled with the arithmetic below, the code of these stores (run only
+                        // by tests) kept pushing the loop out of the instruction cache
+#pragma unroll 1
+                        for (int c = 0; c < kColsPerEpiWarp; ++c) {
+                            const int sum = tc_ld1(taddr + (uint32_t)c);
+                            if (n_ok && m_base + c < p.M) p.acc_dump[((size_t)(m_base + c) * p.N + n) * G + kb] = sum >> 4;
+                        }
+                    }
                     // With twelve epilogue warps (128 registers each) a warp's 64 columns pass through one
                     // 32-register buffer in two turns; otherwise all of them are loaded at once.
                     constexpr int kLdCols = (kEpiWarps == 12 && kColsPerEpiWarp == 64) ? 32 : kColsPerEpiWarp;
@@ -444,19 +478,14 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                             if (lane == 0) mbar_arrive(&sm.acc_empty[a]);
                         }
 #pragma unroll
-                        for (int c = 0; c < kLdCols; ++c) {
-                            // One conversion and one FMA per element. (An integer add of the bits of
+                        for (int c = 0; c < kLdCols; c += 2) {
+                            // One conversion per element and one FMA per two. (An integer add of the bits of
                             // 1.5 * 2^23 plus a float subtract also converts, on the FMA and ALU pipes, but
                             // costs a third instruction; measured 8-16 % slower: issue slots are what this
-                            // loop runs out of, not the conversion unit.)
-                            fsum[c0 + c] = fmaf((float)(int)v[c], sg, fsum[c0 + c]);
-                        }
-                        if (p.acc_dump) {
-#pragma unroll
-                            for (int c = 0; c < kLdCols; ++c) {
-                                const int m = m_base + c0 + c;
-                                if (n_ok && m < p.M) p.acc_dump[((size_t)m * p.N + n) * G + kb] = (int)v[c] >> 4;
-                            }
+                            // loop runs out of, not the conversion unit. Paired FMAs, the issuers' counters and
+                            // the dump's code outside this loop: K, N = 4096, 4096 / 4096, 11008 / 11008, 4096 at
+                            // M = 2048 65.1 / 139.2 / 137.5 -> 61.7 / 135.3 / 133.3 us.)
+                            fma_pair(fsum[c0 + c], fsum[c0 + c + 1], (float)(int)v[c], (float)(int)v[c + 1], sg);
                         }
                     }
                 }
