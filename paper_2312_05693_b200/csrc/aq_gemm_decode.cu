@@ -6,10 +6,10 @@
 //  * a general one (dumps of per-group sums, scales that are not 16-byte aligned, or any M when forced): a CTA owns 32 output channels
 //    (one lane each), its 8 warps split K by 128-k block, products use dp4a on weights
 //    widened to 16*code, warps meet in shared memory;
-//  * a streaming one for M <= 16: a thread-block cluster shares a
+//  * a streaming one for M <= 32: a thread-block cluster shares a
 //    128-channel tile and splits K; in each CTA a producer thread streams 8 KB packed blocks
 //    and their activation codes into a shared-memory ring with TMA, eight consumer warps
-//    multiply (dp4a for one row, the warp-level int8 MMA above). Every CTA keeps the sums over
+//    multiply (dp4a for one row, the warp-level int8 MMA above, on one or two 16-row tiles). Every CTA keeps the sums over
 //    its k range in its own shared memory; the cluster meets once, and every CTA then finishes a
 //    slice of the tile's channels by reading the other CTAs' sums over distributed shared memory
 //    (integer addition is exact in any order). No workspace, no atomics.
@@ -179,7 +179,7 @@ gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
 }
 
 // ---------------------------------------------------------------------------------------
-// Streaming kernel (M <= 16)
+// Streaming kernel (M <= 32)
 // ---------------------------------------------------------------------------------------
 constexpr unsigned long long kStrWaitCycles = 4000000000ull;
 constexpr int kFuseMaxBlocks = 64;        // k blocks per CTA up to which a single row is quantized inside the product kernel
@@ -221,7 +221,7 @@ __device__ __forceinline__ bool str_wait(uint64_t* bar, uint32_t parity, volatil
 // 0.1-0.3 us slower than one.
 template <int MB> struct StreamCfg {
     static constexpr bool kUseMma = MB > 4;
-    static constexpr int kRows = kUseMma ? 16 : MB;
+    static constexpr int kRows = MB;
     static constexpr int kStages = 8;
     static constexpr int kProdLanes = kUseMma ? 1 : 2;
     // Consumer warps: a channel quarter each, kPhases warps per quarter taking the k blocks in turn. A third
@@ -230,6 +230,10 @@ template <int MB> struct StreamCfg {
     // consumer work in flight, not with the time a block waits (with the consumers' arithmetic taken out the
     // same launches take 6.6 / 9.1 / 10.1 us, and the ring is never full either way).
     static constexpr int kPhases = 2;
+    static constexpr int kRowTiles = MB <= 16 ? 1 : 2;           // 16-row tiles of a consumer warp
+    // More than 16 rows: the sum and receive buffers take the place of the operand ring once it has run dry, so that
+    // two CTAs still fit an SM.
+    static constexpr bool kAlias = MB > 16;
     // Two CTAs per SM for both routes. Three single-row CTAs would fit (with 128-byte instead of 1024-byte
     // alignment slack), so that under the stable-weights promise the next launch's CTAs sit, fetching, beside
     // two CTAs of this one; measured slower (M = 1 layer 5.8 / 9.1 / 9.7 -> 6.6 / 9.7 / 11.8 us): what the
@@ -238,24 +242,43 @@ template <int MB> struct StreamCfg {
     static constexpr int kThreads = (1 + kConsumerWarps) * 32;
 };
 
-template <int MB, bool WIDE = false, bool GROUPED = false>
-struct StreamSmem {
-    static constexpr int kRows = StreamCfg<MB>::kRows;
+// this CTA's sums over its k range (per-group scales: the bits of fp32 sums; rows padded by 8 words so that the MMA
+// route's fragment owners, eight rows at the same columns, spread over the banks), and the other CTAs' sums for this
+// CTA's channel slice, by sender (CTAs below this one, then above): `split` - 1 slots of 128 / split channels, or
+// (clusters of 5 to 8) seven slots of 32
+template <int MB, bool WIDE>
+struct StreamSums {
+    static constexpr int kSumStride = kTileN + 8;
+    static constexpr int kRecvStride = WIDE ? 7 * 32 : 96;
+    alignas(16) int sum[StreamCfg<MB>::kRows][kSumStride];
+    alignas(16) int recv[StreamCfg<MB>::kRows][kRecvStride];
+};
+template <int MB, bool GROUPED>
+struct StreamRing {
     static constexpr int kStages = StreamCfg<MB>::kStages;
-    alignas(1024) int8_t x[kStages][kRows * kTileK];       // activation codes of the unit's k block
+    alignas(1024) int8_t x[kStages][StreamCfg<MB>::kRows * kTileK];    // activation codes of the unit's k block
     alignas(128) uint8_t w[kStages][kBlockBytes];          // packed weight block of the unit
     alignas(16) __half sc[GROUPED ? kStages : 1][kTileN];  // per-group scales: those of the unit's k block (= its group)
-    // this CTA's sums (per-group scales: the bits of fp32 sums) over its k range; rows padded by 8 words so that the MMA route's fragment owners (eight
-    // rows at the same columns) spread over the banks
-    static constexpr int kSumStride = kTileN + 8;
-    alignas(16) int sum[kRows][kSumStride];
+};
+template <class Ring, class Sums, bool ALIAS>
+struct StreamBuffers {
+    Ring ring;
+    Sums sums;
+};
+template <class Ring, class Sums>
+struct StreamBuffers<Ring, Sums, true> {
+    union {
+        Ring ring;
+        Sums sums;
+    };
+};
+template <int MB, bool WIDE = false, bool GROUPED = false>
+struct StreamSmem : StreamBuffers<StreamRing<MB, GROUPED>, StreamSums<MB, WIDE>, StreamCfg<MB>::kAlias> {
+    static constexpr int kStages = StreamCfg<MB>::kStages;
+    static constexpr int kRecvStride = StreamSums<MB, WIDE>::kRecvStride;
     // one row quantized by the kernel itself: the codes of this CTA's k range (up to kFuseMaxBlocks blocks)
     alignas(16) int8_t xq[MB == 1 ? kFuseMaxBlocks * kTileK : 16];
     unsigned int warp_max[StreamCfg<MB>::kThreads / 32];
-    // the other CTAs' sums for this CTA's channel slice, by sender: `split` slots of 128 / split channels, or
-    // (clusters of 5 to 8) eight slots of 32
-    static constexpr int kRecvStride = WIDE ? 256 : kTileN;
-    alignas(16) int recv[kRows][kRecvStride];
     alignas(8) uint64_t full[kStages];
     uint64_t empty[kStages];
     volatile uint32_t abort_flag;
@@ -277,6 +300,7 @@ struct StreamParams {
     int early_weights;             // the first ring of weight copies may be issued before the wait for the kernel ahead
     int early_dependents;          // the launch behind this one may be set up from this kernel's start
     int next_packed;
+    int box_rows;                  // rows of the activation tensor map's box: M rounded up to a multiple of 8
     // FUSEQ (one row): the activations themselves; the kernel finds the layer scale, writes the codes of
     // its k range to shared memory (and, from the first channel tile, to q_out) and fills the control block
     const __half* x_row;           // the row's K halves
@@ -306,14 +330,15 @@ template <int MB, bool FUSEQ = false, bool WIDE = false, bool GROUPED = false>
 __global__ void __launch_bounds__(StreamCfg<MB>::kThreads, 2)
 gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const StreamParams p) {
     static_assert(!FUSEQ || MB == 1, "only a single row is quantized inside the product kernel");
-    static_assert(!WIDE || MB == 16, "clusters of 5 to 8 are for the 16-row route");
+    static_assert(!WIDE || MB >= 16, "clusters of 5 to 8 are for the MMA route");
     extern __shared__ uint8_t smem_raw[];
     using Smem = StreamSmem<MB, WIDE, GROUPED>;
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr bool kUseMma = StreamCfg<MB>::kUseMma;
     constexpr int kRows = StreamCfg<MB>::kRows;
     constexpr int kStrStages = StreamCfg<MB>::kStages;
-    constexpr int kPhases = StreamCfg<MB>::kPhases;
+    constexpr int kPhases = StreamCfg<MB>::kPhases, kRowTiles = StreamCfg<MB>::kRowTiles;
+    constexpr bool kAlias = StreamCfg<MB>::kAlias;
     constexpr int kStrConsumerWarps = StreamCfg<MB>::kConsumerWarps;
     constexpr int kStrThreads = StreamCfg<MB>::kThreads;
     cg::cluster_group cluster = cg::this_cluster();
@@ -325,7 +350,8 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
 
     // First meeting of the cluster, arrival only: by the time a CTA writes into another's shared memory
     // (after its k range) every CTA of the cluster has started. The wait comes just before those writes.
-    if (split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    // (Where the receive buffer takes the operand ring's place the meeting is after the k range instead.)
+    if (!kAlias && split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     if (threadIdx.x == 0) {
         if constexpr (kRows > 1)     // start the descriptor's fetch now; the first tile load would wait for it
             asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
@@ -347,17 +373,17 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     auto x_bytes = [&](int kb) -> uint32_t {
         if (FUSEQ) return 0u;                          // the codes are made here, not copied
         return kRows == 1 ? (uint32_t)min(kTileK, p.K - kb * kTileK)
-                          : (uint32_t)((kRows == 16 && p.M <= 8 ? 8 : kRows) * kTileK);   // the tensor map's box: 8 rows when M <= 8
+                          : (uint32_t)(p.box_rows * kTileK);
     };
     auto issue_w = [&](int kb, int s) {
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                      ::"r"(s_u32(&sm.full[s])), "r"((uint32_t)kBlockBytes + (GROUPED ? kTileN * 2u : 0u) + x_bytes(kb)) : "memory");
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(s_u32(sm.w[s])), "l"(wsrc + (size_t)kb * kBlockBytes), "r"((uint32_t)kBlockBytes),
+                     ::"r"(s_u32(sm.ring.w[s])), "l"(wsrc + (size_t)kb * kBlockBytes), "r"((uint32_t)kBlockBytes),
                        "r"(s_u32(&sm.full[s])) : "memory");
         if constexpr (GROUPED)
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(s_u32(sm.sc[s])), "l"(p.w_scales + (size_t)kb * p.Npad + tile * kTileN),
+                         ::"r"(s_u32(sm.ring.sc[s])), "l"(p.w_scales + (size_t)kb * p.Npad + tile * kTileN),
                            "r"((uint32_t)(kTileN * 2)), "r"(s_u32(&sm.full[s])) : "memory");
     };
     auto issue_x = [&](int kb, int s) {
@@ -365,12 +391,12 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
         } else if constexpr (kRows == 1) {
             // one row: its 128 codes are contiguous, a plain bulk copy needs no tensor-map fetch
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(s_u32(sm.x[s])), "l"(p.q + (size_t)kb * kTileK), "r"(x_bytes(kb)),
+                         ::"r"(s_u32(sm.ring.x[s])), "l"(p.q + (size_t)kb * kTileK), "r"(x_bytes(kb)),
                            "r"(s_u32(&sm.full[s])) : "memory");
         } else {
             asm volatile(
                 "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                ::"r"(s_u32(sm.x[s])), "l"(&x_map), "r"(kb * kTileK), "r"(0), "r"(s_u32(&sm.full[s])) : "memory");
+                ::"r"(s_u32(sm.ring.x[s])), "l"(&x_map), "r"(kb * kTileK), "r"(0), "r"(s_u32(&sm.full[s])) : "memory");
         }
     };
     // The weights do not depend on the kernel before this one: the first ring of weight blocks is on its
@@ -508,11 +534,11 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 uint4 wv[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    wv[i] = reinterpret_cast<const uint4*>(sm.w[s])[t * kTileN + quarter * 32 + 8 * i + g];
+                    wv[i] = reinterpret_cast<const uint4*>(sm.ring.w[s])[t * kTileN + quarter * 32 + 8 * i + g];
 #pragma unroll
                 for (int m = 0; m < MB; ++m) {
                     const uint4* xp = FUSEQ ? reinterpret_cast<const uint4*>(sm.xq + (size_t)(kb - kb0) * kTileK + 32 * t)
-                                            : reinterpret_cast<const uint4*>(sm.x[s] + m * kTileK + 32 * t);
+                                            : reinterpret_cast<const uint4*>(sm.ring.x[s] + m * kTileK + 32 * t);
                     const uint4 x0 = xp[0], x1 = xp[1];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -528,7 +554,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                         a = __dp4a((int)((w[3] << 4) & 0xF0F0F0F0u), (int)x1.z, a);
                         a = __dp4a((int)(w[3] & 0xF0F0F0F0u), (int)x1.w, a);
                         if constexpr (GROUPED)
-                            acc[m][i] = __float_as_int(fmaf((float)a, __half2float(sm.sc[s][quarter * 32 + 8 * i + g]),
+                            acc[m][i] = __float_as_int(fmaf((float)a, __half2float(sm.ring.sc[s][quarter * 32 + 8 * i + g]),
                                                             __int_as_float(acc[m][i])));
                         else
                             acc[m][i] = a;
@@ -557,8 +583,8 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 if (phase == ph) {
 #pragma unroll
                     for (int m = 0; m < MB; ++m) {
-                        if (ph == 0) sm.sum[m][r] = mine[m];
-                        else sm.sum[m][r] = add_sums<GROUPED>(sm.sum[m][r], mine[m]);
+                        if (ph == 0) sm.sums.sum[m][r] = mine[m];
+                        else sm.sums.sum[m][r] = add_sums<GROUPED>(sm.sums.sum[m][r], mine[m]);
                     }
                 }
             }
@@ -566,23 +592,22 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             // Warp-level int8 MMA, D[16 rows x 8 channels] += A[16 x 32 k] * B[32 k x 8 channels].
             // Fragment owner: g = lane / 4 (row g and g+8 of A and D; channel g of B),
             // t = lane % 4 (k bytes 4t..4t+3 and 16+4t..; D columns 2t, 2t+1).
-            // Rows 8..15 are not read when M <= 8. (Splitting a block among the four warps of a phase into channel
+            // Rows 8..15 of a 16-row tile are not read when M ends before them, and a tile behind M is left out.
+            // (Splitting a block among the four warps of a phase into channel
             // halves x k halves instead of channel quarters, so that a warp reads half of the activation tile,
             // measured the same within 0.2 us either way.)
             const int g = lane >> 2, t = lane & 3;
-            const bool upper = p.M > 8;
-            int acc[4][4];
+            int acc[kRowTiles][4][4];
+            [[maybe_unused]] float fsum[kRowTiles][4][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[i][c] = 0;
-            [[maybe_unused]] float fsum[4][4];
-            if constexpr (GROUPED) {
+            for (int rt = 0; rt < kRowTiles; ++rt)
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) fsum[i][c] = 0.0f;
-            }
+                    for (int c = 0; c < 4; ++c) {
+                        acc[rt][i][c] = 0;
+                        if constexpr (GROUPED) fsum[rt][i][c] = 0.0f;
+                    }
             for (int kb = kb0 + phase; kb < kb1; kb += kPhases) {
                 const uint32_t it = (uint32_t)(kb - kb0);
                 const int s = (int)(it % kStrStages);
@@ -595,10 +620,6 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                     // word and eight consecutive activation bytes (one 8-byte load per row).
                     // activation rows: 128 bytes, 16-byte chunks XOR-swizzled by row % 8
                     const int x_off = (((2 * j + (t >> 1)) ^ g) << 4) + 8 * (t & 1);
-                    const uint2 xa = *reinterpret_cast<const uint2*>(sm.x[s] + g * kTileK + x_off);
-                    uint2 xb = make_uint2(0u, 0u);
-                    if (upper) xb = *reinterpret_cast<const uint2*>(sm.x[s] + (g + 8) * kTileK + x_off);
-                    const uint32_t a0 = xa.x, a1 = xb.x, a2 = xa.y, a3 = xb.y;
                     // Weight fragments of the four channel passes in one instruction: the 32 units (16 bytes each)
                     // of this chunk and channel quarter are four 8 x 8 matrices of 16-bit elements, one per pass;
                     // lane l gives the address of unit l, and lane (g, t) receives word t of channel 8i + g for
@@ -606,27 +627,38 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                     uint32_t pw[4];
                     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(pw[0]), "=r"(pw[1]), "=r"(pw[2]), "=r"(pw[3])
-                                 : "r"(s_u32(sm.w[s] + (size_t)(j * kTileN + quarter * 32 + lane) * 16)) : "memory");
+                                 : "r"(s_u32(sm.ring.w[s] + (size_t)(j * kTileN + quarter * 32 + lane) * 16)) : "memory");
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint32_t b0 = (pw[i] << 4) & 0xF0F0F0F0u;
-                        const uint32_t b1 = pw[i] & 0xF0F0F0F0u;
-                        asm volatile(
-                            "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-                            "{%8, %9}, {%0, %1, %2, %3};"
-                            : "+r"(acc[i][0]), "+r"(acc[i][1]), "+r"(acc[i][2]), "+r"(acc[i][3])
-                            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                    for (int rt = 0; rt < kRowTiles; ++rt) {
+                        const int row = 16 * rt;
+                        if (rt > 0 && row >= p.M) break;
+                        const uint2 xa = *reinterpret_cast<const uint2*>(sm.ring.x[s] + (row + g) * kTileK + x_off);
+                        uint2 xb = make_uint2(0u, 0u);
+                        if (p.M > row + 8) xb = *reinterpret_cast<const uint2*>(sm.ring.x[s] + (row + g + 8) * kTileK + x_off);
+                        const uint32_t a0 = xa.x, a1 = xb.x, a2 = xa.y, a3 = xb.y;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t b0 = (pw[i] << 4) & 0xF0F0F0F0u;
+                            const uint32_t b1 = pw[i] & 0xF0F0F0F0u;
+                            asm volatile(
+                                "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+                                "{%8, %9}, {%0, %1, %2, %3};"
+                                : "+r"(acc[rt][i][0]), "+r"(acc[rt][i][1]), "+r"(acc[rt][i][2]), "+r"(acc[rt][i][3])
+                                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                        }
                     }
                 }
                 if constexpr (GROUPED) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const float2 sg = __half22float2(*reinterpret_cast<const __half2*>(&sm.sc[s][quarter * 32 + 8 * i + 2 * t]));
+                        const float2 sg = __half22float2(*reinterpret_cast<const __half2*>(&sm.ring.sc[s][quarter * 32 + 8 * i + 2 * t]));
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            fsum[i][c] = fmaf((float)acc[i][c], (c & 1) ? sg.y : sg.x, fsum[i][c]);
-                            acc[i][c] = 0;
-                        }
+                        for (int rt = 0; rt < kRowTiles; ++rt)
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                fsum[rt][i][c] = fmaf((float)acc[rt][i][c], (c & 1) ? sg.y : sg.x, fsum[rt][i][c]);
+                                acc[rt][i][c] = 0;
+                            }
                     }
                 }
                 __syncwarp();
@@ -637,17 +669,20 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             // owns an element in each of them: the first stores, the others add).
 #pragma unroll
             for (int ph = 0; ph < kPhases; ++ph) {
-                if (ph > 0) asm volatile("bar.sync 1, %0;" ::"n"(kStrConsumerWarps * 32) : "memory");
+                // (where the sums take the ring's place, every consumer warp must have read its last block)
+                if (kAlias || ph > 0) asm volatile("bar.sync 1, %0;" ::"n"(kStrConsumerWarps * 32) : "memory");
                 if (phase == ph) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                    for (int rt = 0; rt < kRowTiles; ++rt)
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            int& dst = sm.sum[g + 8 * (c >> 1)][quarter * 32 + 8 * i + 2 * t + (c & 1)];
-                            const int own = GROUPED ? __float_as_int(fsum[i][c]) : acc[i][c];
-                            if (ph == 0) dst = own;
-                            else dst = add_sums<GROUPED>(dst, own);
-                        }
+                        for (int i = 0; i < 4; ++i)
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                int& dst = sm.sums.sum[16 * rt + g + 8 * (c >> 1)][quarter * 32 + 8 * i + 2 * t + (c & 1)];
+                                const int own = GROUPED ? __float_as_int(fsum[rt][i][c]) : acc[rt][i][c];
+                                if (ph == 0) dst = own;
+                                else dst = add_sums<GROUPED>(dst, own);
+                            }
                 }
             }
         }
@@ -684,8 +719,14 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     }
     const int rows = p.M < kRows ? p.M : kRows;
     if (split > 1) {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // everybody has started (arrival at the top)
-        __syncthreads();                                      // this CTA's sums are complete
+        if (kAlias) {
+            __syncthreads();                                  // this CTA's sums are complete, its ring is idle
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // ... and so are the others'
+        } else {
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // everybody has started (arrival at the top)
+            __syncthreads();                                  // this CTA's sums are complete
+        }
         if (ft >= 0) {
             // four consecutive channels at a time (16-byte remote stores) go to the CTA that owns them
             for (int e = ft; e < rows * (kTileN / 4); e += kStrConsumerWarps * 32) {
@@ -693,8 +734,8 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 const int owner = wide ? (((g4 + 1) * split + 31) >> 5) - 1 : ch >> cw_log;
                 const int at = wide ? ch - 4 * ((32 * owner) / split) : ch & (cw - 1);   // place inside the owner's slice
                 if (owner != rank)
-                    *reinterpret_cast<int4*>(cluster.map_shared_rank(&sm.recv[0][0], owner) + m * Smem::kRecvStride + rank * cw + at) =
-                        *reinterpret_cast<const int4*>(&sm.sum[m][ch]);
+                    *reinterpret_cast<int4*>(cluster.map_shared_rank(&sm.sums.recv[0][0], owner) + m * Smem::kRecvStride + (rank - (rank > owner ? 1 : 0)) * cw + at) =
+                        *reinterpret_cast<const int4*>(&sm.sums.sum[m][ch]);
             }
         }
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -707,21 +748,22 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
         // branches around them (rows that do not exist read the last row of the buffer and are dropped):
         // taken one after the other, each behind its own test, they were the longest part of the finish at
         // 16 rows.
-        constexpr int kIt = (kRows + kPhases - 1) / kPhases;      // a pass of the consumer threads covers at least kPhases rows
+        constexpr int kPass = kStrConsumerWarps * 32 / (WIDE ? 32 : kTileN);     // rows that a pass covers at least
+        constexpr int kIt = (kRows + kPass - 1) / kPass;
         const int stride = (kStrConsumerWarps * 32) >> cw_log, m0 = ft >> cw_log;
         int av[kIt];
 #pragma unroll
-        for (int i = 0; i < kIt; ++i) av[i] = i * stride < kRows ? sm.sum[min(m0 + i * stride, kRows - 1)][out_r] : 0;
+        for (int i = 0; i < kIt; ++i) av[i] = i * stride < kRows ? sm.sums.sum[min(m0 + i * stride, kRows - 1)][out_r] : 0;
 #pragma unroll
         for (int k = 1; k < (WIDE ? 8 : 4); ++k) {
             if (k < split) {
                 int c = rank + k;                                             // the k-th other CTA's slot
                 if (c >= split) c -= split;
-                const int col = c * cw + rc;
+                const int col = (c - (c > rank ? 1 : 0)) * cw + rc;
 #pragma unroll
                 for (int i = 0; i < kIt; ++i)
                     if (i * stride < kRows)                               // the same test in every thread
-                        av[i] = add_sums<GROUPED>(av[i], sm.recv[min(m0 + i * stride, kRows - 1)][col]);
+                        av[i] = add_sums<GROUPED>(av[i], sm.sums.recv[min(m0 + i * stride, kRows - 1)][col]);
             }
         }
         auto value = [&](int a) { return GROUPED ? __int_as_float(a) : (float)(a >> 4); };     // integer sums carry a factor 16
@@ -776,8 +818,9 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
     const cuuint64_t strides[1] = {(cuuint64_t)a.K};
-    // 16-row route: rows 8..15 are neither copied nor read when M <= 8
-    const cuuint32_t box[2] = {128u, (cuuint32_t)(StreamCfg<MB>::kRows == 16 && a.M <= 8 ? 8 : StreamCfg<MB>::kRows)};
+    // MMA route: M rounded up to a multiple of 8 rows; what lies behind is neither copied nor read
+    const int box_rows = StreamCfg<MB>::kUseMma ? round_up(a.M, 8) : StreamCfg<MB>::kRows;
+    const cuuint32_t box[2] = {128u, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1u, 1u};
     const CUresult r = reinterpret_cast<EncodeTiledFn>(dev.encode_tiled)(
         &map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t*>(a.q), dims, strides, box, estr,
@@ -790,6 +833,7 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     p.q = a.q;
     p.clear_status = a.after_quantize ? 0 : 1;
     p.next_packed = a.next_packed ? 1 : 0;
+    p.box_rows = box_rows;
     p.w_packed = a.w_packed; p.w_scales = a.w_scales; p.scale_exp = a.scale_exp;
     p.y = a.y; p.acc_dump = a.acc_dump; p.ctl = a.ctl; p.chan_offset = a.chan_offset;
     p.q_next = a.q_next;
@@ -828,7 +872,7 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
 // K = 13824 12.5 / 13.2 -> 9.8 / 10.4 us at M = 4 / 16, K = 5120 6.9 / 7.3 -> 6.0 / 6.5 us; a single row
 // loses with clusters of 8 (N = 4096, K = 5120: 5.1 -> 6.2 us). Plain and chained calls take the same cluster
 // (with per-group scales its size sets the order of the fp32 sums). Returns the cluster size (5 to 8), or 0 for the usual 1, 2 or 4.
-template <bool GROUPED>
+template <int MB, bool GROUPED>
 int wide_split_for(const GemmArgs& a, const DeviceInfo& dev) {
     const int tiles = round_up(a.N, kTileN) / kTileN, KB = k_blocks(a.K);
     if (decode_split(tiles, KB, dev.sm_count) != 4) return 0;
@@ -839,14 +883,14 @@ int wide_split_for(const GemmArgs& a, const DeviceInfo& dev) {
         if (KB / s < 5) continue;
         int known = fits[dev.device][s].load(std::memory_order_relaxed);
         if (known == 0) {
-            using Smem = StreamSmem<16, true, GROUPED>;
+            using Smem = StreamSmem<MB, true, GROUPED>;
             const size_t smem_bytes = sizeof(Smem) + 1024;
             static SmemOptIn opt_in;
             int n = 0;
-            if (opt_in.ensure(gemm_decode_stream_kernel<16, false, true, GROUPED>, dev.device, smem_bytes) == cudaSuccess) {
+            if (opt_in.ensure(gemm_decode_stream_kernel<MB, false, true, GROUPED>, dev.device, smem_bytes) == cudaSuccess) {
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(s, tiles, 1);
-                cfg.blockDim = dim3(StreamCfg<16>::kThreads);
+                cfg.blockDim = dim3(StreamCfg<MB>::kThreads);
                 cfg.dynamicSmemBytes = smem_bytes;
                 cudaLaunchAttribute attr[1];
                 attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -855,7 +899,7 @@ int wide_split_for(const GemmArgs& a, const DeviceInfo& dev) {
                 attr[0].val.clusterDim.z = 1;
                 cfg.attrs = attr;
                 cfg.numAttrs = 1;
-                if (cudaOccupancyMaxActiveClusters(&n, gemm_decode_stream_kernel<16, false, true, GROUPED>, &cfg) != cudaSuccess) {
+                if (cudaOccupancyMaxActiveClusters(&n, gemm_decode_stream_kernel<MB, false, true, GROUPED>, &cfg) != cudaSuccess) {
                     (void)cudaGetLastError();
                     n = 0;
                 }
@@ -897,23 +941,28 @@ bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, int sm_
 }
 
 namespace {
+template <int MB, bool GROUPED>
+cudaError_t launch_stream_mma(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+    if (const int ws = wide_split_for<MB, GROUPED>(a, dev)) return launch_stream<MB, false, true, GROUPED>(a, dev, stream, ws);
+    return launch_stream<MB, false, false, GROUPED>(a, dev, stream);
+}
 template <bool GROUPED>
 cudaError_t launch_stream_rows(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    // one row: dp4a; 2..16 rows: the warp MMA on a 16-row tile (fewer instructions per weight
+    // one row: dp4a; from 2 rows on the warp MMA on 16-row tiles (fewer instructions per weight
     // chunk than dp4a from two rows on; measured faster at M = 4: 7.5 / 11.1 / 13.3 us against
     // 8.1 / 12.8 / 15.2 us on the three 13B shapes)
     if (a.M <= 1 && a.fuse_x) return launch_stream<1, true, false, GROUPED>(a, dev, stream);
     if (a.M <= 1) return launch_stream<1, false, false, GROUPED>(a, dev, stream);
-    if (const int ws = wide_split_for<GROUPED>(a, dev)) return launch_stream<16, false, true, GROUPED>(a, dev, stream, ws);
-    return launch_stream<16, false, false, GROUPED>(a, dev, stream);
+    if (a.M <= 16) return launch_stream_mma<16, GROUPED>(a, dev, stream);
+    return launch_stream_mma<32, GROUPED>(a, dev, stream);
 }
 }  // namespace
 
 cudaError_t launch_gemm_decode(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    if (a.M <= 16 && !a.group) return launch_stream_rows<false>(a, dev, stream);
+    if (a.M <= kFewRows && !a.group) return launch_stream_rows<false>(a, dev, stream);
     // The streaming kernel never holds a group's whole integer sum in one place (a single row's lanes scale their
     // parts of it), so the dump of per-group sums takes the general kernel. Its scales ride in 16-byte copies.
-    if (a.M <= 16 && !a.acc_dump && (reinterpret_cast<uintptr_t>(a.w_scales) & 15u) == 0)
+    if (a.M <= kFewRows && !a.acc_dump && (reinterpret_cast<uintptr_t>(a.w_scales) & 15u) == 0)
         return launch_stream_rows<true>(a, dev, stream);
     if (a.M <= 1) return launch_mb<1>(a, stream);
     if (a.M <= 2) return launch_mb<2>(a, stream);
