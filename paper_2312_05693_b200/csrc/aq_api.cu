@@ -39,12 +39,12 @@ struct Workspace {
     int8_t* codes;
     void* scratch;
     size_t scratch_bytes;
-    float* chan_offset;
     float* split_scratch;
     size_t split_bytes;
 };
 
-// [control block][codes M*K][kernel scratch, M bytes][per-channel offsets of the zero-point variant, N floats]
+// [control block][codes M*K][kernel scratch, M bytes][4 N bytes that earlier versions held per-channel terms in: kept,
+// the size is part of the interface]
 // [fp32 partial outputs of tiles that two CTAs share in the tensor kernel, sized for a 148-SM B200; a
 // device that would need more simply shares no tile]
 constexpr int kPlannedSmCount = 148;
@@ -64,7 +64,6 @@ Workspace carve(void* ws, int M, int K, int N, size_t total_bytes) {
     w.codes = reinterpret_cast<int8_t*>(b + sizeof(Control));
     w.scratch = b + sizeof(Control) + up256((size_t)M * K);
     w.scratch_bytes = up256((size_t)M);
-    w.chan_offset = reinterpret_cast<float*>(b + sizeof(Control) + up256((size_t)M * K) + up256((size_t)M));
     const size_t used = workspace_min_bytes(M, K, N);
     w.split_scratch = reinterpret_cast<float*>(b + used);
     w.split_bytes = total_bytes > used ? total_bytes - used : 0;
@@ -99,13 +98,7 @@ cudaError_t quantize_dispatch(aq_handle_t h, const __half* xh, int M, int K, con
         // the control block
         return launch_quantize_small(xh, M, K, row_idx, bits, scale_mode, clip_shift_or_exp, ctl, q, scale_exp_out,
                                      stream, alpha, k_max, h->weights_stable != 0);
-    const cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(Control), stream);
-    if (e != cudaSuccess) return e;
-    if (scale_mode == AQ_SCALE_DYNAMIC)
-        return launch_quantize_fused(xh, M, K, row_idx, bits, clip_shift_or_exp, ctl, q, scale_exp_out, h->dev, stream,
-                                     alpha, k_max);
-    return launch_quantize(xh, M, K, row_idx, bits, scale_mode, clip_shift_or_exp, ctl, q, scale_exp_out, h->dev,
-                           stream, alpha, k_max);
+    return launch_quantize(xh, M, K, row_idx, bits, scale_mode, clip_shift_or_exp, ctl, q, scale_exp_out, stream, alpha, k_max);
 }
 
 bool trip_args_ok(const uint8_t* alpha, int k_max) { return alpha && k_max >= 0 && k_max <= 4; }
@@ -141,12 +134,9 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
                       (!group || aligned(w_scales, 16));
     if (fuse) {
     } else if (w_offsets) {
-        // zero-point variant: min / max, then e, zp and codes; then the per-channel term -(zp - 2^(b-1)) * r[n]
+        // zero-point variant: min / max, then e, zp and codes; the product adds the term -(zp - 2^(b-1)) * r[n]
         if (!aligned(w_offsets, 4)) return AQ_ERR_ALIGNMENT;
-        e = cudaMemsetAsync(w.ctl, 0, sizeof(Control), stream);
-        if (e == cudaSuccess)
-            e = launch_quantize_asym(xh, M, K, row_idx, bits, w.ctl, w.codes, nullptr, nullptr, h->dev, stream);
-        if (e == cudaSuccess) e = launch_chan_offsets(w_offsets, N, bits, w.ctl, w.chan_offset, stream);
+        e = launch_quantize_asym(xh, M, K, row_idx, bits, w.ctl, w.codes, nullptr, nullptr, stream);
     } else {
         e = quantize_dispatch(h, xh, M, K, row_idx, bits, scale_mode, clip_shift_or_exp, w.ctl, w.codes, nullptr, alpha,
                               k_max, stream);
@@ -161,7 +151,8 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     g.acc_dump = acc_dump;
     g.ctl = w.ctl; g.scratch = w.scratch; g.scratch_bytes = w.scratch_bytes;
     g.split_scratch = w.split_scratch; g.split_bytes = w.split_bytes;
-    g.chan_offset = w_offsets ? w.chan_offset : nullptr;
+    g.chan_offset = w_offsets;
+    g.zp_mid = 1 << (bits - 1);
     g.q_next = q_next; g.next_bits = next_bits; g.next_exp = next_exp;
     g.next_packed = next_packed;
     g.after_quantize = !fuse;
@@ -504,10 +495,8 @@ int aq_quantize_act_asym(aq_handle_t h, const void* x_fp16, int M, int K, int bi
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     Control* ctl = static_cast<Control*>(workspace);
-    cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(Control), stream);
-    if (e == cudaSuccess)
-        e = launch_quantize_asym(static_cast<const __half*>(x_fp16), M, K, row_idx, bits, ctl, q, scale_exp_out,
-                                 zero_point_out, h->dev, stream);
+    const cudaError_t e = launch_quantize_asym(static_cast<const __half*>(x_fp16), M, K, row_idx, bits, ctl, q, scale_exp_out,
+                                               zero_point_out, stream);
     return e == cudaSuccess ? AQ_OK : cuda_fail(h, e);
 }
 

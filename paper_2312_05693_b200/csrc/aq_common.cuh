@@ -46,14 +46,15 @@ __host__ __device__ inline size_t packed_unit_offset(int KB, int nt, int kb, int
 // [kernel scratch].
 // ---------------------------------------------------------------------------------------
 struct Control {
-    unsigned int absmax_bits;   // fp16 bit pattern of max|x| (atomicMax target), cleared per call
+    unsigned int absmax_bits;   // fp16 bit pattern of max|x|
     int scale_exp;              // layer exponent e
     unsigned int status;        // non-zero: a bounded wait gave up
-    unsigned int counter;       // scratch counter
-    unsigned int min_key, max_key;   // zero-point variant: order-preserving keys of min(x), max(x)
+    unsigned int unused[3];
     int zero_point;             // zero-point variant: zp of Eq. 7
-    unsigned int split_flags[57];   // tensor kernel: one bit per (shared tile, epilogue warp), "first half arrived"
-    static constexpr int kMaxSplitTiles = 57 * 32 / 12;   // up to twelve epilogue warps per tile
+    static constexpr int kRangeWords = 29, kSplitWords = 28;
+    unsigned int range[kRangeWords];        // quantize: per cluster, largest magnitudes (fp16 bits) above and below 0
+    unsigned int split_flags[kSplitWords];  // tensor kernel: one bit per (shared tile, epilogue warp), "first half arrived"
+    static constexpr int kMaxSplitTiles = kSplitWords * 32 / 12;   // up to twelve epilogue warps per tile
 };
 static_assert(sizeof(Control) == 256, "control block is 256 bytes");
 
@@ -101,6 +102,22 @@ struct SmemOptIn {
     }
 };
 
+// A launch that may be set up while the kernel ahead of it on the stream drains; the kernels launched this way touch no
+// memory before that kernel has completed.
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), size_t grid, int threads, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned int)grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 cudaError_t launch_pack_w4(const __half* w, int N, int K, int group, uint8_t* packed, __half* scales,
                            cudaStream_t stream);
 cudaError_t launch_unpack_w4(const uint8_t* packed, int N, int K, int8_t* codes, cudaStream_t stream);
@@ -109,10 +126,10 @@ cudaError_t launch_unpack_w4(const uint8_t* packed, int N, int K, int8_t* codes,
 cudaError_t launch_act4_pack(const int8_t* q, size_t count, uint8_t* out, cudaStream_t stream);
 cudaError_t launch_act4_unpack(const uint8_t* packed, size_t count, int8_t* q, cudaStream_t stream);
 
+// Scale (unless given) and codes; fills the control block. alpha / k_max: TRIP factors, see below.
 cudaError_t launch_quantize(const __half* x, int M, int K, const int32_t* row_idx, int bits,
                             int scale_mode, int clip_shift_or_exp, Control* ctl, int8_t* q,
-                            int32_t* scale_exp_out, const DeviceInfo& dev, cudaStream_t stream,
-                            const uint8_t* alpha = nullptr, int k_max = 0);
+                            int32_t* scale_exp_out, cudaStream_t stream, const uint8_t* alpha = nullptr, int k_max = 0);
 
 // Activations of at most 262144 elements: one kernel that also initialises the control block.
 bool quantize_small_fits(int M, int K);
@@ -121,11 +138,6 @@ cudaError_t launch_quantize_small(const __half* x, int M, int K, const int32_t* 
                                   cudaStream_t stream, const uint8_t* alpha = nullptr, int k_max = 0,
                                   bool early_dependents = false);
 
-// Dynamic scale, any size: one cooperative kernel (absmax, exponent, codes). The control block must
-// have been cleared (absmax_bits, counter) on the same stream before.
-cudaError_t launch_quantize_fused(const __half* x, int M, int K, const int32_t* row_idx, int bits, int clip_shift,
-                                  Control* ctl, int8_t* q, int32_t* scale_exp_out, const DeviceInfo& dev,
-                                  cudaStream_t stream, const uint8_t* alpha = nullptr, int k_max = 0);
 // TRIP factors (Eq. 5-8): `alpha` above is NULL or K bytes (16-byte aligned), one factor 0..k_max per
 // input channel: channel k is quantized with the step 2^(e + alpha_k), its code stored shifted left by
 // alpha_k, and the dynamic exponent is lowered by k_max (Eq. 6). The search of Eq. 8:
@@ -133,17 +145,13 @@ cudaError_t launch_trip_calibrate(const __half* x, int M, int K, const int32_t* 
                                   Control* ctl, uint8_t* alpha_out, int32_t* scale_exp_out, const DeviceInfo& dev,
                                   cudaStream_t stream);
 
-// Zero-point variant (Eq. 2, Eq. 5-7 with alpha = 0 and a power-of-two scale): one cooperative kernel
-// finds minimum and maximum, then e, zp and the codes, stored as q - 2^(b-1) in int8. The control block
-// must have been cleared.
+// Zero-point variant (Eq. 2, Eq. 5-7 with alpha = 0 and a power-of-two scale): minimum and maximum, then e, zp and the
+// codes, stored as q - 2^(b-1) in int8; fills the control block.
 cudaError_t launch_quantize_asym(const __half* x, int M, int K, const int32_t* row_idx, int bits, Control* ctl,
-                                 int8_t* q, int32_t* scale_exp_out, int32_t* zero_point_out, const DeviceInfo& dev,
-                                 cudaStream_t stream);
+                                 int8_t* q, int32_t* scale_exp_out, int32_t* zero_point_out, cudaStream_t stream);
 // r[n] = sum_g s_w[n,g] * sum_{k in g} c[n,k], from the packed weights (float [N]).
 cudaError_t launch_weight_offsets(const uint8_t* packed, const __half* scales, int N, int K, int group, float* r,
                                   cudaStream_t stream);
-// off[n] = -(zp - 2^(b-1)) * r[n] with zp from the control block.
-cudaError_t launch_chan_offsets(const float* r, int N, int bits, const Control* ctl, float* off, cudaStream_t stream);
 
 // Log2 codes of Eq. 3 (two kernels: layer maximum, codes) and attention x value on them (aq_attn.cu).
 cudaError_t launch_log2_quantize(const __half* x, long long count, int bits, Control* ctl, int8_t* codes,
@@ -174,7 +182,10 @@ struct GemmArgs {
     __half* y;              // [M][N]
     int32_t* acc_dump;      // NULL or [M][N][G]
     Control* ctl;
-    const float* chan_offset = nullptr;   // NULL or [N]: added to sum_g s*acc before the 2^e factor (zero-point term)
+    // Zero-point term: NULL or r [N]; -(zp - zp_mid) * r[n] is added to sum_g s*acc before the 2^e factor, zp from the
+    // control block.
+    const float* chan_offset = nullptr;
+    int zp_mid = 0;
     // Chaining: when q_next is given the kernels write, instead of y, the next layer's activation codes
     // [M][N] int8: clip(round(y16 / 2^next_exp), -2^(b-1), 2^(b-1)-1), y16 the fp16 value y would have held.
     int8_t* q_next = nullptr;
@@ -186,8 +197,8 @@ struct GemmArgs {
     // status word is already initialised, and the product kernels may be set up (the few-row streaming
     // kernel also starts streaming weights) while that kernel still runs (programmatic dependent launch;
     // they wait for that grid before they touch the codes). Weights cannot be in flight then: the quantize
-    // kernels allow the dependent launch only once everything before them on the stream has completed (the
-    // cooperative one is launched normally, the small one signals after its own wait for the kernel ahead).
+    // kernels allow the dependent launch only once everything before them on the stream has completed (they
+    // signal after their own wait for the kernel ahead).
     bool after_quantize = false;
     // The caller's promise (aq_set_weights_stable) that nothing in flight on the stream writes the packed
     // weights or their scales: the few-row kernel then allows the launch behind it at its very start and puts
@@ -204,6 +215,9 @@ struct GemmArgs {
     void* scratch;          // beyond control block + codes
     size_t scratch_bytes;
 };
+// The factor of the per-channel zero-point term (see GemmArgs::chan_offset).
+__device__ __forceinline__ float offset_factor(const Control* ctl, int zp_mid) { return -(float)(ctl->zero_point - zp_mid); }
+
 // Small accessors for code outside aq_api.cu that is handed a handle.
 int handle_device(aq_handle_t h);
 void handle_record_cuda_error(aq_handle_t h, cudaError_t e);

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kDecThreads)
 gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
                    const uint8_t* __restrict__ w_packed, const __half* __restrict__ w_scales,
                    const int32_t* __restrict__ scale_exp, __half* __restrict__ y,
-                   int32_t* __restrict__ acc_dump, Control* __restrict__ ctl, const float* __restrict__ chan_offset,
+                   int32_t* __restrict__ acc_dump, Control* __restrict__ ctl, const float* __restrict__ chan_offset, int zp_mid,
                    int8_t* __restrict__ q_next, float next_inv, float next_lo, float next_hi, int clear_status,
                    int next_packed) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -155,7 +155,7 @@ gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
     for (int m = warp; m < MB; m += kDecWarps) {
         if (m0 + m >= M) continue;                               // the same for the whole warp
         const bool n_ok = n < N;
-        const float off = chan_offset && n_ok ? chan_offset[n] : 0.0f;
+        const float off = chan_offset && n_ok ? __fmul_rn(offset_factor(ctl, zp_mid), chan_offset[n]) : 0.0f;
         float out;
         if (GROUPED) {
             float s = 0.0f;
@@ -294,6 +294,7 @@ struct StreamParams {
     int32_t* acc_dump;
     Control* ctl;
     const float* chan_offset;
+    int zp_mid;
     int8_t* q_next;
     float next_inv, next_lo, next_hi;
     int clear_status;
@@ -473,8 +474,8 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             }
         }
         if (tile == 0 && rank == 0) {
-            if (threadIdx.x == 0) { p.ctl->scale_exp = e; p.ctl->status = 0; p.ctl->counter = 0; }
-            if (threadIdx.x < 57) p.ctl->split_flags[threadIdx.x] = 0;
+            if (threadIdx.x == 0) { p.ctl->scale_exp = e; p.ctl->status = 0; }
+            if (threadIdx.x < Control::kSplitWords) p.ctl->split_flags[threadIdx.x] = 0;
         }
         const float lo = -(float)(1 << (p.bits - 1)), hi = (float)((1 << (p.bits - 1)) - 1);
         const int v0 = kb0 * (kTileK / 8), v1 = min(kb1 * (kTileK / 8), p.K / 8);       // 8-element vectors of this k range
@@ -715,7 +716,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     if (mine) {
         const float pe = __int_as_float((127 + (FUSEQ ? fused_exp : *p.scale_exp)) << 23);
         sc = GROUPED ? 0.0625f * pe : __half2float(p.w_scales[out_n]) * pe;     // the fp32 sums carry a factor 16
-        if (p.chan_offset) off = p.chan_offset[out_n] * pe;
+        if (p.chan_offset) off = __fmul_rn(offset_factor(p.ctl, p.zp_mid), p.chan_offset[out_n]) * pe;
     }
     const int rows = p.M < kRows ? p.M : kRows;
     if (split > 1) {
@@ -835,7 +836,7 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     p.next_packed = a.next_packed ? 1 : 0;
     p.box_rows = box_rows;
     p.w_packed = a.w_packed; p.w_scales = a.w_scales; p.scale_exp = a.scale_exp;
-    p.y = a.y; p.acc_dump = a.acc_dump; p.ctl = a.ctl; p.chan_offset = a.chan_offset;
+    p.y = a.y; p.acc_dump = a.acc_dump; p.ctl = a.ctl; p.chan_offset = a.chan_offset; p.zp_mid = a.zp_mid;
     p.q_next = a.q_next;
     p.next_inv = ldexpf(1.0f, -a.next_exp);
     p.next_lo = -(float)(1 << (a.next_bits - 1));
@@ -918,12 +919,12 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
     dim3 grid(Npad / 32, (a.M + MB - 1) / MB);
     if (a.group)
         gemm_decode_kernel<MB, true><<<grid, kDecThreads, 0, stream>>>(
-            a.q, a.M, a.K, a.N, Npad, a.w_packed, a.w_scales, a.scale_exp, a.y, a.acc_dump, a.ctl, a.chan_offset,
+            a.q, a.M, a.K, a.N, Npad, a.w_packed, a.w_scales, a.scale_exp, a.y, a.acc_dump, a.ctl, a.chan_offset, a.zp_mid,
             a.q_next, ldexpf(1.0f, -a.next_exp), -(float)(1 << (a.next_bits - 1)), (float)((1 << (a.next_bits - 1)) - 1),
             a.after_quantize ? 0 : 1, a.next_packed ? 1 : 0);
     else
         gemm_decode_kernel<MB, false><<<grid, kDecThreads, 0, stream>>>(
-            a.q, a.M, a.K, a.N, Npad, a.w_packed, a.w_scales, a.scale_exp, a.y, a.acc_dump, a.ctl, a.chan_offset,
+            a.q, a.M, a.K, a.N, Npad, a.w_packed, a.w_scales, a.scale_exp, a.y, a.acc_dump, a.ctl, a.chan_offset, a.zp_mid,
             a.q_next, ldexpf(1.0f, -a.next_exp), -(float)(1 << (a.next_bits - 1)), (float)((1 << (a.next_bits - 1)) - 1),
             a.after_quantize ? 0 : 1, a.next_packed ? 1 : 0);
     return cudaGetLastError();

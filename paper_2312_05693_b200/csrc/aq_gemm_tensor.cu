@@ -95,7 +95,8 @@ struct TensorParams {
     __half* y;
     int32_t* acc_dump;
     Control* ctl;
-    const float* chan_offset;      // NULL or [N]: per-channel term added before the 2^e factor
+    const float* chan_offset;      // NULL or [N]: per-channel term added before the 2^e factor, times offset_factor
+    int zp_mid;
     int split_base;                // SPLIT kernels: CTAs 2j and 2j+1 share tile split_base + j, half of K each
     float* split_scratch;          // [shared tile][half][epilogue warp][column][lane] fp32 partial outputs
     int8_t* q_next;                // chaining: the next layer's codes [M][N] are written instead of y
@@ -367,6 +368,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         const int col0 = half * kColsPerEpiWarp;
         asm volatile("griddepcontrol.wait;" ::: "memory");               // see the activation producer
         const float pe = __int_as_float((127 + *p.scale_exp) << 23);     // 2^e
+        [[maybe_unused]] const float off_factor = OFFSET ? offset_factor(p.ctl, p.zp_mid) : 0.0f;
         [[maybe_unused]] const int G = GROUPED ? KB : 1;
         uint32_t unit = 0;
         [[maybe_unused]] uint32_t g_a = 0, g_ph = 0, g_slot = 0;   // per-group mode: accumulator stage, its parity, scale slot
@@ -381,7 +383,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 const uint32_t aph = (unit / kNumAcc) & 1u;
                 const float sc = __half2float(p.w_scales[n]) * 0.0625f * pe;   // sums carry a factor 16
                 [[maybe_unused]] float off_pe = 0.0f;
-                if constexpr (OFFSET) off_pe = (n_ok ? p.chan_offset[n] : 0.0f) * pe;
+                if constexpr (OFFSET) off_pe = (n_ok ? __fmul_rn(off_factor, p.chan_offset[n]) : 0.0f) * pe;
                 if (!mbar_wait_warp(&sm.acc_full[a], aph, abort_flag, 8u)) goto role_done;
                 tc_fence_after();
                 // all of this warp's sums go to registers and the accumulator returns to the MMA at once,
@@ -510,7 +512,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                     }
                 }
                 if constexpr (OFFSET) {                                  // read after the k loop
-                    const float off_n = n_ok ? p.chan_offset[n] : 0.0f;
+                    const float off_n = n_ok ? __fmul_rn(off_factor, p.chan_offset[n]) : 0.0f;
 #pragma unroll
                     for (int c = 0; c < kColsPerEpiWarp; ++c) fsum[c] += off_n;
                 }
@@ -756,7 +758,7 @@ cudaError_t launch_off(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t st
     p.n_tiles_m = (a.M + BM - 1) / BM;
     p.n_tiles = p.n_tiles_m * (p.Npad / kTileN);
     p.w_packed = a.w_packed; p.w_scales = a.w_scales; p.scale_exp = a.scale_exp;
-    p.y = a.y; p.acc_dump = a.acc_dump; p.ctl = a.ctl; p.chan_offset = a.chan_offset;
+    p.y = a.y; p.acc_dump = a.acc_dump; p.ctl = a.ctl; p.chan_offset = a.chan_offset; p.zp_mid = a.zp_mid;
     p.q_next = a.q_next;
     p.next_inv = ldexpf(1.0f, -a.next_exp);
     p.next_lo = -(float)(1 << (a.next_bits - 1));

@@ -60,7 +60,8 @@ struct WParams {
     __half* y;
     int32_t* acc_dump;
     Control* ctl;
-    const float* chan_offset;
+    const float* chan_offset;      // NULL or [N]: per-channel term, times offset_factor
+    int zp_mid;
     int8_t* q_next;
     float next_inv, next_lo, next_hi;
     int next_packed;
@@ -237,6 +238,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         const int col0 = chalf * kCols;
         asm volatile("griddepcontrol.wait;" ::: "memory");               // see the activation producer
         const float pe = __int_as_float((127 + *p.scale_exp) << 23);     // 2^e
+        [[maybe_unused]] const float off_factor = OFFSET ? offset_factor(p.ctl, p.zp_mid) : 0.0f;
         __half* stage = &sm.ystage[ew][0][0];
         for (int tl = 0; tl < my_tiles; ++tl) {
             const int tile = (int)(blockIdx.x + tl * gridDim.x);
@@ -249,7 +251,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 const int n = (2 * np + h) * kTileN + r;
                 n_ok[h] = n < p.N;
                 sc[h] = __half2float(p.w_scales[n]) * 0.0625f * pe;      // sums carry a factor 16 (n < Npad: the scale array is padded)
-                off_pe[h] = (OFFSET && n_ok[h]) ? p.chan_offset[n] * pe : 0.0f;
+                off_pe[h] = (OFFSET && n_ok[h]) ? __fmul_rn(off_factor, p.chan_offset[n]) * pe : 0.0f;
             }
             // One half after the other: the half's sums (this warp's columns) go to registers and its
             // accumulator returns to its issuer at once, so that conversion and stores overlap the next tile's MMAs.
@@ -379,7 +381,7 @@ cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     p.n_tiles_m = (a.M + kWBM - 1) / kWBM;
     p.n_tiles = p.n_tiles_m * (p.Npad / (2 * kTileN));
     p.w_packed = a.w_packed; p.w_scales = a.w_scales; p.scale_exp = a.scale_exp;
-    p.y = a.y; p.acc_dump = a.acc_dump; p.ctl = a.ctl; p.chan_offset = a.chan_offset;
+    p.y = a.y; p.acc_dump = a.acc_dump; p.ctl = a.ctl; p.chan_offset = a.chan_offset; p.zp_mid = a.zp_mid;
     p.q_next = a.q_next;
     p.next_inv = ldexpf(1.0f, -a.next_exp);
     p.next_lo = -(float)(1 << (a.next_bits - 1));

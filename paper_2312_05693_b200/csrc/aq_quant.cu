@@ -12,8 +12,6 @@ namespace aq {
 
 namespace {
 
-constexpr int kQuantThreads = 256;
-
 // The half2 route with TRIP factors (4-bit codes): lane k multiplies by 2^-(e + alpha_k), built from
 // the factor byte as a half bit pattern (exponent field 15 - e - alpha_k, which must be 1..30),
 // clamps to [-8, 7], rounds by adding and removing 1536, multiplies by 2^alpha_k (exact, |result|
@@ -50,31 +48,6 @@ __device__ __forceinline__ uint4 quantize16_fp32(const uint4& d0, const uint4& d
     const uint2 r0 = quantize8_fp32(d0, e, lo, hi, al ? &a0 : nullptr);
     const uint2 r1 = quantize8_fp32(d1, e, lo, hi, al ? &a1 : nullptr);
     return make_uint4(r0.x, r0.y, r1.x, r1.y);
-}
-
-// ---- quantize: 16 halves in (two 16-byte loads), 16 codes out (one 16-byte store) -----
-__global__ void __launch_bounds__(kQuantThreads)
-quantize_kernel(const uint4* __restrict__ x, int M, int vec_per_row /* 16-element units */,
-                const int32_t* __restrict__ row_idx, int bits, int scale_mode, int clip_shift_or_exp,
-                Control* __restrict__ ctl, uint4* __restrict__ q, int32_t* __restrict__ scale_exp_out,
-                const uint4* __restrict__ alpha, int k_max) {
-    const int e = scale_mode == AQ_SCALE_DYNAMIC
-                      ? layer_exponent_from_bits(ctl->absmax_bits, bits) - clip_shift_or_exp - k_max
-                      : clip_shift_or_exp;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->scale_exp = e;
-        if (scale_exp_out) *scale_exp_out = e;
-    }
-    const float lo = -(float)(1 << (bits - 1)), hi = (float)((1 << (bits - 1)) - 1);
-    const size_t total = (size_t)M * vec_per_row;
-    const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= total) return;
-    const int m = (int)(v / vec_per_row), c = (int)(v % vec_per_row);
-    const size_t src = ((size_t)(row_idx ? row_idx[m] : m) * vec_per_row + c) * 2;
-    const uint4 d0 = __ldg(x + src), d1 = __ldg(x + src + 1);
-    uint4 al;
-    if (alpha) al = __ldg(alpha + c);
-    q[v] = quantize16_fp32(d0, d1, e, lo, hi, alpha ? &al : nullptr);
 }
 
 // ---- small activations (decode): maximum, exponent and codes in ONE kernel -------------
@@ -145,10 +118,9 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
         ctl->absmax_bits = all;
         ctl->scale_exp = e;
         ctl->status = 0;
-        ctl->counter = 0;
         if (scale_exp_out) *scale_exp_out = e;
     }
-    if (rank == 0 && threadIdx.x < 57) ctl->split_flags[threadIdx.x] = 0;    // the product kernel's shared-tile bits
+    if (rank == 0 && threadIdx.x < Control::kSplitWords) ctl->split_flags[threadIdx.x] = 0;    // the product kernel's shared-tile bits
     const float lo = -(float)(1 << (bits - 1)), hi = (float)((1 << (bits - 1)) - 1);
     if (alpha == nullptr && e >= -14 && e <= 14) {           // 2^-e is a normal half: codes in half2 arithmetic
         const __half2 inv2 = __float2half2_rn(__int_as_float((127 - e) << 23));
@@ -175,150 +147,181 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
     }
 }
 
-// ---- larger activations, dynamic scale: maximum, exponent and codes in ONE cooperative kernel ----
-// One CTA per SM takes a contiguous share of X. First pass: 16-byte loads from HBM, running maximum,
-// and the loaded vectors are parked in shared memory (as much of the share as fits). The CTAs then
-// meet at a counter in the control block (all are resident: the launch is cooperative; the wait is
-// bounded all the same), every CTA derives the exponent from the global maximum, and the second
-// pass quantizes from shared memory (from L2 for what did not fit), so X crosses HBM once.
-constexpr int kFusedThreads = 1024;
-constexpr unsigned int kFusedWaitCode = 10;            // status value when the meeting point times out
-constexpr unsigned long long kFusedWaitCycles = 2000000000ull;   // ~1 s
+// ---- larger activations: two kernels, each of them plain (no grid-wide meeting, nothing to clear beforehand) ----
+// range_kernel: clusters of eight CTAs take contiguous shares of X (16-byte loads, eight in flight per thread), find
+// the share's minimum and maximum (symmetric scale: the largest magnitude), meet in distributed shared memory and
+// leave one word per cluster in the control block. quantize_kernel: every warp reads those words (at most one per
+// lane), and quantizes; X is read again, from L2 as far as it fits (126 MB). The second kernel, and the product behind
+// it, are launched with programmatic stream serialization, so that a kernel's launch overlaps its predecessor.
+// What it replaced: one cooperative kernel that parked X in shared memory between a grid-wide meeting, behind a node
+// that cleared the control block. X crossed HBM and L2 once there, but of 12.1 us (2048 x 4096) 4 were the clearing and
+// the cooperative launch and 2 the meeting. In graph replay over rotating inputs: 2048 x 4096 12.1 -> 9.1 us,
+// 2048 x 11008 21.9 -> 18.0 us, 1024 x 5120 10.1 -> 6.6 us, 333 x 5120 8.3 -> 5.5 us.
+constexpr int kRangeThreads = 512, kRangeCtas = 8;
+constexpr int kRangeInFlight = 8;
 
-__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
+__device__ __forceinline__ size_t source_vec(size_t v, int vec_per_row, const int32_t* row_idx) {
+    if (!row_idx) return v;
+    const size_t m = v / (size_t)vec_per_row;
+    return (size_t)row_idx[m] * vec_per_row + (v - m * (size_t)vec_per_row);
 }
 
-__global__ void __launch_bounds__(kFusedThreads, 1)
-quantize_fused_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-element units */,
-                      const int32_t* __restrict__ row_idx, int bits, int clip_shift, Control* __restrict__ ctl,
-                      uint4* __restrict__ q, int32_t* __restrict__ scale_exp_out, unsigned int cache_units,
-                      unsigned int units_per_cta, const uint4* __restrict__ alpha, int k_max) {
-    extern __shared__ uint4 fused_cache[];             // [2][cache_units]: first and second vector of a unit
-    __shared__ unsigned int warp_max[kFusedThreads / 32];
-    __shared__ int e_shared;
-    __shared__ int gave_up;
-    const size_t total = (size_t)M * units_per_row;
-    const size_t u0 = (size_t)blockIdx.x * units_per_cta;
-    const size_t u1 = u0 + units_per_cta < total ? u0 + units_per_cta : total;
-    // a product kernel launched with programmatic stream serialization may be scheduled as soon as this
-    // grid's CTAs leave their SMs (it waits for this grid before it reads the codes); no effect otherwise
+template <bool ASYM>
+__global__ void __cluster_dims__(kRangeCtas, 1, 1) __launch_bounds__(kRangeThreads)
+range_kernel(const uint4* __restrict__ x, size_t vecs /* of 8 halves */, int vec_per_row, const int32_t* __restrict__ row_idx,
+             size_t vecs_per_cta, Control* __restrict__ ctl) {
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ unsigned int warp_max[kRangeThreads / 32], warp_min[kRangeThreads / 32];
+    __shared__ unsigned int peers[kRangeCtas];
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // the kernel ahead may have written X
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-    __half2 m2 = __float2half2_rn(0.0f);
-    // four units (eight 16-byte loads) in flight per thread before the first is used: a CTA's share is a few
-    // units per thread, so the pass is one or two memory round trips rather than one per unit
-    constexpr int kInFlight = 4;
-    for (size_t ub = u0 + threadIdx.x; ub < u1; ub += (size_t)kFusedThreads * kInFlight) {
-        uint4 d0[kInFlight], d1[kInFlight];
+    const size_t v0 = (size_t)blockIdx.x * vecs_per_cta;
+    const size_t v1 = v0 + vecs_per_cta < vecs ? v0 + vecs_per_cta : vecs;
+    __half2 hi2 = __float2half2_rn(0.0f), lo2 = hi2;        // the range always contains 0
+    for (size_t vb = v0 + threadIdx.x; vb < v1; vb += (size_t)kRangeThreads * kRangeInFlight) {
+        uint4 d[kRangeInFlight];
 #pragma unroll
-        for (int i = 0; i < kInFlight; ++i) {
-            const size_t u = ub + (size_t)i * kFusedThreads;
-            if (u < u1) {
-                const int m = (int)(u / units_per_row), c = (int)(u % units_per_row);
-                const size_t src = ((size_t)(row_idx ? row_idx[m] : m) * units_per_row + c) * 2;
-                d0[i] = __ldg(x + src); d1[i] = __ldg(x + src + 1);
-            } else {
-                d0[i] = make_uint4(0u, 0u, 0u, 0u); d1[i] = d0[i];
-            }
+        for (int i = 0; i < kRangeInFlight; ++i) {
+            const size_t v = vb + (size_t)i * kRangeThreads;
+            d[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (v < v1) d[i] = __ldg(x + source_vec(v, vec_per_row, row_idx));
         }
 #pragma unroll
-        for (int i = 0; i < kInFlight; ++i) {
-            const size_t u = ub + (size_t)i * kFusedThreads;
-            if (u < u1) {
-                const unsigned int local = (unsigned int)(u - u0);
-                if (local < cache_units) { fused_cache[local] = d0[i]; fused_cache[cache_units + local] = d1[i]; }
-            }
-            const __half2* h0 = reinterpret_cast<const __half2*>(&d0[i]);
-            const __half2* h1 = reinterpret_cast<const __half2*>(&d1[i]);
+        for (int i = 0; i < kRangeInFlight; ++i) {
+            const __half2* h = reinterpret_cast<const __half2*>(&d[i]);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) m2 = __hmax2(m2, __hmax2(__habs2(h0[k]), __habs2(h1[k])));   // NaN operands are dropped
+            for (int k = 0; k < 4; ++k) {                    // NaN operands are dropped
+                if (ASYM) {
+                    lo2 = __hmin2(lo2, h[k]);
+                    hi2 = __hmax2(hi2, h[k]);
+                } else {
+                    hi2 = __hmax2(hi2, __habs2(h[k]));
+                }
+            }
         }
     }
-    unsigned int bmax = max((unsigned int)__half_as_ushort(__low2half(m2)),
-                            (unsigned int)__half_as_ushort(__high2half(m2)));
-    if (bmax > 0x7C00u) bmax = 0;                                       // never publish NaN
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) bmax = max(bmax, __shfl_xor_sync(0xFFFFFFFFu, bmax, o));
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = bmax;
+    // as magnitudes: bit patterns of non-negative halves order as integers; +-Inf stays Inf here
+    unsigned int bmax = max((unsigned int)__half_as_ushort(__low2half(hi2)), (unsigned int)__half_as_ushort(__high2half(hi2)));
+    unsigned int bmin = 0;
+    if (ASYM) {
+        const __half2 n2 = __habs2(lo2);
+        bmin = max((unsigned int)__half_as_ushort(__low2half(n2)), (unsigned int)__half_as_ushort(__high2half(n2)));
+    }
+    if (bmax > 0x7C00u) bmax = 0;                            // never publish NaN
+    if (bmin > 0x7C00u) bmin = 0;
+    bmax = __reduce_max_sync(0xFFFFFFFFu, bmax);
+    if (ASYM) bmin = __reduce_max_sync(0xFFFFFFFFu, bmin);
+    if ((threadIdx.x & 31) == 0) {
+        warp_max[threadIdx.x >> 5] = bmax;
+        warp_min[threadIdx.x >> 5] = bmin;
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
-        unsigned int b = warp_max[threadIdx.x];
+        bmax = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kRangeThreads / 32 ? warp_max[threadIdx.x] : 0u);
+        bmin = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kRangeThreads / 32 ? warp_min[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) *cluster.map_shared_rank(&peers[cluster.block_rank()], 0) = bmax | (bmin << 16);
+    }
+    cluster.sync();
+    if (cluster.block_rank() == 0 && threadIdx.x == 0) {
+        unsigned int hi = 0, lo = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, o));
-        if (threadIdx.x == 0) {
-            if (b != 0) atomicMax(&ctl->absmax_bits, b);
-            __threadfence();
-            atomicAdd(&ctl->counter, 1u);
-            // meeting point: every CTA has added its maximum once the counter reaches the grid size
-            const long long t0 = clock64();
-            int failed = 0;
-            while (ld_acquire_u32(&ctl->counter) < gridDim.x) {
-                if ((unsigned long long)(clock64() - t0) > kFusedWaitCycles) { failed = 1; break; }
-                __nanosleep(100);
-            }
-            gave_up = failed;
-            e_shared = layer_exponent_from_bits(ld_acquire_u32(&ctl->absmax_bits), bits) - clip_shift - k_max;
+        for (int r = 0; r < kRangeCtas; ++r) {
+            hi = max(hi, peers[r] & 0xFFFFu);
+            lo = max(lo, peers[r] >> 16);
+        }
+        ctl->range[blockIdx.x / kRangeCtas] = hi | (lo << 16);
+    }
+}
+
+// The words of range_kernel, met: largest positive (or absolute) value in the low half, largest magnitude of a negative
+// one in the high half. Whole warps call this.
+__device__ __forceinline__ unsigned int met_range(const Control* ctl, int words) {
+    const unsigned int lane = threadIdx.x & 31;
+    const unsigned int w = lane < (unsigned int)words ? ctl->range[lane] : 0u;
+    return __reduce_max_sync(0xFFFFFFFFu, w & 0xFFFFu) | (__reduce_max_sync(0xFFFFFFFFu, w >> 16) << 16);
+}
+
+// What the product kernel finds in the control block.
+__device__ __forceinline__ void publish_control(Control* ctl, unsigned int absmax_bits, int e, int zp, int32_t* scale_exp_out,
+                                                int32_t* zero_point_out) {
+    if (blockIdx.x != 0) return;
+    if (threadIdx.x == 0) {
+        ctl->absmax_bits = absmax_bits;
+        ctl->scale_exp = e;
+        ctl->zero_point = zp;
+        ctl->status = 0;
+        if (scale_exp_out) *scale_exp_out = e;
+        if (zero_point_out) *zero_point_out = zp;
+    }
+    if (threadIdx.x < Control::kSplitWords) ctl->split_flags[threadIdx.x] = 0;      // the product kernel's shared-tile bits
+}
+
+constexpr int kQuantThreads = 256;
+constexpr int kQuantUnits = 4;                               // units of 16 elements per thread, all loads in flight
+
+// Loads of a thread's units: unit i is u0 + i * kQuantThreads.
+__device__ __forceinline__ void load_units(const uint4* __restrict__ x, size_t u0, size_t total, int units_per_row,
+                                           const int32_t* __restrict__ row_idx, uint4 (&d)[kQuantUnits][2]) {
+#pragma unroll
+    for (int i = 0; i < kQuantUnits; ++i) {
+        const size_t u = u0 + (size_t)i * kQuantThreads;
+        if (u < total) {
+            const size_t src = 2 * source_vec(u, units_per_row, row_idx);
+            d[i][0] = __ldg(x + src);
+            d[i][1] = __ldg(x + src + 1);
         }
     }
-    __syncthreads();
-    if (gave_up) {
-        if (threadIdx.x == 0) atomicCAS(&ctl->status, 0u, kFusedWaitCode);
-        return;
+}
+
+// words > 0: dynamic scale from that many words of range_kernel; 0: the exponent is given
+__global__ void __launch_bounds__(kQuantThreads)
+quantize_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-element units */,
+                const int32_t* __restrict__ row_idx, int bits, int words, int clip_shift_or_exp,
+                Control* __restrict__ ctl, uint4* __restrict__ q, int32_t* __restrict__ scale_exp_out,
+                const uint4* __restrict__ alpha, int k_max) {
+    // After this wait everything ahead (weight packing included) has completed: only now may the product kernel be
+    // set up, which fetches weights before its own wait.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const size_t total = (size_t)M * units_per_row;
+    const size_t u0 = (size_t)blockIdx.x * (kQuantThreads * kQuantUnits) + threadIdx.x;
+    uint4 d[kQuantUnits][2];
+    load_units(x, u0, total, units_per_row, row_idx, d);
+    unsigned int absmax = 0;
+    int e = clip_shift_or_exp;
+    if (words) {
+        absmax = met_range(ctl, words) & 0xFFFFu;
+        e = layer_exponent_from_bits(absmax, bits) - clip_shift_or_exp - k_max;
     }
-    const int e = e_shared;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->scale_exp = e;
-        if (scale_exp_out) *scale_exp_out = e;
-    }
+    publish_control(ctl, absmax, e, 0, scale_exp_out, nullptr);
     const float inv = __int_as_float((127 - e) << 23);      // 2^-e, |e| <= 40
     const float lo = -(float)(1 << (bits - 1)), hi = (float)((1 << (bits - 1)) - 1);
     const bool fast = alpha == nullptr && e >= -14 && e <= 14;   // 2^-e is a normal half
     const bool fast_trip = alpha != nullptr && bits == 4 && e >= -14 && e <= 10;   // so is 2^-(e + alpha), alpha <= 4
     const __half2 inv2 = __float2half2_rn(fast ? inv : 1.0f), lo2 = __float2half2_rn(lo), hi2 = __float2half2_rn(hi);
-#pragma unroll 2
-    for (size_t u = u0 + threadIdx.x; u < u1; u += kFusedThreads) {
-        const unsigned int local = (unsigned int)(u - u0);
-        uint4 d0, d1;
-        if (local < cache_units) {
-            d0 = fused_cache[local]; d1 = fused_cache[cache_units + local];      // this thread's own stores
-        } else {
-            const int m = (int)(u / units_per_row), c = (int)(u % units_per_row);
-            const size_t src = ((size_t)(row_idx ? row_idx[m] : m) * units_per_row + c) * 2;
-            d0 = __ldg(x + src); d1 = __ldg(x + src + 1);
-        }
-        uint32_t out[4];
+#pragma unroll
+    for (int i = 0; i < kQuantUnits; ++i) {
+        const size_t u = u0 + (size_t)i * kQuantThreads;
+        if (u >= total) break;
+        uint4 out;
         if (fast) {
-            quantize8_half2(d0, inv2, lo2, hi2, out[0], out[1]);
-            quantize8_half2(d1, inv2, lo2, hi2, out[2], out[3]);
-            q[u] = make_uint4(out[0], out[1], out[2], out[3]);
-        } else if (fast_trip) {
-            const uint4 al = __ldg(alpha + (size_t)(u % units_per_row));
-            quantize8_half2_trip(d0, e, make_uint2(al.x, al.y), out[0], out[1]);
-            quantize8_half2_trip(d1, e, make_uint2(al.z, al.w), out[2], out[3]);
-            q[u] = make_uint4(out[0], out[1], out[2], out[3]);
+            quantize8_half2(d[i][0], inv2, lo2, hi2, out.x, out.y);
+            quantize8_half2(d[i][1], inv2, lo2, hi2, out.z, out.w);
         } else {
             uint4 al;
             if (alpha) al = __ldg(alpha + (size_t)(u % units_per_row));
-            q[u] = quantize16_fp32(d0, d1, e, lo, hi, alpha ? &al : nullptr);
+            if (fast_trip) {
+                quantize8_half2_trip(d[i][0], e, make_uint2(al.x, al.y), out.x, out.y);
+                quantize8_half2_trip(d[i][1], e, make_uint2(al.z, al.w), out.z, out.w);
+            } else {
+                out = quantize16_fp32(d[i][0], d[i][1], e, lo, hi, alpha ? &al : nullptr);
+            }
         }
+        q[u] = out;
     }
 }
 
 // ---- zero-point variant (Eq. 2, Eq. 5-7 with alpha = 0, power-of-two scale) ---------------
-// Order-preserving map of a float's bits to an unsigned integer, so that atomicMin / atomicMax
-// on the keys give the minimum / maximum value.
-__device__ __forceinline__ unsigned int float_key(float f) {
-    const unsigned int b = __float_as_uint(f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float key_float(unsigned int k) {
-    return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
-}
-constexpr unsigned int kZeroKey = 0x80000000u;         // key of +0.0: the range always contains 0
-
 // 8 halves -> 8 stored codes (q - 2^(b-1)) of the zero-point quantizer in half2 arithmetic, for
 // exponents whose 2^-e is a normal half. The product by 2^-e is exact (or saturates and is clamped);
 // NaN lanes are cleared to 0, which becomes the code zp; clamping rint(t) + zp to [0, qr] equals
@@ -343,71 +346,25 @@ __device__ __forceinline__ void quantize8_half2_asym(const uint4& d, __half2 inv
     w1 = __byte_perm(r[2], r[3], 0x6420);
 }
 
-// One cooperative kernel, as quantize_fused_kernel: first pass minimum and maximum (16-byte loads, the
-// share parked in shared memory), meeting point, e and zp in binary64 by one thread per CTA, second
-// pass codes from shared memory.
-__global__ void __launch_bounds__(kFusedThreads, 1)
-quantize_asym_fused_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-element units */,
-                           const int32_t* __restrict__ row_idx, int bits, Control* __restrict__ ctl,
-                           uint4* __restrict__ q, int32_t* __restrict__ scale_exp_out,
-                           int32_t* __restrict__ zero_point_out, unsigned int cache_units, unsigned int units_per_cta) {
-    extern __shared__ uint4 fused_cache[];             // [2][cache_units]
-    __shared__ unsigned int warp_min[kFusedThreads / 32], warp_maxk[kFusedThreads / 32];
-    __shared__ int params[3];                          // e, zp, gave up
+// Codes from the minimum and maximum that range_kernel left (`words` words), as quantize_kernel.
+__global__ void __launch_bounds__(kQuantThreads)
+quantize_asym_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-element units */,
+                     const int32_t* __restrict__ row_idx, int bits, int words, Control* __restrict__ ctl,
+                     uint4* __restrict__ q, int32_t* __restrict__ scale_exp_out, int32_t* __restrict__ zero_point_out) {
+    __shared__ int params[2];                          // e, zp
+    asm volatile("griddepcontrol.wait;" ::: "memory");                 // see quantize_kernel
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t total = (size_t)M * units_per_row;
-    const size_t u0 = (size_t)blockIdx.x * units_per_cta;
-    const size_t u1 = u0 + units_per_cta < total ? u0 + units_per_cta : total;
-
-    __half2 lo2 = __float2half2_rn(0.0f), hi2 = __float2half2_rn(0.0f);      // the range always contains 0
-#pragma unroll 2
-    for (size_t u = u0 + threadIdx.x; u < u1; u += kFusedThreads) {
-        const int m = (int)(u / units_per_row), c = (int)(u % units_per_row);
-        const size_t src = ((size_t)(row_idx ? row_idx[m] : m) * units_per_row + c) * 2;
-        const uint4 d0 = __ldg(x + src), d1 = __ldg(x + src + 1);
-        const unsigned int local = (unsigned int)(u - u0);
-        if (local < cache_units) { fused_cache[local] = d0; fused_cache[cache_units + local] = d1; }
-        const __half2* h0 = reinterpret_cast<const __half2*>(&d0);
-        const __half2* h1 = reinterpret_cast<const __half2*>(&d1);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {                                        // NaN operands are dropped
-            lo2 = __hmin2(lo2, __hmin2(h0[i], h1[i]));
-            hi2 = __hmax2(hi2, __hmax2(h0[i], h1[i]));
-        }
-    }
-    // +-Inf count as the largest half
-    const float lo = fmaxf(fminf(__low2float(lo2), __high2float(lo2)), -65504.0f);
-    const float hi = fminf(fmaxf(__low2float(hi2), __high2float(hi2)), 65504.0f);
-    unsigned int kmin = float_key(lo), kmax = float_key(hi);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        kmin = min(kmin, __shfl_xor_sync(0xFFFFFFFFu, kmin, o));
-        kmax = max(kmax, __shfl_xor_sync(0xFFFFFFFFu, kmax, o));
-    }
-    if ((threadIdx.x & 31) == 0) { warp_min[threadIdx.x >> 5] = kmin; warp_maxk[threadIdx.x >> 5] = kmax; }
-    __syncthreads();
+    const size_t u0 = (size_t)blockIdx.x * (kQuantThreads * kQuantUnits) + threadIdx.x;
+    uint4 d[kQuantUnits][2];
+    load_units(x, u0, total, units_per_row, row_idx, d);
     if (threadIdx.x < 32) {
-        kmin = warp_min[threadIdx.x];
-        kmax = warp_maxk[threadIdx.x];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            kmin = min(kmin, __shfl_xor_sync(0xFFFFFFFFu, kmin, o));
-            kmax = max(kmax, __shfl_xor_sync(0xFFFFFFFFu, kmax, o));
-        }
+        const unsigned int met = met_range(ctl, words);
         if (threadIdx.x == 0) {
-            // the control block is cleared to 0: keys are stored relative to the key of 0.0
-            if (kmax > kZeroKey) atomicMax(&ctl->max_key, kmax - kZeroKey);
-            if (kmin < kZeroKey) atomicMax(&ctl->min_key, kZeroKey - kmin);
-            __threadfence();
-            atomicAdd(&ctl->counter, 1u);
-            const long long t0 = clock64();
-            int failed = 0;
-            while (ld_acquire_u32(&ctl->counter) < gridDim.x) {
-                if ((unsigned long long)(clock64() - t0) > kFusedWaitCycles) { failed = 1; break; }
-                __nanosleep(100);
-            }
+            // +-Inf count as the largest half
+            const double dhi = (double)__half2float(__ushort_as_half((unsigned short)min(met & 0xFFFFu, 0x7BFFu)));
+            const double dlo = -(double)__half2float(__ushort_as_half((unsigned short)min(met >> 16, 0x7BFFu)));
             const double qr = (double)((1 << bits) - 1);
-            const double dhi = (double)key_float(kZeroKey + ld_acquire_u32(&ctl->max_key));
-            const double dlo = (double)key_float(kZeroKey - ld_acquire_u32(&ctl->min_key));
             const double range = dhi - dlo;
             int ee = 0;
             if (range > 0.0) {
@@ -419,21 +376,11 @@ quantize_asym_fused_kernel(const uint4* __restrict__ x, int M, int units_per_row
             }
             params[0] = ee;
             params[1] = (int)fmin(fmax(rint(ldexp(-dlo, -ee)), 0.0), qr);
-            params[2] = failed;
         }
     }
     __syncthreads();
-    if (params[2]) {
-        if (threadIdx.x == 0) atomicCAS(&ctl->status, 0u, kFusedWaitCode);
-        return;
-    }
     const int e = params[0], zp = params[1];
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->scale_exp = e;
-        ctl->zero_point = zp;
-        if (scale_exp_out) *scale_exp_out = e;
-        if (zero_point_out) *zero_point_out = zp;
-    }
+    publish_control(ctl, 0u, e, zp, scale_exp_out, zero_point_out);
     const int qr_i = (1 << bits) - 1, half_range = 1 << (bits - 1);
     const float inv = __int_as_float((127 - e) << 23);      // 2^-e
     const float fzp = (float)zp, fqr = (float)qr_i;
@@ -441,31 +388,24 @@ quantize_asym_fused_kernel(const uint4* __restrict__ x, int M, int units_per_row
     const __half2 inv2 = __float2half2_rn(fast ? inv : 1.0f);
     const __half2 clo2 = __float2half2_rn(-fzp), chi2 = __float2half2_rn(fqr - fzp);
     const __half2 shift2 = __float2half2_rn((float)(zp - half_range));
-#pragma unroll 2
-    for (size_t u = u0 + threadIdx.x; u < u1; u += kFusedThreads) {
-        const unsigned int local = (unsigned int)(u - u0);
-        uint4 d0, d1;
-        if (local < cache_units) {
-            d0 = fused_cache[local]; d1 = fused_cache[cache_units + local];      // this thread's own stores
-        } else {
-            const int m = (int)(u / units_per_row), c = (int)(u % units_per_row);
-            const size_t src = ((size_t)(row_idx ? row_idx[m] : m) * units_per_row + c) * 2;
-            d0 = __ldg(x + src); d1 = __ldg(x + src + 1);
-        }
+#pragma unroll
+    for (int i = 0; i < kQuantUnits; ++i) {
+        const size_t u = u0 + (size_t)i * kQuantThreads;
+        if (u >= total) break;
         uint32_t out[4];
         if (fast) {
-            quantize8_half2_asym(d0, inv2, clo2, chi2, shift2, out[0], out[1]);
-            quantize8_half2_asym(d1, inv2, clo2, chi2, shift2, out[2], out[3]);
+            quantize8_half2_asym(d[i][0], inv2, clo2, chi2, shift2, out[0], out[1]);
+            quantize8_half2_asym(d[i][1], inv2, clo2, chi2, shift2, out[2], out[3]);
         } else {
-            const __half* h0 = reinterpret_cast<const __half*>(&d0);
-            const __half* h1 = reinterpret_cast<const __half*>(&d1);
+            const __half* h0 = reinterpret_cast<const __half*>(&d[i][0]);
+            const __half* h1 = reinterpret_cast<const __half*>(&d[i][1]);
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
                 uint32_t word = 0;
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    const int i = 4 * w + b;
-                    const float t = __half2float(i < 8 ? h0[i] : h1[i - 8]) * inv;    // exact
+                    const int k = 4 * w + b;
+                    const float t = __half2float(k < 8 ? h0[k] : h1[k - 8]) * inv;    // exact
                     int code = zp;                                                    // NaN: value 0
                     if (t == t) code = (int)fminf(fmaxf(rintf(t) + fzp, 0.0f), fqr);
                     word |= ((uint32_t)(code - half_range) & 0xFFu) << (8 * b);
@@ -475,12 +415,6 @@ quantize_asym_fused_kernel(const uint4* __restrict__ x, int M, int units_per_row
         }
         q[u] = make_uint4(out[0], out[1], out[2], out[3]);
     }
-}
-
-__global__ void chan_offsets_kernel(const float* __restrict__ r, int N, int bits, const Control* __restrict__ ctl,
-                                    float* __restrict__ off) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) off[n] = -(float)(ctl->zero_point - (1 << (bits - 1))) * r[n];
 }
 
 // ---- TRIP calibration (Eq. 8 with the clipping of Eq. 5) ---------------------------------
@@ -677,44 +611,39 @@ gather_rows_kernel(const uint4* __restrict__ x, int vec_per_row, const int32_t* 
 
 }  // namespace
 
-cudaError_t launch_quantize(const __half* x, int M, int K, const int32_t* row_idx, int bits,
-                            int scale_mode, int clip_shift_or_exp, Control* ctl, int8_t* q,
-                            int32_t* scale_exp_out, const DeviceInfo& dev, cudaStream_t stream,
-                            const uint8_t* alpha, int k_max) {
-    (void)dev;
-    const int vec_per_row = K / 16;
-    const size_t total = (size_t)M * vec_per_row;
-    const size_t blocks = (total + kQuantThreads - 1) / kQuantThreads;
-    quantize_kernel<<<(unsigned int)blocks, kQuantThreads, 0, stream>>>(
-        reinterpret_cast<const uint4*>(x), M, vec_per_row, row_idx, bits, scale_mode, clip_shift_or_exp,
-        ctl, reinterpret_cast<uint4*>(q), scale_exp_out, reinterpret_cast<const uint4*>(alpha), k_max);
-    return cudaGetLastError();
+namespace {
+// Returns the number of words range_kernel leaves in the control block.
+template <bool ASYM>
+cudaError_t launch_range(const __half* x, int M, int K, const int32_t* row_idx, Control* ctl, cudaStream_t stream, int& words) {
+    const size_t vecs = (size_t)M * (K / 8);
+    // as many clusters as the control block has words for (232 CTAs of 512 threads, all resident at once), fewer when
+    // a CTA would have less than two vectors per thread
+    const size_t per_cluster = (size_t)kRangeCtas * kRangeThreads * 2;
+    size_t clusters = (vecs + per_cluster - 1) / per_cluster;
+    if (clusters > Control::kRangeWords) clusters = Control::kRangeWords;
+    words = (int)clusters;
+    const size_t ctas = clusters * kRangeCtas;
+    return launch_overlapped(range_kernel<ASYM>, ctas, kRangeThreads, stream, reinterpret_cast<const uint4*>(x), vecs, K / 8, row_idx,
+                             (vecs + ctas - 1) / ctas, ctl);
 }
 
-cudaError_t launch_quantize_fused(const __half* x, int M, int K, const int32_t* row_idx, int bits, int clip_shift,
-                                  Control* ctl, int8_t* q, int32_t* scale_exp_out, const DeviceInfo& dev,
-                                  cudaStream_t stream, const uint8_t* alpha, int k_max) {
-    int units_per_row = K / 16;
-    const size_t total = (size_t)M * units_per_row;
-    size_t grid = (total + kFusedThreads - 1) / kFusedThreads;
-    if (grid > (size_t)dev.sm_count) grid = (size_t)dev.sm_count;
-    unsigned int units_per_cta = (unsigned int)((total + grid - 1) / grid);
-    // shared-memory cache: the CTA's whole share when it fits, else as much as one CTA may hold
-    const size_t reserve = 8192;                       // static shared memory and alignment slack
-    const size_t max_cache = dev.smem_optin > reserve ? (dev.smem_optin - reserve) / 32 : 0;
-    unsigned int cache_units = units_per_cta < max_cache ? units_per_cta : (unsigned int)max_cache;
-    const size_t smem_bytes = (size_t)cache_units * 32;
-    static SmemOptIn opt_in;            // always the device's whole opt-in size: any later share fits
-    if (const cudaError_t e = opt_in.ensure(quantize_fused_kernel, dev.device, dev.smem_optin - reserve); e != cudaSuccess)
-        return e;
-    const uint4* xp = reinterpret_cast<const uint4*>(x);
-    uint4* qp = reinterpret_cast<uint4*>(q);
-    const uint4* ap = reinterpret_cast<const uint4*>(alpha);
-    void* args[] = {&xp, &M, &units_per_row, &row_idx, &bits, &clip_shift, &ctl, &qp, &scale_exp_out, &cache_units,
-                    &units_per_cta, &ap, &k_max};
-    // cooperative: the launch fails rather than start a grid whose CTAs could not all be resident
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(quantize_fused_kernel), dim3((unsigned int)grid),
-                                       dim3(kFusedThreads), args, smem_bytes, stream);
+size_t quantize_grid(int M, int K) {
+    const size_t per_cta = (size_t)kQuantThreads * kQuantUnits;
+    return ((size_t)M * (K / 16) + per_cta - 1) / per_cta;
+}
+}  // namespace
+
+cudaError_t launch_quantize(const __half* x, int M, int K, const int32_t* row_idx, int bits,
+                            int scale_mode, int clip_shift_or_exp, Control* ctl, int8_t* q,
+                            int32_t* scale_exp_out, cudaStream_t stream, const uint8_t* alpha, int k_max) {
+    int words = 0;
+    if (scale_mode == AQ_SCALE_DYNAMIC) {
+        const cudaError_t e = launch_range<false>(x, M, K, row_idx, ctl, stream, words);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_overlapped(quantize_kernel, quantize_grid(M, K), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
+                             row_idx, bits, words, clip_shift_or_exp, ctl, reinterpret_cast<uint4*>(q), scale_exp_out,
+                             reinterpret_cast<const uint4*>(alpha), k_max);
 }
 
 cudaError_t launch_trip_calibrate(const __half* x, int M, int K, const int32_t* row_idx, int bits, int k_max,
@@ -733,32 +662,12 @@ cudaError_t launch_trip_calibrate(const __half* x, int M, int K, const int32_t* 
 }
 
 cudaError_t launch_quantize_asym(const __half* x, int M, int K, const int32_t* row_idx, int bits, Control* ctl,
-                                 int8_t* q, int32_t* scale_exp_out, int32_t* zero_point_out, const DeviceInfo& dev,
-                                 cudaStream_t stream) {
-    int units_per_row = K / 16;
-    const size_t total = (size_t)M * units_per_row;
-    size_t grid = (total + kFusedThreads - 1) / kFusedThreads;
-    if (grid > (size_t)dev.sm_count) grid = (size_t)dev.sm_count;
-    unsigned int units_per_cta = (unsigned int)((total + grid - 1) / grid);
-    const size_t reserve = 8192;
-    const size_t max_cache = dev.smem_optin > reserve ? (dev.smem_optin - reserve) / 32 : 0;
-    unsigned int cache_units = units_per_cta < max_cache ? units_per_cta : (unsigned int)max_cache;
-    const size_t smem_bytes = (size_t)cache_units * 32;
-    static SmemOptIn opt_in;
-    if (const cudaError_t e = opt_in.ensure(quantize_asym_fused_kernel, dev.device, dev.smem_optin - reserve);
-        e != cudaSuccess)
-        return e;
-    const uint4* xp = reinterpret_cast<const uint4*>(x);
-    uint4* qp = reinterpret_cast<uint4*>(q);
-    void* args[] = {&xp, &M, &units_per_row, &row_idx, &bits, &ctl, &qp, &scale_exp_out, &zero_point_out, &cache_units,
-                    &units_per_cta};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(quantize_asym_fused_kernel),
-                                       dim3((unsigned int)grid), dim3(kFusedThreads), args, smem_bytes, stream);
-}
-
-cudaError_t launch_chan_offsets(const float* r, int N, int bits, const Control* ctl, float* off, cudaStream_t stream) {
-    chan_offsets_kernel<<<(N + 255) / 256, 256, 0, stream>>>(r, N, bits, ctl, off);
-    return cudaGetLastError();
+                                 int8_t* q, int32_t* scale_exp_out, int32_t* zero_point_out, cudaStream_t stream) {
+    int words = 0;
+    const cudaError_t e = launch_range<true>(x, M, K, row_idx, ctl, stream, words);
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(quantize_asym_kernel, quantize_grid(M, K), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
+                             row_idx, bits, words, ctl, reinterpret_cast<uint4*>(q), scale_exp_out, zero_point_out);
 }
 
 bool quantize_small_fits(int M, int K) { return (size_t)M * (size_t)K <= kSmallMaxElems; }
