@@ -190,3 +190,42 @@ def test_attn_qk_matches_checker(bits, H, M, J):
     assert_y_close(s.cpu().numpy().reshape(H * M, J), ref.reshape(H * M, J))
     # the integer sums are below 2^24 here, so the scaled fp16 values are the same bits
     assert np.array_equal(s.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("max_bits", [0x3C00, 0x3DA7, 0x3DA8, 0x7BFF, 0x2000, 0x1FFF, 0x1C01, 0x2400, 0x0400, 0x0001])
+def test_byte_factors_of_every_half_below_a_maximum(max_bits):
+    """aq_log2_quantize_factors against the checker on every non-negative half up to a maximum (the bounds of the seven
+    factors all normal halves, or partly subnormal), zeros and NaN among them."""
+    vals = np.concatenate([np.arange(max_bits + 1, dtype=np.uint16), np.array([0x7E00, 0x8000], np.uint16)]).view(np.float16)
+    x = np.concatenate([vals, vals[: -len(vals) % 8]])
+    h = handle()
+    f, mx, ws = h.aq_log2_quantize_factors(dev(x))
+    assert h.aq_check_workspace(ws) == binding.AQ_OK
+    ref, _ = oracle.log2_quantize(x, 4)
+    assert int(mx.item()) & 0xFFFF == max_bits
+    assert np.array_equal(f.cpu().numpy(), np.where(ref > 0, 128 >> np.maximum(ref.astype(np.int32) - 1, 0), 0).astype(np.uint8))
+
+
+@pytest.mark.parametrize("count", [8, 4093, 9_699_328, 10_000_013])
+def test_byte_factors_and_codes_agree_on_every_batch_size(count):
+    """Threads with whole batches of vectors, with a rest, and the ragged tail: the factors are those of the codes."""
+    g = torch.Generator(device="cuda").manual_seed(count)
+    x = torch.rand(count, generator=g, device="cuda").pow_(6).to(torch.float16)
+    h = handle()
+    f, mx, _ = h.aq_log2_quantize_factors(x)
+    c, mc = h.aq_log2_quantize(x, 4)
+    assert torch.equal(mx, mc) and int(mx.item()) == int(x.max().view(torch.int16).item())
+    assert torch.equal(f.to(torch.int32), torch.where(c > 0, 128 >> (c.to(torch.int32) - 1).clamp(min=0), 0))
+
+
+def test_attn_qk_items_with_and_without_whole_boxes_in_turn():
+    """More items than SMs, every second one with rows that end inside a 32-row box (its warps store directly), one tile
+    per item: the staging boxes of the other items alternate from store to store."""
+    H, M, J, D = 210, 176, 72, 128
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q = torch.randint(-9, 10, (H, M, D), generator=g, device="cuda", dtype=torch.int8)
+    k = torch.randint(-9, 10, (H, J, D), generator=g, device="cuda", dtype=torch.int8)
+    e = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s, ws = handle().aq_attn_qk_tc(q, e, k, e)
+    assert handle().aq_check_workspace(ws) == binding.AQ_OK
+    assert torch.equal(s.float(), torch.bmm(q.float(), k.float().transpose(1, 2)).half().float())   # sums below 2^14: exact
