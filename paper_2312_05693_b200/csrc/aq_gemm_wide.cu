@@ -22,7 +22,7 @@ namespace {
 
 constexpr int kWThreads = 20 * 32;
 constexpr int kWFirstUnpack = 4, kWFirstEpi = 12, kWEpiWarps = 8;
-constexpr int kWRegsControl = 48, kWRegsUnpack = 56, kWRegsEpi = 160;     // of the 96 x 640 the launch allocates
+constexpr int kWRegsControl = 40, kWRegsUnpack = 48, kWRegsEpi = 168;     // of the 96 x 640 the launch allocates
 static_assert(128 * kWRegsControl + 256 * kWRegsUnpack + 256 * kWRegsEpi <= kWThreads * 96,
               "register plan exceeds the launch allocation");
 constexpr int kWStageRows = 32;           // tokens per TMA store of an epilogue warp
@@ -42,8 +42,9 @@ struct WSmem {
     alignas(128) uint8_t w[kStages][2][kBlockBytes];           // the two packed weight blocks of a k block
     alignas(128) __half ystage[kWEpiWarps][kWStageRows][32];
     alignas(8) uint64_t tma_full[kStages];                     // both producers' bytes landed -> unpack warps
-    uint64_t smem_empty[kStages];                              // both halves' MMAs done -> TMA producers; unpack warps (slices free)
+    uint64_t smem_empty[kStages];                              // both halves' MMAs done -> TMA producers
     uint64_t a_full[8];                                        // a half's unpack warps stored the slice -> its MMA issuer
+    uint64_t a_empty[8];                                       // MMA done with the slice -> unpack warps
     uint64_t acc_full[2];                                      // a half's last MMAs of the tile done -> epilogue
     uint64_t acc_empty[2];                                     // epilogue has the half's sums in registers -> its issuer
     uint32_t tmem_base;
@@ -101,7 +102,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             mbar_init(&sm.tma_full[s], 2);
             mbar_init(&sm.smem_empty[s], 2);
         }
-        for (int i = 0; i < kWSlices; ++i) mbar_init(&sm.a_full[i], 4);
+        for (int i = 0; i < kWSlices; ++i) {
+            mbar_init(&sm.a_full[i], 4);
+            mbar_init(&sm.a_empty[i], 1);
+        }
         for (int h = 0; h < 2; ++h) {
             mbar_init(&sm.acc_full[h], 1);
             mbar_init(&sm.acc_empty[h], kWEpiWarps);
@@ -130,14 +134,15 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 // behind the call's own quantize kernel (programmatic stream serialization) the codes are
                 // touched only after that grid has completed; the weight producer does not wait
                 if (warp == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-                uint32_t s = 0, ph = 1;
+                uint32_t it = 0;
                 for (int tl = 0; tl < my_tiles; ++tl) {
                     const int tile = (int)(blockIdx.x + tl * gridDim.x);
                     const int mt = tile % p.n_tiles_m, np = tile / p.n_tiles_m;
                     const uint8_t* wsrc0 = p.w_packed + (size_t)(2 * np) * KB * kBlockBytes;
                     const uint8_t* wsrc1 = wsrc0 + (size_t)KB * kBlockBytes;
-                    for (int kb = 0; kb < KB; ++kb) {
-                        if (!mbar_wait(&sm.smem_empty[s], ph, abort_flag, 1u)) goto role_done;
+                    for (int kb = 0; kb < KB; ++kb, ++it) {
+                        const int s = (int)(it % kWStages);
+                        if (!mbar_wait(&sm.smem_empty[s], ((it / kWStages) & 1u) ^ 1u, abort_flag, 1u)) goto role_done;
                         if (warp == 0) {
                             mbar_arrive_expect_tx(&sm.tma_full[s], kWBM * 128);
                             tma_load_2d(sm.x[s], &x_map, kb * kTileK, mt * kWBM, &sm.tma_full[s]);
@@ -146,7 +151,6 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                             tma_load_1d(sm.w[s][0], wsrc0 + (size_t)kb * kBlockBytes, kBlockBytes, &sm.tma_full[s]);
                             tma_load_1d(sm.w[s][1], wsrc1 + (size_t)kb * kBlockBytes, kBlockBytes, &sm.tma_full[s]);
                         }
-                        if (++s == (uint32_t)kWStages) { s = 0; ph ^= 1u; }
                     }
                 }
             }
@@ -154,9 +158,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             // ------------- MMA issuers: warp 1 = channel half 0, warp 3 = half 1
             const int h = warp >> 1;
             if (lane == 0) {
-                // Ring positions and phases are carried in counters, and a block's one commit serves the producers and the
-                // unpack warps alike: this thread's chain of look, four MMAs and commits was the pace of a CTA that has
-                // its SM's L2 path to itself (750 cycles a block with two commits and divisions).
+                // Ring positions and phases are carried in counters: this thread's chain of look, four MMAs and commits
+                // is the pace of a CTA that has its SM's L2 path to itself (without the divisions K = 13824, N = 5120 at
+                // 333 rows 51.4 -> 49.2 us, K = 5120, N = 13824 at 1024 rows 57.7 -> 55.6 us). Also built and measured:
+                // slices freed by the stage's own barrier, so that a commit goes, and the unpack warps loading a block
+                // ahead: 47.0 and 54 us, but 0.8 % slower in a loop of large layers under the power cap.
                 constexpr uint32_t idesc = idesc_i8(128, kWBM);
                 const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm.x[0]));
                 const uint32_t d_addr = tmem_acc + (uint32_t)(h * kWBM);
@@ -173,6 +179,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
                             tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc, (kb == 0 && j == 0) ? 0u : 1u);
+                        tc_commit(&sm.a_empty[ai]);
                         tc_commit(&sm.smem_empty[s]);
                         if (++s == (uint32_t)kWStages) s = 0;
                         ai += 2;
@@ -189,28 +196,24 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         const int h = (warp - kWFirstUnpack) >> 2;
         const int r = quarter * 32 + lane;            // row inside the half's 128-channel block = TMEM lane
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-        // A block's packed words are loaded while the stores of the block before drain; both looks that the next block
-        // needs (its bytes, its slice) are issued together behind those stores.
-        constexpr uint32_t kBack = kWSlices / 2;      // blocks whose slices of this half are in use at once
-        uint32_t s = 0, ph = 0, ai = (uint32_t)h;     // stage of the block, its phase; its slice
-        uint32_t fs = 0, fph = 0;                     // stage whose MMAs free the slice (kBack blocks back), its phase
-        uint4 d[4];
-        auto load = [&](uint32_t stage) {
-            const uint4* src = reinterpret_cast<const uint4*>(sm.w[stage][h]) + r;
+        int pending = -1;                             // slice whose stores have been issued but not published
+        for (uint32_t it = 0; it < total_iters; ++it) {
+            const int s = (int)(it % kWStages);
+            const uint32_t u = it * 2u + (uint32_t)h;
+            const int ai = (int)(u % kWSlices);
+            if (!mbar_wait_warp(&sm.tma_full[s], (it / kWStages) & 1u, abort_flag, 6u)) goto role_done;
+            const uint4* src = reinterpret_cast<const uint4*>(sm.w[s][h]) + r;
+            uint4 d[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) d[j] = src[j * kTileN];
-        };
-        if (total_iters > 0) {
-            if (!mbar_wait_warp(&sm.tma_full[0], 0u, abort_flag, 6u)) goto role_done;
-            load(0);
-        }
-        bool free_slice = true;
-        for (uint32_t it = 0; it < total_iters; ++it) {
-            if (it >= kBack) {
-                if (!__all_sync(0xFFFFFFFFu, free_slice) && !mbar_wait_warp(&sm.smem_empty[fs], fph, abort_flag, 7u)) goto role_done;
-                if (++fs == (uint32_t)kWStages) { fs = 0; fph ^= 1u; }
-                tc_fence_after();
+            if (pending >= 0) {                       // the previous stores had the loads above to finish
+                tc_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.a_full[pending]);
             }
+            if (!mbar_wait_warp(&sm.a_empty[ai], ((u / kWSlices) & 1u) ^ 1u, abort_flag, 7u)) goto role_done;
+            tc_fence_after();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const uint32_t w[4] = {d[j].x, d[j].y, d[j].z, d[j].w};
@@ -220,24 +223,15 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                     v[2 * i] = (w[i] << 4) & 0xF0F0F0F0u;           // 16*code for k0..k0+3
                     v[2 * i + 1] = w[i] & 0xF0F0F0F0u;              // 16*code for k0+4..k0+7
                 }
-                tc_st8(tmem_a + lane_addr + ai * (uint32_t)kAColsPerStage + (uint32_t)(8 * j), v);
+                tc_st8(tmem_a + lane_addr + (uint32_t)(ai * kAColsPerStage + 8 * j), v);
             }
-            if (++s == (uint32_t)kWStages) { s = 0; ph ^= 1u; }
-            const bool more = it + 1 < total_iters;
-            const bool landed = more && mbar_test(&sm.tma_full[s], ph);
-            free_slice = it + 1 >= kBack && mbar_test(&sm.smem_empty[fs], fph);
-            const bool early = __all_sync(0xFFFFFFFFu, landed) != 0;
-            if (early) load(s);
+            pending = ai;
+        }
+        if (pending >= 0) {
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.a_full[ai]);
-            ai += 2;
-            if (ai >= (uint32_t)kWSlices) ai -= kWSlices;
-            if (more && !early) {
-                if (!mbar_wait_warp(&sm.tma_full[s], ph, abort_flag, 6u)) goto role_done;
-                load(s);
-            }
+            if (lane == 0) mbar_arrive(&sm.a_full[pending]);
         }
     } else {
         // ----------------------------------------------------------------------- epilogue
