@@ -160,11 +160,29 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
 constexpr int kRangeThreads = 512, kRangeCtas = 8;
 constexpr int kRangeInFlight = 8;
 
-__device__ __forceinline__ size_t source_vec(size_t v, int vec_per_row, const int32_t* row_idx) {
-    if (!row_idx) return v;
-    const size_t m = v / (size_t)vec_per_row;
-    return (size_t)row_idx[m] * vec_per_row + (v - m * (size_t)vec_per_row);
-}
+// Place of element number v (per_row elements a row) in the gathered rows, carried along in steps: one division at the
+// start instead of one per element (a 64-bit one each cost 8 us on 2458 gathered rows of 7168).
+struct RowWalk {
+    int m, c, step_m, step_c, per_row;
+    __device__ __forceinline__ RowWalk(size_t v, int per_row_, int step) : per_row(per_row_) {
+        if (v <= 0xFFFFFFFFull) {
+            m = (int)((uint32_t)v / (uint32_t)per_row);
+            c = (int)((uint32_t)v - (uint32_t)m * (uint32_t)per_row);
+        } else {
+            const size_t q = v / (size_t)per_row;
+            m = (int)q;
+            c = (int)(v - q * (size_t)per_row);
+        }
+        step_m = step / per_row;
+        step_c = step - step_m * per_row;
+    }
+    __device__ __forceinline__ size_t source(const int32_t* row_idx) const { return (size_t)row_idx[m] * per_row + c; }
+    __device__ __forceinline__ void next() {
+        m += step_m;
+        c += step_c;
+        if (c >= per_row) { c -= per_row; ++m; }
+    }
+};
 
 template <bool ASYM>
 __global__ void __cluster_dims__(kRangeCtas, 1, 1) __launch_bounds__(kRangeThreads)
@@ -178,13 +196,15 @@ range_kernel(const uint4* __restrict__ x, size_t vecs /* of 8 halves */, int vec
     const size_t v0 = (size_t)blockIdx.x * vecs_per_cta;
     const size_t v1 = v0 + vecs_per_cta < vecs ? v0 + vecs_per_cta : vecs;
     __half2 hi2 = __float2half2_rn(0.0f), lo2 = hi2;        // the range always contains 0
+    RowWalk at(row_idx ? v0 + threadIdx.x : 0, vec_per_row, kRangeThreads);
     for (size_t vb = v0 + threadIdx.x; vb < v1; vb += (size_t)kRangeThreads * kRangeInFlight) {
         uint4 d[kRangeInFlight];
 #pragma unroll
         for (int i = 0; i < kRangeInFlight; ++i) {
             const size_t v = vb + (size_t)i * kRangeThreads;
             d[i] = make_uint4(0u, 0u, 0u, 0u);
-            if (v < v1) d[i] = __ldg(x + source_vec(v, vec_per_row, row_idx));
+            if (v < v1) d[i] = __ldg(x + (row_idx ? at.source(row_idx) : v));
+            if (row_idx) at.next();
         }
 #pragma unroll
         for (int i = 0; i < kRangeInFlight; ++i) {
@@ -262,14 +282,16 @@ constexpr int kQuantUnits = 4;                               // units of 16 elem
 // Loads of a thread's units: unit i is u0 + i * kQuantThreads.
 __device__ __forceinline__ void load_units(const uint4* __restrict__ x, size_t u0, size_t total, int units_per_row,
                                            const int32_t* __restrict__ row_idx, uint4 (&d)[kQuantUnits][2]) {
+    RowWalk at(row_idx ? u0 : 0, units_per_row, kQuantThreads);
 #pragma unroll
     for (int i = 0; i < kQuantUnits; ++i) {
         const size_t u = u0 + (size_t)i * kQuantThreads;
         if (u < total) {
-            const size_t src = 2 * source_vec(u, units_per_row, row_idx);
+            const size_t src = 2 * (row_idx ? at.source(row_idx) : u);
             d[i][0] = __ldg(x + src);
             d[i][1] = __ldg(x + src + 1);
         }
+        if (row_idx) at.next();
     }
 }
 
