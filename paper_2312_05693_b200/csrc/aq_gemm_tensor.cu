@@ -848,6 +848,8 @@ cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const De
 }
 
 cudaError_t launch_gemm_tensor(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+    // one scale per channel: two channel blocks share a token tile where the shape allows it
+    if (gemm_wide_applies(a, dev)) return launch_gemm_wide(a, dev, stream);
     if (a.M <= 64) return a.group ? launch_bm<64, true>(a, dev, stream) : launch_bm<64, false>(a, dev, stream);
     if (a.group) {
         // the chained and zero-point variants have no shared-tile launch
@@ -857,8 +859,6 @@ cudaError_t launch_gemm_tensor(const GemmArgs& a, const DeviceInfo& dev, cudaStr
             default: return launch_bm<128, true>(a, dev, stream);
         }
     }
-    // one scale per channel: two channel blocks share a 128-token activation tile where the shape allows it
-    if (gemm_wide_applies(a)) return launch_gemm_wide(a, dev, stream);
     // one scale per channel: the 256-token tile halves the MMA instructions per unit of work
     if (a.M <= 128) return launch_bm<128, false>(a, dev, stream);
     return launch_bm<256, false>(a, dev, stream);

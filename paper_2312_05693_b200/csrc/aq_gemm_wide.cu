@@ -11,10 +11,17 @@
 // Roles: warp 0 = TMA producer of the activation tiles, warp 2 = of the two weight blocks, warps 1 and 3 =
 // MMA issuers (half 0 / half 1), warps 4-7 and 8-11 = unpack (half 0 / half 1), warps 12-19 = epilogue.
 // Needs an even number of 128-channel blocks; other shapes take the kernel of aq_gemm_tensor.cu.
+// CLUSTER (128-token tiles): too few tiles for the SMs (short prompts, narrow layers). The CTAs of
+// a cluster share a tile and take consecutive ranges of its k blocks; the tile's tokens are cut into eight runs, every
+// CTA sends the integer sums of the runs it does not own into their owners' shared memory (the operand ring, idle by
+// then) and finishes its own. Integer additions: the same results in any order; no scratch in memory, no flags.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "aq_common.cuh"
 #include "aq_tc.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace aq {
 
@@ -26,6 +33,8 @@ constexpr int kWRegsControl = 40, kWRegsUnpack = 48, kWRegsEpi = 168;     // of 
 static_assert(128 * kWRegsControl + 256 * kWRegsUnpack + 256 * kWRegsEpi <= kWThreads * 96,
               "register plan exceeds the launch allocation");
 constexpr int kWStageRows = 32;           // tokens per TMA store of an epilogue warp
+constexpr int kExchangeBlocks = 16;       // CLUSTER: what the meetings and the exchange cost, in k blocks (about 6 us)
+constexpr int kWRuns = 8;                 // CLUSTER: token runs of a tile
 template <int BM>
 struct WCfg {
     static constexpr int kStages = BM == 128 ? 6 : 5;          // shared-memory ring: activation tile + two packed weight blocks per stage
@@ -82,9 +91,23 @@ __device__ __forceinline__ void w_stage_code(__half* stage, int c, int lane, int
     }
 }
 
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void w_cluster_meet() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // OFFSET: add the per-channel term of the zero-point variant. CHAIN: write the next layer's codes instead
 // of fp16 outputs.
-template <int BM, bool OFFSET, bool CHAIN>
+template <int BM, bool OFFSET, bool CHAIN, bool CLUSTER>
 __global__ void __launch_bounds__(kWThreads, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap y_map, const WParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -94,8 +117,13 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     constexpr int kCols = WCfg<BM>::kCols;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int KB = p.KB;
-    const int my_tiles = p.n_tiles > (int)blockIdx.x ? (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    const uint32_t total_iters = (uint32_t)my_tiles * (uint32_t)KB;
+    static_assert(!CLUSTER || BM == 128, "runs of 16 tokens");
+    const int rank = CLUSTER ? (int)blockIdx.x : 0, split = CLUSTER ? (int)gridDim.x : 1;
+    const int my_tiles = CLUSTER ? 1 : (p.n_tiles > (int)blockIdx.x ? (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0);
+    const int kb0 = CLUSTER ? KB * rank / split : 0, kb1 = CLUSTER ? KB * (rank + 1) / split : KB;
+    const uint32_t total_iters = (uint32_t)my_tiles * (uint32_t)(kb1 - kb0);
+    auto tile_at = [&](int tl) { return CLUSTER ? (int)blockIdx.y : (int)(blockIdx.x + tl * gridDim.x); };
+    [[maybe_unused]] int met = 0;                    // CLUSTER: meetings this warp has been to
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kWStages; ++s) {
@@ -136,11 +164,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 if (warp == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
                 uint32_t it = 0;
                 for (int tl = 0; tl < my_tiles; ++tl) {
-                    const int tile = (int)(blockIdx.x + tl * gridDim.x);
+                    const int tile = tile_at(tl);
                     const int mt = tile % p.n_tiles_m, np = tile / p.n_tiles_m;
                     const uint8_t* wsrc0 = p.w_packed + (size_t)(2 * np) * KB * kBlockBytes;
                     const uint8_t* wsrc1 = wsrc0 + (size_t)KB * kBlockBytes;
-                    for (int kb = 0; kb < KB; ++kb, ++it) {
+                    for (int kb = kb0; kb < kb1; ++kb, ++it) {
                         const int s = (int)(it % kWStages);
                         if (!mbar_wait(&sm.smem_empty[s], ((it / kWStages) & 1u) ^ 1u, abort_flag, 1u)) goto role_done;
                         if (warp == 0) {
@@ -169,7 +197,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 uint32_t s = 0, ai = (uint32_t)h, ph = 0;
                 for (int tl = 0; tl < my_tiles; ++tl) {
                     if (!mbar_wait(&sm.acc_empty[h], ((uint32_t)tl & 1u) ^ 1u, abort_flag, 4u)) goto role_done;
-                    for (int kb = 0; kb < KB; ++kb) {
+                    for (int kb = kb0; kb < kb1; ++kb) {
                         // the unpack warps publish a slice only after the stage's TMA bytes (activation tile
                         // included) have landed, so this one wait covers both operands
                         if (!mbar_wait(&sm.a_full[ai], ph, abort_flag, 5u)) goto role_done;
@@ -178,7 +206,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                         const uint64_t bdesc = bdesc0 + (uint64_t)(s * (uint32_t)(kWBM * 128 / 16));
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
-                            tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc, (kb == 0 && j == 0) ? 0u : 1u);
+                            tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc, (kb == kb0 && j == 0) ? 0u : 1u);
                         tc_commit(&sm.a_empty[ai]);
                         tc_commit(&sm.smem_empty[s]);
                         if (++s == (uint32_t)kWStages) s = 0;
@@ -247,7 +275,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         [[maybe_unused]] const float off_factor = OFFSET ? offset_factor(p.ctl, p.zp_mid) : 0.0f;
         __half* stage = &sm.ystage[ew][0][0];
         for (int tl = 0; tl < my_tiles; ++tl) {
-            const int tile = (int)(blockIdx.x + tl * gridDim.x);
+            const int tile = tile_at(tl);
             const int mt = tile % p.n_tiles_m, np = tile / p.n_tiles_m;
             const int m_base = mt * kWBM + col0;
             float sc[2], off_pe[2];
@@ -258,6 +286,95 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 n_ok[h] = n < p.N;
                 sc[h] = __half2float(p.w_scales[n]) * 0.0625f * pe;      // sums carry a factor 16 (n < Npad: the scale array is padded)
                 off_pe[h] = (OFFSET && n_ok[h]) ? __fmul_rn(off_factor, p.chan_offset[n]) * pe : 0.0f;
+            }
+            if constexpr (CLUSTER) {
+                // run c of the tile's tokens belongs to CTA c * split / 8; the receiving area of a CTA is laid out as
+                // [sender][run of the slice][half][4 columns][channel][column]. The sums stay in tensor memory and are
+                // read once to be sent and once to be finished.
+                constexpr int kRun = BM / kWRuns, kRunInts = 2 * kRun * kTileN;
+                cg::cluster_group cluster = cg::this_cluster();
+                int* ring = reinterpret_cast<int*>(&sm.x[0][0]);
+                const int slice_runs = (kWRuns + split - 1) / split;     // the most a CTA owns
+                bool ok = true;
+                for (int h = 0; h < 2; ++h) ok = ok && mbar_wait_warp(&sm.acc_full[h], 0u, abort_flag, 8u);
+                tc_fence_after();
+                w_cluster_meet();                                        // every CTA's operand ring is idle
+                met = 1;
+                if (!ok) goto role_done;
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h)
+#pragma unroll 1
+                    for (int c0 = 0; c0 < kCols; c0 += 32) {
+                        uint32_t v[32];
+                        tc_ld32(tmem_acc + lane_addr + (uint32_t)(h * kWBM + col0 + c0), v);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const int c = (col0 + c0) / kRun + i, owner = (c * split) / kWRuns;
+                            if (owner == rank || mt * kWBM + c * kRun >= p.M) continue;
+                            const int first = (owner * kWRuns + split - 1) / split;      // the owner's first run
+                            const int from = rank < owner ? rank : rank - 1;
+                            int4* dst = reinterpret_cast<int4*>(cluster.map_shared_rank(ring, owner) +
+                                                                (size_t)(from * slice_runs + c - first) * kRunInts) + h * (kRun / 4) * kTileN + r;
+#pragma unroll
+                            for (int q = 0; q < kRun / 4; ++q)
+                                dst[q * kTileN] = make_int4((int)v[i * kRun + 4 * q], (int)v[i * kRun + 4 * q + 1],
+                                                            (int)v[i * kRun + 4 * q + 2], (int)v[i * kRun + 4 * q + 3]);
+                        }
+                    }
+                w_cluster_meet();                                        // all sums have arrived; nobody writes here any more
+                met = 2;
+#pragma unroll 1
+                for (int c = rank * kWRuns / split; c < kWRuns; ++c) {
+                    // (this warp's runs among those its CTA owns)
+                    if ((c * split) / kWRuns != rank || c * kRun < col0 || c * kRun >= col0 + kCols || mt * kWBM + c * kRun >= p.M) continue;
+                    const int first = (rank * kWRuns + split - 1) / split, m0 = mt * kWBM + c * kRun;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t v[kRun];
+                        tc_ld16(tmem_acc + lane_addr + (uint32_t)(h * kWBM + c * kRun), v);
+                        tc_wait_ld();
+                        for (int from = 0; from < split - 1; ++from) {
+                            const int4* src = reinterpret_cast<const int4*>(ring + (size_t)(from * slice_runs + c - first) * kRunInts) +
+                                              h * (kRun / 4) * kTileN + r;
+#pragma unroll
+                            for (int q = 0; q < kRun / 4; ++q) {
+                                const int4 o = src[q * kTileN];
+                                v[4 * q] += (uint32_t)o.x;
+                                v[4 * q + 1] += (uint32_t)o.y;
+                                v[4 * q + 2] += (uint32_t)o.z;
+                                v[4 * q + 3] += (uint32_t)o.w;
+                            }
+                        }
+                        const int n = (2 * np + h) * kTileN + r, n0 = (2 * np + h) * kTileN + quarter * 32;
+                        if (p.y_tma) {
+                            if (lane == 0) tma_store_wait_read();
+                            __syncwarp();
+                        }
+#pragma unroll
+                        for (int k = 0; k < kRun; ++k) {
+                            const __half hv = __float2half_rn(OFFSET ? fmaf((float)(int)v[k], sc[h], off_pe[h]) : (float)(int)v[k] * sc[h]);
+                            if (p.y_tma) {
+                                if constexpr (CHAIN)
+                                    w_stage_code(stage, k, lane, w_chain_code(hv, p.next_inv, p.next_lo, p.next_hi), p.next_packed);
+                                else
+                                    stage[k * 32 + lane] = hv;
+                            } else if (n_ok[h] && m0 + k < p.M) {
+                                if constexpr (CHAIN)
+                                    p.q_next[(size_t)(m0 + k) * p.N + n] = (int8_t)w_chain_code(hv, p.next_inv, p.next_lo, p.next_hi);
+                                else
+                                    p.y[(size_t)(m0 + k) * p.N + n] = hv;
+                            }
+                            if (p.acc_dump && n_ok[h] && m0 + k < p.M) p.acc_dump[(size_t)(m0 + k) * p.N + n] = (int)v[k] >> 4;
+                        }
+                        if (p.y_tma) {
+                            fence_proxy_async();
+                            __syncwarp();
+                            if (lane == 0 && n0 < p.N) tma_store_2d(&y_map, stage, (CHAIN && p.next_packed) ? n0 >> 1 : n0, m0);
+                        }
+                    }
+                }
+                goto role_done;
             }
             // One half after the other: the half's sums (this warp's columns) go to registers and its
             // accumulator returns to its issuer at once, so that conversion and stores overlap the next tile's MMAs.
@@ -322,6 +439,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 role_done:
     if (warp >= kWFirstEpi && lane == 0) tma_store_wait_read();   // staging rows live until read
     __syncwarp();
+    if constexpr (CLUSTER)
+        for (; met < 2; ++met) w_cluster_meet();                  // every warp comes to both meetings
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -339,12 +458,13 @@ typedef CUresult (*WEncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-template <int BM, bool OFFSET, bool CHAIN>
-cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+// Tiles in turn on a persistent grid, or one per cluster of `split` CTAs.
+template <int BM, bool OFFSET, bool CHAIN, bool CLUSTER>
+cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int split) {
     constexpr int kWBM = BM;
     const size_t smem_bytes = sizeof(WSmem<BM>) + 1024;
     static SmemOptIn opt_in;
-    if (const cudaError_t e = opt_in.ensure(gemm_wide_kernel<BM, OFFSET, CHAIN>, dev.device, smem_bytes); e != cudaSuccess)
+    if (const cudaError_t e = opt_in.ensure(gemm_wide_kernel<BM, OFFSET, CHAIN, CLUSTER>, dev.device, smem_bytes); e != cudaSuccess)
         return e;
     WEncodeTiledFn enc = reinterpret_cast<WEncodeTiledFn>(dev.encode_tiled);
     CUtensorMap map;
@@ -356,6 +476,7 @@ cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
+    const cuuint32_t store_rows = CLUSTER ? BM / kWRuns : kWStageRows;
     CUtensorMap ymap = map;   // placeholder when the store path is off
     int y_tma = 0;
     if (CHAIN) {
@@ -365,7 +486,7 @@ cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
             const cuuint64_t row_bytes = a.next_packed ? (cuuint64_t)a.N / 2 : (cuuint64_t)a.N;
             const cuuint64_t ydims[2] = {row_bytes, (cuuint64_t)a.M};
             const cuuint64_t ystrides[1] = {row_bytes};
-            const cuuint32_t ybox[2] = {a.next_packed ? 16u : 32u, (cuuint32_t)kWStageRows};
+            const cuuint32_t ybox[2] = {a.next_packed ? 16u : 32u, store_rows};
             if (enc(&ymap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, a.q_next, ydims, ystrides, ybox, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -375,7 +496,7 @@ cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     } else if (a.N % 8 == 0 && (reinterpret_cast<uintptr_t>(a.y) & 15u) == 0) {
         const cuuint64_t ydims[2] = {(cuuint64_t)a.N, (cuuint64_t)a.M};
         const cuuint64_t ystrides[1] = {(cuuint64_t)a.N * 2};
-        const cuuint32_t ybox[2] = {32u, (cuuint32_t)kWStageRows};
+        const cuuint32_t ybox[2] = {32u, store_rows};
         if (enc(&ymap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.y, ydims, ystrides, ybox, estr,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -395,51 +516,108 @@ cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     p.next_packed = a.next_packed ? 1 : 0;
     p.y_tma = y_tma;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(p.n_tiles < dev.sm_count ? p.n_tiles : dev.sm_count);
+    cfg.gridDim = CLUSTER ? dim3(split, p.n_tiles) : dim3(p.n_tiles < dev.sm_count ? p.n_tiles : dev.sm_count);
     cfg.blockDim = dim3(kWThreads);
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = a.after_quantize ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = split;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = a.after_quantize ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<BM, OFFSET, CHAIN>, map, ymap, p);
+    cfg.numAttrs = CLUSTER ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<BM, OFFSET, CHAIN, CLUSTER>, map, ymap, p);
 }
 
 }  // namespace
-
-bool gemm_wide_applies(const GemmArgs& a) {
-    return !a.group && a.M > 128 && (round_up(a.N, kTileN) / kTileN) % 2 == 0;
-}
 
 namespace {
-template <int BM>
-cudaError_t launch_wide_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    if (a.q_next) {
-        if (a.chan_offset) return cudaErrorInvalidValue;       // the two variants are not combined
-        return launch_wide_t<BM, false, true>(a, dev, stream);
+// Clusters of `split` CTAs that run at once (one CTA fills an SM; a GPC holds only so many clusters of a size).
+int wide_clusters(const DeviceInfo& dev, int split) {
+    static std::atomic<int> known[kMaxDevices][9];               // + 1 (0: not asked yet)
+    int k = known[dev.device][split].load(std::memory_order_relaxed);
+    if (k == 0) {
+        const size_t smem_bytes = sizeof(WSmem<128>) + 1024;
+        static SmemOptIn opt_in;
+        int n = 0;
+        if (opt_in.ensure(gemm_wide_kernel<128, false, false, true>, dev.device, smem_bytes) == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(split, 1);
+            cfg.blockDim = dim3(kWThreads);
+            cfg.dynamicSmemBytes = smem_bytes;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = split;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<128, false, false, true>, &cfg) != cudaSuccess) {
+                (void)cudaGetLastError();
+                n = 0;
+            }
+        }
+        k = n + 1;
+        known[dev.device][split].store(k, std::memory_order_relaxed);
     }
-    if (a.chan_offset) return launch_wide_t<BM, true, false>(a, dev, stream);
-    return launch_wide_t<BM, false, false>(a, dev, stream);
+    return k - 1;
+}
+
+// How a shape is run, and what it costs in cycles: rounds of tiles over the SMs x k blocks x the time of a k block, which
+// the L2 -> SM path sets (about 36 bytes per clock and SM measured in this kernel: 32 KB per k block on 128-token tiles,
+// 40 KB on 192-token tiles) unless the tensor pipe's 512 / 768 cycles are longer. 128-token tiles that are few enough
+// for all of them to run at once in clusters may do so: fewer k blocks in a row, at the 730 cycles of an SM that does
+// not share the path with all others, and the exchange. 333 rows, N = 5120 (60 tiles, clusters of two): K = 13824
+// 49.2 -> 35.3 us, K = 5120 23.2 -> 22.7 us; 48 rows: 45.3 -> 22.8 us, 22.5 -> 18.6 us. (Only the last, partial round in
+// clusters behind whole rounds: measured slower, K = 13824, N = 5120 at 1024 rows, 148 + 12 tiles, 68 us against 57.6
+// on 192-token tiles.)
+struct WidePlan {
+    int bm, split;                   // token tile; CTAs that share a tile
+    long cost;
+};
+WidePlan wide_plan(const GemmArgs& a, const DeviceInfo& dev) {
+    const int pairs = round_up(a.N, kTileN) / (2 * kTileN), KB = k_blocks(a.K), sms = dev.sm_count;
+    const int tiles192 = (a.M + 191) / 192 * pairs, tiles128 = (a.M + 127) / 128 * pairs;
+    WidePlan best = {192, 1, (long)((tiles192 + sms - 1) / sms) * KB * 1138};
+    const long cost128 = (long)((tiles128 + sms - 1) / sms) * KB * 910;
+    if (cost128 <= best.cost) best = {128, 1, cost128};
+    for (int s = 2; s <= 8 && s <= KB && s * tiles128 <= sms; ++s) {
+        if (wide_clusters(dev, s) < tiles128) continue;
+        const long c = (long)((KB + s - 1) / s + kExchangeBlocks) * 730;
+        if (c < best.cost) best = {128, s, c};
+    }
+    return best;
+}
+
+template <bool OFFSET, bool CHAIN>
+cudaError_t launch_wide_v(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+    const WidePlan w = wide_plan(a, dev);
+    if (w.bm == 192) return launch_wide_t<192, OFFSET, CHAIN, false>(a, dev, stream, 1);
+    if (w.split == 1) return launch_wide_t<128, OFFSET, CHAIN, false>(a, dev, stream, 1);
+    return launch_wide_t<128, OFFSET, CHAIN, true>(a, dev, stream, w.split);
 }
 }  // namespace
 
-// Token tile: rounds of tiles over the SMs x k blocks x the time of a k block, which the L2 -> SM path sets
-// (about 36 bytes per clock and SM measured in this kernel: 32 KB per k block on 128-token tiles, 40 KB on
-// 192-token tiles) unless the tensor pipe's 512 / 768 cycles are longer.
-int wide_token_tile(int M, int N, int sm_count) {
-    const long pairs = round_up(N, kTileN) / (2 * kTileN);
-    auto cost = [&](int bm, long unit_cycles) {
-        const long tiles = (long)((M + bm - 1) / bm) * pairs;
-        return ((tiles + sm_count - 1) / sm_count) * unit_cycles;
-    };
-    return cost(192, 1138) < cost(128, 910) ? 192 : 128;
+// Whether the pair tiles are the better choice: always from 129 rows on; below, where clusters of them beat the 64- or
+// 128-token tiles of one channel block (655 cycles a k block there).
+bool gemm_wide_applies(const GemmArgs& a, const DeviceInfo& dev) {
+    if (a.group || (round_up(a.N, kTileN) / kTileN) % 2 != 0) return false;
+    if (a.M > 128) return true;
+    const WidePlan w = wide_plan(a, dev);
+    const int tiles = round_up(a.N, kTileN) / kTileN;
+    return w.split > 1 && w.cost < (long)((tiles + dev.sm_count - 1) / dev.sm_count) * k_blocks(a.K) * 655;
 }
 
 cudaError_t launch_gemm_wide(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    return wide_token_tile(a.M, a.N, dev.sm_count) == 192 ? launch_wide_bm<192>(a, dev, stream)
-                                                          : launch_wide_bm<128>(a, dev, stream);
+    if (a.q_next) {
+        if (a.chan_offset) return cudaErrorInvalidValue;       // the two variants are not combined
+        return launch_wide_v<false, true>(a, dev, stream);
+    }
+    if (a.chan_offset) return launch_wide_v<true, false>(a, dev, stream);
+    return launch_wide_v<false, false>(a, dev, stream);
 }
 
 }  // namespace aq

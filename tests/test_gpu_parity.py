@@ -378,6 +378,33 @@ def test_one_scale_per_channel_on_tiles_of_two_channel_blocks(M, K, N):
     assert np.array_equal(gpu["acc"], ref["acc"]) and ref["acc"].max() == 128 * 7 * K
 
 
+@pytest.mark.parametrize("M,K,N", [(130, 1280, 256), (200, 13824, 512), (333, 5120, 5120), (300, 2048, 1016), (129, 416, 768),
+                                   (260, 4096, 250), (1000, 2048, 5120), (640, 8192, 1280), (40, 13824, 512), (100, 4096, 4096)])
+def test_pair_tiles_shared_by_clusters(M, K, N):
+    """One scale per channel where the tiles do not fill the GPU: clusters of two to eight CTAs share a tile's k blocks
+    (uneven ranges and token runs, ragged M and N, a K that ends inside a block; more tiles than SMs once). Sums and outputs as everywhere; plain, chained, packed and zero-point calls."""
+    x = inputs.activations(M, K, seed=M + K, outlier_frac=0.01, outlier_mult=20.0)
+    w = inputs.weights(N, K, seed=N + K)
+    gpu, ref = run_layer_both(x, w, 8, 0, binding.AQ_KERNEL_TENSOR)
+    assert gpu["e"] == ref["e"] and np.array_equal(gpu["q"], ref["q"])
+    assert np.array_equal(gpu["acc"], ref["acc"])
+    assert_y_close(gpu["y"], ref["y"])
+    h = handle()
+    packed, scales = h.aq_pack_w4(dev(w), 0)
+    y = h.aq_linear_w4a8(dev(x), packed, scales, N, 0).cpu().numpy()
+    assert np.array_equal(y.view(np.uint16), gpu["y"].view(np.uint16))
+    e_next = oracle.layer_exponent(y, 4) - 1
+    ref_next = oracle.quantize_act(y, 4, e_next)
+    assert np.array_equal(h.aq_linear_chain(8, dev(x), packed, scales, N, 0, 4, e_next).cpu().numpy(), ref_next)
+    if N % 32 == 0:
+        q4 = h.aq_linear_chain_act4(8, dev(x), packed, scales, N, 0, e_next)
+        assert np.array_equal(q4.cpu().numpy(), oracle.pack_act4(ref_next))
+    codes, sc = oracle.quantize_weights(w, 0)
+    e, zp = oracle.asym_params(x, 8)
+    ya = h.aq_linear_asym(8, dev(x), packed, scales, h.aq_weight_offsets(packed, scales, N, K, 0), N, 0).cpu().numpy()
+    assert_y_close(ya, oracle.linear_asym(oracle.quantize_act_asym(x, 8, e, zp), zp, codes, sc, e, 0)[1])
+
+
 @pytest.mark.parametrize("group", [0, 128])
 def test_several_tiles_per_cta_and_deep_k(group):
     """More tiles than SMs and more k blocks than any ring is deep: every ring and every
