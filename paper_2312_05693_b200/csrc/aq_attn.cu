@@ -353,6 +353,12 @@ constexpr int kConvWarps = 8;                        // warps that turn codes in
 constexpr int tc_threads(int ew, bool convert = false) { return (2 + ew + (convert ? kConvWarps : 0)) * 32; }
 constexpr unsigned long long kTcWaitCycles = 4000000000ull;
 
+// One thread of a converged warp: the compiler then knows that a copy or an MMA has one set of operands (see elect_one in aq_tc.cuh).
+__device__ __forceinline__ bool a_elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ uint32_t a_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ bool a_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
@@ -425,7 +431,7 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
     static_assert(2 * RT * DN <= 512, "two accumulator stages of RT x DN columns in tensor memory");
     constexpr int kRows = RT * 128;                                       // rows of A per item
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(attn_smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int MT = (M + kRows - 1) / kRows;                               // row tiles per head
     const int items = MT * H;                                             // work items; item w = (head w / MT, row tile w % MT)
     const int JB = (J + 127) / 128;
@@ -455,7 +461,7 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
     volatile uint32_t* abort_flag = &sm.abort_flag;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (a_elect_one()) {
             int it = 0;                                                   // stages filled so far, over all items
             bool ok = true;
             for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
@@ -478,7 +484,7 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (a_elect_one()) {
             // D = s32 (2 at bits 4-5), A unsigned 8-bit (0 at bits 7-9), B signed 8-bit (1 at bits 10-12),
             // both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28
             constexpr uint32_t idesc = (2u << 4) | ((A_SIGNED ? 1u : 0u) << 7) | (1u << 10) | ((uint32_t)(DN >> 3) << 17) |

@@ -58,7 +58,7 @@ struct Roles {
 template <int BM>
 struct TileConfig {
     // shared-memory ring depth: activation tile + packed weight block (+ scales) per stage
-    static constexpr int kNumStages = BM >= 192 ? 5 : 6;
+    static constexpr int kNumStages = BM >= 192 ? 5 : BM > 64 ? 7 : 12;
 };
 
 template <int BM, int EPI_WARPS>
@@ -173,7 +173,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
     constexpr int kColsPerEpiWarp = R::kColsPerEpiWarp;   // each quarter's columns are split between two or three warps
     static_assert(kColsPerEpiWarp % 16 == 0 && (!GROUPED || kColsPerEpiWarp % 32 == 0), "epilogue chunking");
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int KB = k_blocks(p.K);      // a last block that K does not fill: zero weight codes meet the tensor map's zero fill
     static_assert(!SPLIT || (GROUPED && !OFFSET && !CHAIN), "only the plain per-group kernel shares tiles");
     const int my_tiles = SPLIT ? 1
@@ -216,30 +216,47 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsControl));
       if (warp == 0 || warp == 2) {
         // ------------- TMA producers: warp 0 streams activation tiles, warp 2 weight blocks (+ scales)
-        if (lane == 0) {
+        if (elect_one()) {
             // Launched behind the call's own quantize kernel with programmatic stream serialization, this
             // grid is set up while that one drains: the codes (and, in the epilogue, the exponent and the
             // offsets) are touched only after it has completed; the weight producer does not wait. A no-op
             // for a normal launch.
-            if (warp == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-            uint32_t it = 0;
-            for (int tl = 0; tl < my_tiles; ++tl) {
-                const int tile = SPLIT ? p.split_base + ((int)blockIdx.x >> 1) : (int)(blockIdx.x + tl * gridDim.x);
-                const int mt = tile % p.n_tiles_m, nt = tile / p.n_tiles_m;
-                const uint8_t* wsrc = p.w_packed + (size_t)nt * KB * kBlockBytes;
-                for (int kb = kb_first; kb < kb_last; ++kb, ++it) {
-                    const int s = (int)(it % kNumStages);
-                    const uint32_t ph = (it / kNumStages) & 1u;
-                    if (!mbar_wait(&sm.smem_empty[s], ph ^ 1u, abort_flag, 1u)) goto role_done;
-                    if (warp == 0) {
-                        mbar_arrive_expect_tx(&sm.tma_full[s], BM * 128);
-                        tma_load_2d(sm.x[s], &x_map, kb * kTileK, mt * BM, &sm.tma_full[s]);
-                    } else {
-                        mbar_arrive_expect_tx(&sm.tma_full[s], kBlockBytes + (GROUPED ? kTileN * 2 : 0));
-                        tma_load_1d(sm.w[s], wsrc + (size_t)kb * kBlockBytes, kBlockBytes, &sm.tma_full[s]);
-                        if (GROUPED)
-                            tma_load_1d(sm.sc[it % Smem::kNumScaleSlots],
-                                        p.w_scales + (size_t)kb * p.Npad + nt * kTileN, kTileN * 2, &sm.tma_full[s]);
+            // Ring positions are carried in counters and addresses are shared-memory words: one thread whose every
+            // instruction waits for the one before paces this loop.
+            uint32_t st = 0, ph = 1u;
+            const uint32_t full0 = smem_u32(sm.tma_full), empty0 = smem_u32(sm.smem_empty);
+            if (warp == 0) {
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                const uint32_t x0 = smem_u32(sm.x[0]);
+                for (int tl = 0; tl < my_tiles; ++tl) {
+                    const int tile = SPLIT ? p.split_base + ((int)blockIdx.x >> 1) : (int)(blockIdx.x + tl * gridDim.x);
+                    const int m0 = tile % p.n_tiles_m * BM;
+                    for (int k = kb_first * kTileK; k < kb_last * kTileK; k += kTileK) {
+                        if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u)) goto role_done;
+                        mbar_arrive_expect_tx_a(full0 + 8u * st, BM * 128);
+                        tma_load_2d_a(x0 + st * (uint32_t)(BM * 128), &x_map, k, m0, full0 + 8u * st);
+                        if (++st == (uint32_t)kNumStages) { st = 0; ph ^= 1u; }
+                    }
+                }
+            } else {
+                const uint32_t w0 = smem_u32(sm.w[0]), sc0 = smem_u32(sm.sc[0]);
+                uint32_t slot = 0;
+                for (int tl = 0; tl < my_tiles; ++tl) {
+                    const int tile = SPLIT ? p.split_base + ((int)blockIdx.x >> 1) : (int)(blockIdx.x + tl * gridDim.x);
+                    const int nt = tile / p.n_tiles_m;
+                    const uint8_t* wsrc = p.w_packed + ((size_t)nt * KB + kb_first) * kBlockBytes;
+                    const __half* ssrc = p.w_scales + (size_t)kb_first * p.Npad + nt * kTileN;
+                    for (int kb = kb_first; kb < kb_last; ++kb) {
+                        if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u)) goto role_done;
+                        mbar_arrive_expect_tx_a(full0 + 8u * st, kBlockBytes + (GROUPED ? kTileN * 2 : 0));
+                        tma_load_1d_a(w0 + st * (uint32_t)kBlockBytes, wsrc, kBlockBytes, full0 + 8u * st);
+                        wsrc += kBlockBytes;
+                        if (GROUPED) {
+                            tma_load_1d_a(sc0 + slot * (uint32_t)(kTileN * 2), ssrc, kTileN * 2, full0 + 8u * st);
+                            ssrc += p.Npad;
+                            if (++slot == (uint32_t)Smem::kNumScaleSlots) slot = 0;
+                        }
+                        if (++st == (uint32_t)kNumStages) { st = 0; ph ^= 1u; }
                     }
                 }
             }
@@ -247,7 +264,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
       } else {
         // ------------- MMA issuers: warp 1 (and warp 3 in grouped mode, taking the odd k blocks)
         const int mma_id = warp >> 1;                  // 0 or 1
-        if (lane == 0 && mma_id < kNumMmaThreads) {
+        if (mma_id < kNumMmaThreads && elect_one()) {
             constexpr uint32_t idesc = idesc_i8(128, BM);
             const uint32_t total_iters = (uint32_t)my_tiles * (uint32_t)(kb_last - kb_first);
             if (GROUPED) {
@@ -280,29 +297,31 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                     if (ai >= (uint32_t)kNumASlices) { ai -= kNumASlices; a_ph ^= 1u; }
                 }
             } else {
-                uint32_t it = 0;
+                uint32_t st = 0, ai = 0, a_ph = 0u;
+                const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm.x[0]));
                 for (int tl = 0; tl < my_tiles; ++tl) {
                     const int a = (int)((uint32_t)tl % kNumAcc);
                     const uint32_t aph = ((uint32_t)tl / kNumAcc) & 1u;
                     if (!mbar_wait(&sm.acc_empty[a], aph ^ 1u, abort_flag, 4u)) goto role_done;
-                    for (int kb = 0; kb < KB; ++kb, ++it) {
-                        const int s = (int)(it % kNumStages);
-                        const int ai = (int)(it % kNumASlices);
+                    const uint32_t d_addr = tmem_acc + (uint32_t)(a * kAccStride);
+                    uint32_t accumulate = 0u;
+                    for (int kb = 0; kb < KB; ++kb) {
                         // the unpack warps publish a slice only after the stage's TMA bytes (activation
                         // tile included) have landed, so this one wait covers both operands
-                        if (!mbar_wait(&sm.a_full[ai], (it / kNumASlices) & 1u, abort_flag, 5u)) goto role_done;
+                        if (!mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 5u)) goto role_done;
                         tc_fence_after();
-                        const uint32_t d_addr = tmem_acc + (uint32_t)(a * kAccStride);
-                        const uint32_t a_addr = tmem_a + (uint32_t)(ai * kAColsPerStage);
-                        const uint64_t bdesc = smem_desc_sw128(smem_u32(sm.x[s]));
+                        const uint32_t a_addr = tmem_a + ai * (uint32_t)kAColsPerStage;
+                        const uint64_t bdesc = bdesc0 + (uint64_t)(st * (uint32_t)(BM * 128 / 16));
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             // 32 k per instruction: 8 TMEM columns of A, 32 bytes along the swizzled row of B
-                            tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc,
-                                         (kb == 0 && j == 0) ? 0u : 1u);
+                            tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc, accumulate);
+                            accumulate = 1u;
                         }
                         tc_commit(&sm.a_empty[ai]);
-                        tc_commit(&sm.smem_empty[s]);
+                        tc_commit(&sm.smem_empty[st]);
+                        if (++st == (uint32_t)kNumStages) st = 0;
+                        if (++ai == (uint32_t)kNumASlices) { ai = 0; a_ph ^= 1u; }
                     }
                     tc_commit(&sm.acc_full[a]);
                 }
@@ -321,12 +340,11 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         // With per-group rescaling the epilogue sets the pace (about four times the MMA time per k block) and
         // one group of unpack warps keeps up; the second group would only poll barriers on the schedulers
         // the epilogue warps issue from (measured: 1-2 % slower with it), so it leaves at once.
-        constexpr int kActiveGroups = GROUPED ? 1 : kUnpackGroups;
+        constexpr int kActiveGroups = GROUPED && BM > 64 ? 1 : kUnpackGroups;
         if (group >= kActiveGroups) goto role_done;
+        uint32_t s = (uint32_t)group, s_ph = 0u, ai = (uint32_t)group, a_ph = 1u;
         for (uint32_t it = group; it < total_iters; it += kActiveGroups) {
-            const int s = (int)(it % kNumStages);
-            const int ai = (int)(it % kNumASlices);
-            if (!mbar_wait_warp(&sm.tma_full[s], (it / kNumStages) & 1u, abort_flag, 6u)) goto role_done;
+            if (!mbar_wait_warp(&sm.tma_full[s], s_ph, abort_flag, 6u)) goto role_done;
             const uint4* src = reinterpret_cast<const uint4*>(sm.w[s]) + r;
             uint4 d[4];
 #pragma unroll
@@ -337,7 +355,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm.a_full[pending]);
             }
-            if (!mbar_wait_warp(&sm.a_empty[ai], ((it / kNumASlices) & 1u) ^ 1u, abort_flag, 7u)) goto role_done;
+            if (!mbar_wait_warp(&sm.a_empty[ai], a_ph, abort_flag, 7u)) goto role_done;
             tc_fence_after();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -350,7 +368,11 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 }
                 tc_st8(tmem_a + lane_addr + (uint32_t)(ai * kAColsPerStage + 8 * j), v);
             }
-            pending = ai;
+            pending = (int)ai;
+            s += kActiveGroups;
+            if (s >= (uint32_t)kNumStages) { s -= kNumStages; s_ph ^= 1u; }
+            ai += kActiveGroups;
+            if (ai >= (uint32_t)kNumASlices) { ai -= kNumASlices; a_ph ^= 1u; }
         }
         if (pending >= 0) {
             tc_wait_st();
@@ -601,7 +623,7 @@ struct ProbeSmem {
 __global__ void __launch_bounds__(128, 1) int8_probe_kernel(int iters, int a_from_tmem, Control* ctl) {
     extern __shared__ uint8_t smem_raw[];
     ProbeSmem& sm = *reinterpret_cast<ProbeSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     uint32_t* words = reinterpret_cast<uint32_t*>(sm.a);
     for (int i = threadIdx.x; i < (int)(sizeof(sm.a) + sizeof(sm.b)) / 4; i += blockDim.x) {
         uint32_t v = (uint32_t)i * 2654435761u + blockIdx.x * 40503u;       // any bytes will do
@@ -638,7 +660,7 @@ __global__ void __launch_bounds__(128, 1) int8_probe_kernel(int iters, int a_fro
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && elect_one()) {
         constexpr uint32_t idesc = idesc_i8(128, 256);
         constexpr int kBatch = 32;
         const uint64_t adesc = smem_desc_sw128(smem_u32(sm.a)), bdesc = smem_desc_sw128(smem_u32(sm.b));

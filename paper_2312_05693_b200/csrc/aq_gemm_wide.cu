@@ -115,7 +115,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int kWBM = BM, kWStages = WCfg<BM>::kStages, kWSlices = WCfg<BM>::kSlices, kWAccCols = WCfg<BM>::kAccCols;
     constexpr int kCols = WCfg<BM>::kCols;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int KB = p.KB;
     static_assert(!CLUSTER || BM == 128, "runs of 16 tokens");
     const int rank = CLUSTER ? (int)blockIdx.x : 0, split = CLUSTER ? (int)gridDim.x : 1;
@@ -158,26 +158,36 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWRegsControl));
         if (warp == 0 || warp == 2) {
             // ------------- TMA producers
-            if (lane == 0) {
-                // behind the call's own quantize kernel (programmatic stream serialization) the codes are
-                // touched only after that grid has completed; the weight producer does not wait
-                if (warp == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-                uint32_t it = 0;
-                for (int tl = 0; tl < my_tiles; ++tl) {
-                    const int tile = tile_at(tl);
-                    const int mt = tile % p.n_tiles_m, np = tile / p.n_tiles_m;
-                    const uint8_t* wsrc0 = p.w_packed + (size_t)(2 * np) * KB * kBlockBytes;
-                    const uint8_t* wsrc1 = wsrc0 + (size_t)KB * kBlockBytes;
-                    for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                        const int s = (int)(it % kWStages);
-                        if (!mbar_wait(&sm.smem_empty[s], ((it / kWStages) & 1u) ^ 1u, abort_flag, 1u)) goto role_done;
-                        if (warp == 0) {
-                            mbar_arrive_expect_tx(&sm.tma_full[s], kWBM * 128);
-                            tma_load_2d(sm.x[s], &x_map, kb * kTileK, mt * kWBM, &sm.tma_full[s]);
-                        } else {
-                            mbar_arrive_expect_tx(&sm.tma_full[s], 2 * kBlockBytes);
-                            tma_load_1d(sm.w[s][0], wsrc0 + (size_t)kb * kBlockBytes, kBlockBytes, &sm.tma_full[s]);
-                            tma_load_1d(sm.w[s][1], wsrc1 + (size_t)kb * kBlockBytes, kBlockBytes, &sm.tma_full[s]);
+            if (elect_one()) {
+                uint32_t st = 0, ph = 1u;
+                const uint32_t full0 = smem_u32(sm.tma_full), empty0 = smem_u32(sm.smem_empty);
+                if (warp == 0) {
+                    // behind the call's own quantize kernel (programmatic stream serialization) the codes are
+                    // touched only after that grid has completed; the weight producer does not wait
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    const uint32_t x0 = smem_u32(sm.x[0]);
+                    for (int tl = 0; tl < my_tiles; ++tl) {
+                        const int m0 = tile_at(tl) % p.n_tiles_m * kWBM;
+                        for (int k = kb0 * kTileK; k < kb1 * kTileK; k += kTileK) {
+                            if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u)) goto role_done;
+                            mbar_arrive_expect_tx_a(full0 + 8u * st, kWBM * 128);
+                            tma_load_2d_a(x0 + st * (uint32_t)(kWBM * 128), &x_map, k, m0, full0 + 8u * st);
+                            if (++st == (uint32_t)kWStages) { st = 0; ph ^= 1u; }
+                        }
+                    }
+                } else {
+                    const uint32_t w0 = smem_u32(sm.w[0][0]);
+                    for (int tl = 0; tl < my_tiles; ++tl) {
+                        const int np = tile_at(tl) / p.n_tiles_m;
+                        const uint8_t* src = p.w_packed + ((size_t)(2 * np) * KB + kb0) * kBlockBytes;
+                        for (int kb = kb0; kb < kb1; ++kb) {
+                            if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u)) goto role_done;
+                            mbar_arrive_expect_tx_a(full0 + 8u * st, 2 * kBlockBytes);
+                            const uint32_t dst = w0 + st * (uint32_t)(2 * kBlockBytes);
+                            tma_load_1d_a(dst, src, kBlockBytes, full0 + 8u * st);
+                            tma_load_1d_a(dst + kBlockBytes, src + (size_t)KB * kBlockBytes, kBlockBytes, full0 + 8u * st);
+                            src += kBlockBytes;
+                            if (++st == (uint32_t)kWStages) { st = 0; ph ^= 1u; }
                         }
                     }
                 }
@@ -185,7 +195,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         } else {
             // ------------- MMA issuers: warp 1 = channel half 0, warp 3 = half 1
             const int h = warp >> 1;
-            if (lane == 0) {
+            if (elect_one()) {
                 // Ring positions and phases are carried in counters: this thread's chain of look, four MMAs and commits
                 // is the pace of a CTA that has its SM's L2 path to itself (without the divisions K = 13824, N = 5120 at
                 // 333 rows 51.4 -> 49.2 us, K = 5120, N = 13824 at 1024 rows 57.7 -> 55.6 us). Also built and measured:
@@ -225,11 +235,9 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         const int r = quarter * 32 + lane;            // row inside the half's 128-channel block = TMEM lane
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         int pending = -1;                             // slice whose stores have been issued but not published
+        uint32_t s = 0, s_ph = 0u, ai = (uint32_t)h, a_ph = 1u;
         for (uint32_t it = 0; it < total_iters; ++it) {
-            const int s = (int)(it % kWStages);
-            const uint32_t u = it * 2u + (uint32_t)h;
-            const int ai = (int)(u % kWSlices);
-            if (!mbar_wait_warp(&sm.tma_full[s], (it / kWStages) & 1u, abort_flag, 6u)) goto role_done;
+            if (!mbar_wait_warp(&sm.tma_full[s], s_ph, abort_flag, 6u)) goto role_done;
             const uint4* src = reinterpret_cast<const uint4*>(sm.w[s][h]) + r;
             uint4 d[4];
 #pragma unroll
@@ -240,7 +248,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm.a_full[pending]);
             }
-            if (!mbar_wait_warp(&sm.a_empty[ai], ((u / kWSlices) & 1u) ^ 1u, abort_flag, 7u)) goto role_done;
+            if (!mbar_wait_warp(&sm.a_empty[ai], a_ph, abort_flag, 7u)) goto role_done;
             tc_fence_after();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -253,7 +261,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 }
                 tc_st8(tmem_a + lane_addr + (uint32_t)(ai * kAColsPerStage + 8 * j), v);
             }
-            pending = ai;
+            pending = (int)ai;
+            if (++s == (uint32_t)kWStages) { s = 0; s_ph ^= 1u; }
+            ai += 2;
+            if (ai >= (uint32_t)kWSlices) { ai -= kWSlices; a_ph ^= 1u; }
         }
         if (pending >= 0) {
             tc_wait_st();
