@@ -15,11 +15,12 @@
 // One persistent CTA per SM walks a static list of (channel tile, token tile) pairs.
 // Warp roles: 0 and 2 = TMA producers (activations / weights), 1 and 3 = MMA issuers (warp 1
 // also owns the TMEM allocation; warp 3 only works in per-group mode), 4-11 = weight unpack
-// (two groups of four taking alternate k blocks; only the first group works in per-group mode),
+// (two groups of four taking alternate k blocks; only the first group works in per-group mode above 64 tokens),
 // 12-19 = epilogue; registers are moved from
-// the first two roles to the epilogue with setmaxnreg. One thread spends about 55 cycles per
-// MMA instruction and about 100 per TMA instruction, which is why issue is spread over
-// threads and why the tile is 256 tokens wide where tensor memory allows it. Two (one scale per channel)
+// the first two roles to the epilogue with setmaxnreg. The issuing threads are chosen with elect.sync: then the
+// compiler knows that one thread is active, and a k block's four MMAs and three commits take about 100 cycles of
+// it, a producer's turn about 300. Behind `lane == 0` they took 500 each, and that, not memory or the tensor
+// cores, was the pace of every shape with few tokens. Two (one scale per channel)
 // or three (per-group scales) accumulator stages in TMEM let the epilogue of one
 // accumulation overlap the MMAs of the next ones. Every wait is bounded; on expiry the CTA records a status
 // word, stops issuing work and leaves through the common exit that frees TMEM.
@@ -58,6 +59,9 @@ struct Roles {
 template <int BM>
 struct TileConfig {
     // shared-memory ring depth: activation tile + packed weight block (+ scales) per stage
+    // (64 tokens: a turn of the ring, from the copy's issue to the MMA's commit, takes about 3500 cycles. Twelve stages,
+    // both unpack groups and elected issuers: a layer of 48 rows 4096 x 4096 18.6 -> 14.3 us, 4096 x 11008 19.0 -> 15.0 us,
+    // 11008 x 4096 27.4 -> 21.9 us; with one scale per channel, 4096 x 4224, 17.4 -> 11.6 us.)
     static constexpr int kNumStages = BM >= 192 ? 5 : BM > 64 ? 7 : 12;
 };
 
@@ -337,8 +341,8 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const uint32_t total_iters = (uint32_t)my_tiles * (uint32_t)(kb_last - kb_first);
         int pending = -1;                             // slice whose store has been issued but not published
-        // With per-group rescaling the epilogue sets the pace (about four times the MMA time per k block) and
-        // one group of unpack warps keeps up; the second group would only poll barriers on the schedulers
+        // With per-group rescaling and more than 64 tokens the epilogue sets the pace (about four times the MMA time per
+        // k block) and one group of unpack warps (about 500 cycles a block) keeps up; the second group would only poll barriers on the schedulers
         // the epilogue warps issue from (measured: 1-2 % slower with it), so it leaves at once.
         constexpr int kActiveGroups = GROUPED && BM > 64 ? 1 : kUnpackGroups;
         if (group >= kActiveGroups) goto role_done;

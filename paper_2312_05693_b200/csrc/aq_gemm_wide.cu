@@ -196,11 +196,9 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             // ------------- MMA issuers: warp 1 = channel half 0, warp 3 = half 1
             const int h = warp >> 1;
             if (elect_one()) {
-                // Ring positions and phases are carried in counters: this thread's chain of look, four MMAs and commits
-                // is the pace of a CTA that has its SM's L2 path to itself (without the divisions K = 13824, N = 5120 at
-                // 333 rows 51.4 -> 49.2 us, K = 5120, N = 13824 at 1024 rows 57.7 -> 55.6 us). Also built and measured:
-                // slices freed by the stage's own barrier, so that a commit goes, and the unpack warps loading a block
-                // ahead: 47.0 and 54 us, but 0.8 % slower in a loop of large layers under the power cap.
+                // One thread's chain of look, four MMAs and commits: elected threads, and ring positions and phases in counters,
+                // here and in the producers (K = 5120, N = 13824 at 1024 rows 55.6 -> 47.4 us; K = 13824, N = 5120 at 333 rows,
+                // in clusters, 35.3 -> 31.1 us).
                 constexpr uint32_t idesc = idesc_i8(128, kWBM);
                 const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm.x[0]));
                 const uint32_t d_addr = tmem_acc + (uint32_t)(h * kWBM);

@@ -14,7 +14,8 @@ constexpr int kAColsPerStage = 32;            // 128 k of int8 = 32 TMEM columns
 constexpr unsigned long long kWaitCycles = 4000000000ull;   // ~2 s
 
 // ------------------------------------------------------------------------- PTX wrappers
-// One thread of a converged warp.
+// One thread of a converged warp. Copies, MMAs and commits take uniform operands: behind elect.sync the compiler knows that
+// there is one thread's set of them (behind `lane == 0` it does not, and each such instruction costs some 100 cycles more).
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
