@@ -194,6 +194,12 @@ __device__ __forceinline__ bool str_try_wait(uint64_t* bar, uint32_t parity) {
         : "=r"(ok) : "r"(s_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
+// One thread of a converged warp: the compiler then knows that a copy has one set of operands (see elect_one in aq_tc.cuh).
+__device__ __forceinline__ bool s_elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 // Bounded wait; false when the limit ran out or another thread of the CTA already gave up.
 __device__ __forceinline__ bool str_wait(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
     if (str_try_wait(bar, parity)) return true;
@@ -213,17 +219,10 @@ __device__ __forceinline__ bool str_wait(uint64_t* bar, uint32_t parity, volatil
 // loads are free of bank conflicts.
 // Ring depth 8 (64 KB of weights in flight per CTA, two CTAs per SM): 9 stages for 16 rows and 12 for one
 // row, which shared memory would allow, measured no faster.
-// Producer lanes: a wait, an expect and two copies per block are four shared-memory-pipe instructions of a
-// hundred cycles and more each next to the working consumers, so one lane cannot issue faster than a block
-// per ~500 cycles, which bounds a CTA that streams alone on its SM. With two lanes of the warp in lockstep
-// (lane l takes the blocks l, l + 2, ... of the k range) the single-row kernel gains 0.3-1.1 us per launch;
-// four lanes gain no more, eight lose, and with 16 rows (tensor-map copies of the codes) two lanes measured
-// 0.1-0.3 us slower than one.
 template <int MB> struct StreamCfg {
     static constexpr bool kUseMma = MB > 4;
     static constexpr int kRows = MB;
     static constexpr int kStages = 8;
-    static constexpr int kProdLanes = kUseMma ? 1 : 2;
     // Consumer warps: a channel quarter each, kPhases warps per quarter taking the k blocks in turn. A third
     // warp per quarter measured slower with 16 rows (7.6 / 11.4 / 13.6 -> 8.5 / 12.0 / 14.4 us on the 13B
     // shapes) although a warp holds a block for 600-700 cycles there: the stream slows with the amount of
@@ -343,7 +342,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     constexpr int kStrConsumerWarps = StreamCfg<MB>::kConsumerWarps;
     constexpr int kStrThreads = StreamCfg<MB>::kThreads;
     cg::cluster_group cluster = cg::this_cluster();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int KB = k_blocks(p.K);
     const int rank = blockIdx.x, split = gridDim.x;
     const int tile = blockIdx.y;
@@ -410,15 +409,15 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     // promise that nothing in flight writes the weights, the weights are fetched first. With that promise
     // the launch behind this one is also allowed from the start, so that its CTAs take the places of this
     // grid's CTAs as they leave and have their first ring on the way while this grid finishes.
-    // The producer is kProdLanes lanes of warp 0 in lockstep, lane l taking the blocks l, l + kProdLanes, ...
-    constexpr int kProdLanes = StreamCfg<MB>::kProdLanes;
-    const bool producer = warp == 0 && lane < kProdLanes;
+    // The producer is one elected thread of warp 0 (a block per about 250 cycles; behind `lane == 0` about 500, which two lanes
+    // in lockstep had halved for the single-row kernel). M = 1 layers on 5120 x 5120 / 13824 x 5120 (K x N) 6.9 / 10.6 ->
+    // 6.4 / 10.2 us, M = 16 on 3072 x 768 6.4 -> 6.3 us.
     const int ring = min(kStrStages, kb1 - kb0);      // blocks of the first ring
     int issued = 0;
     if (p.early_dependents) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (p.early_weights) {     // behind this call's own quantize kernel, or the caller has promised stable weights
-        if (producer)
-            for (int i = lane; i < ring; i += kProdLanes) issue_w(kb0 + i, i);
+        if (warp == 0 && s_elect_one())
+            for (int i = 0; i < ring; ++i) issue_w(kb0 + i, i);
         issued = ring;
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -426,8 +425,8 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     [[maybe_unused]] int fused_exp = 0;
     if constexpr (FUSEQ) {
         // ---- the layer scale and this CTA's codes (Eq. 1, Eq. 2 / Eq. 5 with zp = 0; one scale for the layer)
-        if (producer)
-            for (int i = issued + lane; i < ring; i += kProdLanes) issue_w(kb0 + i, i);   // weights on their way meanwhile
+        if (warp == 0 && s_elect_one())
+            for (int i = issued; i < ring; ++i) issue_w(kb0 + i, i);   // weights on their way meanwhile
         issued = ring;
         const uint4* xv = reinterpret_cast<const uint4*>(p.x_row + (p.row_idx ? (size_t)p.row_idx[0] * p.K : 0));
         int e = p.clip_shift_or_exp;
@@ -502,9 +501,9 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
         __syncthreads();
     }
     if (warp == 0) {
-        if (producer) {
-            for (int i = lane; i < issued; i += kProdLanes) issue_x(kb0 + i, i);
-            for (int kb = kb0 + issued + lane; kb < kb1; kb += kProdLanes) {
+        if (s_elect_one()) {
+            for (int i = 0; i < issued; ++i) issue_x(kb0 + i, i);
+            for (int kb = kb0 + issued; kb < kb1; ++kb) {
                 const uint32_t i = (uint32_t)(kb - kb0);
                 const int s = (int)(i % kStrStages);
                 if (!str_wait(&sm.empty[s], ((i / kStrStages) & 1u) ^ 1u, abort_flag)) break;
