@@ -70,17 +70,16 @@ Workspace carve(void* ws, int M, int K, int N, size_t total_bytes) {
     return w;
 }
 
-// Up to 32 rows the streaming kernel: the tensor-core kernels' tiles of 128 channels are too few for the GPU there
-// (K = N = 4096, per-group scales: 20.7 -> 9.4 us at 17 rows, 21.2 -> 10.1 us at 32; K = N = 1024, 24 rows 10.4 -> 4.9
-// us). Beyond, two more 16-row tiles of the warp-level MMA cost more than that on wide layers (48 rows, K = 4096,
-// N = 11008: 28.8 against 21.9 us). It has no dump of per-group sums, which takes the tensor-core kernel.
-int kernel_for(aq_handle_t h, int M, bool group_dump) {
+// Up to 16 rows the streaming kernel. Beyond, its second 16-row tile of the warp-level MMA costs more than the tensor-core
+// kernels' tiles of 128 channels in clusters (layers of 20 rows, K = N = 5120 11.5 against 10.5 us; of 32 rows 12.3 / 11.0 us,
+// K = 5120, N = 13824 18.8 / 13.0 us, K = 11008, N = 4096 in groups of 128 22.2 / 16.3 us).
+int kernel_for(aq_handle_t h, int M) {
     const int choice = h->kernel_choice;
-    return choice == AQ_KERNEL_AUTO ? (M <= 16 || (M <= kFewRows && !group_dump) ? AQ_KERNEL_DECODE : AQ_KERNEL_TENSOR) : choice;
+    return choice == AQ_KERNEL_AUTO ? (M <= 16 ? AQ_KERNEL_DECODE : AQ_KERNEL_TENSOR) : choice;
 }
 
 int run_gemm(aq_handle_t h, const GemmArgs& g, cudaStream_t stream) {
-    const int choice = kernel_for(h, g.M, g.group && g.acc_dump);
+    const int choice = kernel_for(h, g.M);
     GemmArgs a = g;
     a.weights_stable = h->weights_stable != 0;
     const cudaError_t e = choice == AQ_KERNEL_DECODE ? launch_gemm_decode(a, h->dev, stream)
@@ -129,7 +128,7 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     if (alpha && !aligned(alpha, 16)) return AQ_ERR_ALIGNMENT;
     cudaError_t e = cudaSuccess;
     // a single row on the few-row kernel: that kernel finds the scale and makes the codes itself
-    const bool fuse = !w_offsets && !alpha && kernel_for(h, M, group && acc_dump) == AQ_KERNEL_DECODE &&
+    const bool fuse = !w_offsets && !alpha && kernel_for(h, M) == AQ_KERNEL_DECODE &&
                       decode_can_fuse_quantize(M, K, N, group, acc_dump != nullptr, h->dev.sm_count) &&
                       (!group || aligned(w_scales, 16));
     if (fuse) {
@@ -379,11 +378,7 @@ int aq_gemm_w4(aq_handle_t h, const int8_t* q, int M, int K, const void* w_packe
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const Workspace w = carve(workspace, M, K, N, workspace_bytes_);
-    if (kernel_for(h, M, group_size && acc_dump) == AQ_KERNEL_TENSOR) {       // the decode kernels clear the status word themselves
-        const cudaError_t e = cudaMemsetAsync(w.ctl, 0, sizeof(Control), stream);
-        if (e != cudaSuccess) return cuda_fail(h, e);
-    }
-    GemmArgs g;
+    GemmArgs g;                    // the kernels clear the status word themselves
     g.q = q; g.M = M; g.K = K; g.N = N; g.group = group_size;
     g.w_packed = static_cast<const uint8_t*>(w_packed);
     g.w_scales = static_cast<const __half*>(w_scales);

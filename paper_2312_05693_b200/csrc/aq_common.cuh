@@ -224,13 +224,13 @@ void handle_record_cuda_error(aq_handle_t h, cudaError_t e);
 
 cudaError_t launch_gemm_tensor(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 // One scale per channel on tiles of 256 channels x 128 tokens (aq_gemm_wide.cu), for shapes it applies to.
-bool gemm_wide_applies(const GemmArgs& a, const DeviceInfo& dev);
+bool gemm_wide_applies(const GemmArgs& a, const DeviceInfo& dev, long other);
 cudaError_t launch_gemm_wide(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 // Bytes of split_scratch the tensor kernel can use for these sizes on a GPU with sm_count SMs (0: none).
 size_t tensor_split_scratch_bytes(int M, int K, int N, int group, int sm_count);
 // Tensor-core rate probe: every SM issues iters x 4 MMAs of 128 x 256 x 32 (int8) on resident operands.
 cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const DeviceInfo& dev, cudaStream_t stream);
-constexpr int kFewRows = 32;         // rows up to which AQ_KERNEL_AUTO takes the few-row kernels
+constexpr int kFewRows = 32;         // rows up to which the streaming kernel runs (AQ_KERNEL_AUTO takes it up to 16)
 cudaError_t launch_gemm_decode(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, int sm_count);
 

@@ -24,10 +24,13 @@
 // or three (per-group scales) accumulator stages in TMEM let the epilogue of one
 // accumulation overlap the MMAs of the next ones. Every wait is bounded; on expiry the CTA records a status
 // word, stops issuing work and leaves through the common exit that frees TMEM.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "aq_common.cuh"
 #include "aq_tc.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace aq {
 
@@ -41,12 +44,12 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kRegsControl = 40, kRegsUnpack = 48;
 // The warps behind the control warpgroup are unpack warps, then epilogue warps. Eight epilogue warps (two per
 // TMEM lane quarter, half of the token columns each) follow two groups of unpack warps; the per-group
-// kernels with 96- or 192-token tiles run twelve (three per quarter, a third of the columns each) behind
+// kernels with 192-token tiles run twelve (three per quarter, a third of the columns each) behind
 // the one unpack group they need: there the per-group rescaling sets the pace, and a third warp per
 // scheduler hides the latency of the other two's barrier and tensor-memory round trips.
 template <int BM, bool GROUPED>
 struct Roles {
-    static constexpr int kEpiWarps = (GROUPED && (BM == 96 || BM == 192)) ? 12 : 8;
+    static constexpr int kEpiWarps = (GROUPED && BM == 192) ? 12 : 8;
     static constexpr int kFirstEpiWarp = kWarps - kEpiWarps;
     static constexpr int kRegsEpilogue = kEpiWarps == 12 ? 128 : 168;
     static constexpr int kColsPerEpiWarp = BM / (kEpiWarps / 4);
@@ -107,6 +110,7 @@ struct TensorParams {
     float next_inv, next_lo, next_hi;   // 2^-next_exp and the code range of the next layer
     int next_packed;               // chaining: 4-bit codes leave two per byte (even channel in the low nibble)
     int y_tma;                     // outputs leave through y_map (needs N % 8 == 0 and a 16-byte aligned y)
+    int clear_status;              // no quantize kernel of the call has set the control block up
 };
 
 // One column of this thread's row, waited for.
@@ -148,8 +152,12 @@ __device__ __forceinline__ void stage_code(__half* stage, int c, int lane, int c
 // change with them. SPLIT (per-group scales only): the launch covers the tiles of a last, partial round;
 // every tile is shared by two CTAs that take half of the k range each, leave fp32 partial sums in
 // scratch, and whichever epilogue warp arrives second adds the other's sums and writes the outputs
-// (nobody waits).
-template <int BM, bool GROUPED, bool OFFSET, bool CHAIN, bool SPLIT = false>
+// (nobody waits). CLUSTER: tiles so few that all of them run at once in clusters of two to eight
+// CTAs (up to a few hundred rows on narrow layers). The CTAs of a cluster share a tile and take consecutive ranges of its
+// k blocks; every epilogue warp sends the sums (fp32 with per-group scales, otherwise integers) of the token runs that
+// another CTA finishes into that CTA's operand ring (idle by then), the cluster meets, and each adds what it received to
+// its own in the order of the senders' ranks.
+template <int BM, bool GROUPED, bool OFFSET, bool CHAIN, bool SPLIT = false, bool CLUSTER = false>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap y_map,
                    const TensorParams p) {
@@ -163,7 +171,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
     // accumulator stages in tensor memory: three for per-group rescaling, otherwise as many
     // 2 (or 1 for the 256-token tile) as leave room for the weight-slice ring
     constexpr int kNumAcc = GROUPED ? (BM > 128 ? 2 : 3) : (BM >= 256 ? 1 : 2);
-    constexpr int kAccStride = BM == 96 ? 128 : BM;   // columns between accumulator stages
+    constexpr int kAccStride = BM;                    // columns between accumulator stages
     constexpr int kNumMmaThreads = GROUPED ? 2 : 1;   // issuers alternate k blocks when every block has its own accumulator
     constexpr int kAccCols = kNumAcc * kAccStride;
     // the rest of tensor memory (up to 8 slices) is the ring of unpacked weight slices (A operand)
@@ -180,13 +188,20 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int KB = k_blocks(p.K);      // a last block that K does not fill: zero weight codes meet the tensor map's zero fill
     static_assert(!SPLIT || (GROUPED && !OFFSET && !CHAIN), "only the plain per-group kernel shares tiles");
-    const int my_tiles = SPLIT ? 1
+    static_assert(!CLUSTER || (!SPLIT && BM <= 192), "what a CTA receives fits its operand ring");
+    const int rank = CLUSTER ? (int)blockIdx.x : 0, split = CLUSTER ? (int)gridDim.x : 1;
+    [[maybe_unused]] int met = 0;                    // CLUSTER: meetings this warp has been to
+    auto tile_at = [&](int tl) {
+        return CLUSTER ? (int)blockIdx.y : SPLIT ? p.split_base + ((int)blockIdx.x >> 1) : (int)(blockIdx.x + tl * gridDim.x);
+    };
+    const int my_tiles = SPLIT || CLUSTER ? 1
                                : (p.n_tiles > (int)blockIdx.x
                                       ? (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0);
-    // the k blocks of a work item: all of them, or one half when the tile is shared
-    const int kb_first = SPLIT ? (((int)blockIdx.x & 1) ? KB / 2 : 0) : 0;
-    const int kb_last = SPLIT ? (((int)blockIdx.x & 1) ? KB : KB / 2) : KB;
+    // the k blocks of a work item: all of them, or a range of them when the tile is shared
+    const int kb_first = CLUSTER ? KB * rank / split : SPLIT ? (((int)blockIdx.x & 1) ? KB / 2 : 0) : 0;
+    const int kb_last = CLUSTER ? KB * (rank + 1) / split : SPLIT ? (((int)blockIdx.x & 1) ? KB : KB / 2) : KB;
 
+    if (p.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) p.ctl->status = 0;   // nothing has given up yet
     if (threadIdx.x == 0) {
         for (int s = 0; s < kNumStages; ++s) {
             mbar_init(&sm.tma_full[s], 2);
@@ -233,7 +248,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 const uint32_t x0 = smem_u32(sm.x[0]);
                 for (int tl = 0; tl < my_tiles; ++tl) {
-                    const int tile = SPLIT ? p.split_base + ((int)blockIdx.x >> 1) : (int)(blockIdx.x + tl * gridDim.x);
+                    const int tile = tile_at(tl);
                     const int m0 = tile % p.n_tiles_m * BM;
                     for (int k = kb_first * kTileK; k < kb_last * kTileK; k += kTileK) {
                         if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u)) goto role_done;
@@ -246,7 +261,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 const uint32_t w0 = smem_u32(sm.w[0]), sc0 = smem_u32(sm.sc[0]);
                 uint32_t slot = 0;
                 for (int tl = 0; tl < my_tiles; ++tl) {
-                    const int tile = SPLIT ? p.split_base + ((int)blockIdx.x >> 1) : (int)(blockIdx.x + tl * gridDim.x);
+                    const int tile = tile_at(tl);
                     const int nt = tile / p.n_tiles_m;
                     const uint8_t* wsrc = p.w_packed + ((size_t)nt * KB + kb_first) * kBlockBytes;
                     const __half* ssrc = p.w_scales + (size_t)kb_first * p.Npad + nt * kTileN;
@@ -309,7 +324,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                     if (!mbar_wait(&sm.acc_empty[a], aph ^ 1u, abort_flag, 4u)) goto role_done;
                     const uint32_t d_addr = tmem_acc + (uint32_t)(a * kAccStride);
                     uint32_t accumulate = 0u;
-                    for (int kb = 0; kb < KB; ++kb) {
+                    for (int kb = kb_first; kb < kb_last; ++kb) {
                         // the unpack warps publish a slice only after the stage's TMA bytes (activation
                         // tile included) have landed, so this one wait covers both operands
                         if (!mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 5u)) goto role_done;
@@ -398,8 +413,54 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         [[maybe_unused]] const int G = GROUPED ? KB : 1;
         uint32_t unit = 0;
         [[maybe_unused]] uint32_t g_a = 0, g_ph = 0, g_slot = 0;   // per-group mode: accumulator stage, its parity, scale slot
+        // CLUSTER: a warp's columns in runs of four tokens, run c finished by CTA c * split / kRuns; a CTA receives (its own share
+        // too) at [sender][epilogue warp][run of its slice][lane], four tokens of a channel (16 bytes) a slot, in its operand
+        // ring. The loops over a CTA's own runs are rolled: this code runs once, and what it costs is mostly fetching it
+        // (with the runs unrolled K = N = 4096 at 200 rows took 1.4 us longer).
+        constexpr int kRuns = kColsPerEpiWarp / 4, kSlot = kEpiWarps * 512, kRing = kNumStages * (BM * 128 + kBlockBytes);
+        static_assert(!CLUSTER || (2 * kSlot * ((kRuns + 1) / 2) <= kRing && 3 * kSlot * ((kRuns + 2) / 3) <= kRing &&
+                                   4 * kSlot * ((kRuns + 3) / 4) <= kRing && 5 * kSlot * ((kRuns + 4) / 5) <= kRing &&
+                                   6 * kSlot * ((kRuns + 5) / 6) <= kRing && 7 * kSlot * ((kRuns + 6) / 7) <= kRing &&
+                                   8 * kSlot * ((kRuns + 7) / 8) <= kRing),
+                      "the operand ring (activation tiles, then weight blocks) holds what a CTA receives");
+        [[maybe_unused]] const int slice_runs = (kRuns + split - 1) / split;
+        [[maybe_unused]] const int run_first = (rank * kRuns + split - 1) / split, run_last = ((rank + 1) * kRuns + split - 1) / split;
+        [[maybe_unused]] uint4* ring = reinterpret_cast<uint4*>(&sm) + (warp - kFirstEpiWarp) * slice_runs * 32 + lane;
+        [[maybe_unused]] auto send_run = [&](int c, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+            const int owner = (c * split) / kRuns, first = (owner * kRuns + split - 1) / split;
+            *(cg::this_cluster().map_shared_rank(ring, owner) + (rank * kEpiWarps * slice_runs + c - first) * 32) = make_uint4(v0, v1, v2, v3);
+        };
+        [[maybe_unused]] auto whole_run = [&](int c) {
+            uint4 o = ring[(c - run_first) * 32];
+#pragma unroll 1
+            for (int from = 1; from < split; ++from) {
+                const uint4 g = ring[(from * kEpiWarps * slice_runs + c - run_first) * 32];
+                if (GROUPED) {
+                    o.x = __float_as_uint(__uint_as_float(o.x) + __uint_as_float(g.x));
+                    o.y = __float_as_uint(__uint_as_float(o.y) + __uint_as_float(g.y));
+                    o.z = __float_as_uint(__uint_as_float(o.z) + __uint_as_float(g.z));
+                    o.w = __float_as_uint(__uint_as_float(o.w) + __uint_as_float(g.w));
+                } else {
+                    o.x += g.x; o.y += g.y; o.z += g.z; o.w += g.w;
+                }
+            }
+            return o;
+        };
+        // ... and the output of one token of such a run (all lanes of the warp together)
+        [[maybe_unused]] auto put = [&](int m, int n, bool n_ok, __half hv) {
+            if constexpr (CHAIN) {
+                const int code = chain_code(hv, p.next_inv, p.next_lo, p.next_hi);
+                const int hi = __shfl_down_sync(0xFFFFFFFFu, code, 1);
+                if (n_ok && m < p.M) {
+                    if (!p.next_packed) p.q_next[(size_t)m * p.N + n] = (int8_t)code;
+                    else if (!(lane & 1)) p.q_next[((size_t)m * p.N + n) >> 1] = (int8_t)((code & 0xF) | (hi << 4));
+                }
+            } else if (n_ok && m < p.M) {
+                p.y[(size_t)m * p.N + n] = hv;
+            }
+        };
         for (int tl = 0; tl < my_tiles; ++tl) {
-            const int tile = SPLIT ? p.split_base + ((int)blockIdx.x >> 1) : (int)(blockIdx.x + tl * gridDim.x);
+            const int tile = tile_at(tl);
             const int mt = tile % p.n_tiles_m, nt = tile / p.n_tiles_m;
             const int n = nt * kTileN + r;
             const int m_base = mt * BM + col0;
@@ -422,6 +483,26 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm.acc_empty[a]);
+                if constexpr (CLUSTER) {
+                    cluster_meet();                                      // every CTA's operand ring is idle
+#pragma unroll
+                    for (int c = 0; c < kRuns; ++c)
+                        if (m_base + 4 * c < p.M) send_run(c, v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                    cluster_meet();                                      // all sums have arrived; nobody writes here any more
+                    met = 2;
+#pragma unroll 1
+                    for (int c = run_first; c < run_last && m_base + 4 * c < p.M; ++c) {
+                        const uint4 o = whole_run(c);
+                        const int sums[4] = {(int)o.x, (int)o.y, (int)o.z, (int)o.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int m = m_base + 4 * c + i;
+                            put(m, n, n_ok, __float2half_rn(OFFSET ? fmaf((float)sums[i], sc, off_pe) : (float)sums[i] * sc));
+                            if (p.acc_dump && n_ok && m < p.M) p.acc_dump[(size_t)m * p.N + n] = sums[i] >> 4;
+                        }
+                    }
+                    goto role_done;
+                }
                 if (p.y_tma) {
                     __half* stage = &sm.ystage[warp - kFirstEpiWarp][0][0];
                     const int n0 = nt * kTileN + quarter * 32;
@@ -537,6 +618,26 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                         for (int c = 0; c < kColsPerEpiWarp; ++c) fsum[c] += __ldcg(other + c * 32 + lane);
                     }
                 }
+                if constexpr (CLUSTER) {
+                    cluster_meet();
+#pragma unroll
+                    for (int c = 0; c < kRuns; ++c)
+                        if (m_base + 4 * c < p.M)
+                            send_run(c, __float_as_uint(fsum[4 * c]), __float_as_uint(fsum[4 * c + 1]), __float_as_uint(fsum[4 * c + 2]),
+                                     __float_as_uint(fsum[4 * c + 3]));
+                    cluster_meet();
+                    met = 2;
+                    const float off_n = OFFSET && n_ok ? __fmul_rn(off_factor, p.chan_offset[n]) : 0.0f;
+#pragma unroll 1
+                    for (int c = run_first; c < run_last && m_base + 4 * c < p.M; ++c) {
+                        const uint4 o = whole_run(c);
+                        const float sums[4] = {__uint_as_float(o.x), __uint_as_float(o.y), __uint_as_float(o.z), __uint_as_float(o.w)};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            put(m_base + 4 * c + i, n, n_ok, __float2half_rn((OFFSET ? sums[i] + off_n : sums[i]) * pe));
+                    }
+                    goto role_done;
+                }
                 if constexpr (OFFSET) {                                  // read after the k loop
                     const float off_n = n_ok ? __fmul_rn(off_factor, p.chan_offset[n]) : 0.0f;
 #pragma unroll
@@ -583,6 +684,8 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
 role_done:
     if (warp >= kFirstEpiWarp && lane == 0) tma_store_wait_read();   // staging rows live until read
     __syncwarp();
+    if constexpr (CLUSTER)
+        for (; met < 2; ++met) cluster_meet();                       // every warp comes to both meetings
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -705,21 +808,98 @@ inline bool round_is_shared(int rem, int sms, int k_blocks, int bm) {
     return rem > 0 && 2 * rem <= sms && k_blocks >= split_min_k_blocks(bm) && rem <= Control::kMaxSplitTiles;
 }
 
-// Token tile of the per-group kernels. Up to 64 tokens: 64. Otherwise 128 (eight epilogue warps, three
-// accumulator stages) or 192 (twelve epilogue warps, two stages), whichever gives the shorter schedule:
+// Clusters of `split` CTAs that run at once (one CTA fills an SM; a GPC holds only so many of a size).
+template <int BM, bool GROUPED>
+int tile_clusters(const DeviceInfo& dev, int split) {
+    static std::atomic<int> known[kMaxDevices][9];               // + 1 (0: not asked yet)
+    int k = known[dev.device][split].load(std::memory_order_relaxed);
+    if (k == 0) {
+        const size_t smem_bytes = sizeof(SharedStorage<BM, Roles<BM, GROUPED>::kEpiWarps>) + 1024;
+        auto kernel = gemm_tensor_kernel<BM, GROUPED, false, false, false, true>;
+        static SmemOptIn opt_in;
+        int n = 0;
+        if (opt_in.ensure(kernel, dev.device, smem_bytes) == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(split, 1);
+            cfg.blockDim = dim3(kThreads);
+            cfg.dynamicSmemBytes = smem_bytes;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = split;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+                (void)cudaGetLastError();
+                n = 0;
+            }
+        }
+        k = n + 1;
+        known[dev.device][split].store(k, std::memory_order_relaxed);
+    }
+    return k - 1;
+}
+
+// How a per-group product is run: token tile and CTAs that share a tile. Up to 64 tokens the tile is 64. Otherwise 128 (eight
+// epilogue warps, three accumulator stages) or 192 (twelve epilogue warps, two stages), whichever gives the shorter schedule:
 // rounds of tiles over the SMs (a shared last round counts half) x tile height x the measured cost per
-// token column and k block (about 7.6 cycles with 128-token tiles, 6.6 with 192-token tiles).
-int grouped_token_tile(int M, int K, int N, int sms, bool may_share) {
-    if (M <= 64) return 64;
-    const int kbs = K / kTileK, n_tiles_n = round_up(N, kTileN) / kTileN;
-    auto cost = [&](int bm, float per_col) {
+// token column and k block (about 7.6 cycles with 128-token tiles, 6.6 with 192-token tiles, 9 with 64-token tiles).
+// Tiles few enough for all of them to run at once in clusters do so when the k blocks saved outweigh the exchange (layers of
+// 48 rows, K x N = 4096 x 4096 14.3 -> 10.8 us, 11008 x 4096 21.9 -> 15.7 us, 5120 x 5120 17.6 -> 13.3 us; of 128 rows,
+// 11008 x 4096 30.9 -> 22.5 us; but 48 rows, 1024 x 4096 7.1 -> 8.3 us, left alone). They also replaced shared tiles where those made up the
+// whole launch (333 rows, 4096 x 4096 23.1 -> 21.3 us).
+struct GroupedPlan {
+    int bm, split;
+};
+constexpr float kExchangeCycles = 4500.0f, kSharedRoundCycles = 2500.0f;
+GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_share, bool clusters) {
+    const int kbs = K / kTileK, n_tiles_n = round_up(N, kTileN) / kTileN, sms = dev.sm_count;
+    GroupedPlan best = {64, 1};
+    float best_cost = 3.0e38f;
+    auto consider = [&](int bm, float per_col) {
         const long tiles = (long)((M + bm - 1) / bm) * n_tiles_n;
         const long rounds = tiles / sms;
         const int rem = (int)(tiles % sms);
-        const float last = rem == 0 ? 0.0f : (may_share && round_is_shared(rem, sms, kbs, bm) ? 0.5f : 1.0f);
-        return ((float)rounds + last) * (float)bm * per_col;
+        const bool halves = may_share && rounds > 0 && round_is_shared(rem, sms, kbs, bm);
+        const float last = rem == 0 ? 0.0f : halves ? 0.5f : 1.0f;
+        const float block = (float)bm * per_col, plain = ((float)rounds + last) * (float)kbs * block + (halves ? kSharedRoundCycles : 0.0f);
+        if (plain < best_cost) { best_cost = plain; best = {bm, 1}; }
+        if (!clusters) return;
+        for (int s = 2; s <= 8 && s <= kbs && s * tiles <= sms; ++s) {
+            const float shared = (float)((kbs + s - 1) / s) * block + kExchangeCycles;
+            if (shared >= best_cost) continue;
+            const int fit = bm == 64 ? tile_clusters<64, true>(dev, s) : bm == 128 ? tile_clusters<128, true>(dev, s) : tile_clusters<192, true>(dev, s);
+            if (fit >= tiles) { best_cost = shared; best = {bm, s}; }
+        }
     };
-    return cost(192, 6.6f) < cost(128, 7.6f) ? 192 : 128;
+    if (M <= 64) {
+        consider(64, 9.0f);
+    } else {
+        consider(128, 7.6f);
+        consider(192, 6.6f);
+    }
+    return best;
+}
+
+// One scale per channel, tiles of one channel block: 64 tokens up to 64 rows, 128 up to 128 rows, or more while the tiles
+// fill one round; in clusters where the k blocks saved outweigh the exchange (cycles as above).
+struct ChannelPlan {
+    int bm, split;
+    long cost;
+};
+constexpr int kNarrow64 = 420, kNarrow128 = 600;     // cycles per k block
+ChannelPlan channel_plan(int M, int K, int N, const DeviceInfo& dev) {
+    const int KB = k_blocks(K), sms = dev.sm_count, bm = M <= 64 ? 64 : 128, block = M <= 64 ? kNarrow64 : kNarrow128;
+    const long tiles = (long)((M + bm - 1) / bm) * (round_up(N, kTileN) / kTileN);
+    if (M > 128 && tiles > sms) return {256, 1, 0x7fffffffL};
+    ChannelPlan best = {bm, 1, (tiles + sms - 1) / sms * KB * block};
+    for (int s = 2; s <= 8 && s <= KB && s * tiles <= sms; ++s) {
+        const long c = (long)((KB + s - 1) / s) * block + (long)kExchangeCycles;
+        if (c >= best.cost) continue;
+        if ((bm == 64 ? tile_clusters<64, false>(dev, s) : tile_clusters<128, false>(dev, s)) >= tiles) best = {bm, s, c};
+    }
+    return best;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -727,13 +907,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 // tile_limit >= 0: only the first tile_limit tiles (whole rounds). SPLIT: the tiles from split_base on, two CTAs each.
-template <int BM, bool GROUPED, bool OFFSET, bool CHAIN, bool SPLIT = false>
+// CLUSTER: one tile per cluster of `cluster` CTAs.
+template <int BM, bool GROUPED, bool OFFSET, bool CHAIN, bool SPLIT = false, bool CLUSTER = false>
 cudaError_t launch_off(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int tile_limit = -1,
-                       int split_base = 0, int split_tiles = 0) {
+                       int split_base = 0, int split_tiles = 0, int cluster = 1) {
     using Smem = SharedStorage<BM, Roles<BM, GROUPED>::kEpiWarps>;
     const size_t smem_bytes = sizeof(Smem) + 1024;
     static SmemOptIn opt_in;
-    if (const cudaError_t e = opt_in.ensure(gemm_tensor_kernel<BM, GROUPED, OFFSET, CHAIN, SPLIT>, dev.device, smem_bytes);
+    if (const cudaError_t e = opt_in.ensure(gemm_tensor_kernel<BM, GROUPED, OFFSET, CHAIN, SPLIT, CLUSTER>, dev.device, smem_bytes);
         e != cudaSuccess)
         return e;
     CUtensorMap map;
@@ -793,6 +974,7 @@ cudaError_t launch_off(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t st
     if (tile_limit >= 0) p.n_tiles = tile_limit;
     p.split_base = split_base;
     p.split_scratch = a.split_scratch;
+    p.clear_status = !a.after_quantize && split_base == 0 ? 1 : 0;
     const int grid = SPLIT ? 2 * split_tiles : (p.n_tiles < dev.sm_count ? p.n_tiles : dev.sm_count);
     if constexpr (SPLIT) {
         // This launch depends on nothing the preceding whole-round launch writes (other tiles of y; the
@@ -805,7 +987,7 @@ cudaError_t launch_off(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t st
         cfg.stream = stream;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = split_base > 0 ? 1 : 0;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, gemm_tensor_kernel<BM, GROUPED, OFFSET, CHAIN, SPLIT>, map, ymap, p);
@@ -813,28 +995,37 @@ cudaError_t launch_off(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t st
         // Behind the call's own quantize kernel the launch may overlap that kernel's drain (the kernel
         // waits for it before it reads what it wrote).
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid);
+        cfg.gridDim = CLUSTER ? dim3(cluster, p.n_tiles) : dim3(grid);
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = smem_bytes;
         cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[0].val.programmaticStreamSerializationAllowed = a.after_quantize ? 1 : 0;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = cluster;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = a.after_quantize ? 1 : 0;
-        return cudaLaunchKernelEx(&cfg, gemm_tensor_kernel<BM, GROUPED, OFFSET, CHAIN, SPLIT>, map, ymap, p);
+        cfg.numAttrs = CLUSTER ? 2 : 1;
+        return cudaLaunchKernelEx(&cfg, gemm_tensor_kernel<BM, GROUPED, OFFSET, CHAIN, SPLIT, CLUSTER>, map, ymap, p);
     }
 }
 
 template <int BM, bool GROUPED>
-cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    if (a.q_next) {
-        if (a.chan_offset) return cudaErrorInvalidValue;       // the two variants are not combined
-        return launch_off<BM, GROUPED, false, true>(a, dev, stream);
+cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int cluster = 1) {
+    if (a.q_next && a.chan_offset) return cudaErrorInvalidValue;       // the two variants are not combined
+    if constexpr (BM <= 192) {
+        if (cluster > 1) {
+            if (a.q_next) return launch_off<BM, GROUPED, false, true, false, true>(a, dev, stream, -1, 0, 0, cluster);
+            if (a.chan_offset) return launch_off<BM, GROUPED, true, false, false, true>(a, dev, stream, -1, 0, 0, cluster);
+            return launch_off<BM, GROUPED, false, false, false, true>(a, dev, stream, -1, 0, 0, cluster);
+        }
     }
+    if (a.q_next) return launch_off<BM, GROUPED, false, true>(a, dev, stream);
     if (a.chan_offset) return launch_off<BM, GROUPED, true, false>(a, dev, stream);
     if constexpr (GROUPED) {
-        // A last round that would leave more than half of the SMs idle is run as shared tiles, when the
+        // Behind whole rounds: a last round that would leave more than half of the SMs idle is run as shared tiles, when the
         // reduction is deep enough for half a tile to outweigh the second launch and the exchange of
         // partial sums (measured with 128-token tiles: a loss of 2-5 us at K = 4096, a gain of 8 us at
         // K = 11008; with 192-token tiles a gain of 2 us at K = 4096 already).
@@ -842,12 +1033,14 @@ cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t str
         const int n_tiles = ((a.M + BM - 1) / BM) * (round_up(a.N, kTileN) / kTileN);
         const int rounds = n_tiles / sms, rem = n_tiles % sms;
         const size_t need = (size_t)rem * 2 * BM * kTileN * sizeof(float);
-        if (round_is_shared(rem, sms, a.K / kTileK, BM) && a.split_scratch &&
+        if (rounds > 0 && round_is_shared(rem, sms, a.K / kTileK, BM) && a.split_scratch &&
             a.split_bytes >= need && (reinterpret_cast<uintptr_t>(a.split_scratch) & 15u) == 0) {
-            if (rounds > 0) {
-                const cudaError_t e = launch_off<BM, true, false, false>(a, dev, stream, rounds * sms);
+            if (!a.after_quantize) {
+                const cudaError_t e = cudaMemsetAsync(a.ctl->split_flags, 0, sizeof(a.ctl->split_flags), stream);
                 if (e != cudaSuccess) return e;
             }
+            const cudaError_t e = launch_off<BM, true, false, false>(a, dev, stream, rounds * sms);
+            if (e != cudaSuccess) return e;
             return launch_off<BM, true, false, false, true>(a, dev, stream, -1, rounds * sms, rem);
         }
     }
@@ -858,7 +1051,9 @@ cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t str
 
 size_t tensor_split_scratch_bytes(int M, int K, int N, int group, int sm_count) {
     if (!group) return 0;
-    const int bm = grouped_token_tile(M, K, N, sm_count, true);
+    DeviceInfo dev = {};
+    dev.sm_count = sm_count;
+    const int bm = grouped_plan(M, K, N, dev, true, false).bm;     // the most that the plan with clusters uses
     const int n_tiles = ((M + bm - 1) / bm) * (round_up(N, kTileN) / kTileN);
     const int rem = n_tiles % sm_count;
     if (!round_is_shared(rem, sm_count, K / kTileK, bm)) return 0;
@@ -874,20 +1069,23 @@ cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const De
 }
 
 cudaError_t launch_gemm_tensor(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    // one scale per channel: two channel blocks share a token tile where the shape allows it
-    if (gemm_wide_applies(a, dev)) return launch_gemm_wide(a, dev, stream);
-    if (a.M <= 64) return a.group ? launch_bm<64, true>(a, dev, stream) : launch_bm<64, false>(a, dev, stream);
     if (a.group) {
         // the chained and zero-point variants have no shared-tile launch
-        switch (grouped_token_tile(a.M, a.K, a.N, dev.sm_count, !a.q_next && !a.chan_offset)) {
-            case 96: return launch_bm<96, true>(a, dev, stream);
-            case 192: return launch_bm<192, true>(a, dev, stream);
-            default: return launch_bm<128, true>(a, dev, stream);
+        const GroupedPlan g = grouped_plan(a.M, a.K, a.N, dev, !a.q_next && !a.chan_offset, true);
+        switch (g.bm) {
+            case 64: return launch_bm<64, true>(a, dev, stream, g.split);
+            case 192: return launch_bm<192, true>(a, dev, stream, g.split);
+            default: return launch_bm<128, true>(a, dev, stream, g.split);
         }
     }
-    // one scale per channel: the 256-token tile halves the MMA instructions per unit of work
-    if (a.M <= 128) return launch_bm<128, false>(a, dev, stream);
-    return launch_bm<256, false>(a, dev, stream);
+    // one scale per channel: two channel blocks share a token tile where the shape allows it and that is the shorter schedule
+    const ChannelPlan c = channel_plan(a.M, a.K, a.N, dev);
+    if (gemm_wide_applies(a, dev, c.cost)) return launch_gemm_wide(a, dev, stream);
+    switch (c.bm) {
+        case 64: return launch_bm<64, false>(a, dev, stream, c.split);
+        case 128: return launch_bm<128, false>(a, dev, stream, c.split);
+        default: return launch_bm<256, false>(a, dev, stream);    // halves the MMA instructions per unit of work
+    }
 }
 
 }  // namespace aq

@@ -75,6 +75,7 @@ struct WParams {
     float next_inv, next_lo, next_hi;
     int next_packed;
     int y_tma;
+    int clear_status;              // no quantize kernel of the call has set the control block up
 };
 
 __device__ __forceinline__ int w_chain_code(__half hv, float inv, float lo, float hi) {
@@ -100,10 +101,6 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16]) {
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void w_cluster_meet() {
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
 
 // OFFSET: add the per-channel term of the zero-point variant. CHAIN: write the next layer's codes instead
 // of fp16 outputs.
@@ -125,6 +122,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     auto tile_at = [&](int tl) { return CLUSTER ? (int)blockIdx.y : (int)(blockIdx.x + tl * gridDim.x); };
     [[maybe_unused]] int met = 0;                    // CLUSTER: meetings this warp has been to
 
+    if (p.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) p.ctl->status = 0;   // nothing has given up yet
     if (threadIdx.x == 0) {
         for (int s = 0; s < kWStages; ++s) {
             mbar_init(&sm.tma_full[s], 2);
@@ -307,7 +305,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 bool ok = true;
                 for (int h = 0; h < 2; ++h) ok = ok && mbar_wait_warp(&sm.acc_full[h], 0u, abort_flag, 8u);
                 tc_fence_after();
-                w_cluster_meet();                                        // every CTA's operand ring is idle
+                cluster_meet();                                        // every CTA's operand ring is idle
                 met = 1;
                 if (!ok) goto role_done;
 #pragma unroll 1
@@ -331,7 +329,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                                                             (int)v[i * kRun + 4 * q + 2], (int)v[i * kRun + 4 * q + 3]);
                         }
                     }
-                w_cluster_meet();                                        // all sums have arrived; nobody writes here any more
+                cluster_meet();                                        // all sums have arrived; nobody writes here any more
                 met = 2;
 #pragma unroll 1
                 for (int c = rank * kWRuns / split; c < kWRuns; ++c) {
@@ -449,7 +447,7 @@ role_done:
     if (warp >= kWFirstEpi && lane == 0) tma_store_wait_read();   // staging rows live until read
     __syncwarp();
     if constexpr (CLUSTER)
-        for (; met < 2; ++met) w_cluster_meet();                  // every warp comes to both meetings
+        for (; met < 2; ++met) cluster_meet();                  // every warp comes to both meetings
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -524,6 +522,7 @@ cudaError_t launch_wide_t(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     p.next_hi = (float)((1 << (a.next_bits - 1)) - 1);
     p.next_packed = a.next_packed ? 1 : 0;
     p.y_tma = y_tma;
+    p.clear_status = a.after_quantize ? 0 : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = CLUSTER ? dim3(split, p.n_tiles) : dim3(p.n_tiles < dev.sm_count ? p.n_tiles : dev.sm_count);
     cfg.blockDim = dim3(kWThreads);
@@ -610,14 +609,11 @@ cudaError_t launch_wide_v(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
 }
 }  // namespace
 
-// Whether the pair tiles are the better choice: always from 129 rows on; below, where clusters of them beat the 64- or
-// 128-token tiles of one channel block (655 cycles a k block there).
-bool gemm_wide_applies(const GemmArgs& a, const DeviceInfo& dev) {
+// Whether the pair tiles are the better choice: where their schedule is no longer than `other`, that of the tiles of one
+// channel block (in cycles).
+bool gemm_wide_applies(const GemmArgs& a, const DeviceInfo& dev, long other) {
     if (a.group || (round_up(a.N, kTileN) / kTileN) % 2 != 0) return false;
-    if (a.M > 128) return true;
-    const WidePlan w = wide_plan(a, dev);
-    const int tiles = round_up(a.N, kTileN) / kTileN;
-    return w.split > 1 && w.cost < (long)((tiles + dev.sm_count - 1) / dev.sm_count) * k_blocks(a.K) * 655;
+    return wide_plan(a, dev).cost <= other;
 }
 
 cudaError_t launch_gemm_wide(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {

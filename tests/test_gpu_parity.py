@@ -405,6 +405,35 @@ def test_pair_tiles_shared_by_clusters(M, K, N):
     assert_y_close(ya, oracle.linear_asym(oracle.quantize_act_asym(x, 8, e, zp), zp, codes, sc, e, 0)[1])
 
 
+@pytest.mark.parametrize("M,K,N,group", [(33, 1280, 200, 128), (64, 11008, 512, 128), (49, 4096, 4096, 128), (65, 2048, 2048, 128),
+                                         (128, 5120, 1016, 128), (190, 4096, 4096, 128), (333, 4096, 4096, 128), (129, 13824, 250, 128),
+                                         (17, 416, 136, 0), (33, 1024, 384, 0), (64, 13824, 5120, 0), (47, 5120, 5120, 0),
+                                         (65, 4096, 1152, 0), (128, 2048, 1000, 0), (200, 2048, 2048, 0), (333, 5120, 5120, 0)])
+def test_tiles_of_one_channel_block_shared_by_clusters(M, K, N, group):
+    """Clusters of two to eight CTAs share the k blocks of a 64-, 128- or 192-token tile of one channel block (uneven ranges and
+    token runs, ragged M and N, a K that ends inside a block): sums, plain, chained, packed and zero-point outputs."""
+    x = inputs.activations(M, K, seed=M + K, outlier_frac=0.01, outlier_mult=20.0)
+    w = inputs.weights(N, K, seed=N + K)
+    gpu, ref = run_layer_both(x, w, 8, group, binding.AQ_KERNEL_TENSOR)
+    assert gpu["e"] == ref["e"] and np.array_equal(gpu["q"], ref["q"])
+    assert np.array_equal(gpu["acc"], ref["acc"])
+    assert_y_close(gpu["y"], ref["y"])
+    h = handle()
+    packed, scales = h.aq_pack_w4(dev(w), group)
+    y = h.aq_linear_w4a8(dev(x), packed, scales, N, group).cpu().numpy()
+    assert_y_close(y, ref["y"])
+    e_next = oracle.layer_exponent(y, 4) - 1
+    ref_next = oracle.quantize_act(y, 4, e_next)
+    assert np.array_equal(h.aq_linear_chain(8, dev(x), packed, scales, N, group, 4, e_next).cpu().numpy(), ref_next)
+    if N % 32 == 0:
+        q4 = h.aq_linear_chain_act4(8, dev(x), packed, scales, N, group, e_next)
+        assert np.array_equal(q4.cpu().numpy(), oracle.pack_act4(ref_next))
+    codes, sc = oracle.quantize_weights(w, group)
+    e, zp = oracle.asym_params(x, 8)
+    ya = h.aq_linear_asym(8, dev(x), packed, scales, h.aq_weight_offsets(packed, scales, N, K, group), N, group).cpu().numpy()
+    assert_y_close(ya, oracle.linear_asym(oracle.quantize_act_asym(x, 8, e, zp), zp, codes, sc, e, group)[1])
+
+
 @pytest.mark.parametrize("group", [0, 128])
 def test_several_tiles_per_cta_and_deep_k(group):
     """More tiles than SMs and more k blocks than any ring is deep: every ring and every
