@@ -341,7 +341,7 @@ def bench_zero_point(h, reps=30):
     ms = _event_ms(step, reps)
     ops = sum(2.0 * M * s.K * s.N for s in wl.shapes)
     return {"workload": wl.name + " with zero point", "ms_per_step": ms, "TOPS": ops / (ms * 1e-3) / 1e12,
-            "note": "one cooperative quantize kernel (min/max, e and zp, codes) plus the per-channel term"}
+            "note": "range and quantize kernels (min/max; e, zp and codes); the per-channel term in the product kernel"}
 
 
 def bench_chain(h, reps=30):
@@ -801,9 +801,9 @@ def main():
                 "h2d_bytes_per_step": int(sum(M * s.K * 2 for s in wl.shapes)),
                 "d2h_bytes_per_step": int(sum(M * s.N * 2 for s in wl.shapes)),
                 "ms_per_step": e2e_ms, "api": "aq_linear_host_async, one stream per layer"},
-        # per layer: the fused quantize kernel and the product kernel, which is two launches where the tiles of a
+        # per layer: the range and quantize kernels and the product kernel, which is two launches where the tiles of a
         # partial last round are shared between CTA pairs (the workspace then has room for their partial sums)
-        "gpu_launches": args.steps * sum(2 + (binding.aq_workspace_bytes(M, s.K, s.N, wl.group_size) >
+        "gpu_launches": args.steps * sum(3 + (binding.aq_workspace_bytes(M, s.K, s.N, wl.group_size) >
                                               binding.aq_workspace_bytes(M, s.K, s.N, 0)) for s in wl.shapes),
         "clocks": clocks,
         "roofline": roofline,
