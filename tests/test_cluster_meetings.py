@@ -1,0 +1,47 @@
+"""A CTA may write into another CTA's shared memory only once that CTA has started, so every kernel that maps a peer's
+shared memory has to wait for its cluster before it does. Read off the sources: the race cannot be provoked."""
+import glob
+import os
+import re
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_2312_05693_b200", "csrc")
+WAIT = re.compile(r"barrier\.cluster\.wait|cluster_started_wait\(\)|cluster_meet\(\)|cluster\.sync\(\)")
+
+
+def kernels():
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        for part in open(path).read().split("__global__")[1:]:
+            part = re.sub(r"//[^\n]*", "", part)
+            if "map_shared_rank" in part:
+                yield pytest.param(part, id=re.search(r"(\w+_kernel)\(", part).group(1))
+
+
+@pytest.mark.parametrize("body", list(kernels()))
+def test_remote_stores_come_behind_a_wait_for_the_cluster(body):
+    first = body.index("map_shared_rank")
+    helper = re.search(r"auto (\w+) = \[&\]\([^)]*\) \{[^{}]*map_shared_rank", body)     # a store inside a lambda counts where it is called
+    if helper:
+        first = body.index(helper.group(1) + "(", helper.end())
+    assert WAIT.search(body, 0, first), "stores into a peer's shared memory before the cluster is known to have started"
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,K", [(1, 32), (1, 64), (3, 32), (3, 96), (16, 4096), (17, 16384)])
+def test_every_share_of_the_cluster_reaches_the_scale(M, K):
+    """One value at a time carries the scale, from the first to the last share of a cluster; CTAs without a share of X are
+    at the meeting at once. Codes and exponents as the checker's."""
+    import oracle
+    from gpu_util import dev, handle
+    h = handle()
+    for at in sorted({0, M * K - 1, *range(0, M * K, max(8, M * K // 16))}):
+        x = np.full(M * K, 0.125, np.float16)
+        x[at] = -37.5
+        x = x.reshape(M, K)
+        q, e = h.aq_quantize_act(dev(x), 8)
+        assert int(e.item()) == oracle.layer_exponent(x, 8)
+        assert np.array_equal(q.cpu().numpy(), oracle.quantize_act(x, 8, int(e.item())))
+        qa, ea, zp = h.aq_quantize_act_asym(dev(x), 8)
+        assert (int(ea.item()), int(zp.item())) == oracle.asym_params(x, 8)
