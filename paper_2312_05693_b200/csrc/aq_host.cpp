@@ -100,13 +100,21 @@ void check(int status, const char* what) {
     }
     throw Bad{};
 }
-// The C call runs without the interpreter lock, as through ctypes.
+// The C call runs without the interpreter lock, as through ctypes. The lock comes back on every way out: a tensor without
+// storage (sparse, fake) throws when f asks for its address, and that becomes a Python exception above.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    Unlocked() = default;
+    Unlocked(const Unlocked&) = delete;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
 template <class F>
 void call(const char* what, F&& f) {
     int status;
-    Py_BEGIN_ALLOW_THREADS
-    status = f();
-    Py_END_ALLOW_THREADS
+    {
+        Unlocked unlocked;
+        status = f();
+    }
     check(status, what);
 }
 at::Tensor workspace_for(const at::Tensor& given, int M, int K, int N, int group, const at::Tensor& like) {

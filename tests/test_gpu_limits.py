@@ -83,3 +83,19 @@ def test_sizes_beyond_the_limits_are_refused():
     with pytest.raises(binding.AgileqError) as ei:
         h.aq_quantize_act(x, 8)
     assert ei.value.status == binding.AQ_ERR_SHAPE
+
+
+def test_a_tensor_without_storage_raises():
+    """Its address is asked for while the interpreter lock is released: an exception in Python, and the next call runs."""
+    h = handle()
+    q = torch.ones((4, 128), dtype=torch.int8, device="cuda")
+    packed, scales = h.aq_pack_w4(torch.ones((8, 128), dtype=torch.float16, device="cuda"), 0)
+    e = torch.zeros(1, dtype=torch.int32, device="cuda")
+    y = torch.zeros((4, 8), dtype=torch.float16, device="cuda")
+    ws = h.alloc_workspace(4, 128, 8, 0)
+    with pytest.raises(RuntimeError, match="storage"):
+        h.aq_gemm_w4(q.to_sparse(), packed, scales, 8, 0, e, y=y, workspace=ws)
+    with pytest.raises(RuntimeError, match="storage"):
+        h.aq_token_select(torch.ones(8, device="cuda").to_sparse(), 4)
+    assert h.aq_gemm_w4(q, packed, scales, 8, 0, e, y=y, workspace=ws) is y
+    assert torch.allclose(y, torch.full_like(y, 128.0), rtol=1e-3)
