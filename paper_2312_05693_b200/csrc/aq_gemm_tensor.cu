@@ -847,12 +847,18 @@ int tile_clusters(const DeviceInfo& dev, int split) {
 // token column and k block (about 7.6 cycles with 128-token tiles, 6.6 with 192-token tiles, 9 with 64-token tiles).
 // Tiles few enough for all of them to run at once in clusters do so when the k blocks saved outweigh the exchange (layers of
 // 48 rows, K x N = 4096 x 4096 14.3 -> 10.8 us, 11008 x 4096 21.9 -> 15.7 us, 5120 x 5120 17.6 -> 13.3 us; of 128 rows,
-// 11008 x 4096 30.9 -> 22.5 us; but 48 rows, 1024 x 4096 7.1 -> 8.3 us, left alone). They also replaced shared tiles where those made up the
-// whole launch (333 rows, 4096 x 4096 23.1 -> 21.3 us).
+// 11008 x 4096 30.9 -> 22.5 us). They also replaced shared tiles where those made up the
+// whole launch (333 rows, 4096 x 4096 23.1 -> 21.3 us). What the exchange costs grows with the tile and the cluster: over 512 <= K <= 11008,
+// 256 <= N <= 4096, 24 to 512 rows (450 layers, every cluster size forced), 1.9 us + 0.14 for each CTA beyond two with 64-token
+// tiles, 3.4 + 0.22 with 128 and 3.6 + 0.25 with 192. One figure for all of them (4500 cycles) put short reductions into
+// clusters that lose: 768 x 768 at 333 rows 10.0 us plain, 11.7 us in clusters; 1024 x 1152 at 192 rows 10.2 / 13.7 us.
 struct GroupedPlan {
     int bm, split;
 };
-constexpr float kExchangeCycles = 4500.0f, kSharedRoundCycles = 2500.0f;
+constexpr float kSharedRoundCycles = 2500.0f;
+float grouped_exchange_cycles(int bm, int split) {
+    return bm == 64 ? 3800.0f + 280.0f * (float)(split - 2) : bm == 128 ? 6700.0f + 430.0f * (float)(split - 2) : 7050.0f + 500.0f * (float)(split - 2);
+}
 GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_share, bool clusters) {
     const int kbs = K / kTileK, n_tiles_n = round_up(N, kTileN) / kTileN, sms = dev.sm_count;
     GroupedPlan best = {64, 1};
@@ -867,7 +873,7 @@ GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_sh
         if (plain < best_cost) { best_cost = plain; best = {bm, 1}; }
         if (!clusters) return;
         for (int s = 2; s <= 8 && s <= kbs && s * tiles <= sms; ++s) {
-            const float shared = (float)((kbs + s - 1) / s) * block + kExchangeCycles;
+            const float shared = (float)((kbs + s - 1) / s) * block + grouped_exchange_cycles(bm, s);
             if (shared >= best_cost) continue;
             const int fit = bm == 64 ? tile_clusters<64, true>(dev, s) : bm == 128 ? tile_clusters<128, true>(dev, s) : tile_clusters<192, true>(dev, s);
             if (fit >= tiles) { best_cost = shared; best = {bm, s}; }
@@ -883,19 +889,19 @@ GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_sh
 }
 
 // One scale per channel, tiles of one channel block: 64 tokens up to 64 rows, 128 up to 128 rows, or more while the tiles
-// fill one round; in clusters where the k blocks saved outweigh the exchange (cycles as above).
+// fill one round; in clusters where the k blocks saved outweigh the exchange.
 struct ChannelPlan {
     int bm, split;
     long cost;
 };
-constexpr int kNarrow64 = 420, kNarrow128 = 600;     // cycles per k block
+constexpr int kNarrow64 = 420, kNarrow128 = 600, kExchangeCycles = 4500;     // cycles per k block; of the exchange
 ChannelPlan channel_plan(int M, int K, int N, const DeviceInfo& dev) {
     const int KB = k_blocks(K), sms = dev.sm_count, bm = M <= 64 ? 64 : 128, block = M <= 64 ? kNarrow64 : kNarrow128;
     const long tiles = (long)((M + bm - 1) / bm) * (round_up(N, kTileN) / kTileN);
     if (M > 128 && tiles > sms) return {256, 1, 0x7fffffffL};
     ChannelPlan best = {bm, 1, (tiles + sms - 1) / sms * KB * block};
     for (int s = 2; s <= 8 && s <= KB && s * tiles <= sms; ++s) {
-        const long c = (long)((KB + s - 1) / s) * block + (long)kExchangeCycles;
+        const long c = (long)((KB + s - 1) / s) * block + kExchangeCycles;
         if (c >= best.cost) continue;
         if ((bm == 64 ? tile_clusters<64, false>(dev, s) : tile_clusters<128, false>(dev, s)) >= tiles) best = {bm, s, c};
     }
