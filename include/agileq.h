@@ -91,7 +91,8 @@ size_t aq_packed_w4_bytes(int N, int K);
  * this number beside them and repacks when a later library reports another one. */
 int aq_packed_w4_layout_version(void);
 /* Bytes of the fp16 scale buffer: [G][Npad], G = 1 (group_size 0) or K/128, Npad = N
- * rounded up to 128; element (g, n) at index g*Npad + n. */
+ * rounded up to 128; element (g, n) at index g*Npad + n. Any 2-byte aligned address is accepted; per-group
+ * scales on a 16-byte aligned one (as an allocation gives) are read in bulk, others one by one (slower). */
 size_t aq_scales_bytes(int N, int K, int group_size);
 /* Bytes of scratch that aq_quantize_act / aq_linear_* / aq_gemm_w4 / aq_token_select should get
  * for these sizes (M = rows actually multiplied). Always a multiple of 256. */

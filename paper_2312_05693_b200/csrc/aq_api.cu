@@ -82,8 +82,11 @@ int run_gemm(aq_handle_t h, const GemmArgs& g, cudaStream_t stream) {
     const int choice = kernel_for(h, g.M);
     GemmArgs a = g;
     a.weights_stable = h->weights_stable != 0;
-    const cudaError_t e = choice == AQ_KERNEL_DECODE ? launch_gemm_decode(a, h->dev, stream)
-                                                     : launch_gemm_tensor(a, h->dev, stream);
+    // The tensor-core kernel takes per-group scales in bulk copies, which start on 16 bytes; scales that lie elsewhere (any
+    // 2-byte address is accepted) go to the kernel that loads them one by one.
+    const bool loose_scales = g.group != 0 && !aligned(g.w_scales, 16);
+    const cudaError_t e = choice == AQ_KERNEL_DECODE || loose_scales ? launch_gemm_decode(a, h->dev, stream)
+                                                                     : launch_gemm_tensor(a, h->dev, stream);
     return e == cudaSuccess ? AQ_OK : cuda_fail(h, e);
 }
 

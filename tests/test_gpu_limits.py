@@ -99,3 +99,32 @@ def test_a_tensor_without_storage_raises():
         h.aq_token_select(torch.ones(8, device="cuda").to_sparse(), 4)
     assert h.aq_gemm_w4(q, packed, scales, 8, 0, e, y=y, workspace=ws) is y
     assert torch.allclose(y, torch.full_like(y, 128.0), rtol=1e-3)
+
+
+@pytest.mark.parametrize("kernel", [binding.AQ_KERNEL_AUTO, binding.AQ_KERNEL_TENSOR])
+@pytest.mark.parametrize("M,K,N,group", [(1, 256, 200, 128), (9, 384, 136, 128), (40, 512, 264, 128), (200, 256, 136, 128), (40, 256, 264, 0)])
+def test_scales_on_any_two_byte_address(M, K, N, group, kernel):
+    """The scales one, two and four elements behind a 16-byte boundary: sums exact, outputs within the layer's tolerance,
+    chained codes those of the plain call."""
+    x = inputs.activations(M, K, seed=M, outlier_frac=0.01, outlier_mult=20.0)
+    w = inputs.weights(N, K, seed=N)
+    h = handle()
+    packed, scales = h.aq_pack_w4(dev(w), group)
+    codes, sc = oracle.quantize_weights(w, group)
+    ref = oracle.linear(x, codes, sc, 8, group, 0, 0, want_acc=True)
+    h.aq_set_kernel(kernel)
+    try:
+        for shift in (1, 2, 4):
+            room = torch.zeros(scales.numel() + 8, dtype=torch.float16, device="cuda")
+            loose = room[shift:shift + scales.numel()]
+            loose.copy_(scales.view(-1))
+            y = h.aq_linear_w4a8(dev(x), packed, loose, N, group)
+            acc = torch.zeros((M, N, K // 128 if group else 1), dtype=torch.int32, device="cuda")
+            h.aq_linear_w4a8(dev(x), packed, loose, N, group, acc_dump=acc)
+            assert np.array_equal(acc.cpu().numpy(), ref["acc"])
+            assert_y_close(y.cpu().numpy(), ref["y"])
+            e_next = oracle.layer_exponent(y.cpu().numpy(), 8) - 1
+            q = h.aq_linear_chain(8, dev(x), packed, loose, N, group, 8, e_next)
+            assert np.array_equal(q.cpu().numpy(), oracle.quantize_act(y.cpu().numpy(), 8, e_next))
+    finally:
+        h.aq_set_kernel(binding.AQ_KERNEL_AUTO)
