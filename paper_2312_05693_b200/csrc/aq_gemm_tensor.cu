@@ -187,7 +187,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
 
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int KB = k_blocks(p.K);      // a last block that K does not fill: zero weight codes meet the tensor map's zero fill
-    static_assert(!SPLIT || (GROUPED && !OFFSET && !CHAIN), "only the plain per-group kernel shares tiles");
+    static_assert(!SPLIT || (GROUPED && !OFFSET), "tiles of a last round are shared with per-group scales, without a zero point");
     static_assert(!CLUSTER || (!SPLIT && BM <= 192), "what a CTA receives fits its operand ring");
     const int rank = CLUSTER ? (int)blockIdx.x : 0, split = CLUSTER ? (int)gridDim.x : 1;
     [[maybe_unused]] int met = 0;                    // CLUSTER: meetings this warp has been to
@@ -1028,13 +1028,13 @@ cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t str
             return launch_off<BM, GROUPED, false, false, false, true>(a, dev, stream, -1, 0, 0, cluster);
         }
     }
-    if (a.q_next) return launch_off<BM, GROUPED, false, true>(a, dev, stream);
     if (a.chan_offset) return launch_off<BM, GROUPED, true, false>(a, dev, stream);
     if constexpr (GROUPED) {
         // Behind whole rounds: a last round that would leave more than half of the SMs idle is run as shared tiles, when the
         // reduction is deep enough for half a tile to outweigh the second launch and the exchange of
         // partial sums (measured with 128-token tiles: a loss of 2-5 us at K = 4096, a gain of 8 us at
-        // K = 11008; with 192-token tiles a gain of 2 us at K = 4096 already).
+        // K = 11008; with 192-token tiles a gain of 2 us at K = 4096 already). Chained calls share the same tiles as plain
+        // ones: where a sum is cut decides its last fp32 rounding, and the codes are those of the plain call's outputs.
         const int sms = dev.sm_count;
         const int n_tiles = ((a.M + BM - 1) / BM) * (round_up(a.N, kTileN) / kTileN);
         const int rounds = n_tiles / sms, rem = n_tiles % sms;
@@ -1045,11 +1045,14 @@ cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t str
                 const cudaError_t e = cudaMemsetAsync(a.ctl->split_flags, 0, sizeof(a.ctl->split_flags), stream);
                 if (e != cudaSuccess) return e;
             }
-            const cudaError_t e = launch_off<BM, true, false, false>(a, dev, stream, rounds * sms);
+            const cudaError_t e = a.q_next ? launch_off<BM, true, false, true>(a, dev, stream, rounds * sms)
+                                           : launch_off<BM, true, false, false>(a, dev, stream, rounds * sms);
             if (e != cudaSuccess) return e;
-            return launch_off<BM, true, false, false, true>(a, dev, stream, -1, rounds * sms, rem);
+            return a.q_next ? launch_off<BM, true, false, true, true>(a, dev, stream, -1, rounds * sms, rem)
+                            : launch_off<BM, true, false, false, true>(a, dev, stream, -1, rounds * sms, rem);
         }
     }
+    if (a.q_next) return launch_off<BM, GROUPED, false, true>(a, dev, stream);
     return launch_off<BM, GROUPED, false, false>(a, dev, stream);
 }
 
@@ -1076,8 +1079,8 @@ cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const De
 
 cudaError_t launch_gemm_tensor(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
     if (a.group) {
-        // the chained and zero-point variants have no shared-tile launch
-        const GroupedPlan g = grouped_plan(a.M, a.K, a.N, dev, !a.q_next && !a.chan_offset, true);
+        // the zero-point variant has no shared-tile launch
+        const GroupedPlan g = grouped_plan(a.M, a.K, a.N, dev, !a.chan_offset, true);
         switch (g.bm) {
             case 64: return launch_bm<64, true>(a, dev, stream, g.split);
             case 192: return launch_bm<192, true>(a, dev, stream, g.split);

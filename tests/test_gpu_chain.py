@@ -38,6 +38,33 @@ def test_chain_codes_equal_quantized_plain_output(kernel, next_bits, M, K, N, gr
     assert ref.min() == -(1 << (next_bits - 1)) or ref.max() == (1 << (next_bits - 1)) - 1   # it did clip
 
 
+@pytest.mark.parametrize("M,K,N", [(200, 8192, 11008), (1000, 8192, 4096), (1500, 8192, 3000), (60, 8192, 19072)])
+def test_chain_codes_where_the_last_round_of_tiles_is_shared(M, K, N):
+    """Per-group scales, whole rounds of 128-, 192- or 64-token tiles and a last one whose tiles two CTAs share, half of
+    the reduction each: the chained and packed codes are still those of the plain call. The groups' scales spread over
+    seven octaves, so that the fp32 sums round (with like scales most of them are exact, and where a sum is cut would not show)."""
+    x = dev(inputs.activations(M, K, seed=M))
+    g = torch.Generator(device="cuda").manual_seed(N)
+    w = torch.randn((N, K // 128, 128), generator=g, device="cuda")
+    w *= torch.exp2(-7.0 * torch.rand((N, K // 128, 1), generator=g, device="cuda"))
+    w = (0.3 * w).reshape(N, K).to(torch.float16)
+    h = handle()
+    packed, scales = h.aq_pack_w4(w, 128)
+    ws = h.alloc_workspace(M, K, N, 128)
+    assert ws.numel() > binding.aq_workspace_min_bytes(M, K, N, 128)            # it does share tiles
+    y = h.aq_linear_w4a8(x, packed, scales, N, 128, workspace=ws).cpu().numpy()
+    assert h.aq_check_workspace(ws) == binding.AQ_OK
+    for bits in (8, 4):
+        e_next = oracle.layer_exponent(y, bits) - 1
+        ref = oracle.quantize_act(y, bits, e_next)
+        q = h.aq_linear_chain(8, x, packed, scales, N, 128, bits, e_next, workspace=ws)
+        assert h.aq_check_workspace(ws) == binding.AQ_OK
+        assert np.array_equal(q.cpu().numpy(), ref)
+    if N % 32 == 0:
+        q4 = h.aq_linear_chain_act4(8, x, packed, scales, N, 128, e_next, workspace=ws)
+        assert np.array_equal(q4.cpu().numpy(), oracle.pack_act4(ref))
+
+
 def test_two_chained_layers_match_checker_on_the_codes():
     M, K, N1, N2, group = 200, 512, 384, 256, 128
     x = inputs.activations(M, K, seed=42, outlier_frac=0.01, outlier_mult=20.0)
