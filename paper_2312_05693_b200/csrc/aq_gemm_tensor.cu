@@ -886,47 +886,54 @@ int tile_clusters(const DeviceInfo& dev, int split) {
 
 // How a per-group product is run: token tile and CTAs that share a tile. Up to 64 tokens the tile is 64. Otherwise 128 (eight
 // epilogue warps, three accumulator stages) or 192 (twelve epilogue warps, two stages), whichever gives the shorter schedule:
-// rounds of tiles over the SMs (a shared last round counts half) x tile height x the measured cost per
-// token column and k block (about 7.6 cycles with 128-token tiles, 6.6 with 192-token tiles, 9 with 64-token tiles).
-// Tiles few enough for all of them to run at once in clusters do so when the k blocks saved outweigh the exchange (layers of
-// 48 rows, K x N = 4096 x 4096 14.3 -> 10.8 us, 11008 x 4096 21.9 -> 15.7 us, 5120 x 5120 17.6 -> 13.3 us; of 128 rows,
-// 11008 x 4096 30.9 -> 22.5 us). They also replaced shared tiles where those made up the
-// whole launch (333 rows, 4096 x 4096 23.1 -> 21.3 us). What the exchange costs grows with the tile and the cluster: over 512 <= K <= 11008,
-// 256 <= N <= 4096, 24 to 512 rows (450 layers, every cluster size forced), 1.9 us + 0.14 for each CTA beyond two with 64-token
-// tiles, 3.4 + 0.22 with 128 and 3.6 + 0.25 with 192. One figure for all of them (4500 cycles) put short reductions into
-// clusters that lose: 768 x 768 at 333 rows 10.0 us plain, 11.7 us in clusters; 1024 x 1152 at 192 rows 10.2 / 13.7 us.
+// rounds of tiles over the SMs, a last round whose tiles two CTAs share, or all tiles at once in clusters, where the k blocks
+// saved outweigh the exchange (layers of 48 rows, K x N = 4096 x 4096 14.3 -> 10.8 us, 11008 x 4096 21.9 -> 15.7 us, 5120 x 5120
+// 17.6 -> 13.3 us; of 128 rows, 11008 x 4096 30.9 -> 22.5 us).
+// The times are fitted to layer calls with every schedule forced: 48 to 3000 rows, 768 <= K <= 13824, 768 <= N <= 22016 without
+// clusters (2332 calls, relative error 2.6 %), 24 to 512 rows, 512 <= K <= 11008, 256 <= N <= 4096 with them (4492). Of 936 layers
+// without clusters the schedule taken is within 1 % of the best in all; of 450 with them within 3 % in 95 % and 8 % in all. (In
+// cycles per token column, as measured before the issuing threads were elected, and one figure for every exchange: 17 % and
+// 42 % off at the worst. 500 rows, 8192 x 11008 took 87.6 us on shared 128-token tiles, 79.8 on whole 192-token tiles; 1024 x 1152
+// at 192 rows 13.7 us in a cluster, 10.2 without.)
 struct GroupedPlan {
     int bm, split;
 };
-constexpr float kSharedRoundCycles = 2500.0f;
-float grouped_exchange_cycles(int bm, int split) {
-    return bm == 64 ? 3800.0f + 280.0f * (float)(split - 2) : bm == 128 ? 6700.0f + 430.0f * (float)(split - 2) : 7050.0f + 500.0f * (float)(split - 2);
+struct GroupedTimes {                // microseconds
+    float call, round, block;        // layer call; round of tiles, k block of it
+    float shared, shared_block;      // a last round of shared tiles: launch and exchange, k block of half a tile
+    float exchange, exchange_cta;    // clusters of two; each CTA more
+};
+constexpr GroupedTimes grouped_times(int bm) {
+    return bm == 64 ? GroupedTimes{4.56f, 0.91f, 0.266f, 6.44f, 0.317f, 1.9f, 0.06f}
+         : bm == 128 ? GroupedTimes{6.45f, 0.96f, 0.440f, 8.05f, 0.423f, 2.9f, 0.14f}
+                     : GroupedTimes{6.63f, 1.47f, 0.499f, 9.23f, 0.523f, 3.85f, 0.41f};
 }
 GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_share, bool clusters) {
     const int kbs = K / kTileK, n_tiles_n = round_up(N, kTileN) / kTileN, sms = dev.sm_count;
     GroupedPlan best = {64, 1};
-    float best_cost = 3.0e38f;
-    auto consider = [&](int bm, float per_col) {
+    float best_time = 3.0e38f;
+    auto consider = [&](int bm) {
+        const GroupedTimes t = grouped_times(bm);
         const long tiles = (long)((M + bm - 1) / bm) * n_tiles_n;
-        const long rounds = tiles / sms;
         const int rem = (int)(tiles % sms);
-        const bool halves = may_share && rounds > 0 && round_is_shared(rem, sms, kbs, bm);
-        const float last = rem == 0 ? 0.0f : halves ? 0.5f : 1.0f;
-        const float block = (float)bm * per_col, plain = ((float)rounds + last) * (float)kbs * block + (halves ? kSharedRoundCycles : 0.0f);
-        if (plain < best_cost) { best_cost = plain; best = {bm, 1}; }
+        const bool halves = may_share && tiles >= sms && round_is_shared(rem, sms, kbs, bm);
+        const long rounds = tiles / sms + (rem > 0 && !halves ? 1 : 0);
+        const float plain = t.call + (float)rounds * (t.round + (float)kbs * t.block) +
+                            (halves ? t.shared + (float)((kbs + 1) / 2) * t.shared_block : 0.0f);
+        if (plain < best_time) { best_time = plain; best = {bm, 1}; }
         if (!clusters) return;
         for (int s = 2; s <= 8 && s <= kbs && s * tiles <= sms; ++s) {
-            const float shared = (float)((kbs + s - 1) / s) * block + grouped_exchange_cycles(bm, s);
-            if (shared >= best_cost) continue;
+            const float shared = t.call + t.round + (float)((kbs + s - 1) / s) * t.block + t.exchange + (float)(s - 2) * t.exchange_cta;
+            if (shared >= best_time) continue;
             const int fit = bm == 64 ? tile_clusters<64, true>(dev, s) : bm == 128 ? tile_clusters<128, true>(dev, s) : tile_clusters<192, true>(dev, s);
-            if (fit >= tiles) { best_cost = shared; best = {bm, s}; }
+            if (fit >= tiles) { best_time = shared; best = {bm, s}; }
         }
     };
     if (M <= 64) {
-        consider(64, 9.0f);
+        consider(64);
     } else {
-        consider(128, 7.6f);
-        consider(192, 6.6f);
+        consider(128);
+        consider(192);
     }
     return best;
 }
