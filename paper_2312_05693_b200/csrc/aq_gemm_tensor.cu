@@ -846,9 +846,11 @@ __global__ void __launch_bounds__(128, 1) int8_probe_kernel(int iters, int a_fro
 // tiles, where half a tile is worth more (see launch_bm).
 constexpr int split_min_k_blocks(int bm) { return bm >= 192 ? 32 : 64; }
 
-// Whether a last, partial round of `rem` tiles is run as shared tiles.
-inline bool round_is_shared(int rem, int sms, int k_blocks, int bm) {
-    return rem > 0 && 2 * rem <= sms && k_blocks >= split_min_k_blocks(bm) && rem <= Control::kMaxSplitTiles;
+// Tiles of a last, partial round behind whole ones that are run as shared tiles (0: none). The plan, the launch and the size of
+// the scratch all ask here.
+inline int shared_tiles(long tiles, int sms, int k_blocks, int bm) {
+    const int rem = (int)(tiles % sms);
+    return tiles >= sms && 2 * rem <= sms && k_blocks >= split_min_k_blocks(bm) && rem <= Control::kMaxSplitTiles ? rem : 0;
 }
 
 // Clusters of `split` CTAs that run at once (one CTA fills an SM; a GPC holds only so many of a size).
@@ -893,7 +895,7 @@ int tile_clusters(const DeviceInfo& dev, int split) {
 // clusters (2332 calls, relative error 2.6 %), 24 to 512 rows, 512 <= K <= 11008, 256 <= N <= 4096 with them (4492). Of 936 layers
 // without clusters the schedule taken is within 1 % of the best in all; of 450 with them within 3 % in 95 % and 8 % in all. (In
 // cycles per token column, as measured before the issuing threads were elected, and one figure for every exchange: 17 % and
-// 42 % off at the worst. 500 rows, 8192 x 11008 took 87.6 us on shared 128-token tiles, 79.8 on whole 192-token tiles; 1024 x 1152
+// 42 % off at the worst. 500 rows, 8192 x 11008 took 87.6 us on shared 128-token tiles, 75.2 on whole 192-token tiles; 1024 x 1152
 // at 192 rows 13.7 us in a cluster, 10.2 without.)
 struct GroupedPlan {
     int bm, split;
@@ -915,9 +917,8 @@ GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_sh
     auto consider = [&](int bm) {
         const GroupedTimes t = grouped_times(bm);
         const long tiles = (long)((M + bm - 1) / bm) * n_tiles_n;
-        const int rem = (int)(tiles % sms);
-        const bool halves = may_share && tiles >= sms && round_is_shared(rem, sms, kbs, bm);
-        const long rounds = tiles / sms + (rem > 0 && !halves ? 1 : 0);
+        const bool halves = may_share && shared_tiles(tiles, sms, kbs, bm) > 0;
+        const long rounds = halves ? tiles / sms : (tiles + sms - 1) / sms;
         const float plain = t.call + (float)rounds * (t.round + (float)kbs * t.block) +
                             (halves ? t.shared + (float)((kbs + 1) / 2) * t.shared_block : 0.0f);
         if (plain < best_time) { best_time = plain; best = {bm, 1}; }
@@ -1087,19 +1088,18 @@ cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t str
         // ones: where a sum is cut decides its last fp32 rounding, and the codes are those of the plain call's outputs.
         const int sms = dev.sm_count;
         const int n_tiles = ((a.M + BM - 1) / BM) * (round_up(a.N, kTileN) / kTileN);
-        const int rounds = n_tiles / sms, rem = n_tiles % sms;
+        const int rem = shared_tiles(n_tiles, sms, a.K / kTileK, BM), whole = n_tiles - rem;
         const size_t need = (size_t)rem * 2 * BM * kTileN * sizeof(float);
-        if (rounds > 0 && round_is_shared(rem, sms, a.K / kTileK, BM) && a.split_scratch &&
-            a.split_bytes >= need && (reinterpret_cast<uintptr_t>(a.split_scratch) & 15u) == 0) {
+        if (rem > 0 && a.split_scratch && a.split_bytes >= need && (reinterpret_cast<uintptr_t>(a.split_scratch) & 15u) == 0) {
             if (!a.after_quantize) {
                 const cudaError_t e = cudaMemsetAsync(a.ctl->split_flags, 0, sizeof(a.ctl->split_flags), stream);
                 if (e != cudaSuccess) return e;
             }
-            const cudaError_t e = a.q_next ? launch_off<BM, true, false, true>(a, dev, stream, rounds * sms)
-                                           : launch_off<BM, true, false, false>(a, dev, stream, rounds * sms);
+            const cudaError_t e = a.q_next ? launch_off<BM, true, false, true>(a, dev, stream, whole)
+                                           : launch_off<BM, true, false, false>(a, dev, stream, whole);
             if (e != cudaSuccess) return e;
-            return a.q_next ? launch_off<BM, true, false, true, true>(a, dev, stream, -1, rounds * sms, rem)
-                            : launch_off<BM, true, false, false, true>(a, dev, stream, -1, rounds * sms, rem);
+            return a.q_next ? launch_off<BM, true, false, true, true>(a, dev, stream, -1, whole, rem)
+                            : launch_off<BM, true, false, false, true>(a, dev, stream, -1, whole, rem);
         }
     }
     if (a.q_next) return launch_off<BM, GROUPED, false, true>(a, dev, stream);
@@ -1114,9 +1114,7 @@ size_t tensor_split_scratch_bytes(int M, int K, int N, int group, int sm_count) 
     dev.sm_count = sm_count;
     const int bm = grouped_plan(M, K, N, dev, true, false).bm;     // the most that the plan with clusters uses
     const int n_tiles = ((M + bm - 1) / bm) * (round_up(N, kTileN) / kTileN);
-    const int rem = n_tiles % sm_count;
-    if (!round_is_shared(rem, sm_count, K / kTileK, bm)) return 0;
-    return (size_t)rem * 2 * bm * kTileN * sizeof(float);
+    return (size_t)shared_tiles(n_tiles, sm_count, K / kTileK, bm) * 2 * bm * kTileN * sizeof(float);
 }
 
 cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const DeviceInfo& dev, cudaStream_t stream) {

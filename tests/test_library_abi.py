@@ -63,6 +63,9 @@ def test_which_shapes_fit_the_built_in_scratch_buffer():
     # the per-group kernel's optional area is what separates the two size functions
     assert binding.aq_workspace_bytes(2048, 4096, 4096, 128) > binding.aq_workspace_min_bytes(2048, 4096, 4096, 128)
     assert binding.aq_workspace_bytes(2048, 4096, 4096, 0) == binding.aq_workspace_min_bytes(2048, 4096, 4096, 0)
+    # tiles are shared behind whole rounds only: no scratch where the tiles do not fill the SMs once
+    for M in (17, 48, 128, 200):
+        assert binding.aq_workspace_bytes(M, 11008, 4096, 128) == binding.aq_workspace_min_bytes(M, 11008, 4096, 128)
 
 
 def test_null_handle_is_rejected_without_touching_a_device():
