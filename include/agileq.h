@@ -57,8 +57,8 @@ typedef enum aq_status {
 enum { AQ_SCALE_DYNAMIC = 0, AQ_SCALE_STATIC = 1 };
 
 /* Which matrix-product kernel aq_linear_* / aq_gemm_w4 uses. AUTO picks the decode kernel
- * for M <= 32 and the tensor-core kernel otherwise; the others force one (for tests and
- * measurements). All give identical integer sums. */
+ * for M <= 16 and the tensor-core kernel otherwise; the others force one (for tests and
+ * measurements). All give identical integer sums; fp32 sums of per-group products are added in another order. */
 enum { AQ_KERNEL_AUTO = 0, AQ_KERNEL_TENSOR = 1, AQ_KERNEL_DECODE = 2 };
 
 const char* aq_status_string(int status);
@@ -75,7 +75,7 @@ int aq_set_kernel(aq_handle_t h, int kernel);
 /* A scheduling promise, not part of the paper's method; off by default. enabled != 0 tells the library that,
  * for every later call on this handle, no work still in flight on the call's stream when the call is enqueued
  * writes the packed weights or weight scales the call reads (the usual case: weights are packed once, before
- * inference starts). The few-row kernels (M <= 32) then let the launch behind them be
+ * inference starts). The few-row kernels (M <= 16) then let the launch behind them be
  * set up from their start and fetch their first 64 KB of weights per CTA before they wait for the kernel ahead
  * of them; everything else a call reads or writes still waits for that kernel. Results are the same bit for
  * bit; consecutive few-row calls on one stream overlap by a microsecond or two. With the promise broken (a

@@ -70,12 +70,12 @@ Workspace carve(void* ws, int M, int K, int N, size_t total_bytes) {
     return w;
 }
 
-// Up to 16 rows the streaming kernel. Beyond, its second 16-row tile of the warp-level MMA costs more than the tensor-core
-// kernels' tiles of 128 channels in clusters (layers of 20 rows, K = N = 5120 11.5 against 10.5 us; of 32 rows 12.3 / 11.0 us,
-// K = 5120, N = 13824 18.8 / 13.0 us, K = 11008, N = 4096 in groups of 128 22.2 / 16.3 us).
+// Up to 16 rows the streaming kernel. Beyond, a second 16-row tile of its warp-level MMA cost more than the tensor-core kernels'
+// tiles of 128 channels in clusters (layers of 20 rows, K = N = 5120 11.5 against 10.5 us; of 32 rows 12.3 / 11.0 us, K = 5120,
+// N = 13824 18.8 / 13.0 us, K = 11008, N = 4096 in groups of 128 22.2 / 16.3 us).
 int kernel_for(aq_handle_t h, int M) {
     const int choice = h->kernel_choice;
-    return choice == AQ_KERNEL_AUTO ? (M <= 16 ? AQ_KERNEL_DECODE : AQ_KERNEL_TENSOR) : choice;
+    return choice == AQ_KERNEL_AUTO ? (M <= kFewRows ? AQ_KERNEL_DECODE : AQ_KERNEL_TENSOR) : choice;
 }
 
 int run_gemm(aq_handle_t h, const GemmArgs& g, cudaStream_t stream) {

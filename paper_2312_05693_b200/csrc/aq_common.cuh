@@ -230,7 +230,7 @@ cudaError_t launch_gemm_wide(const GemmArgs& a, const DeviceInfo& dev, cudaStrea
 size_t tensor_split_scratch_bytes(int M, int K, int N, int group, int sm_count);
 // Tensor-core rate probe: every SM issues iters x 4 MMAs of 128 x 256 x 32 (int8) on resident operands.
 cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const DeviceInfo& dev, cudaStream_t stream);
-constexpr int kFewRows = 32;         // rows up to which the streaming kernel runs (AQ_KERNEL_AUTO takes it up to 16)
+constexpr int kFewRows = 16;         // rows up to which the streaming kernel runs, and AQ_KERNEL_AUTO takes it
 cudaError_t launch_gemm_decode(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, int sm_count);
 

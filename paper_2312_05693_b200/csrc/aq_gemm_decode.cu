@@ -6,13 +6,14 @@
 //  * a general one (dumps of per-group sums, scales that are not 16-byte aligned, or any M when forced): a CTA owns 32 output channels
 //    (one lane each), its 8 warps split K by 128-k block, products use dp4a on weights
 //    widened to 16*code, warps meet in shared memory;
-//  * a streaming one for M <= 32: a thread-block cluster shares a
+//  * a streaming one for M <= 16: a thread-block cluster shares a
 //    128-channel tile and splits K; in each CTA a producer thread streams 8 KB packed blocks
 //    and their activation codes into a shared-memory ring with TMA, eight consumer warps
-//    multiply (dp4a for one row, the warp-level int8 MMA above, on one or two 16-row tiles). Every CTA keeps the sums over
-//    its k range in its own shared memory; the cluster meets once, and every CTA then finishes a
-//    slice of the tile's channels by reading the other CTAs' sums over distributed shared memory
-//    (integer addition is exact in any order). No workspace, no atomics.
+//    multiply (dp4a for one row, the warp-level int8 MMA on a 16-row tile above). Every CTA keeps the sums over
+//    its k range in its own shared memory and writes those of the channels it does not finish into the shared
+//    memory of the CTA that does; the cluster meets once, and every CTA finishes its slice of the tile's channels
+//    (integer sums are exact in any order, fp32 ones are added in an order that does not depend on timing). No
+//    workspace, no atomics.
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -179,7 +180,7 @@ gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
 }
 
 // ---------------------------------------------------------------------------------------
-// Streaming kernel (M <= 32)
+// Streaming kernel (M <= 16)
 // ---------------------------------------------------------------------------------------
 constexpr unsigned long long kStrWaitCycles = 4000000000ull;
 constexpr int kFuseMaxBlocks = 64;        // k blocks per CTA up to which a single row is quantized inside the product kernel
@@ -229,10 +230,6 @@ template <int MB> struct StreamCfg {
     // consumer work in flight, not with the time a block waits (with the consumers' arithmetic taken out the
     // same launches take 6.6 / 9.1 / 10.1 us, and the ring is never full either way).
     static constexpr int kPhases = 2;
-    static constexpr int kRowTiles = MB <= 16 ? 1 : 2;           // 16-row tiles of a consumer warp
-    // More than 16 rows: the sum and receive buffers take the place of the operand ring once it has run dry, so that
-    // two CTAs still fit an SM.
-    static constexpr bool kAlias = MB > 16;
     // Two CTAs per SM for both routes. Three single-row CTAs would fit (with 128-byte instead of 1024-byte
     // alignment slack), so that under the stable-weights promise the next launch's CTAs sit, fetching, beside
     // two CTAs of this one; measured slower (M = 1 layer 5.8 / 9.1 / 9.7 -> 6.6 / 9.7 / 11.8 us): what the
@@ -259,20 +256,10 @@ struct StreamRing {
     alignas(128) uint8_t w[kStages][kBlockBytes];          // packed weight block of the unit
     alignas(16) __half sc[GROUPED ? kStages : 1][kTileN];  // per-group scales: those of the unit's k block (= its group)
 };
-template <class Ring, class Sums, bool ALIAS>
-struct StreamBuffers {
-    Ring ring;
-    Sums sums;
-};
-template <class Ring, class Sums>
-struct StreamBuffers<Ring, Sums, true> {
-    union {
-        Ring ring;
-        Sums sums;
-    };
-};
 template <int MB, bool WIDE = false, bool GROUPED = false>
-struct StreamSmem : StreamBuffers<StreamRing<MB, GROUPED>, StreamSums<MB, WIDE>, StreamCfg<MB>::kAlias> {
+struct StreamSmem {
+    StreamRing<MB, GROUPED> ring;
+    StreamSums<MB, WIDE> sums;
     static constexpr int kStages = StreamCfg<MB>::kStages;
     static constexpr int kRecvStride = StreamSums<MB, WIDE>::kRecvStride;
     // one row quantized by the kernel itself: the codes of this CTA's k range (up to kFuseMaxBlocks blocks)
@@ -300,7 +287,7 @@ struct StreamParams {
     int early_weights;             // the first ring of weight copies may be issued before the wait for the kernel ahead
     int early_dependents;          // the launch behind this one may be set up from this kernel's start
     int next_packed;
-    int box_rows;                  // rows of the activation tensor map's box: M rounded up to a multiple of 8
+    int box_rows;                  // rows of the activation tensor map's box: 8 when M <= 8 (MMA route)
     // FUSEQ (one row): the activations themselves; the kernel finds the layer scale, writes the codes of
     // its k range to shared memory (and, from the first channel tile, to q_out) and fills the control block
     const __half* x_row;           // the row's K halves
@@ -330,15 +317,14 @@ template <int MB, bool FUSEQ = false, bool WIDE = false, bool GROUPED = false>
 __global__ void __launch_bounds__(StreamCfg<MB>::kThreads, 2)
 gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const StreamParams p) {
     static_assert(!FUSEQ || MB == 1, "only a single row is quantized inside the product kernel");
-    static_assert(!WIDE || MB >= 16, "clusters of 5 to 8 are for the MMA route");
+    static_assert(!WIDE || MB == 16, "clusters of 5 to 8 are for the MMA route");
     extern __shared__ uint8_t smem_raw[];
     using Smem = StreamSmem<MB, WIDE, GROUPED>;
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr bool kUseMma = StreamCfg<MB>::kUseMma;
     constexpr int kRows = StreamCfg<MB>::kRows;
     constexpr int kStrStages = StreamCfg<MB>::kStages;
-    constexpr int kPhases = StreamCfg<MB>::kPhases, kRowTiles = StreamCfg<MB>::kRowTiles;
-    constexpr bool kAlias = StreamCfg<MB>::kAlias;
+    constexpr int kPhases = StreamCfg<MB>::kPhases;
     constexpr int kStrConsumerWarps = StreamCfg<MB>::kConsumerWarps;
     constexpr int kStrThreads = StreamCfg<MB>::kThreads;
     cg::cluster_group cluster = cg::this_cluster();
@@ -350,8 +336,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
 
     // First meeting of the cluster, arrival only: by the time a CTA writes into another's shared memory
     // (after its k range) every CTA of the cluster has started. The wait comes just before those writes.
-    // (Where the receive buffer takes the operand ring's place the meeting is after the k range instead.)
-    if (!kAlias && split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    if (split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     if (threadIdx.x == 0) {
         if constexpr (kRows > 1)     // start the descriptor's fetch now; the first tile load would wait for it
             asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
@@ -592,22 +577,21 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             // Warp-level int8 MMA, D[16 rows x 8 channels] += A[16 x 32 k] * B[32 k x 8 channels].
             // Fragment owner: g = lane / 4 (row g and g+8 of A and D; channel g of B),
             // t = lane % 4 (k bytes 4t..4t+3 and 16+4t..; D columns 2t, 2t+1).
-            // Rows 8..15 of a 16-row tile are not read when M ends before them, and a tile behind M is left out.
+            // Rows 8..15 are not read when M <= 8.
             // (Splitting a block among the four warps of a phase into channel
             // halves x k halves instead of channel quarters, so that a warp reads half of the activation tile,
             // measured the same within 0.2 us either way.)
             const int g = lane >> 2, t = lane & 3;
-            int acc[kRowTiles][4][4];
-            [[maybe_unused]] float fsum[kRowTiles][4][4];
+            const bool upper = p.M > 8;
+            int acc[4][4];
+            [[maybe_unused]] float fsum[4][4];
 #pragma unroll
-            for (int rt = 0; rt < kRowTiles; ++rt)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        acc[rt][i][c] = 0;
-                        if constexpr (GROUPED) fsum[rt][i][c] = 0.0f;
-                    }
+                for (int c = 0; c < 4; ++c) {
+                    acc[i][c] = 0;
+                    if constexpr (GROUPED) fsum[i][c] = 0.0f;
+                }
             for (int kb = kb0 + phase; kb < kb1; kb += kPhases) {
                 const uint32_t it = (uint32_t)(kb - kb0);
                 const int s = (int)(it % kStrStages);
@@ -628,24 +612,19 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(pw[0]), "=r"(pw[1]), "=r"(pw[2]), "=r"(pw[3])
                                  : "r"(s_u32(sm.ring.w[s] + (size_t)(j * kTileN + quarter * 32 + lane) * 16)) : "memory");
+                    const uint2 xa = *reinterpret_cast<const uint2*>(sm.ring.x[s] + g * kTileK + x_off);
+                    uint2 xb = make_uint2(0u, 0u);
+                    if (upper) xb = *reinterpret_cast<const uint2*>(sm.ring.x[s] + (g + 8) * kTileK + x_off);
+                    const uint32_t a0 = xa.x, a1 = xb.x, a2 = xa.y, a3 = xb.y;
 #pragma unroll
-                    for (int rt = 0; rt < kRowTiles; ++rt) {
-                        const int row = 16 * rt;
-                        if (rt > 0 && row >= p.M) break;
-                        const uint2 xa = *reinterpret_cast<const uint2*>(sm.ring.x[s] + (row + g) * kTileK + x_off);
-                        uint2 xb = make_uint2(0u, 0u);
-                        if (p.M > row + 8) xb = *reinterpret_cast<const uint2*>(sm.ring.x[s] + (row + g + 8) * kTileK + x_off);
-                        const uint32_t a0 = xa.x, a1 = xb.x, a2 = xa.y, a3 = xb.y;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint32_t b0 = (pw[i] << 4) & 0xF0F0F0F0u;
-                            const uint32_t b1 = pw[i] & 0xF0F0F0F0u;
-                            asm volatile(
-                                "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-                                "{%8, %9}, {%0, %1, %2, %3};"
-                                : "+r"(acc[rt][i][0]), "+r"(acc[rt][i][1]), "+r"(acc[rt][i][2]), "+r"(acc[rt][i][3])
-                                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-                        }
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t b0 = (pw[i] << 4) & 0xF0F0F0F0u;
+                        const uint32_t b1 = pw[i] & 0xF0F0F0F0u;
+                        asm volatile(
+                            "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+                            "{%8, %9}, {%0, %1, %2, %3};"
+                            : "+r"(acc[i][0]), "+r"(acc[i][1]), "+r"(acc[i][2]), "+r"(acc[i][3])
+                            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
                     }
                 }
                 if constexpr (GROUPED) {
@@ -653,12 +632,10 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                     for (int i = 0; i < 4; ++i) {
                         const float2 sg = __half22float2(*reinterpret_cast<const __half2*>(&sm.ring.sc[s][quarter * 32 + 8 * i + 2 * t]));
 #pragma unroll
-                        for (int rt = 0; rt < kRowTiles; ++rt)
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                fsum[rt][i][c] = fmaf((float)acc[rt][i][c], (c & 1) ? sg.y : sg.x, fsum[rt][i][c]);
-                                acc[rt][i][c] = 0;
-                            }
+                        for (int c = 0; c < 4; ++c) {
+                            fsum[i][c] = fmaf((float)acc[i][c], (c & 1) ? sg.y : sg.x, fsum[i][c]);
+                            acc[i][c] = 0;
+                        }
                     }
                 }
                 __syncwarp();
@@ -669,20 +646,17 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             // owns an element in each of them: the first stores, the others add).
 #pragma unroll
             for (int ph = 0; ph < kPhases; ++ph) {
-                // (where the sums take the ring's place, every consumer warp must have read its last block)
-                if (kAlias || ph > 0) asm volatile("bar.sync 1, %0;" ::"n"(kStrConsumerWarps * 32) : "memory");
+                if (ph > 0) asm volatile("bar.sync 1, %0;" ::"n"(kStrConsumerWarps * 32) : "memory");
                 if (phase == ph) {
 #pragma unroll
-                    for (int rt = 0; rt < kRowTiles; ++rt)
+                    for (int i = 0; i < 4; ++i)
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                int& dst = sm.sums.sum[16 * rt + g + 8 * (c >> 1)][quarter * 32 + 8 * i + 2 * t + (c & 1)];
-                                const int own = GROUPED ? __float_as_int(fsum[rt][i][c]) : acc[rt][i][c];
-                                if (ph == 0) dst = own;
-                                else dst = add_sums<GROUPED>(dst, own);
-                            }
+                        for (int c = 0; c < 4; ++c) {
+                            int& dst = sm.sums.sum[g + 8 * (c >> 1)][quarter * 32 + 8 * i + 2 * t + (c & 1)];
+                            const int own = GROUPED ? __float_as_int(fsum[i][c]) : acc[i][c];
+                            if (ph == 0) dst = own;
+                            else dst = add_sums<GROUPED>(dst, own);
+                        }
                 }
             }
         }
@@ -719,14 +693,8 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     }
     const int rows = p.M < kRows ? p.M : kRows;
     if (split > 1) {
-        if (kAlias) {
-            __syncthreads();                                  // this CTA's sums are complete, its ring is idle
-            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // ... and so are the others'
-        } else {
-            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // everybody has started (arrival at the top)
-            __syncthreads();                                  // this CTA's sums are complete
-        }
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // everybody has started (arrival at the top)
+        __syncthreads();                                      // this CTA's sums are complete
         if (ft >= 0) {
             // four consecutive channels at a time (16-byte remote stores) go to the CTA that owns them
             for (int e = ft; e < rows * (kTileN / 4); e += kStrConsumerWarps * 32) {
@@ -818,7 +786,7 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
     const cuuint64_t strides[1] = {(cuuint64_t)a.K};
-    // MMA route: M rounded up to a multiple of 8 rows; what lies behind is neither copied nor read
+    // MMA route: 8 or 16 rows; rows 8..15 are neither copied nor read when M <= 8
     const int box_rows = StreamCfg<MB>::kUseMma ? round_up(a.M, 8) : StreamCfg<MB>::kRows;
     const cuuint32_t box[2] = {128u, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1u, 1u};
@@ -953,8 +921,7 @@ cudaError_t launch_stream_rows(const GemmArgs& a, const DeviceInfo& dev, cudaStr
     // 8.1 / 12.8 / 15.2 us on the three 13B shapes)
     if (a.M <= 1 && a.fuse_x) return launch_stream<1, true, false, GROUPED>(a, dev, stream);
     if (a.M <= 1) return launch_stream<1, false, false, GROUPED>(a, dev, stream);
-    if (a.M <= 16) return launch_stream_mma<16, GROUPED>(a, dev, stream);
-    return launch_stream_mma<32, GROUPED>(a, dev, stream);
+    return launch_stream_mma<16, GROUPED>(a, dev, stream);
 }
 }  // namespace
 

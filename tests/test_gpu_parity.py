@@ -241,34 +241,40 @@ def test_decode_clusters_of_five_to_eight(M, K, N):
         assert np.array_equal(q_next.cpu().numpy(), oracle.quantize_act(gpu["y"], 8, e_next))
 
 
+@pytest.mark.parametrize("kernel", [pytest.param(binding.AQ_KERNEL_AUTO, id="auto"), *KERNELS])
 @pytest.mark.parametrize("group", [0, 128])
 @pytest.mark.parametrize("M,K,N", [(17, 128, 1), (17, 11008, 4096), (20, 9216, 5760), (24, 5120, 392), (25, 384, 4096),
                                    (32, 640, 136), (32, 13824, 5120), (33, 1280, 200)])
-def test_17_to_32_rows(M, K, N, group):
-    """The streaming kernel on two 16-row tiles (the second partly missing; clusters of one to eight CTAs; 33 rows take
-    the tensor-core kernel): codes exact, sums exact where one scale spans K (integer additions in any order), outputs
-    within tolerance; chained and packed codes agree with the plain call bit for bit."""
+def test_17_to_32_rows(M, K, N, group, kernel):
+    """Just beyond the few-row range, where AUTO takes the tensor-core kernels (clusters of one to eight CTAs), and the
+    general few-row kernel when it is forced: codes exact, sums exact where one scale spans K, outputs within
+    tolerance; chained and packed codes agree with the plain call bit for bit."""
     x = inputs.activations(M, K, seed=M + K, outlier_frac=0.01, outlier_mult=20.0)
     w = inputs.weights(N, K, seed=N + K)
-    gpu, ref = run_layer_both(x, w, 8, group, binding.AQ_KERNEL_AUTO, want_acc=group == 0)
+    gpu, ref = run_layer_both(x, w, 8, group, kernel, want_acc=group == 0)
     assert gpu["e"] == ref["e"] and np.array_equal(gpu["q"], ref["q"])
     if group == 0:
         assert np.array_equal(gpu["acc"], ref["acc"])
     assert_y_close(gpu["y"], ref["y"])
     h = handle()
     packed, scales = h.aq_pack_w4(dev(w), group)
-    y = h.aq_linear_w4a8(dev(x), packed, scales, N, group).cpu().numpy()
-    if group == 0:
-        assert np.array_equal(y.view(np.uint16), gpu["y"].view(np.uint16))
-    e_next = oracle.layer_exponent(y, 4) - 1
-    ref_next = oracle.quantize_act(y, 4, e_next)
-    assert np.array_equal(h.aq_linear_chain(8, dev(x), packed, scales, N, group, 4, e_next).cpu().numpy(), ref_next)
-    if N % 32 == 0:
-        q4 = h.aq_linear_chain_act4(8, dev(x), packed, scales, N, group, e_next)
-        assert np.array_equal(q4.cpu().numpy(), oracle.pack_act4(ref_next))
-    codes, sc = oracle.quantize_weights(w, group)
-    e, zp = oracle.asym_params(x, 8)
-    ya = h.aq_linear_asym(8, dev(x), packed, scales, h.aq_weight_offsets(packed, scales, N, K, group), N, group).cpu().numpy()
+    h.aq_set_kernel(kernel)
+    try:
+        y = h.aq_linear_w4a8(dev(x), packed, scales, N, group).cpu().numpy()
+        if group == 0:
+            assert np.array_equal(y.view(np.uint16), gpu["y"].view(np.uint16))
+        e_next = oracle.layer_exponent(y, 4) - 1
+        ref_next = oracle.quantize_act(y, 4, e_next)
+        assert np.array_equal(h.aq_linear_chain(8, dev(x), packed, scales, N, group, 4, e_next).cpu().numpy(), ref_next)
+        if N % 32 == 0:
+            q4 = h.aq_linear_chain_act4(8, dev(x), packed, scales, N, group, e_next)
+            assert np.array_equal(q4.cpu().numpy(), oracle.pack_act4(ref_next))
+        codes, sc = oracle.quantize_weights(w, group)
+        e, zp = oracle.asym_params(x, 8)
+        r = h.aq_weight_offsets(packed, scales, N, K, group)
+        ya = h.aq_linear_asym(8, dev(x), packed, scales, r, N, group).cpu().numpy()
+    finally:
+        h.aq_set_kernel(binding.AQ_KERNEL_AUTO)
     assert_y_close(ya, oracle.linear_asym(oracle.quantize_act_asym(x, 8, e, zp), zp, codes, sc, e, group)[1])
 
 
