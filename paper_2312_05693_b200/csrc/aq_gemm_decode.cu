@@ -240,12 +240,13 @@ template <int MB> struct StreamCfg {
 
 // this CTA's sums over its k range (per-group scales: the bits of fp32 sums; rows padded by 8 words so that the MMA
 // route's fragment owners, eight rows at the same columns, spread over the banks), and the other CTAs' sums for this
-// CTA's channel slice, by sender (CTAs below this one, then above): `split` - 1 slots of 128 / split channels, or
-// (clusters of 5 to 8) seven slots of 32
+// CTA's channel slice, by sender: `split` slots of 128 / split channels, or (clusters of 5 to 8) eight slots of 32. (Without
+// the slot of the CTA itself, which stays empty, every address takes a comparison of ranks: layers of 2 to 16 rows of
+// 4096 x 4096 took 6.7-7.5 us instead of 6.5-7.3, 5120 x 5120 8.1-8.7 instead of 7.9-8.6.)
 template <int MB, bool WIDE>
 struct StreamSums {
     static constexpr int kSumStride = kTileN + 8;
-    static constexpr int kRecvStride = WIDE ? 7 * 32 : 96;
+    static constexpr int kRecvStride = WIDE ? 8 * 32 : kTileN;
     alignas(16) int sum[StreamCfg<MB>::kRows][kSumStride];
     alignas(16) int recv[StreamCfg<MB>::kRows][kRecvStride];
 };
@@ -702,7 +703,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 const int owner = wide ? (((g4 + 1) * split + 31) >> 5) - 1 : ch >> cw_log;
                 const int at = wide ? ch - 4 * ((32 * owner) / split) : ch & (cw - 1);   // place inside the owner's slice
                 if (owner != rank)
-                    *reinterpret_cast<int4*>(cluster.map_shared_rank(&sm.sums.recv[0][0], owner) + m * Smem::kRecvStride + (rank - (rank > owner ? 1 : 0)) * cw + at) =
+                    *reinterpret_cast<int4*>(cluster.map_shared_rank(&sm.sums.recv[0][0], owner) + m * Smem::kRecvStride + rank * cw + at) =
                         *reinterpret_cast<const int4*>(&sm.sums.sum[m][ch]);
             }
         }
@@ -727,7 +728,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             if (k < split) {
                 int c = rank + k;                                             // the k-th other CTA's slot
                 if (c >= split) c -= split;
-                const int col = (c - (c > rank ? 1 : 0)) * cw + rc;
+                const int col = c * cw + rc;
 #pragma unroll
                 for (int i = 0; i < kIt; ++i)
                     if (i * stride < kRows)                               // the same test in every thread
