@@ -431,7 +431,11 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
     static_assert(2 * RT * DN <= 512, "two accumulator stages of RT x DN columns in tensor memory");
     constexpr int kRows = RT * 128;                                       // rows of A per item
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(attn_smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    // Elected issuing threads pay everywhere but where codes are converted for items of 128 rows: there the paced issue of
+    // `lane == 0` leaves the converting warps more of the shared-memory pipe (40 heads, 1000 x 1008 32.5 -> 31.1 us, 12 heads,
+    // 2000 x 2000 38.4 -> 35.8; items of 256 rows the other way round, 40 heads, 2048 x 1008 46.1 elected, 47.1 paced).
+    constexpr bool kElect = !CONVERT || RT > 1;
+    const int warp = kElect ? __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0) : (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int MT = (M + kRows - 1) / kRows;                               // row tiles per head
     const int items = MT * H;                                             // work items; item w = (head w / MT, row tile w % MT)
     const int JB = (J + 127) / 128;
@@ -461,7 +465,7 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
     volatile uint32_t* abort_flag = &sm.abort_flag;
 
     if (warp == 0) {
-        if (a_elect_one()) {
+        if (kElect ? a_elect_one() : lane == 0) {
             int it = 0;                                                   // stages filled so far, over all items
             bool ok = true;
             for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
@@ -484,7 +488,7 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
             }
         }
     } else if (warp == 1) {
-        if (a_elect_one()) {
+        if (kElect ? a_elect_one() : lane == 0) {
             // D = s32 (2 at bits 4-5), A unsigned 8-bit (0 at bits 7-9), B signed 8-bit (1 at bits 10-12),
             // both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28
             constexpr uint32_t idesc = (2u << 4) | ((A_SIGNED ? 1u : 0u) << 7) | (1u << 10) | ((uint32_t)(DN >> 3) << 17) |
