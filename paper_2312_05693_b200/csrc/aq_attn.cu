@@ -12,7 +12,8 @@ constexpr int kLog2Ctas = 4;                            // CTAs of 256 threads p
 constexpr int kLog2InFlight = 8;                        // 16-byte loads a thread has in flight
 
 // ---- layer-wide max |x| as an fp16 bit pattern (NaN ignored, Inf counts as 65504) -------------
-// 16-byte loads where the pointer allows; the first thread also takes the ragged tail.
+// 16-byte loads where the pointer allows; what they leave (the ragged tail, or all of an array that lies elsewhere) goes round
+// the threads one by one.
 __global__ void __launch_bounds__(256, kLog2Ctas)
 log2_absmax_kernel(const __half* __restrict__ x, long long count, Control* __restrict__ ctl) {
     unsigned int b = 0;
@@ -50,8 +51,7 @@ log2_absmax_kernel(const __half* __restrict__ x, long long count, Control* __res
         take(mw & 0xFFFFu);
         take(mw >> 16);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (long long i = nvec * 8; i < count; ++i) take(__half_as_ushort(x[i]));
+    for (long long i = nvec * 8 + at; i < count; i += stride) take(__half_as_ushort(x[i]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, o));
     if ((threadIdx.x & 31) == 0 && b != 0) atomicMax(&ctl->absmax_bits, b);
@@ -248,12 +248,11 @@ log2_codes_kernel(const __half* __restrict__ x, long long count, int bits, Contr
         if (as_factors) { out[0] = log2_factors4(out[0], bad); out[1] = log2_factors4(out[1], bad); }
         *reinterpret_cast<uint2*>(codes + 8 * i) = make_uint2(out[0], out[1]);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (long long i = nvec * 8; i < count; ++i) {
-            const int c = log2_code(__half_as_ushort(x[i]), mb_bits, eb, t_up, t_down, kmax);
-            bad |= as_factors && c < 0;
-            codes[i] = as_factors ? (int8_t)(uint8_t)(c > 0 ? (128u >> (c - 1)) : 0u) : (int8_t)c;
-        }
+    for (long long i = nvec * 8 + (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
+        const int c = log2_code(__half_as_ushort(x[i]), mb_bits, eb, t_up, t_down, kmax);
+        bad |= as_factors && c < 0;
+        codes[i] = as_factors ? (int8_t)(uint8_t)(c > 0 ? (128u >> (c - 1)) : 0u) : (int8_t)c;
+    }
     if (bad) atomicCAS(&ctl->status, 0u, 11u);
 }
 

@@ -229,3 +229,26 @@ def test_attn_qk_items_with_and_without_whole_boxes_in_turn():
     s, ws = handle().aq_attn_qk_tc(q, e, k, e)
     assert handle().aq_check_workspace(ws) == binding.AQ_OK
     assert torch.equal(s.float(), torch.bmm(q.float(), k.float().transpose(1, 2)).half().float())   # sums below 2^14: exact
+
+
+@pytest.mark.parametrize("count", [1, 7, 4093, 1_000_003])
+def test_log2_codes_of_an_array_off_a_16_byte_boundary(count):
+    """Every element is then taken one by one, by all threads: codes of both widths and factors as of the same values on a
+    boundary, a negative input among the factors' inputs reported."""
+    g = torch.Generator(device="cuda").manual_seed(count)
+    room = torch.rand(count + 8, generator=g, device="cuda").pow_(6).to(torch.float16)
+    room[3 + count // 2] = 0.97
+    loose = room[3:3 + count]
+    x = loose.clone()
+    h = handle()
+    for bits in (4, 8):
+        a, ma = h.aq_log2_quantize(loose, bits)
+        b, mb = h.aq_log2_quantize(x, bits)
+        assert torch.equal(a, b) and torch.equal(ma, mb)
+    fa, ma, ws = h.aq_log2_quantize_factors(loose)
+    assert h.aq_check_workspace(ws) == binding.AQ_OK
+    fb, mb, _ = h.aq_log2_quantize_factors(x)
+    assert torch.equal(fa, fb) and torch.equal(ma, mb)
+    room[3 + count - 1] = -0.5
+    _, _, ws = h.aq_log2_quantize_factors(loose)
+    assert h.aq_check_workspace(ws) == binding.AQ_ERR_INVALID_ARG
