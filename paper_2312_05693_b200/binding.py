@@ -125,7 +125,11 @@ def _host():
     global _native
     if _native is None:
         load()
-        from . import _aq_host
+        try:
+            from . import _aq_host
+        except ImportError as e:
+            raise ImportError("the native half of the binding cannot be loaded: build it for this interpreter and torch with "
+                              "`python -m paper_2312_05693_b200.build`") from e
         _aq_host.set_error(AgileqError)
         _native = _aq_host
     return _native
