@@ -321,9 +321,9 @@ PyObject* attn_v(PyObject* const* v, Py_ssize_t n) {
     const int on_factors = a.integer();
     const at::Tensor &p = a.tensor(), mx = a.optional(), &vc = a.tensor(), ve = a.optional();
     at::Tensor y = a.optional(), ws = a.optional();
-    int H, M, J, H2, J2, D;
+    int H, M, J;
     sizes3(p, H, M, J);
-    sizes3(vc, H2, J2, D);
+    const int D = (int)vc.size(2);
     if (!y.defined()) y = make({H, M, D}, at::kHalf, p);
     if (!ws.defined()) ws = make({(int64_t)aq_attn_workspace_bytes(H, M, J, D)}, at::kByte, p);
     void* s = stream();
@@ -346,9 +346,9 @@ PyObject* attn_qk(PyObject* const* v, Py_ssize_t n) {
     const aq_handle_t h = a.handle();
     const at::Tensor &q = a.tensor(), qe = a.optional(), &k = a.tensor(), ke = a.optional();
     at::Tensor sc = a.optional(), ws = a.optional();
-    int H, M, D, H2, J, D2;
+    int H, M, D;
     sizes3(q, H, M, D);
-    sizes3(k, H2, J, D2);
+    const int J = (int)k.size(1);
     if (!sc.defined()) sc = make({H, M, J}, at::kHalf, q);
     if (!ws.defined()) ws = make({256}, at::kByte, q);
     void* s = stream();

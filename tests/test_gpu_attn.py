@@ -252,3 +252,16 @@ def test_log2_codes_of_an_array_off_a_16_byte_boundary(count):
     room[3 + count - 1] = -0.5
     _, _, ws = h.aq_log2_quantize_factors(loose)
     assert h.aq_check_workspace(ws) == binding.AQ_ERR_INVALID_ARG
+
+
+def test_codes_of_keys_and_values_with_dimensions_of_one_behind():
+    """Only the sizes that the calls use are asked of k and v: a trailing dimension of one changes nothing."""
+    H, M, J, D = 2, 40, 64, 128
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v = (torch.randint(-9, 10, (H, n, D), generator=g, device="cuda", dtype=torch.int8) for n in (M, J, J))
+    p = torch.randint(0, 9, (H, M, J), generator=g, device="cuda", dtype=torch.int8)
+    e = torch.zeros(1, dtype=torch.int32, device="cuda")
+    mx = torch.full((1,), 0x3C00, dtype=torch.int32, device="cuda")
+    h = handle()
+    assert torch.equal(h.aq_attn_qk_tc(q, e, k.unsqueeze(-1), e)[0], h.aq_attn_qk_tc(q, e, k, e)[0])
+    assert torch.equal(h.aq_attn_v_log2_tc(p, mx, v.unsqueeze(-1), e)[0], h.aq_attn_v_log2_tc(p, mx, v, e)[0])
