@@ -299,6 +299,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 // [sender][run of the slice][half][4 columns][channel][column]. The sums stay in tensor memory and are
                 // read once to be sent and once to be finished.
                 constexpr int kRun = BM / kWRuns, kRunInts = 2 * kRun * kTileN;
+                constexpr int kRing = kWStages * (BM * 128 + 2 * kBlockBytes), kRunBytes = kRunInts * 4;
+                static_assert(offsetof(Smem, x) + sizeof(sm.x) == offsetof(Smem, w) && 4 * kRunBytes <= kRing && 2 * 3 * kRunBytes <= kRing &&
+                                  3 * 2 * kRunBytes <= kRing && 4 * 2 * kRunBytes <= kRing && 5 * 2 * kRunBytes <= kRing &&
+                                  6 * 2 * kRunBytes <= kRing && 7 * kRunBytes <= kRing,
+                              "the operand ring (activation tiles, then weight blocks) holds what a CTA receives in clusters of two to eight");
                 cg::cluster_group cluster = cg::this_cluster();
                 int* ring = reinterpret_cast<int*>(&sm.x[0][0]);
                 const int slice_runs = (kWRuns + split - 1) / split;     // the most a CTA owns
@@ -581,7 +586,9 @@ int wide_clusters(const DeviceInfo& dev, int split) {
 // not share the path with all others, and the exchange. 333 rows, N = 5120 (60 tiles, clusters of two): K = 13824
 // 49.2 -> 35.3 us, K = 5120 23.2 -> 22.7 us; 48 rows: 45.3 -> 22.8 us, 22.5 -> 18.6 us. (Only the last, partial round in
 // clusters behind whole rounds: measured slower, K = 13824, N = 5120 at 1024 rows, 148 + 12 tiles, 68 us against 57.6
-// on 192-token tiles.)
+// on 192-token tiles.) All these cycles and times are from before the issuing threads were elected. Since then a block of a
+// 128-token tile takes about 780 cycles (K = 5120, N = 13824 at 1024 rows, three rounds, 47.4 us), and K = 13824, N = 5120 at
+// 333 rows 31.1 us in clusters where the rule says 26: whole tiles are priced some 40 % too high against clusters.
 struct WidePlan {
     int bm, split;                   // token tile; CTAs that share a tile
     long cost;

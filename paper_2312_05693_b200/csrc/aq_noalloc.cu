@@ -51,7 +51,7 @@ extern "C" int aq_linear_w4a8_noalloc(aq_handle_t h, const void* x_fp16, int M, 
     void* scratch = nullptr;
     const int rc = scratch_address(h, &scratch);
     if (rc != AQ_OK) return rc;
-    // aq_linear_w4a8 clears the control block (the only part that must start at zero) itself;
+    // Nothing has to start at zero: the kernels of aq_linear_w4a8 write every word of the control block that they read, and
     // the codes are fully rewritten before they are read.
     return aq_linear_w4a8(h, x_fp16, M, K, w_packed, w_scales, N, group_size, scale_mode, clip_shift_or_exp,
                           nullptr, y_fp16, nullptr, scratch, AQ_NOALLOC_SCRATCH_BYTES, stream);

@@ -98,7 +98,7 @@ def test_quantize_act_static_rowidx_and_nonfinite():
 
 @pytest.mark.parametrize("bits", [8, 4])
 def test_quantize_act_one_pass_kernel_edges(bits):
-    # sizes above the small-activation limit take the cooperative one-pass kernel: ragged split over
+    # sizes above the small-activation limit take the range and quantize kernels: ragged split over
     # the CTAs, exact ties, non-finite values, gathered (repeated, permuted) rows, and exponents on
     # both sides of the half-precision fast path
     M, K = 701, 1152

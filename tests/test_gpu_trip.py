@@ -1,5 +1,5 @@
 """Per-channel TRIP factors (paper Eq. 5-8, Sec. 4.4) on the GPU against the CPU checker: the Eq. 8
-search, the Eq. 5 quantizer with factors (all three quantize kernels: small, one-pass cooperative,
+search, the Eq. 5 quantizer with factors (small activations in one kernel, larger ones in two,
 given exponent) and the whole W4A4 layer through both product kernels."""
 import numpy as np
 import pytest
