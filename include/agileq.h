@@ -127,7 +127,8 @@ int aq_quantize_act(aq_handle_t h, const void* x_fp16, int M, int K, int bits, i
 
 /* ---- the layer (paper Sec. 4.4): quantize, integer product, floating-point output
  * y_fp16 [M,N] row-major. acc_dump: NULL, or int32 [M][N][G] (G as in aq_scales_bytes)
- * receiving the integer sums (test aid; slows the call). row_idx as above. */
+ * receiving the integer sums (test aid; slows the call; with per-group scales and M <= 16 it takes another
+ * kernel, whose fp32 sums may round differently). row_idx as above. */
 int aq_linear_w4a8(aq_handle_t h, const void* x_fp16, int M, int K, const void* w_packed,
                    const void* w_scales, int N, int group_size, int scale_mode,
                    int clip_shift_or_exp, const int32_t* row_idx, void* y_fp16,
@@ -212,7 +213,8 @@ int aq_linear_w4a4_asym(aq_handle_t h, const void* x_fp16, int M, int K, const v
  * As aq_linear_w4a8 / aq_linear_w4a4, but instead of the fp16 outputs the call writes the NEXT layer's
  * activation codes q_next [M,N] int8 row-major: q_next = clip(round(y16 / 2^next_exp), -2^(b-1),
  * 2^(b-1)-1) with b = next_bits (8 or 4), where y16 is exactly the fp16 value the plain call would have
- * written (so the codes equal aq_quantize_act of that output with the static exponent next_exp; NaN -> 0).
+ * written, on the same workspace size and acc_dump or none in both (so the codes equal aq_quantize_act of that
+ * output with the static exponent next_exp; NaN -> 0).
  * The next layer then runs on the codes with aq_gemm_w4 (its scale_exp = next_exp on the device). The
  * exponent has to be known beforehand (calibration), since a layer-wide maximum of y does not exist
  * before the layer has finished. -40 <= next_exp <= 40. */
@@ -281,7 +283,7 @@ int aq_attn_v_log2(aq_handle_t h, const int8_t* p_codes, const uint32_t* p_max_b
 /* The same result on the tensor cores for a non-negative P (a softmax output), 4-bit codes: the factor
  * 2^(kmax - k) is then an unsigned byte and the sums are a u8 x s8 -> s32 contraction over j
  * (tcgen05.mma kind::i8, operands staged by TMA, accumulator in tensor memory). D is 64 or 128,
- * J % 16 == 0; y must be 16-byte aligned. The workspace (aq_attn_workspace_bytes) holds a control block
+ * J % 16 == 0; p_codes and y must be 16-byte aligned. The workspace (aq_attn_workspace_bytes) holds a control block
  * and the transposed value codes (the codes of P become byte factors tile by tile inside the product kernel). A negative code in P is an error: it is counted as 0
  * and aq_check_workspace on this workspace then returns AQ_ERR_INVALID_ARG. */
 /* Query x key scores on int8 (or 4-bit, stored in int8) codes of aq_quantize_act, reduction over the head

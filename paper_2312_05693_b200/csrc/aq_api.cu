@@ -610,7 +610,7 @@ static int attn_v_tc_impl(aq_handle_t h, bool p_is_factors, const int8_t* p_code
     if (H < 1 || H > 65535 || M < 1 || J < 16 || J > 65536 || J % 16 != 0 || (D != 64 && D != 128)) return AQ_ERR_SHAPE;
     if ((long long)H * M > 0x7FFFFFFFll || (long long)H * D > 0x7FFFFFFFll) return AQ_ERR_SHAPE;
     if (!workspace || workspace_bytes_ < aq_attn_workspace_bytes(H, M, J, D)) return AQ_ERR_WORKSPACE;
-    if (!aligned(p_codes, p_is_factors ? 16 : 4) || !aligned(v_codes, 1) || !aligned(y_fp16, 16) || !aligned(p_max_bits, 4) ||
+    if (!aligned(p_codes, 16) || !aligned(v_codes, 1) || !aligned(y_fp16, 16) || !aligned(p_max_bits, 4) ||
         !aligned(v_scale_exp, 4) || !aligned(workspace, 256))
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);

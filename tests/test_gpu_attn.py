@@ -254,6 +254,17 @@ def test_log2_codes_of_an_array_off_a_16_byte_boundary(count):
     assert h.aq_check_workspace(ws) == binding.AQ_ERR_INVALID_ARG
 
 
+def test_codes_of_p_off_a_16_byte_boundary_are_refused_by_name():
+    """They are read by tensor map, which wants 16 bytes: an alignment error, not a failed CUDA call."""
+    H, M, J, D = 1, 32, 32, 64
+    room = torch.ones(H * M * J + 16, dtype=torch.int8, device="cuda")
+    e = torch.zeros(1, dtype=torch.int32, device="cuda")
+    v = torch.ones((H, J, D), dtype=torch.int8, device="cuda")
+    with pytest.raises(binding.AgileqError) as err:
+        handle().aq_attn_v_log2_tc(room[4:4 + H * M * J].view(H, M, J), e, v, e)
+    assert err.value.status == binding.AQ_ERR_ALIGNMENT
+
+
 def test_codes_of_keys_and_values_with_dimensions_of_one_behind():
     """Only the sizes that the calls use are asked of k and v: a trailing dimension of one changes nothing."""
     H, M, J, D = 2, 40, 64, 128
