@@ -52,6 +52,7 @@ def load():
         raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2312_05693_b200.build` "
                           "(there is no fallback implementation)")
     L = C.CDLL(LIB_PATH)
+    # every entry point, also those that the native half calls: a program may use the library returned here directly
     vp, i32, sz = C.c_void_p, C.c_int, C.c_size_t
     L.aq_status_string.restype = C.c_char_p
     L.aq_status_string.argtypes = [i32]
