@@ -13,8 +13,8 @@
 //     by TMA with the 128-byte swizzle and read through an MMA shared-memory descriptor.
 //
 // One persistent CTA per SM walks a static list of (channel tile, token tile) pairs.
-// Warp roles: 0 and 2 = TMA producers (activations / weights), 1 and 3 = MMA issuers (warp 1
-// also owns the TMEM allocation; warp 3 only works in per-group mode), 4-11 = weight unpack
+// Warp roles: 0 and 2 = TMA producers (activations / weights), 1 = MMA issuer (and owner of the TMEM
+// allocation), 3 = watches the accumulator barriers for the epilogue (per-group mode), 4-11 = weight unpack
 // (two groups of four taking alternate k blocks; only the first group works in per-group mode above 64 tokens),
 // 12-19 = epilogue; registers are moved from
 // the first two roles to the epilogue with setmaxnreg. The issuing threads are chosen with elect.sync: then the
@@ -37,7 +37,7 @@ namespace aq {
 namespace {
 
 constexpr int kUnpackGroups = 2;              // groups of four unpack warps; group g takes k blocks g, g+2, ...
-constexpr int kFirstUnpackWarp = 4;           // warps 0-3 (one warpgroup): two TMA producers, two MMA issuers
+constexpr int kFirstUnpackWarp = 4;           // warps 0-3 (one warpgroup): two TMA producers, the MMA issuer
 constexpr int kWarps = 20;
 constexpr int kThreads = kWarps * 32;
 // Registers per thread after the roles split (setmaxnreg works on aligned groups of four warps):
@@ -113,6 +113,18 @@ struct TensorParams {
     int clear_status;              // no quantize kernel of the call has set the control block up
 };
 
+__device__ __forceinline__ __half ld_shared_half(uint32_t addr) {
+    unsigned short v;
+    asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
+    return __ushort_as_half(v);
+}
+// Waits for a phase that is sure to come, whatever has given up elsewhere (all lanes of a warp; limited all the same).
+__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
+    const long long t0 = clock64();
+    bool late = false;
+    while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)) && !late)
+        late = __any_sync(0xFFFFFFFFu, (unsigned long long)(clock64() - t0) > kWaitCycles);
+}
 // One column of this thread's row, waited for.
 __device__ __forceinline__ int tc_ld1(uint32_t taddr) {
     uint32_t v;
@@ -217,7 +229,6 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
     // 2 (or 1 for the 256-token tile) as leave room for the weight-slice ring
     constexpr int kNumAcc = GROUPED ? (BM > 128 ? 2 : 3) : (BM >= 256 ? 1 : 2);
     constexpr int kAccStride = BM;                    // columns between accumulator stages
-    constexpr int kNumMmaThreads = GROUPED ? 2 : 1;   // issuers alternate k blocks when every block has its own accumulator
     constexpr int kAccCols = kNumAcc * kAccStride;
     // the rest of tensor memory (up to 8 slices) is the ring of unpacked weight slices (A operand)
     constexpr int kNumASlices = (512 - kAccCols) / kAColsPerStage >= 8 ? 8 : (512 - kAccCols) / kAColsPerStage;
@@ -326,39 +337,64 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
             }
         }
       } else {
-        // ------------- MMA issuers: warp 1 (and warp 3 in grouped mode, taking the odd k blocks)
-        const int mma_id = warp >> 1;                  // 0 or 1
-        if (mma_id < kNumMmaThreads && elect_one()) {
-            constexpr uint32_t idesc = idesc_i8(128, BM);
-            const uint32_t total_iters = (uint32_t)my_tiles * (uint32_t)(kb_last - kb_first);
-            if (GROUPED) {
-                // Every k block is one accumulation into its own accumulator stage. Ring positions and phases are
-                // carried in counters (steps of kNumMmaThreads): the divisions that gave them from the block's number
-                // were most of this loop, one thread whose every instruction waits for the one before.
-                uint32_t a = (uint32_t)mma_id % kNumAcc, st = (uint32_t)mma_id, ai = (uint32_t)mma_id;
-                uint32_t acc_ph = 1u, a_ph = 0u;
-                const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm.x[0]));
-                for (uint32_t it = mma_id; it < total_iters; it += kNumMmaThreads) {
-                    const bool got_a = mbar_try_wait(&sm.a_full[ai], a_ph);       // both asked before either answer is used
-                    const bool got_acc = mbar_try_wait(&sm.acc_empty[a], acc_ph);
-                    if (!got_acc && !mbar_wait(&sm.acc_empty[a], acc_ph, abort_flag, 2u)) goto role_done;
-                    if (!got_a && !mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 3u)) goto role_done;
+        if (GROUPED && warp == 3) {
+            // ------------- watcher: tells the epilogue warps, through a named barrier per lane quarter and accumulator stage,
+            // that an accumulation is complete. A look at an mbarrier costs a warp some 200 cycles in this kernel even where
+            // the phase is long over, a named barrier some 30, and the epilogue's chain per block sets the pace (K, N = 4096,
+            // 11008 at M = 2048: 124 -> 120 us).
+            // A stage's barrier is not arrived at again before its warps have come by: the next accumulation in it needs
+            // their release. When a wait has given up, no accumulation follows; the remaining arrivals are then paced by
+            // those releases themselves, so that the epilogue warps, which wait without a limit, all come through.
+            uint32_t ph = 0;                                           // a bit per accumulator stage
+            bool live = true;
+            for (int tl = 0; tl < my_tiles; ++tl) {
+                uint32_t a = 0;
+                for (int kb = kb_first; kb < kb_last; ++kb) {
+                    if (live) live = mbar_wait_warp(&sm.acc_full[a], (ph >> a) & 1u, abort_flag, 9u);
+                    if (!live) drain_wait(&sm.acc_empty[a], ((ph >> a) & 1u) ^ 1u);
                     tc_fence_after();
-                    const uint32_t d_addr = tmem_acc + a * (uint32_t)kAccStride;
-                    const uint32_t a_addr = tmem_a + ai * (uint32_t)kAColsPerStage;
-                    const uint64_t bdesc = bdesc0 + (uint64_t)(st * (uint32_t)(BM * 128 / 16));
+                    tc_fence_before();
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc, j > 0 ? 1u : 0u);
-                    tc_commit(&sm.acc_full[a]);
-                    tc_commit(&sm.a_empty[ai]);
-                    tc_commit(&sm.smem_empty[st]);
-                    a += kNumMmaThreads;
-                    if (a >= (uint32_t)kNumAcc) { a -= kNumAcc; acc_ph ^= 1u; }
-                    st += kNumMmaThreads;
-                    if (st >= (uint32_t)kNumStages) st -= kNumStages;
-                    ai += kNumMmaThreads;
-                    if (ai >= (uint32_t)kNumASlices) { ai -= kNumASlices; a_ph ^= 1u; }
+                    for (int q = 0; q < 4; ++q)
+                        asm volatile("bar.arrive %0, %1;" ::"r"(1 + q * kNumAcc + (int)a), "n"(32 + kEpiWarps * 8) : "memory");
+                    ph ^= 1u << a;
+                    if (++a == (uint32_t)kNumAcc) a = 0;
+                }
+            }
+        }
+        // ------------- MMA issuer (one thread: a second one taking the odd k blocks of per-group products changes nothing
+        // since both are elected threads)
+        if (warp == 1 && elect_one()) {
+            constexpr uint32_t idesc = idesc_i8(128, BM);
+            if (GROUPED) {
+                // Every k block is one accumulation into its own accumulator stage; a tile's first block takes stage 0. Ring
+                // positions and phases are carried in counters: the divisions that gave them from the block's number
+                // were most of this loop, one thread whose every instruction waits for the one before.
+                uint32_t st = 0, ai = 0, a_ph = 0u, acc_ph = ~0u;             // acc_ph: a bit per accumulator stage
+                const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sm.x[0]));
+                for (int tl = 0; tl < my_tiles; ++tl) {
+                    uint32_t a = 0;
+                    for (int kb = kb_first; kb < kb_last; ++kb) {
+                        const uint32_t a_bit = (acc_ph >> a) & 1u;
+                        const bool got_a = mbar_try_wait(&sm.a_full[ai], a_ph);       // both asked before either answer is used
+                        const bool got_acc = mbar_try_wait(&sm.acc_empty[a], a_bit);
+                        if (!got_acc && !mbar_wait(&sm.acc_empty[a], a_bit, abort_flag, 2u)) goto role_done;
+                        if (!got_a && !mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 3u)) goto role_done;
+                        tc_fence_after();
+                        const uint32_t d_addr = tmem_acc + a * (uint32_t)kAccStride;
+                        const uint32_t a_addr = tmem_a + ai * (uint32_t)kAColsPerStage;
+                        const uint64_t bdesc = bdesc0 + (uint64_t)(st * (uint32_t)(BM * 128 / 16));
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            tc_mma_i8_ts(d_addr, a_addr + 8 * j, bdesc + (uint64_t)(2 * j), idesc, j > 0 ? 1u : 0u);
+                        tc_commit(&sm.acc_full[a]);
+                        tc_commit(&sm.a_empty[ai]);
+                        tc_commit(&sm.smem_empty[st]);
+                        acc_ph ^= 1u << a;
+                        if (++a == (uint32_t)kNumAcc) a = 0;
+                        if (++st == (uint32_t)kNumStages) st = 0;
+                        if (++ai == (uint32_t)kNumASlices) { ai = 0; a_ph ^= 1u; }
+                    }
                 }
             } else {
                 uint32_t st = 0, ai = 0, a_ph = 0u;
@@ -457,7 +493,13 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         [[maybe_unused]] const float off_factor = OFFSET ? offset_factor(p.ctl, p.zp_mid) : 0.0f;
         [[maybe_unused]] const int G = GROUPED ? KB : 1;
         uint32_t unit = 0;
-        [[maybe_unused]] uint32_t g_a = 0, g_ph = 0, g_slot = 0;   // per-group mode: accumulator stage, its parity, scale slot
+        // per-group mode: the next block's scale, the lane that releases a stage. (The scale is read from a shared-memory
+        // address: stepped as a pointer it was read with generic loads, 5 % of the kernel's time.)
+        [[maybe_unused]] uint32_t sc_addr = smem_u32(&sm.sc[0][r]);
+        [[maybe_unused]] const uint32_t sc_end = sc_addr + Smem::kNumScaleSlots * kTileN * 2;
+        [[maybe_unused]] const bool releases = elect_one();
+        [[maybe_unused]] const uint32_t acc_empty0 = smem_u32(sm.acc_empty);
+        [[maybe_unused]] const uint32_t taddr0 = __shfl_sync(0xFFFFFFFFu, tmem_acc + lane_addr + (uint32_t)col0, 0);
         // CLUSTER: a warp's columns in runs of four tokens, run c finished by CTA c * split / kRuns; a CTA receives (its own share
         // too) at [sender][epilogue warp][run of its slice][lane], four tokens of a channel (16 bytes) a slot, in its operand
         // ring. The loops over a CTA's own runs are rolled: this code runs once, and what it costs is mostly fetching it
@@ -595,18 +637,22 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 float fsum[kColsPerEpiWarp];                             // fp32 partial outputs
 #pragma unroll
                 for (int c = 0; c < kColsPerEpiWarp; ++c) fsum[c] = 0.0f;
-                for (int kb = kb_first; kb < kb_last; ++kb) {
-                    // ring positions are carried in counters (g_a, g_ph, g_slot): no division per block
-                    const int a = (int)g_a;
-                    if (!mbar_wait_warp(&sm.acc_full[a], g_ph, abort_flag, 9u)) goto role_done;
+                // One k block, in accumulator stage `a`. Unrolled over the stages, so that a block's barriers and columns are
+                // constants beside a few registers, and with its releasing lane chosen before the loop, a block takes a warp
+                // some fifteen instructions less of what is not arithmetic (with the watcher, K, N = 4096, 4096 / 4096, 11008 at
+                // M = 2048 58.9 / 127.0 -> 56.1 / 120.5 us). What a block costs an epilogue warp, in
+                // cycles: the named barrier and the loop 100, the first load with the scale 130, the second with the release 150, and
+                // 460 of conversions and FMAs, which the three warps of a scheduler want at the same time.
+                auto block = [&](const uint32_t a, int kb) {
+                    asm volatile("bar.sync %0, %1;" ::"r"(1 + quarter * kNumAcc + (int)a), "n"(32 + kEpiWarps * 8) : "memory");   // the watcher's word
                     tc_fence_after();
                     // This block's MMAs are complete, so its stage (scales included) had landed: the
                     // issuer saw the unpack warps' signal, which they gave after seeing the TMA barrier.
-                    const float sg = __half2float(sm.sc[g_slot][r]) * 0.0625f;
-                    if (++g_a == (uint32_t)kNumAcc) { g_a = 0; g_ph ^= 1u; }
-                    if (++g_slot == (uint32_t)Smem::kNumScaleSlots) g_slot = 0;
+                    const float sg = __half2float(ld_shared_half(sc_addr)) * 0.0625f;
+                    sc_addr += kTileN * 2;
+                    if (sc_addr == sc_end) sc_addr -= Smem::kNumScaleSlots * kTileN * 2;
                     static_assert(kColsPerEpiWarp == 32 || kColsPerEpiWarp == 64, "epilogue register plan");
-                    const uint32_t taddr = tmem_acc + lane_addr + (uint32_t)(a * kAccStride + col0);
+                    const uint32_t taddr = taddr0 + a * (uint32_t)kAccStride;
                     if (p.acc_dump) {
                         // a rolled loop of its own: unrolled with the arithmetic below, the code of these stores (run only
                         // by tests) kept pushing the loop out of the instruction cache
@@ -629,20 +675,25 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                             // the sums are in registers: the accumulator stage goes back to the MMA at once
                             tc_fence_before();
                             __syncwarp();
-                            if (lane == 0) mbar_arrive(&sm.acc_empty[a]);
+                            if (releases) mbar_arrive_a(acc_empty0 + 8u * a);
                         }
 #pragma unroll
                         for (int c = 0; c < kLdCols; c += 2) {
                             // One conversion per element and one FMA per two. (An integer add of the bits of
                             // 1.5 * 2^23 plus a float subtract also converts, on the FMA and ALU pipes, but
-                            // costs a third instruction; measured 8-16 % slower: issue slots are what this
-                            // loop runs out of, not the conversion unit. Paired FMAs, the issuers' counters and
+                            // costs a third instruction; measured 8-16 % slower. Paired FMAs, the issuers' counters and
                             // the dump's code outside this loop: K, N = 4096, 4096 / 4096, 11008 / 11008, 4096 at
                             // M = 2048 65.1 / 139.2 / 137.5 -> 61.7 / 135.3 / 133.3 us.)
                             fma_pair(fsum[c0 + c], fsum[c0 + c + 1], (float)(int)v[c], (float)(int)v[c + 1], sg);
                         }
                     }
+                };
+                for (int kb = kb_first; kb < kb_last; kb += kNumAcc) {
+#pragma unroll
+                    for (int a = 0; a < kNumAcc; ++a)
+                        if (kb + a < kb_last) block((uint32_t)a, kb + a);
                 }
+                if (__any_sync(0xFFFFFFFFu, *abort_flag != 0)) goto role_done;   // some wait gave up: these are not the tile's sums
                 [[maybe_unused]] bool emit = true;
                 if constexpr (SPLIT) {
                     const int ew = warp - kFirstEpiWarp, slot = (int)blockIdx.x >> 1, hf = (int)blockIdx.x & 1;
