@@ -562,9 +562,8 @@ int aq_log2_quantize(aq_handle_t h, const void* x_fp16, long long count, int bit
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     Control* ctl = static_cast<Control*>(workspace);
-    cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(Control), stream);
-    if (e == cudaSuccess)
-        e = launch_log2_quantize(static_cast<const __half*>(x_fp16), count, bits, ctl, codes, max_bits_out, h->dev, stream);
+    const cudaError_t e =
+        launch_log2_quantize(static_cast<const __half*>(x_fp16), count, bits, ctl, codes, max_bits_out, h->dev, stream);
     return e == cudaSuccess ? AQ_OK : cuda_fail(h, e);
 }
 
@@ -576,9 +575,8 @@ int aq_log2_quantize_factors(aq_handle_t h, const void* x_fp16, long long count,
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     Control* ctl = static_cast<Control*>(workspace);
-    cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(Control), stream);
-    if (e == cudaSuccess)
-        e = launch_log2_quantize(static_cast<const __half*>(x_fp16), count, 4, ctl, reinterpret_cast<int8_t*>(factors),
+    const cudaError_t e =
+        launch_log2_quantize(static_cast<const __half*>(x_fp16), count, 4, ctl, reinterpret_cast<int8_t*>(factors),
                                  max_bits_out, h->dev, stream, true);
     return e == cudaSuccess ? AQ_OK : cuda_fail(h, e);
 }
@@ -615,9 +613,8 @@ static int attn_v_tc_impl(aq_handle_t h, bool p_is_factors, const int8_t* p_code
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     Control* ctl = static_cast<Control*>(workspace);
-    cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(Control), stream);
-    if (e == cudaSuccess)
-        e = launch_attn_v_log2_tc(p_codes, p_max_bits, v_codes, v_scale_exp, H, M, J, D, static_cast<__half*>(y_fp16), ctl,
+    const cudaError_t e =
+        launch_attn_v_log2_tc(p_codes, p_max_bits, v_codes, v_scale_exp, H, M, J, D, static_cast<__half*>(y_fp16), ctl,
                                   static_cast<uint8_t*>(workspace) + sizeof(Control), h->dev, stream, p_is_factors);
     return e == cudaSuccess ? AQ_OK : cuda_fail(h, e);
 }
@@ -648,9 +645,8 @@ int aq_attn_qk_tc(aq_handle_t h, const int8_t* q_codes, const int32_t* q_scale_e
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     Control* ctl = static_cast<Control*>(workspace);
-    cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(Control), stream);
-    if (e == cudaSuccess)
-        e = launch_attn_qk_tc(q_codes, q_scale_exp, k_codes, k_scale_exp, H, M, J, D, static_cast<__half*>(s_fp16), ctl,
+    const cudaError_t e =
+        launch_attn_qk_tc(q_codes, q_scale_exp, k_codes, k_scale_exp, H, M, J, D, static_cast<__half*>(s_fp16), ctl,
                               h->dev, stream);
     return e == cudaSuccess ? AQ_OK : cuda_fail(h, e);
 }

@@ -3,19 +3,28 @@
 #include <cuda.h>
 
 #include "aq_common.cuh"
+#include "aq_quant_math.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace aq {
 
 namespace {
 
-constexpr int kLog2Ctas = 4;                            // CTAs of 256 threads per SM, all resident at once
+constexpr int kLog2Ctas = 4;                            // CTAs of 256 threads per SM, all resident at once (codes)
+constexpr int kLog2MaxThreads = 512;                    // the maximum: clusters of eight CTAs, two CTAs per SM, all resident at once
 constexpr int kLog2InFlight = 8;                        // 16-byte loads a thread has in flight
 
 // ---- layer-wide max |x| as an fp16 bit pattern (NaN ignored, Inf counts as 65504) -------------
 // 16-byte loads where the pointer allows; what they leave (the ragged tail, or all of an array that lies elsewhere) goes round
 // the threads one by one.
-__global__ void __launch_bounds__(256, kLog2Ctas)
+// Every cluster leaves its word in the control block; the first CTA sets the status word up.
+__global__ void __cluster_dims__(kRangeCtas, 1, 1) __launch_bounds__(kLog2MaxThreads, 2)
 log2_absmax_kernel(const __half* __restrict__ x, long long count, Control* __restrict__ ctl) {
+    cluster_started_arrive();
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched while the kernel ahead drains
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->status = 0;
     unsigned int b = 0;
     auto take = [&](unsigned int hb) {
         hb &= 0x7FFFu;
@@ -52,9 +61,9 @@ log2_absmax_kernel(const __half* __restrict__ x, long long count, Control* __res
         take(mw >> 16);
     }
     for (long long i = nvec * 8 + at; i < count; i += stride) take(__half_as_ushort(x[i]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, o));
-    if ((threadIdx.x & 31) == 0 && b != 0) atomicMax(&ctl->absmax_bits, b);
+    __shared__ unsigned int peers[kRangeCtas];
+    cluster_started_wait();
+    leave_range<false, kLog2MaxThreads>(ctl, b, 0u, peers, cg::this_cluster().map_shared_rank(&peers[cg::this_cluster().block_rank()], 0));
 }
 
 // A positive fp16 bit pattern as mant * 2^expo with 1024 <= mant < 2048.
@@ -149,14 +158,18 @@ __device__ __forceinline__ __half2 log2_fast2(__half2 x2, const Log2Fast& f) {
 }
 
 __global__ void __launch_bounds__(256, kLog2Ctas)
-log2_codes_kernel(const __half* __restrict__ x, long long count, int bits, Control* __restrict__ ctl,
+log2_codes_kernel(const __half* __restrict__ x, long long count, int bits, int words, Control* __restrict__ ctl,
                   int8_t* __restrict__ codes, uint32_t* __restrict__ max_bits_out, int as_factors) {
     // as_factors (4-bit codes of a non-negative input): instead of the code c the byte 2^(kmax - k) = 128 >> (c - 1)
     // is written (0 for a zero), the form the tensor-core product takes; a negative value is reported (status 11)
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched while the maximum's kernel drains
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     bool bad = false;
-    const unsigned int mb_bits = ctl->absmax_bits;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && max_bits_out) *max_bits_out = mb_bits;
+    const unsigned int mb_bits = met_range(ctl, words);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctl->absmax_bits = mb_bits;
+        if (max_bits_out) *max_bits_out = mb_bits;
+    }
     const int kmax = (1 << (bits - 1)) - 1;
     int mb = 1024, eb = 0, t_up = 0, t_down = 0;
     if (mb_bits) half_parts(mb_bits, mb, eb);
@@ -301,9 +314,17 @@ attn_v_log2_kernel(const int8_t* __restrict__ pcodes, const uint32_t* __restrict
 // operands stored j-major. tcgen05.mma kind::i8 reads both from shared memory (128-byte swizzle,
 // staged by TMA); the accumulator [128 query rows x D] lives in tensor memory.
 
+// The first kernel of a call (launched while the kernel ahead drains) sets the control block up.
+__device__ __forceinline__ void begin_attn_call(Control* ctl) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) ctl->status = 0;
+}
+
 // [H][J][D] int8 -> [H][D][J] int8 through a 32 x 32 shared-memory tile.
 __global__ void __launch_bounds__(256)
-transpose_i8_kernel(const int8_t* __restrict__ in, int J, int D, int8_t* __restrict__ out) {
+transpose_i8_kernel(const int8_t* __restrict__ in, int J, int D, int8_t* __restrict__ out, Control* __restrict__ ctl) {
+    begin_attn_call(ctl);
     __shared__ int8_t tile[32][33];
     const int h = blockIdx.z, j0 = blockIdx.x * 32, d0 = blockIdx.y * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;          // 32 x 8
@@ -321,7 +342,8 @@ transpose_i8_kernel(const int8_t* __restrict__ in, int J, int D, int8_t* __restr
 // The same through a 64 x 64 tile with 4-byte accesses on both sides (D and J multiples of 4, 4-byte aligned
 // buffers): a warp reads and writes 64-byte row pieces as words instead of 32 single bytes.
 __global__ void __launch_bounds__(256)
-transpose_i8_words_kernel(const int8_t* __restrict__ in, int J, int D, int8_t* __restrict__ out) {
+transpose_i8_words_kernel(const int8_t* __restrict__ in, int J, int D, int8_t* __restrict__ out, Control* __restrict__ ctl) {
+    begin_attn_call(ctl);
     __shared__ __align__(4) int8_t tile[64][68];                      // [j][d], rows padded to 68 bytes
     const int h = blockIdx.z, j0 = blockIdx.x * 64, d0 = blockIdx.y * 64;
 #pragma unroll
@@ -406,8 +428,8 @@ struct AttnSmem {
 };
 
 // Batched int8 contraction y[h][m][n] = scale * sum_k A[h*M + m][k] * B[h*NB + n][k] (both operands
-// k-major). A work item is (128 rows of A, head): all tiles of DN rows of B for those rows. The grid is
-// persistent: CTA c takes the items c, c + gridDim.x, ..., and the ring of operand stages and the two
+// k-major). A work item is (128 rows of A, head) and all tiles of DN rows of B for those rows, or one of `parts` runs
+// of those tiles (see attn_parts). The grid is persistent: CTA c takes the items c, c + gridDim.x, ..., and the ring of operand stages and the two
 // accumulator stages in tensor memory run on across items, so the producer fetches the next item's tiles
 // while the epilogue of the last tile of this one still writes (a CTA's 16 k steps of one item alone were
 // mostly fill and drain). With RT = 2 an item is 256 rows of A, two accumulators of 128 rows that share
@@ -422,7 +444,8 @@ template <int DN, bool A_SIGNED, int RT = 1, int EW = 4, bool CONVERT = false>
 __global__ void __launch_bounds__(tc_threads(EW, CONVERT), 1)
 attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map,
                  const __grid_constant__ CUtensorMap y_map, const uint32_t* __restrict__ max_bits, const int32_t* __restrict__ e1, const int32_t* __restrict__ e2,
-                 int e_off, int H, int M, int J /* length of k */, int NB, __half* __restrict__ y, Control* __restrict__ ctl) {
+                 int e_off, int H, int M, int J /* length of k */, int NB, int parts, int clear_status, __half* __restrict__ y,
+                 Control* __restrict__ ctl) {
     extern __shared__ uint8_t attn_smem_raw[];
     using Smem = AttnSmem<DN, RT, EW>;
     static_assert(EW == 4 || (EW == 8 && DN % 64 == 0), "epilogue warps: one or two per lane quarter");
@@ -436,9 +459,18 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
     constexpr bool kElect = !CONVERT || RT > 1;
     const int warp = kElect ? __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0) : (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int MT = (M + kRows - 1) / kRows;                               // row tiles per head
-    const int items = MT * H;                                             // work items; item w = (head w / MT, row tile w % MT)
+    const int items = MT * H * parts;                                     // work items, see below
     const int JB = (J + 127) / 128;
-    const int NT = (NB + DN - 1) / DN;                                    // tiles of B rows per item
+    const int NT = (NB + DN - 1) / DN;                                    // tiles of B rows
+    const int tiles_per_part = (NT + parts - 1) / parts;
+    // item w: head, first row, and the tiles [nt0, nt1) of B rows
+    auto item_at = [&](int w, int& h, int& m0, int& nt0, int& nt1) {
+        const int rows = parts > 1 ? w / parts : w;
+        nt0 = (w - rows * parts) * tiles_per_part;
+        nt1 = min(NT, nt0 + tiles_per_part);
+        h = rows / MT;
+        m0 = (rows - h * MT) * kRows;
+    };
     if (threadIdx.x == 0) {
         for (int s = 0; s < kTcStages; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(a_smem_u32(&sm.full[s])) : "memory");
@@ -462,15 +494,22 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = sm.tmem_base;
     volatile uint32_t* abort_flag = &sm.abort_flag;
+    // Set up while the kernel ahead drains; nothing is read or written before it has completed. The launch behind this one is not
+    // allowed early: its waiting CTAs on the SMs cost this kernel more than the launch gap (scores, byte factors and attention x
+    // value of 32 heads, 2048 x 2048: 216.1 us with plain launches, 217.5 with early ones behind this kernel, 198.7 as it is).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) ctl->status = 0;
 
     if (warp == 0) {
         if (kElect ? a_elect_one() : lane == 0) {
             int it = 0;                                                   // stages filled so far, over all items
             bool ok = true;
             for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
-              const int h = w / MT, m0 = (w % MT) * kRows;
-              for (int i = 0; i < NT * JB; ++i, ++it) {
-                const int nt = i / JB, jb = i % JB, n0 = nt * DN;
+              int h, m0, nt0, nt1;
+              item_at(w, h, m0, nt0, nt1);
+              for (int nt = nt0; nt < nt1 && ok; ++nt)
+              for (int jb = 0; jb < JB; ++jb, ++it) {
+                const int n0 = nt * DN;
                 const int s = it % kTcStages;
                 if (!a_wait(&sm.empty[s], ((it / kTcStages) & 1) ^ 1, abort_flag)) { ok = false; break; }
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
@@ -494,8 +533,10 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
                                        ((uint32_t)(128 >> 4) << 24);
             bool ok = true;
             int it = 0, tc = 0;                                           // stages and tiles consumed so far, over all items
-            for (int w = blockIdx.x; w < items && ok; w += gridDim.x)
-            for (int nt = 0; nt < NT && ok; ++nt, ++tc) {
+            for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
+            int h, m0, nt0, nt1;
+            item_at(w, h, m0, nt0, nt1);
+            for (int nt = nt0; nt < nt1 && ok; ++nt, ++tc) {
               const int a = tc & 1;
               ok = a_wait(&sm.acc_empty[a], ((tc >> 1) & 1) ^ 1, abort_flag);      // the epilogue has drained this stage
               if (!ok) break;
@@ -527,6 +568,7 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              ::"r"(a_smem_u32(&sm.acc_full[a])) : "memory");
             }
+            }
         }
     } else if (CONVERT && warp >= 2 + EW) {
         // ---- codes -> byte factors, in place, on every A tile that has landed (the map is bytewise, so the
@@ -538,7 +580,9 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
         int it = 0;
         bool ok = true;
         for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
-            for (int i = 0; i < NT * JB && ok; ++i, ++it) {
+            int h, m0, nt0, nt1;
+            item_at(w, h, m0, nt0, nt1);
+            for (int i = 0; i < (nt1 - nt0) * JB && ok; ++i, ++it) {
                 const int s = it % kTcStages;
                 ok = __all_sync(0xFFFFFFFFu, a_wait(&sm.full[s], (it / kTcStages) & 1, abort_flag) ? 1 : 0) != 0;
                 if (!ok) break;
@@ -577,8 +621,9 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
         int next_box = 0;
         bool alive = true;
         for (int w = blockIdx.x; w < items && alive; w += gridDim.x) {
-          const int h = w / MT, m0_item = (w % MT) * kRows;
-          for (int nt = 0; nt < NT; ++nt, ++tc) {
+          int h, m0_item, nt0, nt1;
+          item_at(w, h, m0_item, nt0, nt1);
+          for (int nt = nt0; nt < nt1; ++nt, ++tc) {
             const int a = tc & 1, n0 = nt * DN;
             if (!(__all_sync(0xFFFFFFFFu, a_wait(&sm.acc_full[a], (tc >> 1) & 1, abort_flag) ? 1 : 0) != 0)) { alive = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -677,10 +722,24 @@ typedef CUresult (*AttnEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, 
                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// Into how many runs an item's tiles of B rows are cut: as few as give the busiest CTA the fewest tiles. (Whole, the 512 items
+// of 16 tiles that 32 heads of 2048 x 2048 scores have are four rounds, 64 tiles, on 148 SMs whose share is 55.4; in halves 56.)
+inline int attn_parts(long row_items, int tiles, int sms) {
+    int best = 1;
+    long best_tiles = (row_items + sms - 1) / sms * tiles;
+    for (int p = 2; p <= tiles && row_items * p <= 0x7FFFFFFFl; ++p) {
+        const int per = (tiles + p - 1) / p;
+        if ((p - 1) * per >= tiles) continue;                            // the last run would be empty
+        const long most = (row_items * p + sms - 1) / sms * per;
+        if (most < best_tiles) { best_tiles = most; best = p; }
+    }
+    return best;
+}
+
 template <int DN, bool A_SIGNED, int RT = 1, int EW = 4, bool CONVERT = false>
 cudaError_t launch_attn_tc(const void* w, const int8_t* vt, const uint32_t* max_bits, const int32_t* e1, const int32_t* e2,
                            int e_off, int H, int M, int J, int NB, __half* y, Control* ctl, const DeviceInfo& dev,
-                           cudaStream_t stream) {
+                           cudaStream_t stream, bool first_of_call = false) {
     using Smem = AttnSmem<DN, RT, EW>;
     const size_t smem_bytes = sizeof(Smem) + 1024;
     static SmemOptIn opt_in;
@@ -710,11 +769,12 @@ cudaError_t launch_attn_tc(const void* w, const int8_t* vt, const uint32_t* max_
     if (enc(&ymap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, y, ydims, ystrides, ybox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    const int items = ((M + RT * 128 - 1) / (RT * 128)) * H;
-    dim3 grid(items < dev.sm_count ? items : dev.sm_count);
-    attn_v_tc_kernel<DN, A_SIGNED, RT, EW, CONVERT><<<grid, tc_threads(EW, CONVERT), smem_bytes, stream>>>(amap, bmap, ymap, max_bits, e1, e2, e_off, H, M,
-                                                                            J, NB, y, ctl);
-    return cudaGetLastError();
+    const long row_items = (long)((M + RT * 128 - 1) / (RT * 128)) * H;
+    const int parts = attn_parts(row_items, (NB + DN - 1) / DN, dev.sm_count);
+    const long items = row_items * parts;
+    return launch_overlapped_smem(attn_v_tc_kernel<DN, A_SIGNED, RT, EW, CONVERT>, dim3((unsigned int)(items < dev.sm_count ? items : dev.sm_count)),
+                             tc_threads(EW, CONVERT), stream, smem_bytes, amap, bmap, ymap, max_bits, e1, e2, e_off, H, M, J, NB, parts,
+                             first_of_call ? 1 : 0, y, ctl);
 }
 
 }  // namespace
@@ -735,10 +795,9 @@ cudaError_t launch_attn_v_log2_tc(const int8_t* pcodes, const uint32_t* max_bits
     // codes or byte factors: the product kernel reads either
     const uint8_t* w = reinterpret_cast<const uint8_t*>(pcodes);
     if (J % 4 == 0 && D % 4 == 0 && (reinterpret_cast<uintptr_t>(vq) & 3u) == 0 && (reinterpret_cast<uintptr_t>(vt) & 3u) == 0)
-        transpose_i8_words_kernel<<<dim3((J + 63) / 64, (D + 63) / 64, H), 256, 0, stream>>>(vq, J, D, vt);
+        e = launch_overlapped(transpose_i8_words_kernel, dim3((J + 63) / 64, (D + 63) / 64, H), 256, stream, vq, J, D, vt, ctl);
     else
-        transpose_i8_kernel<<<dim3((J + 31) / 32, (D + 31) / 32, H), 256, 0, stream>>>(vq, J, D, vt);
-    e = cudaGetLastError();
+        e = launch_overlapped(transpose_i8_kernel, dim3((J + 31) / 32, (D + 31) / 32, H), 256, stream, vq, J, D, vt, ctl);
     if (e != cudaSuccess) return e;
     const bool wide_items = M % 256 == 0;       // items of 256 query rows share every value tile; whole items only
     if (p_is_factors)
@@ -754,19 +813,23 @@ cudaError_t launch_attn_v_log2_tc(const int8_t* pcodes, const uint32_t* max_bits
 cudaError_t launch_attn_qk_tc(const int8_t* qc, const int32_t* e_q, const int8_t* kc, const int32_t* e_k, int H, int M,
                               int J, int D, __half* s_out, Control* ctl, const DeviceInfo& dev, cudaStream_t stream) {
     // one k step per tile (k = D = 128): the epilogue, 64 KB of scores per tile and row block, sets the pace
-    return launch_attn_tc<128, true, 1, 8>(qc, kc, nullptr, e_q, e_k, 0, H, M, D, J, s_out, ctl, dev, stream);
+    return launch_attn_tc<128, true, 1, 8>(qc, kc, nullptr, e_q, e_k, 0, H, M, D, J, s_out, ctl, dev, stream, true);
 }
 
 cudaError_t launch_log2_quantize(const __half* x, long long count, int bits, Control* ctl, int8_t* codes,
                                  uint32_t* max_bits_out, const DeviceInfo& dev, cudaStream_t stream, bool as_factors) {
+    // as many clusters as the control block has words for (232 CTAs: two per SM of most), fewer for small arrays
+    long long clusters = (count / 8 + kRangeCtas * kLog2MaxThreads - 1) / (kRangeCtas * kLog2MaxThreads);
+    if (clusters > Control::kRangeWords) clusters = Control::kRangeWords;
+    if (clusters < 1) clusters = 1;
+    const cudaError_t e = launch_overlapped(log2_absmax_kernel, dim3((unsigned int)clusters * kRangeCtas), kLog2MaxThreads, stream, x, count, ctl);
+    if (e != cudaSuccess) return e;
     long long blocks = (count / 8 + 255) / 256;
     const long long cap = (long long)dev.sm_count * kLog2Ctas;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    log2_absmax_kernel<<<(unsigned int)blocks, 256, 0, stream>>>(x, count, ctl);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_overlapped(log2_codes_kernel, (size_t)blocks, 256, stream, x, count, bits, ctl, codes, max_bits_out, as_factors ? 1 : 0);
+    return launch_overlapped(log2_codes_kernel, dim3((unsigned int)blocks), 256, stream, x, count, bits, (int)clusters, ctl, codes, max_bits_out,
+                             as_factors ? 1 : 0);
 }
 
 cudaError_t launch_attn_v_log2(const int8_t* pcodes, const uint32_t* max_bits, const int8_t* vq, const int32_t* e_v,

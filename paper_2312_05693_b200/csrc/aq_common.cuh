@@ -105,10 +105,11 @@ struct SmemOptIn {
 // A launch that may be set up while the kernel ahead of it on the stream drains; the kernels launched this way touch no
 // memory before that kernel has completed.
 template <class... Params, class... Args>
-cudaError_t launch_overlapped(void (*kernel)(Params...), size_t grid, int threads, cudaStream_t stream, Args... args) {
+cudaError_t launch_overlapped_smem(void (*kernel)(Params...), dim3 grid, int threads, cudaStream_t stream, size_t smem_bytes, Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned int)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -116,6 +117,10 @@ cudaError_t launch_overlapped(void (*kernel)(Params...), size_t grid, int thread
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, int threads, cudaStream_t stream, Args... args) {
+    return launch_overlapped_smem(kernel, grid, threads, stream, 0, args...);
 }
 
 cudaError_t launch_pack_w4(const __half* w, int N, int K, int group, uint8_t* packed, __half* scales,

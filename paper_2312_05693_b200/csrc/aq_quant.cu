@@ -50,13 +50,6 @@ __device__ __forceinline__ uint4 quantize16_fp32(const uint4& d0, const uint4& d
     return make_uint4(r0.x, r0.y, r1.x, r1.y);
 }
 
-// A CTA may write into another one's shared memory only once that one has started, which being scheduled together does
-// not promise: every thread arrives at its kernel's top and waits just before the kernel's first remote store (a CTA
-// whose share of X is empty gets there at once). Behind the loads the wait costs next to nothing: without it and with
-// it 2.11 / 2.12 us on 6 x 4096, 3.44 / 3.47 us on 48 x 4096, 9.68 / 9.67 us on 2048 x 4096 (quantize calls, graph replay).
-__device__ __forceinline__ void cluster_started_arrive() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
-__device__ __forceinline__ void cluster_started_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-
 // ---- small activations (decode): maximum, exponent and codes in ONE kernel -------------
 // One cluster of 8 CTAs x 512 threads holds the whole activation in registers (up to 8 vectors of
 // 8 halves per thread), so x is read once; the CTAs' maxima are exchanged through distributed
@@ -166,7 +159,7 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
 // that cleared the control block. X crossed HBM and L2 once there, but of 12.1 us (2048 x 4096) 4 were the clearing and
 // the cooperative launch and 2 the meeting. In graph replay over rotating inputs: 2048 x 4096 12.1 -> 9.1 us,
 // 2048 x 11008 21.9 -> 18.0 us, 1024 x 5120 10.1 -> 6.6 us, 333 x 5120 8.3 -> 5.5 us.
-constexpr int kRangeThreads = 512, kRangeCtas = 8;
+constexpr int kRangeThreads = 512;
 constexpr int kRangeInFlight = 8;
 
 // Place of element number v (per_row elements a row) in the gathered rows, carried along in steps: one division at the
@@ -197,9 +190,6 @@ template <bool ASYM>
 __global__ void __cluster_dims__(kRangeCtas, 1, 1) __launch_bounds__(kRangeThreads)
 range_kernel(const uint4* __restrict__ x, size_t vecs /* of 8 halves */, int vec_per_row, const int32_t* __restrict__ row_idx,
              size_t vecs_per_cta, Control* __restrict__ ctl) {
-    cg::cluster_group cluster = cg::this_cluster();
-    __shared__ unsigned int warp_max[kRangeThreads / 32], warp_min[kRangeThreads / 32];
-    __shared__ unsigned int peers[kRangeCtas];
     cluster_started_arrive();
     asm volatile("griddepcontrol.wait;" ::: "memory");      // the kernel ahead may have written X
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -237,39 +227,9 @@ range_kernel(const uint4* __restrict__ x, size_t vecs /* of 8 halves */, int vec
         const __half2 n2 = __habs2(lo2);
         bmin = max((unsigned int)__half_as_ushort(__low2half(n2)), (unsigned int)__half_as_ushort(__high2half(n2)));
     }
-    if (bmax > 0x7C00u) bmax = 0;                            // never publish NaN
-    if (bmin > 0x7C00u) bmin = 0;
-    bmax = __reduce_max_sync(0xFFFFFFFFu, bmax);
-    if (ASYM) bmin = __reduce_max_sync(0xFFFFFFFFu, bmin);
-    if ((threadIdx.x & 31) == 0) {
-        warp_max[threadIdx.x >> 5] = bmax;
-        warp_min[threadIdx.x >> 5] = bmin;
-    }
+    __shared__ unsigned int peers[kRangeCtas];
     cluster_started_wait();
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        bmax = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kRangeThreads / 32 ? warp_max[threadIdx.x] : 0u);
-        bmin = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kRangeThreads / 32 ? warp_min[threadIdx.x] : 0u);
-        if (threadIdx.x == 0) *cluster.map_shared_rank(&peers[cluster.block_rank()], 0) = bmax | (bmin << 16);
-    }
-    cluster.sync();
-    if (cluster.block_rank() == 0 && threadIdx.x == 0) {
-        unsigned int hi = 0, lo = 0;
-#pragma unroll
-        for (int r = 0; r < kRangeCtas; ++r) {
-            hi = max(hi, peers[r] & 0xFFFFu);
-            lo = max(lo, peers[r] >> 16);
-        }
-        ctl->range[blockIdx.x / kRangeCtas] = hi | (lo << 16);
-    }
-}
-
-// The words of range_kernel, met: largest positive (or absolute) value in the low half, largest magnitude of a negative
-// one in the high half. Whole warps call this.
-__device__ __forceinline__ unsigned int met_range(const Control* ctl, int words) {
-    const unsigned int lane = threadIdx.x & 31;
-    const unsigned int w = lane < (unsigned int)words ? ctl->range[lane] : 0u;
-    return __reduce_max_sync(0xFFFFFFFFu, w & 0xFFFFu) | (__reduce_max_sync(0xFFFFFFFFu, w >> 16) << 16);
+    leave_range<ASYM, kRangeThreads>(ctl, bmax, bmin, peers, cg::this_cluster().map_shared_rank(&peers[cg::this_cluster().block_rank()], 0));
 }
 
 // What the product kernel finds in the control block.
@@ -656,7 +616,7 @@ cudaError_t launch_range(const __half* x, int M, int K, const int32_t* row_idx, 
     if (clusters > Control::kRangeWords) clusters = Control::kRangeWords;
     words = (int)clusters;
     const size_t ctas = clusters * kRangeCtas;
-    return launch_overlapped(range_kernel<ASYM>, ctas, kRangeThreads, stream, reinterpret_cast<const uint4*>(x), vecs, K / 8, row_idx,
+    return launch_overlapped(range_kernel<ASYM>, dim3((unsigned int)ctas), kRangeThreads, stream, reinterpret_cast<const uint4*>(x), vecs, K / 8, row_idx,
                              (vecs + ctas - 1) / ctas, ctl);
 }
 
@@ -674,7 +634,7 @@ cudaError_t launch_quantize(const __half* x, int M, int K, const int32_t* row_id
         const cudaError_t e = launch_range<false>(x, M, K, row_idx, ctl, stream, words);
         if (e != cudaSuccess) return e;
     }
-    return launch_overlapped(quantize_kernel, quantize_grid(M, K), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
+    return launch_overlapped(quantize_kernel, dim3((unsigned int)quantize_grid(M, K)), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
                              row_idx, bits, words, clip_shift_or_exp, ctl, reinterpret_cast<uint4*>(q), scale_exp_out,
                              reinterpret_cast<const uint4*>(alpha), k_max);
 }
@@ -699,7 +659,7 @@ cudaError_t launch_quantize_asym(const __half* x, int M, int K, const int32_t* r
     int words = 0;
     const cudaError_t e = launch_range<true>(x, M, K, row_idx, ctl, stream, words);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(quantize_asym_kernel, quantize_grid(M, K), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
+    return launch_overlapped(quantize_asym_kernel, dim3((unsigned int)quantize_grid(M, K)), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
                              row_idx, bits, words, ctl, reinterpret_cast<uint4*>(q), scale_exp_out, zero_point_out);
 }
 

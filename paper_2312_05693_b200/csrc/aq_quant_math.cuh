@@ -2,6 +2,8 @@
 // shared by the quantize kernels and the decode kernel that quantizes its own activations.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "aq_common.cuh"
 
 namespace aq {
@@ -59,6 +61,57 @@ __device__ __forceinline__ uint2 quantize8_fp32(const uint4& d, int e, float lo,
         out[w] = word;
     }
     return make_uint2(out[0], out[1]);
+}
+
+// A CTA may write into another one's shared memory only once that one has started, which being scheduled together does
+// not promise: every thread arrives at its kernel's top and waits just before the kernel's first remote store (a CTA
+// whose share of X is empty gets there at once). Behind the loads the wait costs next to nothing: without it and with
+// it 2.11 / 2.12 us on 6 x 4096, 3.44 / 3.47 us on 48 x 4096, 9.68 / 9.67 us on 2048 x 4096 (quantize calls, graph replay).
+__device__ __forceinline__ void cluster_started_arrive() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_started_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// ---- the largest magnitudes of a whole array, without a word that has to be cleared beforehand: every cluster of
+// kRangeCtas CTAs leaves one word in the control block, and whoever needs the outcome reads all of them.
+constexpr int kRangeCtas = 8;
+// What a CTA's threads have seen: bit patterns of halves, the largest positive (or absolute) value and (TWO_SIDED) the largest
+// magnitude of a negative one. All threads of all CTAs of the cluster call this, once, behind cluster_started_wait(). peers: a
+// shared-memory word per CTA of the cluster; peer_slot: this CTA's word of them in the cluster's first CTA.
+template <bool TWO_SIDED, int THREADS>
+__device__ __forceinline__ void leave_range(Control* ctl, unsigned int bmax, unsigned int bmin, const unsigned int* peers, unsigned int* peer_slot) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ unsigned int warp_max[THREADS / 32], warp_min[THREADS / 32];
+    if (bmax > 0x7C00u) bmax = 0;                            // never publish NaN
+    if (bmin > 0x7C00u) bmin = 0;
+    bmax = __reduce_max_sync(0xFFFFFFFFu, bmax);
+    if (TWO_SIDED) bmin = __reduce_max_sync(0xFFFFFFFFu, bmin);
+    if ((threadIdx.x & 31) == 0) {
+        warp_max[threadIdx.x >> 5] = bmax;
+        warp_min[threadIdx.x >> 5] = bmin;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        bmax = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < THREADS / 32 ? warp_max[threadIdx.x] : 0u);
+        bmin = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < THREADS / 32 ? warp_min[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) *peer_slot = bmax | (bmin << 16);
+    }
+    cluster.sync();
+    if (cluster.block_rank() == 0 && threadIdx.x == 0) {
+        unsigned int hi = 0, lo = 0;
+#pragma unroll
+        for (int r = 0; r < kRangeCtas; ++r) {
+            hi = max(hi, peers[r] & 0xFFFFu);
+            lo = max(lo, peers[r] >> 16);
+        }
+        ctl->range[blockIdx.x / kRangeCtas] = hi | (lo << 16);
+    }
+}
+// The words of leave_range, met: largest positive (or absolute) value in the low half, largest magnitude of a negative
+// one in the high half. Whole warps call this.
+__device__ __forceinline__ unsigned int met_range(const Control* ctl, int words) {
+    const unsigned int lane = threadIdx.x & 31;
+    const unsigned int w = lane < (unsigned int)words ? ctl->range[lane] : 0u;
+    return __reduce_max_sync(0xFFFFFFFFu, w & 0xFFFFu) | (__reduce_max_sync(0xFFFFFFFFu, w >> 16) << 16);
 }
 }  // namespace
 
