@@ -130,9 +130,9 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     const __half* xh = static_cast<const __half*>(x);
     if (alpha && !aligned(alpha, 16)) return AQ_ERR_ALIGNMENT;
     cudaError_t e = cudaSuccess;
-    // a single row on the few-row kernel: that kernel finds the scale and makes the codes itself
+    // a single row, or a few short ones, on the few-row kernel: that kernel finds the scale and makes the codes itself
     const bool fuse = !w_offsets && !alpha && kernel_for(h, M) == AQ_KERNEL_DECODE &&
-                      decode_can_fuse_quantize(M, K, N, group, acc_dump != nullptr, h->dev.sm_count) &&
+                      decode_can_fuse_quantize(M, K, N, group, acc_dump != nullptr, h->weights_stable != 0, h->dev) &&
                       (!group || aligned(w_scales, 16));
     if (fuse) {
     } else if (w_offsets) {

@@ -212,7 +212,7 @@ struct GemmArgs {
     // fp32 partial outputs of tiles whose k range two CTAs share (tensor kernel, per-group scales)
     float* split_scratch = nullptr;
     size_t split_bytes = 0;
-    // One row (M = 1): the few-row streaming kernel quantizes the activations itself (no quantize kernel runs
+    // One row, or a few short ones: the few-row streaming kernel quantizes the activations itself (no quantize kernel runs
     // ahead); q then receives the codes, the control block the exponent.
     const __half* fuse_x = nullptr;
     const int32_t* fuse_row_idx = nullptr;
@@ -237,6 +237,6 @@ size_t tensor_split_scratch_bytes(int M, int K, int N, int group, int sm_count);
 cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const DeviceInfo& dev, cudaStream_t stream);
 constexpr int kFewRows = 16;         // rows up to which the streaming kernel runs, and AQ_KERNEL_AUTO takes it
 cudaError_t launch_gemm_decode(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream);
-bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, int sm_count);
+bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool weights_stable, const DeviceInfo& dev);
 
 }  // namespace aq

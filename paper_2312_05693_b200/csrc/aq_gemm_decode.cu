@@ -184,6 +184,10 @@ gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
 // ---------------------------------------------------------------------------------------
 constexpr unsigned long long kStrWaitCycles = 4000000000ull;
 constexpr int kFuseMaxBlocks = 64;        // k blocks per CTA up to which a single row is quantized inside the product kernel
+// Several rows: what the product kernel can quantize itself, kFuseVecs vectors of eight elements per thread (M * K <= 27648) and
+// kFuseTileBytes of codes of a CTA's k range (8 or 16 rows), and what is left to it: see decode_can_fuse_quantize.
+constexpr int kFuseVecs = 12, kFuseTileBytes = 20 * 1024;
+constexpr long kFuseElems = 12288, kFuseWeightBytes = 4l << 20;
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ bool str_try_wait(uint64_t* bar, uint32_t parity) {
@@ -250,16 +254,16 @@ struct StreamSums {
     alignas(16) int sum[StreamCfg<MB>::kRows][kSumStride];
     alignas(16) int recv[StreamCfg<MB>::kRows][kRecvStride];
 };
-template <int MB, bool GROUPED>
+template <int MB, bool GROUPED, bool FUSEQ>
 struct StreamRing {
     static constexpr int kStages = StreamCfg<MB>::kStages;
-    alignas(1024) int8_t x[kStages][StreamCfg<MB>::kRows * kTileK];    // activation codes of the unit's k block
+    alignas(1024) int8_t x[FUSEQ && MB > 1 ? 1 : kStages][FUSEQ && MB > 1 ? kFuseTileBytes : StreamCfg<MB>::kRows * kTileK];   // activation codes of the unit's k block (FUSEQ: of all of the CTA's)
     alignas(128) uint8_t w[kStages][kBlockBytes];          // packed weight block of the unit
     alignas(16) __half sc[GROUPED ? kStages : 1][kTileN];  // per-group scales: those of the unit's k block (= its group)
 };
-template <int MB, bool WIDE = false, bool GROUPED = false>
+template <int MB, bool WIDE = false, bool GROUPED = false, bool FUSEQ = false>
 struct StreamSmem {
-    StreamRing<MB, GROUPED> ring;
+    StreamRing<MB, GROUPED, FUSEQ> ring;
     StreamSums<MB, WIDE> sums;
     static constexpr int kStages = StreamCfg<MB>::kStages;
     static constexpr int kRecvStride = StreamSums<MB, WIDE>::kRecvStride;
@@ -289,11 +293,11 @@ struct StreamParams {
     int early_dependents;          // the launch behind this one may be set up from this kernel's start
     int next_packed;
     int box_rows;                  // rows of the activation tensor map's box: 8 when M <= 8 (MMA route)
-    // FUSEQ (one row): the activations themselves; the kernel finds the layer scale, writes the codes of
+    // FUSEQ: the activations themselves; the kernel finds the layer scale, writes the codes of
     // its k range to shared memory (and, from the first channel tile, to q_out) and fills the control block
-    const __half* x_row;           // the row's K halves
-    const int32_t* row_idx;        // NULL or one index: the row is x_row + row_idx[0] * K
-    int8_t* q_out;                 // [K] codes
+    const __half* x_row;           // the rows, K halves each
+    const int32_t* row_idx;        // NULL or M indices: row m is x_row + row_idx[m] * K
+    int8_t* q_out;                 // [M][K] codes
     int bits, scale_mode, clip_shift_or_exp;
 };
 
@@ -317,10 +321,9 @@ __device__ __forceinline__ int add_sums(int a, int b) {
 template <int MB, bool FUSEQ = false, bool WIDE = false, bool GROUPED = false>
 __global__ void __launch_bounds__(StreamCfg<MB>::kThreads, 2)
 gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const StreamParams p) {
-    static_assert(!FUSEQ || MB == 1, "only a single row is quantized inside the product kernel");
     static_assert(!WIDE || MB == 16, "clusters of 5 to 8 are for the MMA route");
     extern __shared__ uint8_t smem_raw[];
-    using Smem = StreamSmem<MB, WIDE, GROUPED>;
+    using Smem = StreamSmem<MB, WIDE, GROUPED, FUSEQ>;
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr bool kUseMma = StreamCfg<MB>::kUseMma;
     constexpr int kRows = StreamCfg<MB>::kRows;
@@ -339,7 +342,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     // (after its k range) every CTA of the cluster has started. The wait comes just before those writes.
     if (split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     if (threadIdx.x == 0) {
-        if constexpr (kRows > 1)     // start the descriptor's fetch now; the first tile load would wait for it
+        if constexpr (kRows > 1 && !FUSEQ)     // start the descriptor's fetch now; the first tile load would wait for it
             asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
         for (int s = 0; s < kStrStages; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(&sm.full[s])) : "memory");
@@ -409,7 +412,79 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) p.ctl->status = 0;   // nothing has given up yet
     [[maybe_unused]] int fused_exp = 0;
-    if constexpr (FUSEQ) {
+    if constexpr (FUSEQ && MB > 1) {
+        // ---- several rows: every CTA reads all of them, once, into registers, finds the layer's scale, and makes the codes it
+        // multiplies. What it replaces, a quantize kernel ahead of this one, is one launch more, with its drain, this kernel's
+        // wait and the codes' way through L2. (A CTA that reads only its k range and exchanges its largest magnitude with the
+        // others of its cluster pays a meeting instead: 6 x 4096 x 4096 7.3 us behind a quantize kernel, 7.9 with the meeting.)
+        if (warp == 0 && s_elect_one())
+            for (int i = issued; i < ring; ++i) issue_w(kb0 + i, i);   // weights on their way meanwhile
+        issued = ring;
+        const int per_row = p.K / 8, total = p.M * per_row;              // vectors of eight elements
+        const int step_m = kStrThreads / per_row, step_c = kStrThreads - step_m * per_row;
+        const int m_start = (int)threadIdx.x / per_row, c_start = (int)threadIdx.x - m_start * per_row;
+        uint4 keep[kFuseVecs];
+        {
+            int m = m_start, c = c_start;
+#pragma unroll
+            for (int i = 0; i < kFuseVecs; ++i) {
+                keep[i] = make_uint4(0, 0, 0, 0);
+                if ((int)threadIdx.x + i * kStrThreads < total)
+                    keep[i] = __ldg(reinterpret_cast<const uint4*>(p.x_row) + (size_t)(p.row_idx ? p.row_idx[m] : m) * per_row + c);
+                m += step_m;
+                c += step_c;
+                if (c >= per_row) { c -= per_row; ++m; }
+            }
+        }
+        int e = p.clip_shift_or_exp;
+        if (p.scale_mode == AQ_SCALE_DYNAMIC) {
+            __half2 m2 = __float2half2_rn(0.0f);
+#pragma unroll
+            for (int i = 0; i < kFuseVecs; ++i) {
+                const __half2* h = reinterpret_cast<const __half2*>(&keep[i]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) m2 = __hmax2(m2, __habs2(h[k]));   // NaN operands are dropped; absent vectors are zero
+            }
+            unsigned int bmax = max((unsigned int)__half_as_ushort(__low2half(m2)), (unsigned int)__half_as_ushort(__high2half(m2)));
+            if (bmax > 0x7C00u) bmax = 0;
+            bmax = __reduce_max_sync(0xFFFFFFFFu, bmax);
+            if (lane == 0) sm.warp_max[warp] = bmax;
+            __syncthreads();
+            unsigned int all = 0;
+#pragma unroll
+            for (int w = 0; w < kStrThreads / 32; ++w) all = max(all, sm.warp_max[w]);
+            e = layer_exponent_from_bits(all, p.bits) - p.clip_shift_or_exp;
+            if (tile == 0 && rank == 0 && threadIdx.x == 0) p.ctl->absmax_bits = all;
+        }
+        if (tile == 0 && rank == 0) {
+            if (threadIdx.x == 0) p.ctl->scale_exp = e;
+            if (threadIdx.x < Control::kSplitWords) p.ctl->split_flags[threadIdx.x] = 0;
+        }
+        const float lo = -(float)(1 << (p.bits - 1)), hi = (float)((1 << (p.bits - 1)) - 1);
+        const bool fast = e >= -14 && e <= 14;             // 2^-e is a normal half: codes in half2 arithmetic
+        const __half2 inv2 = __float2half2_rn(fast ? __int_as_float((127 - e) << 23) : 1.0f);
+        const __half2 lo2 = __float2half2_rn(lo), hi2 = __float2half2_rn(hi);
+        const int c_first = kb0 * (kTileK / 8), c_last = kb1 * (kTileK / 8);      // this CTA's k range
+        int m = m_start, c = c_start;
+#pragma unroll
+        for (int i = 0; i < kFuseVecs; ++i) {
+            if ((int)threadIdx.x + i * kStrThreads < total && c >= c_first && c < c_last) {
+                uint2 code;
+                if (fast) quantize8_half2(keep[i], inv2, lo2, hi2, code.x, code.y);
+                else code = quantize8_fp32(keep[i], e, lo, hi, nullptr);
+                // rows of 128 bytes by k block, 16-byte chunks swizzled by row % 8 as a tensor-map copy leaves them
+                const int at = c - c_first;
+                *reinterpret_cast<uint2*>(sm.ring.x[0] + ((at >> 4) * p.box_rows + m) * kTileK + ((((at & 15) >> 1) ^ (m & 7)) << 4) + 8 * (at & 1)) = code;
+                if (tile == 0) *reinterpret_cast<uint2*>(p.q_out + (size_t)m * p.K + 8 * c) = code;
+            }
+            m += step_m;
+            c += step_c;
+            if (c >= per_row) { c -= per_row; ++m; }
+        }
+        fused_exp = e;
+        __syncthreads();
+    }
+    if constexpr (FUSEQ && MB == 1) {
         // ---- the layer scale and this CTA's codes (Eq. 1, Eq. 2 / Eq. 5 with zp = 0; one scale for the layer)
         if (warp == 0 && s_elect_one())
             for (int i = issued; i < ring; ++i) issue_w(kb0 + i, i);   // weights on their way meanwhile
@@ -597,6 +672,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 const uint32_t it = (uint32_t)(kb - kb0);
                 const int s = (int)(it % kStrStages);
                 if (!__all_sync(0xFFFFFFFFu, str_wait(&sm.full[s], (it / kStrStages) & 1u, abort_flag) ? 1 : 0)) break;
+                const int8_t* xt = FUSEQ ? sm.ring.x[0] + (kb - kb0) * p.box_rows * kTileK : sm.ring.x[s];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     // The sum over k does not depend on which k sits in which slot of the instruction, as long
@@ -613,9 +689,9 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(pw[0]), "=r"(pw[1]), "=r"(pw[2]), "=r"(pw[3])
                                  : "r"(s_u32(sm.ring.w[s] + (size_t)(j * kTileN + quarter * 32 + lane) * 16)) : "memory");
-                    const uint2 xa = *reinterpret_cast<const uint2*>(sm.ring.x[s] + g * kTileK + x_off);
+                    const uint2 xa = *reinterpret_cast<const uint2*>(xt + g * kTileK + x_off);
                     uint2 xb = make_uint2(0u, 0u);
-                    if (upper) xb = *reinterpret_cast<const uint2*>(sm.ring.x[s] + (g + 8) * kTileK + x_off);
+                    if (upper) xb = *reinterpret_cast<const uint2*>(xt + (g + 8) * kTileK + x_off);
                     const uint32_t a0 = xa.x, a1 = xb.x, a2 = xa.y, a3 = xb.y;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -779,19 +855,19 @@ inline int decode_split(int tiles, int KB, int sm_count) {
 
 template <int MB, bool FUSEQ, bool WIDE, bool GROUPED>
 cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int wide_split = 0) {
-    using Smem = StreamSmem<MB, WIDE, GROUPED>;
+    using Smem = StreamSmem<MB, WIDE, GROUPED, FUSEQ>;
     const size_t smem_bytes = sizeof(Smem) + 1024;
     static SmemOptIn opt_in;
     if (const cudaError_t e = opt_in.ensure(gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED>, dev.device, smem_bytes); e != cudaSuccess)
         return e;
-    CUtensorMap map;
+    CUtensorMap map = {};
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
     const cuuint64_t strides[1] = {(cuuint64_t)a.K};
     // MMA route: 8 or 16 rows; rows 8..15 are neither copied nor read when M <= 8
     const int box_rows = StreamCfg<MB>::kUseMma ? round_up(a.M, 8) : StreamCfg<MB>::kRows;
     const cuuint32_t box[2] = {128u, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1u, 1u};
-    const CUresult r = reinterpret_cast<EncodeTiledFn>(dev.encode_tiled)(
+    const CUresult r = FUSEQ ? CUDA_SUCCESS : reinterpret_cast<EncodeTiledFn>(dev.encode_tiled)(      // (FUSEQ: nothing is fetched through it)
         &map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t*>(a.q), dims, strides, box, estr,
         CU_TENSOR_MAP_INTERLEAVE_NONE,
         StreamCfg<MB>::kUseMma ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -842,8 +918,8 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
 // loses with clusters of 8 (N = 4096, K = 5120: 5.1 -> 6.2 us). Plain and chained calls take the same cluster
 // (with per-group scales its size sets the order of the fp32 sums). Returns the cluster size (5 to 8), or 0 for the usual 1, 2 or 4.
 template <int MB, bool GROUPED>
-int wide_split_for(const GemmArgs& a, const DeviceInfo& dev) {
-    const int tiles = round_up(a.N, kTileN) / kTileN, KB = k_blocks(a.K);
+int wide_split_for(int K, int N, const DeviceInfo& dev) {
+    const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
     if (decode_split(tiles, KB, dev.sm_count) != 4) return 0;
     static std::atomic<int> fits[kMaxDevices][9];               // clusters of s that run at once, + 1 (0: not asked yet)
     int s = (2 * dev.sm_count) / tiles;
@@ -900,20 +976,30 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
 
 }  // namespace
 
-// One row and a k range per CTA that fits the kernel's code buffer: the product kernel can quantize the row itself
-// (one launch for the layer). Dumps of per-group sums are left to the general kernel.
-bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, int sm_count) {
-    if (M != 1 || (group && dump)) return false;
+// Whether the product kernel quantizes the rows itself (one launch for the layer). Dumps of per-group sums are left to the general
+// kernel. A single row: where a CTA's k range fits its code buffer. Several rows: up to kFuseElems elements of X, where that
+// takes the GPU as long as a quantize kernel ahead (in graph replay, two launches / one: 16 x 768 x 768 5.80 / 5.72 us, 2 x 5120 x 5120
+// 7.76 / 7.51; beyond, every CTA reading all of X costs more: 16 x 1664 x 1664 6.23 / 7.08, 6 x 4096 x 4096 7.34 / 8.36) and a program
+// that launches call by call saves the launch (16 x 768 x 768 7.07 -> 5.96 us). Without the promise of stable weights their
+// fetch starts only behind the kernel ahead, which a quantize kernel of the call would have hidden: then small weights only
+// (16 x 768 x 768 5.46 / 5.55, 3 x 928 x 2048 4.86 / 4.95; but 4 x 2048 x 5504 6.40 / 6.83, 2 x 5120 x 5120 7.85 / 8.19).
+bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool weights_stable, const DeviceInfo& dev) {
+    if (M > kFewRows || (group && dump)) return false;
     const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
-    const int split = decode_split(tiles, KB, sm_count);
-    return (KB + split - 1) / split + 1 <= kFuseMaxBlocks;
+    int split = decode_split(tiles, KB, dev.sm_count);
+    if (M == 1) return (KB + split - 1) / split + 1 <= kFuseMaxBlocks;
+    static_assert(kFuseElems <= 8L * kFuseVecs * StreamCfg<kFewRows>::kThreads, "all of X in a CTA's registers");
+    if ((long)M * K > kFuseElems || (!weights_stable && (long)tiles * KB * kBlockBytes > kFuseWeightBytes)) return false;
+    if (const int ws = group ? wide_split_for<kFewRows, true>(K, N, dev) : wide_split_for<kFewRows, false>(K, N, dev)) split = ws;
+    return (KB + split - 1) / split * round_up(M, 8) * kTileK <= kFuseTileBytes;
 }
 
 namespace {
 template <int MB, bool GROUPED>
 cudaError_t launch_stream_mma(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    if (const int ws = wide_split_for<MB, GROUPED>(a, dev)) return launch_stream<MB, false, true, GROUPED>(a, dev, stream, ws);
-    return launch_stream<MB, false, false, GROUPED>(a, dev, stream);
+    if (const int ws = wide_split_for<MB, GROUPED>(a.K, a.N, dev))
+        return a.fuse_x ? launch_stream<MB, true, true, GROUPED>(a, dev, stream, ws) : launch_stream<MB, false, true, GROUPED>(a, dev, stream, ws);
+    return a.fuse_x ? launch_stream<MB, true, false, GROUPED>(a, dev, stream) : launch_stream<MB, false, false, GROUPED>(a, dev, stream);
 }
 template <bool GROUPED>
 cudaError_t launch_stream_rows(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
