@@ -177,6 +177,8 @@ cudaError_t launch_token_select(const float* scores, int M, int n_keep, int32_t*
 cudaError_t launch_token_compact(const __half* x, int K, const int32_t* idx, int n_keep, __half* out,
                                  const DeviceInfo& dev, cudaStream_t stream);
 
+constexpr unsigned long long kWaitCycles = 4000000000ull;   // limit of a wait on an mbarrier: about 2 s
+
 // Integer product + floating-point output on quantized codes.
 struct GemmArgs {
     const int8_t* q;        // [M][K]
@@ -212,6 +214,8 @@ struct GemmArgs {
     // fp32 partial outputs of tiles whose k range two CTAs share (tensor kernel, per-group scales)
     float* split_scratch = nullptr;
     size_t split_bytes = 0;
+    // Limit of the waits of gemm_tensor_kernel.
+    unsigned long long wait_cycles = kWaitCycles;
     // One row, or a few short ones: the few-row streaming kernel quantizes the activations itself (no quantize kernel runs
     // ahead); q then receives the codes, the control block the exponent.
     const __half* fuse_x = nullptr;

@@ -22,8 +22,9 @@
 // it, a producer's turn about 300. Behind `lane == 0` they took 500 each, and that, not memory or the tensor
 // cores, was the pace of every shape with few tokens. Two (one scale per channel)
 // or three (per-group scales) accumulator stages in TMEM let the epilogue of one
-// accumulation overlap the MMAs of the next ones. Every wait is bounded; on expiry the CTA records a status
-// word, stops issuing work and leaves through the common exit that frees TMEM.
+// accumulation overlap the MMAs of the next ones. Every wait on an mbarrier is bounded; on expiry the CTA records a status
+// word, stops issuing work and leaves through the common exit that frees TMEM. The named barriers have no limit; the watcher
+// arrives at them whatever has given up, and says which tile is the last (see there).
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -91,6 +92,7 @@ struct SharedStorage {
     uint64_t acc_empty[3];                           // epilogue -> MMA
     uint32_t tmem_base;
     volatile uint32_t abort_flag;
+    volatile int given_up;                           // per-group mode: the tile the watcher gave up in, the CTA's last
 };
 
 struct TensorParams {
@@ -111,6 +113,7 @@ struct TensorParams {
     int next_packed;               // chaining: 4-bit codes leave two per byte (even channel in the low nibble)
     int y_tma;                     // outputs leave through y_map (needs N % 8 == 0 and a 16-byte aligned y)
     int clear_status;              // no quantize kernel of the call has set the control block up
+    unsigned long long wait_cycles;   // limit of a wait
 };
 
 __device__ __forceinline__ __half ld_shared_half(uint32_t addr) {
@@ -118,12 +121,12 @@ __device__ __forceinline__ __half ld_shared_half(uint32_t addr) {
     asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
     return __ushort_as_half(v);
 }
-// Waits for a phase that is sure to come, whatever has given up elsewhere (all lanes of a warp; limited all the same).
-__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
-    const long long t0 = clock64();
-    bool late = false;
-    while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)) && !late)
-        late = __any_sync(0xFFFFFFFFu, (unsigned long long)(clock64() - t0) > kWaitCycles);
+// Waits for a phase that only needs the epilogue warps to go on, and so is sure to come, whatever has given up elsewhere (all
+// lanes of a warp). Limited all the same: in tries, since on a GPU that is taken away from all warps for a while only the clock
+// goes on, and over all such waits together (a tile takes some 10^3 of them).
+constexpr uint32_t kDrainTries = 1u << 22;
+__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, uint32_t& tries_left) {
+    while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)) && tries_left > 0) --tries_left;
 }
 // One column of this thread's row, waited for.
 __device__ __forceinline__ int tc_ld1(uint32_t taddr) {
@@ -272,6 +275,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
             mbar_init(&sm.acc_empty[a], kEpiWarps);
         }
         sm.abort_flag = 0;
+        sm.given_up = -1;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -307,7 +311,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                     const int tile = tile_at(tl);
                     const int m0 = tile % p.n_tiles_m * BM;
                     for (int k = kb_first * kTileK; k < kb_last * kTileK; k += kTileK) {
-                        if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u)) goto role_done;
+                        if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u, p.wait_cycles)) goto role_done;
                         mbar_arrive_expect_tx_a(full0 + 8u * st, BM * 128);
                         tma_load_2d_a(x0 + st * (uint32_t)(BM * 128), &x_map, k, m0, full0 + 8u * st);
                         if (++st == (uint32_t)kNumStages) { st = 0; ph ^= 1u; }
@@ -322,7 +326,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                     const uint8_t* wsrc = p.w_packed + ((size_t)nt * KB + kb_first) * kBlockBytes;
                     const __half* ssrc = p.w_scales + (size_t)kb_first * p.Npad + nt * kTileN;
                     for (int kb = kb_first; kb < kb_last; ++kb) {
-                        if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u)) goto role_done;
+                        if (!mbar_wait_a(empty0 + 8u * st, ph, abort_flag, 1u, p.wait_cycles)) goto role_done;
                         mbar_arrive_expect_tx_a(full0 + 8u * st, kBlockBytes + (GROUPED ? kTileN * 2 : 0));
                         tma_load_1d_a(w0 + st * (uint32_t)kBlockBytes, wsrc, kBlockBytes, full0 + 8u * st);
                         wsrc += kBlockBytes;
@@ -343,15 +347,30 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
             // the phase is long over, a named barrier some 30, and the epilogue's chain per block sets the pace (K, N = 4096,
             // 11008 at M = 2048: 124 -> 120 us).
             // A stage's barrier is not arrived at again before its warps have come by: the next accumulation in it needs
-            // their release. When a wait has given up, no accumulation follows; the remaining arrivals are then paced by
-            // those releases themselves, so that the epilogue warps, which wait without a limit, all come through.
+            // their release.
+            // Who can give up here, and raise the flag: the two producers (1), the MMA issuer (2, 3), the unpack warps (6, 7)
+            // and this warp (9). The first three only stop: what they would have made never comes, and this warp sees the
+            // flag, or its own limit, in its wait for it. So it alone decides. The epilogue warps, which wait without a
+            // limit, never look at the flag; once a wait here has ended without its phase they get the rest of the tile's arrivals
+            // all the same, each behind their release of the stage's previous block, and before the tile's last arrival
+            // the word that this tile is given up. It is written once and names the tile, so a warp that is still at
+            // an earlier tile's end does not take it for its own. Behind that tile all of them leave, and so does this warp:
+            // no barrier is left with a part of its warps, and the CTA is through a tile's worth of arrivals after the limit.
+            // That the releases come rests on the epilogue warps waiting for no one but this warp, once the kernel ahead has
+            // completed; so this warp waits for that kernel too before it watches.
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             uint32_t ph = 0;                                           // a bit per accumulator stage
             bool live = true;
-            for (int tl = 0; tl < my_tiles; ++tl) {
+            uint32_t tries_left = kDrainTries;
+            for (int tl = 0; tl < my_tiles && live; ++tl) {
                 uint32_t a = 0;
                 for (int kb = kb_first; kb < kb_last; ++kb) {
-                    if (live) live = mbar_wait_warp(&sm.acc_full[a], (ph >> a) & 1u, abort_flag, 9u);
-                    if (!live) drain_wait(&sm.acc_empty[a], ((ph >> a) & 1u) ^ 1u);
+                    if (live) live = mbar_wait_warp(&sm.acc_full[a], (ph >> a) & 1u, abort_flag, 9u, p.wait_cycles);
+                    if (!live) {
+                        drain_wait(&sm.acc_empty[a], ((ph >> a) & 1u) ^ 1u, tries_left);
+                        if (kb == kb_last - 1 && lane == 0) sm.given_up = tl;
+                        __syncwarp();
+                    }
                     tc_fence_after();
                     tc_fence_before();
 #pragma unroll
@@ -378,8 +397,8 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                         const uint32_t a_bit = (acc_ph >> a) & 1u;
                         const bool got_a = mbar_try_wait(&sm.a_full[ai], a_ph);       // both asked before either answer is used
                         const bool got_acc = mbar_try_wait(&sm.acc_empty[a], a_bit);
-                        if (!got_acc && !mbar_wait(&sm.acc_empty[a], a_bit, abort_flag, 2u)) goto role_done;
-                        if (!got_a && !mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 3u)) goto role_done;
+                        if (!got_acc && !mbar_wait(&sm.acc_empty[a], a_bit, abort_flag, 2u, p.wait_cycles)) goto role_done;
+                        if (!got_a && !mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 3u, p.wait_cycles)) goto role_done;
                         tc_fence_after();
                         const uint32_t d_addr = tmem_acc + a * (uint32_t)kAccStride;
                         const uint32_t a_addr = tmem_a + ai * (uint32_t)kAColsPerStage;
@@ -402,13 +421,13 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 for (int tl = 0; tl < my_tiles; ++tl) {
                     const int a = (int)((uint32_t)tl % kNumAcc);
                     const uint32_t aph = ((uint32_t)tl / kNumAcc) & 1u;
-                    if (!mbar_wait(&sm.acc_empty[a], aph ^ 1u, abort_flag, 4u)) goto role_done;
+                    if (!mbar_wait(&sm.acc_empty[a], aph ^ 1u, abort_flag, 4u, p.wait_cycles)) goto role_done;
                     const uint32_t d_addr = tmem_acc + (uint32_t)(a * kAccStride);
                     uint32_t accumulate = 0u;
                     for (int kb = kb_first; kb < kb_last; ++kb) {
                         // the unpack warps publish a slice only after the stage's TMA bytes (activation
                         // tile included) have landed, so this one wait covers both operands
-                        if (!mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 5u)) goto role_done;
+                        if (!mbar_wait(&sm.a_full[ai], a_ph, abort_flag, 5u, p.wait_cycles)) goto role_done;
                         tc_fence_after();
                         const uint32_t a_addr = tmem_a + ai * (uint32_t)kAColsPerStage;
                         const uint64_t bdesc = bdesc0 + (uint64_t)(st * (uint32_t)(BM * 128 / 16));
@@ -444,7 +463,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         if (group >= kActiveGroups) goto role_done;
         uint32_t s = (uint32_t)group, s_ph = 0u, ai = (uint32_t)group, a_ph = 1u;
         for (uint32_t it = group; it < total_iters; it += kActiveGroups) {
-            if (!mbar_wait_warp(&sm.tma_full[s], s_ph, abort_flag, 6u)) goto role_done;
+            if (!mbar_wait_warp(&sm.tma_full[s], s_ph, abort_flag, 6u, p.wait_cycles)) goto role_done;
             const uint4* src = reinterpret_cast<const uint4*>(sm.w[s]) + r;
             uint4 d[4];
 #pragma unroll
@@ -455,7 +474,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm.a_full[pending]);
             }
-            if (!mbar_wait_warp(&sm.a_empty[ai], a_ph, abort_flag, 7u)) goto role_done;
+            if (!mbar_wait_warp(&sm.a_empty[ai], a_ph, abort_flag, 7u, p.wait_cycles)) goto role_done;
             tc_fence_after();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -558,7 +577,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 const float sc = __half2float(p.w_scales[n]) * 0.0625f * pe;   // sums carry a factor 16
                 [[maybe_unused]] float off_pe = 0.0f;
                 if constexpr (OFFSET) off_pe = (n_ok ? __fmul_rn(off_factor, p.chan_offset[n]) : 0.0f) * pe;
-                if (!mbar_wait_warp(&sm.acc_full[a], aph, abort_flag, 8u)) goto role_done;
+                if (!mbar_wait_warp(&sm.acc_full[a], aph, abort_flag, 8u, p.wait_cycles)) goto role_done;
                 tc_fence_after();
                 // all of this warp's sums go to registers and the accumulator returns to the MMA at once,
                 // so that the conversion and the stores below overlap the next tile's MMAs
@@ -693,7 +712,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                     for (int a = 0; a < kNumAcc; ++a)
                         if (kb + a < kb_last) block((uint32_t)a, kb + a);
                 }
-                if (__any_sync(0xFFFFFFFFu, *abort_flag != 0)) goto role_done;   // some wait gave up: these are not the tile's sums
+                if (__any_sync(0xFFFFFFFFu, sm.given_up == tl)) goto role_done;   // the watcher's word: these are not the tile's sums
                 [[maybe_unused]] bool emit = true;
                 if constexpr (SPLIT) {
                     const int ew = warp - kFirstEpiWarp, slot = (int)blockIdx.x >> 1, hf = (int)blockIdx.x & 1;
@@ -1083,6 +1102,7 @@ cudaError_t launch_off(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t st
     p.split_base = split_base;
     p.split_scratch = a.split_scratch;
     p.clear_status = !a.after_quantize && split_base == 0 ? 1 : 0;
+    p.wait_cycles = a.wait_cycles;
     const int grid = SPLIT ? 2 * split_tiles : (p.n_tiles < dev.sm_count ? p.n_tiles : dev.sm_count);
     if constexpr (SPLIT) {
         // This launch depends on nothing the preceding whole-round launch writes (other tiles of y; the

@@ -11,7 +11,6 @@ namespace aq {
 namespace {
 
 constexpr int kAColsPerStage = 32;            // 128 k of int8 = 32 TMEM columns per lane
-constexpr unsigned long long kWaitCycles = 4000000000ull;   // ~2 s
 
 // ------------------------------------------------------------------------- PTX wrappers
 // One thread of a converged warp. Copies, MMAs and commits take uniform operands: behind elect.sync the compiler knows that
@@ -49,14 +48,15 @@ __device__ __forceinline__ bool mbar_try_wait_a(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) { return mbar_try_wait_a(smem_u32(bar), parity); }
 // Bounded wait. Returns false when the limit ran out or another role already gave up.
 // `code` (non-zero) names the wait; the first wait that gives up leaves its code in the flag.
-__device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t code) {
+__device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t code,
+                                            unsigned long long limit = kWaitCycles) {
     if (mbar_try_wait_a(bar, parity)) return true;
     const long long t0 = clock64();
     uint32_t spins = 0;
     while (!mbar_try_wait_a(bar, parity)) {
         if ((++spins & 0x3FFu) == 0) {
             if (*abort_flag) return false;
-            if ((unsigned long long)(clock64() - t0) > kWaitCycles) {
+            if ((unsigned long long)(clock64() - t0) > limit) {
                 if (*abort_flag == 0) *abort_flag = code;
                 return false;
             }
@@ -64,13 +64,14 @@ __device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, volat
     }
     return true;
 }
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t code) {
-    return mbar_wait_a(smem_u32(bar), parity, abort_flag, code);
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t code,
+                                          unsigned long long limit = kWaitCycles) {
+    return mbar_wait_a(smem_u32(bar), parity, abort_flag, code, limit);
 }
 // The same for a whole warp: all lanes agree on the outcome before any warp-wide instruction.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
-                                               uint32_t code) {
-    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, code) ? 1 : 0) != 0;
+                                               uint32_t code, unsigned long long limit = kWaitCycles) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, code, limit) ? 1 : 0) != 0;
 }
 __device__ __forceinline__ void tma_load_2d_a(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
     asm volatile(
