@@ -128,7 +128,9 @@ int aq_quantize_act(aq_handle_t h, const void* x_fp16, int M, int K, int bits, i
 /* ---- the layer (paper Sec. 4.4): quantize, integer product, floating-point output
  * y_fp16 [M,N] row-major. acc_dump: NULL, or int32 [M][N][G] (G as in aq_scales_bytes)
  * receiving the integer sums (test aid; slows the call; with per-group scales and M <= 16 it takes another
- * kernel, whose fp32 sums may round differently). row_idx as above. */
+ * kernel, whose fp32 sums may round differently). row_idx as above.
+ * The outputs (of the chained calls too) may lie over x: all of it is read before any of them is written. The one exception is a
+ * single row that row_idx names (M = 1): there they must not. */
 int aq_linear_w4a8(aq_handle_t h, const void* x_fp16, int M, int K, const void* w_packed,
                    const void* w_scales, int N, int group_size, int scale_mode,
                    int clip_shift_or_exp, const int32_t* row_idx, void* y_fp16,

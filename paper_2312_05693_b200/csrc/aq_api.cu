@@ -103,6 +103,11 @@ cudaError_t quantize_dispatch(aq_handle_t h, const __half* xh, int M, int K, con
     return launch_quantize(xh, M, K, row_idx, bits, scale_mode, clip_shift_or_exp, ctl, q, scale_exp_out, stream, alpha, k_max);
 }
 
+inline bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+    const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+    return a && b && pa < pb + b_bytes && pb < pa + a_bytes;
+}
+
 bool trip_args_ok(const uint8_t* alpha, int k_max) { return alpha && k_max >= 0 && k_max <= 4; }
 
 int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void* w_packed,
@@ -130,8 +135,15 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     const __half* xh = static_cast<const __half*>(x);
     if (alpha && !aligned(alpha, 16)) return AQ_ERR_ALIGNMENT;
     cudaError_t e = cudaSuccess;
-    // a single row, or a few short ones, on the few-row kernel: that kernel finds the scale and makes the codes itself
-    const bool fuse = !w_offsets && !alpha && kernel_for(h, M) == AQ_KERNEL_DECODE &&
+    // A single row, or a few short ones, on the few-row kernel: that kernel finds the scale and makes the codes itself. Every CTA
+    // then reads all of X, and writes its outputs when others may not have read yet, so nothing that the call writes may
+    // lie over what it reads: those calls quantize in a launch ahead, as calls with more rows do. Which rows an index names
+    // is not known here: several indexed rows are quantized ahead too (a single one is not: see the header).
+    const size_t x_bytes = (size_t)M * K * sizeof(__half), outs = (size_t)M * N;
+    const bool apart = row_idx ? M == 1
+                               : !overlap(x, x_bytes, y, outs * sizeof(__half)) && !overlap(x, x_bytes, q_next, next_packed ? outs / 2 : outs) &&
+                                     !overlap(x, x_bytes, acc_dump, outs * sizeof(int32_t)) && !overlap(x, x_bytes, workspace, workspace_bytes_);
+    const bool fuse = apart && !w_offsets && !alpha && kernel_for(h, M) == AQ_KERNEL_DECODE &&
                       decode_can_fuse_quantize(M, K, N, group, acc_dump != nullptr, h->weights_stable != 0, h->dev) &&
                       (!group || aligned(w_scales, 16));
     if (fuse) {

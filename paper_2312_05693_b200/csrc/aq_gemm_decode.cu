@@ -296,7 +296,7 @@ struct StreamParams {
     // FUSEQ: the activations themselves; the kernel finds the layer scale, writes the codes of
     // its k range to shared memory (and, from the first channel tile, to q_out) and fills the control block
     const __half* x_row;           // the rows, K halves each
-    const int32_t* row_idx;        // NULL or M indices: row m is x_row + row_idx[m] * K
+    const int32_t* row_idx;        // one row: NULL or its index, the row is x_row + row_idx[0] * K
     int8_t* q_out;                 // [M][K] codes
     int bits, scale_mode, clip_shift_or_exp;
 };
@@ -424,17 +424,11 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
         const int step_m = kStrThreads / per_row, step_c = kStrThreads - step_m * per_row;
         const int m_start = (int)threadIdx.x / per_row, c_start = (int)threadIdx.x - m_start * per_row;
         uint4 keep[kFuseVecs];
-        {
-            int m = m_start, c = c_start;
 #pragma unroll
-            for (int i = 0; i < kFuseVecs; ++i) {
-                keep[i] = make_uint4(0, 0, 0, 0);
-                if ((int)threadIdx.x + i * kStrThreads < total)
-                    keep[i] = __ldg(reinterpret_cast<const uint4*>(p.x_row) + (size_t)(p.row_idx ? p.row_idx[m] : m) * per_row + c);
-                m += step_m;
-                c += step_c;
-                if (c >= per_row) { c -= per_row; ++m; }
-            }
+        for (int i = 0; i < kFuseVecs; ++i) {
+            keep[i] = make_uint4(0, 0, 0, 0);
+            if ((int)threadIdx.x + i * kStrThreads < total)
+                keep[i] = __ldg(reinterpret_cast<const uint4*>(p.x_row) + (int)threadIdx.x + i * kStrThreads);
         }
         int e = p.clip_shift_or_exp;
         if (p.scale_mode == AQ_SCALE_DYNAMIC) {
