@@ -184,10 +184,10 @@ gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
 // ---------------------------------------------------------------------------------------
 constexpr unsigned long long kStrWaitCycles = 4000000000ull;
 constexpr int kFuseMaxBlocks = 64;        // k blocks per CTA up to which a single row is quantized inside the product kernel
-// Several rows: what the product kernel can quantize itself, kFuseVecs vectors of eight elements per thread (M * K <= 27648) and
-// kFuseTileBytes of codes of a CTA's k range (8 or 16 rows), and what is left to it: see decode_can_fuse_quantize.
-constexpr int kFuseVecs = 12, kFuseTileBytes = 20 * 1024;
+// Several rows: what is left to the product kernel to quantize (see decode_can_fuse_quantize) and the codes of a CTA's k range
+// that it has room for (8 or 16 rows).
 constexpr long kFuseElems = 12288, kFuseWeightBytes = 4l << 20;
+constexpr int kFuseTileBytes = 20 * 1024;
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ bool str_try_wait(uint64_t* bar, uint32_t parity) {
@@ -241,6 +241,10 @@ template <int MB> struct StreamCfg {
     static constexpr int kConsumerWarps = 4 * kPhases;
     static constexpr int kThreads = (1 + kConsumerWarps) * 32;
 };
+
+// Vectors of eight elements that a thread holds of the rows quantized here: all of kFuseElems, and no more, since the unrolled loops
+// over them are fetched and run whatever X holds (with 12 of them 16 x 768 x 768 took 5.0 us in graph replay, with 6 4.5).
+constexpr int kFuseVecs = (int)((kFuseElems / 8 + StreamCfg<kFewRows>::kThreads - 1) / StreamCfg<kFewRows>::kThreads);
 
 // this CTA's sums over its k range (per-group scales: the bits of fp32 sums; rows padded by 8 words so that the MMA
 // route's fragment owners, eight rows at the same columns, spread over the banks), and the other CTAs' sums for this
@@ -971,18 +975,21 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
 }  // namespace
 
 // Whether the product kernel quantizes the rows itself (one launch for the layer). Dumps of per-group sums are left to the general
-// kernel. A single row: where a CTA's k range fits its code buffer. Several rows: up to kFuseElems elements of X, where that
-// takes the GPU as long as a quantize kernel ahead (in graph replay, two launches / one: 16 x 768 x 768 5.80 / 5.72 us, 2 x 5120 x 5120
-// 7.76 / 7.51; beyond, every CTA reading all of X costs more: 16 x 1664 x 1664 6.23 / 7.08, 6 x 4096 x 4096 7.34 / 8.36) and a program
-// that launches call by call saves the launch (16 x 768 x 768 7.07 -> 5.96 us). Without the promise of stable weights their
-// fetch starts only behind the kernel ahead, which a quantize kernel of the call would have hidden: then small weights only
-// (16 x 768 x 768 5.46 / 5.55, 3 x 928 x 2048 4.86 / 4.95; but 4 x 2048 x 5504 6.40 / 6.83, 2 x 5120 x 5120 7.85 / 8.19).
+// kernel. A single row: where a CTA's k range fits its code buffer. Several rows: up to kFuseElems elements of X. us with two
+// launches / one, graph replay and call by call, without the promise of stable weights and with it:
+//   16 x 768 x 768     5.26 / 4.55   6.20 / 5.01     5.63 / 4.49   6.37 / 4.93
+//   3 x 928 x 2048     4.93 / 3.72   5.78 / 4.20     5.15 / 3.95   5.80 / 4.39
+//   2 x 4096 x 2048 *  5.58 / 5.05   6.47 / 5.40     6.62 / 5.20   7.60 / 5.56      (* groups of 128)
+//   2 x 5120 x 5120         -             -          8.08 / 6.72   9.12 / 7.16
+// Beyond the line it would pay too, up to what more vectors a thread cost the calls below it (eight vectors, 18432 elements: 16 x 1024 x 1024
+// 5.14 / 4.04   5.90 / 4.58     5.56 / 4.14   6.14 / 4.48; 16 x 768 x 768 0.1 more); it lies where it was drawn before the kernel was that short.
+// Without the promise the weights' fetch starts only behind the kernel ahead, which a quantize kernel of the call would have
+// hidden: then small weights only (before the kernel was that short 4 x 2048 x 5504 took 6.40 / 6.83, 2 x 5120 x 5120 7.85 / 8.19).
 bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool weights_stable, const DeviceInfo& dev) {
     if (M > kFewRows || (group && dump)) return false;
     const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
     int split = decode_split(tiles, KB, dev.sm_count);
     if (M == 1) return (KB + split - 1) / split + 1 <= kFuseMaxBlocks;
-    static_assert(kFuseElems <= 8L * kFuseVecs * StreamCfg<kFewRows>::kThreads, "all of X in a CTA's registers");
     if ((long)M * K > kFuseElems || (!weights_stable && (long)tiles * KB * kBlockBytes > kFuseWeightBytes)) return false;
     if (const int ws = group ? wide_split_for<kFewRows, true>(K, N, dev) : wide_split_for<kFewRows, false>(K, N, dev)) split = ws;
     return (KB + split - 1) / split * round_up(M, 8) * kTileK <= kFuseTileBytes;
