@@ -2,6 +2,7 @@
 // product on its codes, where every product is a shift of the int8 value code.
 #include <cuda.h>
 
+#include "aq_attn_parts.cuh"
 #include "aq_common.cuh"
 #include "aq_quant_math.cuh"
 
@@ -721,20 +722,6 @@ attn_v_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constan
 typedef CUresult (*AttnEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// Into how many runs an item's tiles of B rows are cut: as few as give the busiest CTA the fewest tiles. (Whole, the 512 items
-// of 16 tiles that 32 heads of 2048 x 2048 scores have are four rounds, 64 tiles, on 148 SMs whose share is 55.4; in halves 56.)
-inline int attn_parts(long row_items, int tiles, int sms) {
-    int best = 1;
-    long best_tiles = (row_items + sms - 1) / sms * tiles;
-    for (int p = 2; p <= tiles && row_items * p <= 0x7FFFFFFFl; ++p) {
-        const int per = (tiles + p - 1) / p;
-        if ((p - 1) * per >= tiles) continue;                            // the last run would be empty
-        const long most = (row_items * p + sms - 1) / sms * per;
-        if (most < best_tiles) { best_tiles = most; best = p; }
-    }
-    return best;
-}
 
 template <int DN, bool A_SIGNED, int RT = 1, int EW = 4, bool CONVERT = false>
 cudaError_t launch_attn_tc(const void* w, const int8_t* vt, const uint32_t* max_bits, const int32_t* e1, const int32_t* e2,
