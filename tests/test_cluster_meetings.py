@@ -11,21 +11,37 @@ CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_231
 WAIT = re.compile(r"barrier\.cluster\.wait|cluster_started_wait\(\)|cluster_meet\(\)|cluster\.sync\(\)")
 
 
+REMOTE = re.compile(r"map_shared_rank|leave_range\b")           # leave_range stores through a pointer that its caller has mapped
+
+
 def kernels():
     for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
         for part in open(path).read().split("__global__")[1:]:
             part = re.sub(r"//[^\n]*", "", part)
-            if "map_shared_rank" in part:
+            if REMOTE.search(part):
                 yield pytest.param(part, id=re.search(r"(\w+_kernel)\(", part).group(1))
 
 
 @pytest.mark.parametrize("body", list(kernels()))
 def test_remote_stores_come_behind_a_wait_for_the_cluster(body):
-    first = body.index("map_shared_rank")
+    first = REMOTE.search(body).start()
     helper = re.search(r"auto (\w+) = \[&\]\([^)]*\) \{[^{}]*map_shared_rank", body)     # a store inside a lambda counts where it is called
     if helper:
         first = body.index(helper.group(1) + "(", helper.end())
     assert WAIT.search(body, 0, first), "stores into a peer's shared memory before the cluster is known to have started"
+
+
+def test_the_headers_map_no_peer_themselves():
+    """What the headers hold is not read as part of a kernel above: the only store into a peer there goes through a pointer that
+    the kernel hands in."""
+    stores = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cuh"))):
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        assert "map_shared_rank" not in code and "mapa" not in code, path
+        stores += re.findall(r"\*\s*(peer_\w+)\s*=", code)
+    assert stores == ["peer_slot"]
+    users = [k.id for k in kernels() if "leave_range" in k.values[0]]
+    assert sorted(users) == ["log2_absmax_kernel", "range_kernel"]
 
 
 @pytest.mark.gpu
