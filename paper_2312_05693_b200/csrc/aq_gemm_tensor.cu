@@ -357,27 +357,36 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
             // an earlier tile's end does not take it for its own. Behind that tile all of them leave, and so does this warp:
             // no barrier is left with a part of its warps, and the CTA is through a tile's worth of arrivals after the limit.
             // That the releases come rests on the epilogue warps waiting for no one but this warp, once the kernel ahead has
-            // completed; so this warp waits for that kernel too before it watches.
-            asm volatile("griddepcontrol.wait;" ::: "memory");
+            // completed; so this warp waits for that kernel too before the first such arrival.
             uint32_t ph = 0;                                           // a bit per accumulator stage
             bool live = true;
-            uint32_t tries_left = kDrainTries;
+            auto tell = [&](uint32_t a) {
+                tc_fence_after();
+                tc_fence_before();
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    asm volatile("bar.arrive %0, %1;" ::"r"(1 + q * kNumAcc + (int)a), "n"(32 + kEpiWarps * 8) : "memory");
+                ph ^= 1u << a;
+            };
             for (int tl = 0; tl < my_tiles && live; ++tl) {
                 uint32_t a = 0;
-                for (int kb = kb_first; kb < kb_last; ++kb) {
-                    if (live) live = mbar_wait_warp(&sm.acc_full[a], (ph >> a) & 1u, abort_flag, 9u, p.wait_cycles);
-                    if (!live) {
+                int kb = kb_first;
+                for (; kb < kb_last; ++kb) {
+                    live = mbar_wait_warp(&sm.acc_full[a], (ph >> a) & 1u, abort_flag, 9u, p.wait_cycles);
+                    if (!live) break;
+                    tell(a);
+                    if (++a == (uint32_t)kNumAcc) a = 0;
+                }
+                if (!live) {
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    uint32_t tries_left = kDrainTries;
+                    for (; kb < kb_last; ++kb) {
                         drain_wait(&sm.acc_empty[a], ((ph >> a) & 1u) ^ 1u, tries_left);
                         if (kb == kb_last - 1 && lane == 0) sm.given_up = tl;
                         __syncwarp();
+                        tell(a);
+                        if (++a == (uint32_t)kNumAcc) a = 0;
                     }
-                    tc_fence_after();
-                    tc_fence_before();
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        asm volatile("bar.arrive %0, %1;" ::"r"(1 + q * kNumAcc + (int)a), "n"(32 + kEpiWarps * 8) : "memory");
-                    ph ^= 1u << a;
-                    if (++a == (uint32_t)kNumAcc) a = 0;
                 }
             }
         }

@@ -18,7 +18,7 @@ def outcome(verdict, warps, tiles, blocks, issued, watcher_waits=True):
     ends: a step that no other one can release ("stuck"), a wait for a release that never comes ("late").
     verdict "watcher": the watcher's word names the tile. "flag": every warp looks at the flag for itself.
     The warps start when the kernel ahead has completed; a wait for their releases may run out before that, not after.
-    watcher_waits: the watcher starts then too."""
+    watcher_waits: the watcher, too, arrives for blocks that never came only then (others have not come before)."""
     total = tiles * blocks
     # (block, live, word) of the watcher; per warp (block, state: 0 arrive, 1 blocked, 2 release, 3 tile's end, 4 left); arrivals at
     # a barrier per stage; releases per block; whether the flag is up; whether the kernel ahead has completed
@@ -101,8 +101,9 @@ def test_the_kernel_takes_these_steps():
     src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "aq_gemm_tensor.cu")).read())
     watcher = src[src.index("if (GROUPED && warp == 3)"):src.index("if (warp == 1 && elect_one())")]
     assert re.search(r"for \(int tl = 0; tl < my_tiles && live; \+\+tl\)", watcher)
-    assert watcher.index("griddepcontrol.wait") < watcher.index("for (int tl")
-    assert watcher.index("sm.given_up = tl") < watcher.index("bar.arrive")
+    given_up = watcher[watcher.index("if (!live) {"):]
+    assert given_up.index("griddepcontrol.wait") < given_up.index("drain_wait(") < given_up.index("sm.given_up = tl") < given_up.index("tell(a)")
+    assert watcher.count("bar.arrive") == 1 and watcher.count("tell(a)") == 2
     epilogue = src[src.index("auto block = [&]"):src.index("role_done:")]
     assert "abort_flag" not in epilogue and "sm.given_up == tl" in epilogue
 
