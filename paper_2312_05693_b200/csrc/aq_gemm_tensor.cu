@@ -970,12 +970,13 @@ int tile_clusters(const DeviceInfo& dev, int split) {
 // rounds of tiles over the SMs, a last round whose tiles two CTAs share, or all tiles at once in clusters, where the k blocks
 // saved outweigh the exchange (layers of 48 rows, K x N = 4096 x 4096 14.3 -> 10.8 us, 11008 x 4096 21.9 -> 15.7 us, 5120 x 5120
 // 17.6 -> 13.3 us; of 128 rows, 11008 x 4096 30.9 -> 22.5 us).
-// The times are fitted to layer calls with every schedule forced: 48 to 3000 rows, 768 <= K <= 13824, 768 <= N <= 22016 without
-// clusters (2332 calls, relative error 2.6 %), 24 to 512 rows, 512 <= K <= 11008, 256 <= N <= 4096 with them (4492). Of 936 layers
-// without clusters the schedule taken is within 1 % of the best in all; of 450 with them within 3 % in 95 % and 8 % in all. (In
-// cycles per token column, as measured before the issuing threads were elected, and one figure for every exchange: 17 % and
-// 42 % off at the worst. 500 rows, 8192 x 11008 took 87.6 us on shared 128-token tiles, 75.2 on whole 192-token tiles; 1024 x 1152
-// at 192 rows 13.7 us in a cluster, 10.2 without.)
+// The times were fitted to layer calls with every schedule forced: 48 to 3000 rows, 768 <= K <= 13824, 768 <= N <= 22016 without
+// clusters (2332 calls), 24 to 512 rows, 512 <= K <= 11008, 256 <= N <= 4096 with them (4492), before the epilogue waited at named
+// barriers (a block of a 192-token tile is priced at 0.499 us and takes some 0.45). They still rank: with every schedule forced on the
+// kernel as it is, of 300 layers without clusters, 65 to 3000 rows, the schedule taken is the best but for one (1.6 % off). Of
+// 300 with clusters, 24 to 512 rows, it is within 3 % of the best in 70 %, within 8 % in 89 %, 22 % off at the worst: on short k
+// ranges (K near 1024, up to 350 rows) the exchange is priced too high, 102 rows of 1024 x 297 take 11.4 us on whole tiles and 9.3 in
+// clusters of four.
 struct GroupedPlan {
     int bm, split;
 };
