@@ -3,16 +3,21 @@
 #include "../paper_2312_05693_b200/csrc/aq_common.cuh"
 
 namespace {
-__global__ void busy_kernel(long long cycles) {
+__device__ unsigned long long now_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+__global__ void busy_kernel(unsigned long long ns) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long t0 = clock64();
-    for (int i = 0; i < 100000000 && clock64() - t0 < cycles; ++i) {}
+    const unsigned long long t0 = now_ns();
+    for (int i = 0; i < 100000000 && now_ns() - t0 < ns; ++i) {}
 }
 }  // namespace
 
 // ms: from the start of the kernel ahead to the end of the product. Returns a CUDA error code.
 extern "C" int starved_product(int device, int M, int K, int N, const void* codes, const void* packed, const void* scales, void* y,
-                               void* ctl, void* scratch, size_t scratch_bytes, long long busy_cycles, unsigned long long wait_cycles,
+                               void* ctl, void* scratch, size_t scratch_bytes, unsigned long long busy_ns, unsigned long long wait_cycles,
                                float* ms) {
     aq::DeviceInfo dev = {};
     dev.device = device;
@@ -39,7 +44,7 @@ extern "C" int starved_product(int device, int M, int K, int N, const void* code
     a.after_quantize = true;                       // may start while the kernel ahead runs
     a.wait_cycles = wait_cycles;
     cudaEventRecord(begin, stream);
-    busy_kernel<<<1, 32, 0, stream>>>(busy_cycles);
+    busy_kernel<<<1, 32, 0, stream>>>(busy_ns);
     e = aq::launch_gemm_tensor(a, dev, stream);
     cudaEventRecord(end, stream);
     const cudaError_t done = cudaStreamSynchronize(stream);
