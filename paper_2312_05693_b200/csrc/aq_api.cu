@@ -143,13 +143,17 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     const bool apart = row_idx ? M == 1
                                : !overlap(x, x_bytes, y, outs * sizeof(__half)) && !overlap(x, x_bytes, q_next, next_packed ? outs / 2 : outs) &&
                                      !overlap(x, x_bytes, acc_dump, outs * sizeof(int32_t)) && !overlap(x, x_bytes, workspace, workspace_bytes_);
-    const bool fuse = apart && !w_offsets && !alpha && kernel_for(h, M) == AQ_KERNEL_DECODE &&
-                      decode_can_fuse_quantize(M, K, N, group, acc_dump != nullptr, h->weights_stable != 0, h->dev) &&
+    if (w_offsets && !aligned(w_offsets, 4)) return AQ_ERR_ALIGNMENT;
+    const bool plain = !w_offsets && !alpha;
+    // TRIP factors are read by that kernel as well, and rows named by an index with them or a zero point are left to the kernel ahead
+    const bool factors_apart = !alpha || (!overlap(alpha, K, y, outs * sizeof(__half)) && !overlap(alpha, K, q_next, next_packed ? outs / 2 : outs) &&
+                                          !overlap(alpha, K, acc_dump, outs * sizeof(int32_t)) && !overlap(alpha, K, workspace, workspace_bytes_));
+    const bool fuse = apart && factors_apart && (plain || !row_idx) && kernel_for(h, M) == AQ_KERNEL_DECODE &&
+                      decode_can_fuse_quantize(M, K, N, group, acc_dump != nullptr, plain, h->weights_stable != 0, h->dev) &&
                       (!group || aligned(w_scales, 16));
     if (fuse) {
     } else if (w_offsets) {
         // zero-point variant: min / max, then e, zp and codes; the product adds the term -(zp - 2^(b-1)) * r[n]
-        if (!aligned(w_offsets, 4)) return AQ_ERR_ALIGNMENT;
         e = launch_quantize_asym(xh, M, K, row_idx, bits, w.ctl, w.codes, nullptr, nullptr, stream);
     } else {
         e = quantize_dispatch(h, xh, M, K, row_idx, bits, scale_mode, clip_shift_or_exp, w.ctl, w.codes, nullptr, alpha,
@@ -173,6 +177,7 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     if (fuse) {
         g.fuse_x = xh; g.fuse_row_idx = row_idx; g.fuse_bits = bits; g.fuse_scale_mode = scale_mode;
         g.fuse_clip_shift_or_exp = clip_shift_or_exp;
+        g.fuse_alpha = alpha; g.fuse_k_max = k_max;
     }
     return run_gemm(h, g, stream);
 }

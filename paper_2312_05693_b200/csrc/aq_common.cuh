@@ -221,6 +221,8 @@ struct GemmArgs {
     const __half* fuse_x = nullptr;
     const int32_t* fuse_row_idx = nullptr;
     int fuse_bits = 8, fuse_scale_mode = 0, fuse_clip_shift_or_exp = 0;
+    const uint8_t* fuse_alpha = nullptr;        // NULL or TRIP factors
+    int fuse_k_max = 0;
     void* scratch;          // beyond control block + codes
     size_t scratch_bytes;
 };
@@ -241,6 +243,7 @@ size_t tensor_split_scratch_bytes(int M, int K, int N, int group, int sm_count);
 cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const DeviceInfo& dev, cudaStream_t stream);
 constexpr int kFewRows = 16;         // rows up to which the streaming kernel runs, and AQ_KERNEL_AUTO takes it
 cudaError_t launch_gemm_decode(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream);
-bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool weights_stable, const DeviceInfo& dev);
+// plain: neither a zero point nor TRIP factors
+bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool plain, bool weights_stable, const DeviceInfo& dev);
 
 }  // namespace aq

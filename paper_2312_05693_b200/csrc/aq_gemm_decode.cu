@@ -11,16 +11,13 @@
 //    and their activation codes into a shared-memory ring with TMA, eight consumer warps
 //    multiply (dp4a for one row, the warp-level int8 MMA on a 16-row tile above). Every CTA keeps the sums over
 //    its k range in its own shared memory and writes those of the channels it does not finish into the shared
-//    memory of the CTA that does; the cluster meets once, and every CTA finishes its slice of the tile's channels
+//    memory of the CTA that does, whose barrier counts them, and every CTA finishes its slice of the tile's channels
 //    (integer sums are exact in any order, fp32 ones are added in an order that does not depend on timing). No
 //    workspace, no atomics.
-#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "aq_common.cuh"
 #include "aq_quant_math.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace aq {
 
@@ -183,11 +180,12 @@ gemm_decode_kernel(const int8_t* __restrict__ q, int M, int K, int N, int Npad,
 // Streaming kernel (M <= 16)
 // ---------------------------------------------------------------------------------------
 constexpr unsigned long long kStrWaitCycles = 4000000000ull;
+// For what its cluster's other CTAs send a CTA waits longer: one of them that gave up elsewhere sends all the same.
+constexpr unsigned long long kStrPeerCycles = 4 * kStrWaitCycles;
 constexpr int kFuseMaxBlocks = 64;        // k blocks per CTA up to which a single row is quantized inside the product kernel
-// Several rows: what is left to the product kernel to quantize (see decode_can_fuse_quantize) and the codes of a CTA's k range
-// that it has room for (8 or 16 rows).
-constexpr long kFuseElems = 12288, kFuseWeightBytes = 4l << 20;
-constexpr int kFuseTileBytes = 20 * 1024;
+// Several rows (see decode_can_fuse_quantize): vectors of eight elements that a consumer thread holds at most while it quantizes them.
+constexpr int kSliceVecs = 10;
+constexpr long kFuseElems = 12288, kFuseWeightBytes = 4l << 20, kSliceElemsFrom = 16384;
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ bool str_try_wait(uint64_t* bar, uint32_t parity) {
@@ -219,6 +217,14 @@ __device__ __forceinline__ bool str_wait(uint64_t* bar, uint32_t parity, volatil
     return true;
 }
 
+// Bounded wait for what the cluster's other CTAs send, also after this CTA has given up elsewhere: it must be there when it comes.
+__device__ __forceinline__ void str_wait_peers(uint64_t* bar, volatile uint32_t* abort_flag) {
+    if (str_try_wait(bar, 0u)) return;
+    const long long t0 = clock64();
+    while (!str_try_wait(bar, 0u))
+        if ((unsigned long long)(clock64() - t0) > kStrPeerCycles) { *abort_flag = 1; return; }
+}
+
 // One row uses dp4a with one lane per channel; more rows use the warp-level int8 MMA
 // (m16n8k32) on 16 rows, with the activation tile stored 128-byte swizzled so that fragment
 // loads are free of bank conflicts.
@@ -242,13 +248,9 @@ template <int MB> struct StreamCfg {
     static constexpr int kThreads = (1 + kConsumerWarps) * 32;
 };
 
-// Vectors of eight elements that a thread holds of the rows quantized here: all of kFuseElems, and no more, since the unrolled loops
-// over them are fetched and run whatever X holds (with 12 of them 16 x 768 x 768 took 5.0 us in graph replay, with 6 4.5).
-constexpr int kFuseVecs = (int)((kFuseElems / 8 + StreamCfg<kFewRows>::kThreads - 1) / StreamCfg<kFewRows>::kThreads);
-
 // this CTA's sums over its k range (per-group scales: the bits of fp32 sums; rows padded by 8 words so that the MMA
 // route's fragment owners, eight rows at the same columns, spread over the banks), and the other CTAs' sums for this
-// CTA's channel slice, by sender: `split` slots of 128 / split channels, or (clusters of 5 to 8) eight slots of 32. (Without
+// CTA's channel slice, by sender: `split` slots of 128 / split channels, or (WIDE) slots of 32, of 64 where three CTAs share. (Without
 // the slot of the CTA itself, which stays empty, every address takes a comparison of ranks: layers of 2 to 16 rows of
 // 4096 x 4096 took 6.7-7.5 us instead of 6.5-7.3, 5120 x 5120 8.1-8.7 instead of 7.9-8.6.)
 template <int MB, bool WIDE>
@@ -261,7 +263,8 @@ struct StreamSums {
 template <int MB, bool GROUPED, bool FUSEQ>
 struct StreamRing {
     static constexpr int kStages = StreamCfg<MB>::kStages;
-    alignas(1024) int8_t x[FUSEQ && MB > 1 ? 1 : kStages][FUSEQ && MB > 1 ? kFuseTileBytes : StreamCfg<MB>::kRows * kTileK];   // activation codes of the unit's k block (FUSEQ: of all of the CTA's)
+    // activation codes of the unit's k block; several rows quantized here: those of all of the CTA's k range
+    alignas(1024) int8_t x[FUSEQ && MB > 1 ? 1 : kStages][FUSEQ && MB > 1 ? kSliceVecs * 8 * StreamCfg<MB>::kConsumerWarps * 32 : StreamCfg<MB>::kRows * kTileK];
     alignas(128) uint8_t w[kStages][kBlockBytes];          // packed weight block of the unit
     alignas(16) __half sc[GROUPED ? kStages : 1][kTileN];  // per-group scales: those of the unit's k block (= its group)
 };
@@ -274,11 +277,13 @@ struct StreamSmem {
     // one row quantized by the kernel itself: the codes of this CTA's k range (up to kFuseMaxBlocks blocks)
     alignas(16) int8_t xq[MB == 1 ? kFuseMaxBlocks * kTileK : 16];
     unsigned int warp_max[StreamCfg<MB>::kThreads / 32];
+    unsigned int seen[FUSEQ && MB > 1 ? 8 * StreamCfg<MB>::kConsumerWarps : 1];       // several rows: what the warps of the cluster's CTAs saw of X
     alignas(8) uint64_t full[kStages];
     uint64_t empty[kStages];
+    uint64_t got;                          // the other CTAs' sums are there
+    uint64_t met;                          // all of `seen` is there
     volatile uint32_t abort_flag;
 };
-
 struct StreamParams {
     int M, K, N, Npad;
     const int8_t* q;
@@ -296,19 +301,20 @@ struct StreamParams {
     int early_weights;             // the first ring of weight copies may be issued before the wait for the kernel ahead
     int early_dependents;          // the launch behind this one may be set up from this kernel's start
     int next_packed;
-    int box_rows;                  // rows of the activation tensor map's box: 8 when M <= 8 (MMA route)
-    // FUSEQ: the activations themselves; the kernel finds the layer scale, writes the codes of
+    int box_rows;                  // MMA route: rows of a k block's codes in shared memory
+    // FUSEQ: the activations themselves; the kernel finds the layer scale (several rows: or scale and zero point), writes the codes of
     // its k range to shared memory (and, from the first channel tile, to q_out) and fills the control block
     const __half* x_row;           // the rows, K halves each
     const int32_t* row_idx;        // one row: NULL or its index, the row is x_row + row_idx[0] * K
     int8_t* q_out;                 // [M][K] codes
     int bits, scale_mode, clip_shift_or_exp;
+    const uint8_t* alpha;          // several rows: NULL or the TRIP factors, K bytes, none above k_max
+    int k_max;
 };
 
 // grid = (split, channel tiles), cluster = (split, 1, 1): the CTAs of a cluster share a channel
 // tile and take consecutive k ranges; CTA r adds up and writes its slice of the tile's channels:
-// [r, r+1) * 128 / split for split 1, 2, 4; WIDE (split 5 to 8, 16-row route only) the groups of four
-// channels [32 r / split, 32 (r + 1) / split).
+// [r, r+1) * 128 / split for split 1, 2, 4; WIDE (split 3, 5 to 8) the groups of four channels [32 r / split, 32 (r + 1) / split).
 //
 // GROUPED (one scale per 128 k): a k block is one group, so a block's integer sums are scaled and added in fp32 as
 // soon as the block is done, by the warp that made them; what the warps, and the CTAs of the cluster, then add up
@@ -322,12 +328,144 @@ __device__ __forceinline__ int add_sums(int a, int b) {
     return GROUPED ? __float_as_int(__int_as_float(a) + __int_as_float(b)) : a + b;
 }
 
+// The codes of this CTA's k range, from X itself; the layer's exponent and zero point. The consumer warps call this. A step takes
+// kTileN * 2 vectors of eight elements, one a thread: the rows side by side, each in runs of 16 / (rows rounded up to a power of two)
+// k blocks, so that a step's places, in X and in the codes, lie a fixed distance behind the step's before it. HELD: steps (vectors a
+// thread holds).
+__host__ __device__ inline int slice_row_log(int M) {
+    int log = 0;
+    while ((1 << log) < M) ++log;
+    return log;
+}
+template <int MB, bool WIDE, bool GROUPED, int HELD>
+__device__ __forceinline__ void slice_codes(const StreamParams& p, StreamSmem<MB, WIDE, GROUPED, true>& sm, int8_t* x_tile, int kb0, int per_row,
+                                            int row_log, int rank, int split, int tile, int& e_out, int& zp_out) {
+    constexpr int kThreads = StreamCfg<MB>::kConsumerWarps * 32, kWarps = kThreads / 32;
+    const int tid = (int)threadIdx.x - 32, warp = tid >> 5, lane = tid & 31;
+    const int wide = kThreads >> row_log;                        // vectors of a row in a step
+    const int m = tid >> (8 - row_log), c = tid & (wide - 1);
+    static_assert(kThreads == 256, "the shifts above");
+    const int left = m < p.M ? per_row - c : 0;                  // of this thread's row, from its first vector on
+    const uint4* const x = reinterpret_cast<const uint4*>(p.x_row) + (size_t)m * (p.K / 8) + kb0 * (kTileK / 8) + c;
+    uint4 held[HELD];
+#pragma unroll
+    for (int i = 0; i < HELD; ++i) {
+        held[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (i * wide < left) held[i] = __ldg(x + i * wide);
+    }
+    const bool asym = p.chan_offset != nullptr;
+    __half2 hi2 = __float2half2_rn(0.0f), lo2 = hi2;             // absent vectors are zero; a zero point's range contains it anyway
+    if (asym) {
+#pragma unroll
+        for (int i = 0; i < HELD; ++i) {
+            const __half2* h = reinterpret_cast<const __half2*>(&held[i]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {                        // NaN operands are dropped
+                lo2 = __hmin2(lo2, h[k]);
+                hi2 = __hmax2(hi2, h[k]);
+            }
+        }
+        lo2 = __habs2(lo2);
+    } else {
+#pragma unroll
+        for (int i = 0; i < HELD; ++i) {
+            const __half2* h = reinterpret_cast<const __half2*>(&held[i]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) hi2 = __hmax2(hi2, __habs2(h[k]));
+        }
+    }
+    const unsigned int bmax = max((unsigned int)__half_as_ushort(__low2half(hi2)), (unsigned int)__half_as_ushort(__high2half(hi2)));
+    const unsigned int bmin = max((unsigned int)__half_as_ushort(__low2half(lo2)), (unsigned int)__half_as_ushort(__high2half(lo2)));
+    unsigned int seen = __reduce_max_sync(0xFFFFFFFFu, bmax) | (asym ? __reduce_max_sync(0xFFFFFFFFu, bmin) << 16 : 0u);
+    if (split > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");        // everybody has started
+    if (lane < split) {
+        uint32_t slot, bar;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(slot) : "r"(s_u32(&sm.seen[rank * kWarps + warp])), "r"(lane));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(s_u32(&sm.met)), "r"(lane));
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(slot), "r"(seen), "r"(bar) : "memory");
+    }
+    __syncwarp();
+    str_wait_peers(&sm.met, &sm.abort_flag);
+    __syncwarp();
+    seen = 0;
+    for (int i = lane; i < split * kWarps; i += 32) seen = __vmaxu2(seen, sm.seen[i]);
+    seen = __reduce_max_sync(0xFFFFFFFFu, seen & 0xFFFFu) | (asym ? __reduce_max_sync(0xFFFFFFFFu, seen >> 16) << 16 : 0u);
+    int e = p.clip_shift_or_exp, zp = 0;
+    if (asym) zero_point_scale(seen & 0xFFFFu, seen >> 16, p.bits, e, zp);
+    else if (p.scale_mode == AQ_SCALE_DYNAMIC) e = layer_exponent_from_bits(seen, p.bits) - p.clip_shift_or_exp - p.k_max;
+    if (tile == 0 && rank == 0) {
+        if (tid == 0) {
+            p.ctl->scale_exp = e;
+            p.ctl->zero_point = zp;
+            p.ctl->absmax_bits = asym ? 0u : seen;
+        }
+        if (tid < Control::kSplitWords) p.ctl->split_flags[tid] = 0;
+    }
+    e_out = e;
+    zp_out = zp;
+    // rows of 128 bytes by k block, 16-byte chunks swizzled by row % 8 as a tensor-map copy leaves them
+    int8_t* const at = x_tile + ((c >> 4) * p.box_rows + m) * kTileK + ((((c & 15) >> 1) ^ (m & 7)) << 4) + 8 * (c & 1);
+    const int step = (wide >> 4) * p.box_rows * kTileK;
+    int8_t* const q = p.q_out + (size_t)m * p.K + kb0 * kTileK + 8 * c;
+    const int top = 1 << (p.bits - 1);
+    if (!p.alpha && e >= -14 && e <= 14) {                       // 2^-e is a normal half: codes in half2 arithmetic
+        // without a zero point: the same with a shift of zero
+        const __half2 inv2 = __float2half2_rn(__int_as_float((127 - e) << 23));
+        const __half2 clo2 = __float2half2_rn((float)(asym ? -zp : -top)), chi2 = __float2half2_rn((float)(asym ? 2 * top - 1 - zp : top - 1));
+        const __half2 shift2 = __float2half2_rn((float)(asym ? zp - top : 0));
+#pragma unroll
+        for (int i = 0; i < HELD; ++i) {
+            if (i * wide < left) {
+                uint2 code;
+                quantize8_half2_asym(held[i], inv2, clo2, chi2, shift2, code.x, code.y);
+                *reinterpret_cast<uint2*>(at + i * step) = code;
+                if (tile == 0) *reinterpret_cast<uint2*>(q + i * wide * 8) = code;
+            }
+        }
+        return;
+    }
+    if (p.alpha && p.bits == 4 && e >= -14 && e <= 10) {         // so is 2^-(e + alpha), alpha <= 4
+        const uint2* const al = reinterpret_cast<const uint2*>(p.alpha) + kb0 * (kTileK / 8) + c;
+        uint2 a[HELD];
+#pragma unroll
+        for (int i = 0; i < HELD; ++i)
+            if (i * wide < left) a[i] = __ldg(al + i * wide);
+#pragma unroll
+        for (int i = 0; i < HELD; ++i) {
+            if (i * wide < left) {
+                uint2 code;
+                quantize8_half2_trip(held[i], e, a[i], code.x, code.y);
+                *reinterpret_cast<uint2*>(at + i * step) = code;
+                if (tile == 0) *reinterpret_cast<uint2*>(q + i * wide * 8) = code;
+            }
+        }
+        return;
+    }
+    // The other exponents: X is read again, in a loop that is not unrolled (unrolled with all quantizers in it the code
+    // was longer than the instruction cache holds: 16 x 13824 x 5120 28 us instead of 20)
+#pragma unroll 1
+    for (int i = 0; i * wide < left; ++i) {
+        const uint4 d = __ldg(x + i * wide);
+        uint2 code;
+        if (asym) {
+            code = quantize8_fp32_asym(d, __int_as_float((127 - e) << 23), zp, p.bits);
+        } else if (p.alpha) {
+            const uint2 al = __ldg(reinterpret_cast<const uint2*>(p.alpha) + kb0 * (kTileK / 8) + c + i * wide);
+            code = quantize8_fp32(d, e, -(float)top, (float)(top - 1), &al);
+        } else {
+            code = quantize8_fp32(d, e, -(float)top, (float)(top - 1), nullptr);
+        }
+        *reinterpret_cast<uint2*>(at + i * step) = code;
+        if (tile == 0) *reinterpret_cast<uint2*>(q + i * wide * 8) = code;
+    }
+}
+
 template <int MB, bool FUSEQ = false, bool WIDE = false, bool GROUPED = false>
 __global__ void __launch_bounds__(StreamCfg<MB>::kThreads, 2)
 gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const StreamParams p) {
-    static_assert(!WIDE || MB == 16, "clusters of 5 to 8 are for the MMA route");
     extern __shared__ uint8_t smem_raw[];
     using Smem = StreamSmem<MB, WIDE, GROUPED, FUSEQ>;
+    constexpr bool kSlices = FUSEQ && MB > 1;
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr bool kUseMma = StreamCfg<MB>::kUseMma;
     constexpr int kRows = StreamCfg<MB>::kRows;
@@ -335,16 +473,17 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     constexpr int kPhases = StreamCfg<MB>::kPhases;
     constexpr int kStrConsumerWarps = StreamCfg<MB>::kConsumerWarps;
     constexpr int kStrThreads = StreamCfg<MB>::kThreads;
-    cg::cluster_group cluster = cg::this_cluster();
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int KB = k_blocks(p.K);
     const int rank = blockIdx.x, split = gridDim.x;
     const int tile = blockIdx.y;
     const int kb0 = (int)((long long)KB * rank / split), kb1 = (int)((long long)KB * (rank + 1) / split);
 
-    // First meeting of the cluster, arrival only: by the time a CTA writes into another's shared memory
-    // (after its k range) every CTA of the cluster has started. The wait comes just before those writes.
-    if (split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    int8_t* const x_tile = sm.ring.x[0];                     // FUSEQ: codes of the k range
+
+    // Channel slices: CTA r finishes channels [r, r + 1) * 128 / split for split 1, 2, 4 (divisions are shifts); WIDE: the groups of four
+    // channels [32 r / split, 32 (r + 1) / split), at most 28 channels.
+    const int g_first = (32 * rank) / split, g_count = (32 * (rank + 1)) / split - g_first;
     if (threadIdx.x == 0) {
         if constexpr (kRows > 1 && !FUSEQ)     // start the descriptor's fetch now; the first tile load would wait for it
             asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
@@ -353,7 +492,20 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_u32(&sm.empty[s])), "r"(4) : "memory");   // the four quarter warps of the block's phase
         }
         sm.abort_flag = 0;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(&sm.got)) : "memory");
+        if constexpr (kSlices) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(&sm.met)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (split > 1)            // this CTA's channels of every row from each of the others
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                         ::"r"(s_u32(&sm.got)), "r"((uint32_t)((split - 1) * min(p.M, kRows) * g_count * 16)) : "memory");
+        if constexpr (kSlices)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s_u32(&sm.met)), "r"((uint32_t)(split * kStrConsumerWarps * 4)) : "memory");
+    }
+    if (split > 1) {
+        __syncwarp();
+        // Meeting of the cluster, arrival only: by the time a CTA writes into another's shared memory (after its k range; by slices
+        // before it) every CTA of the cluster has started and its barriers are set up. The wait comes just before those writes.
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     }
     __syncthreads();
     volatile uint32_t* abort_flag = &sm.abort_flag;
@@ -415,72 +567,25 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) p.ctl->status = 0;   // nothing has given up yet
-    [[maybe_unused]] int fused_exp = 0;
-    if constexpr (FUSEQ && MB > 1) {
-        // ---- several rows: every CTA reads all of them, once, into registers, finds the layer's scale, and makes the codes it
-        // multiplies. What it replaces, a quantize kernel ahead of this one, is one launch more, with its drain, this kernel's
-        // wait and the codes' way through L2. (A CTA that reads only its k range and exchanges its largest magnitude with the
-        // others of its cluster pays a meeting instead: 6 x 4096 x 4096 7.3 us behind a quantize kernel, 7.9 with the meeting.)
+    [[maybe_unused]] int fused_exp = 0, fused_zp = 0;
+    if constexpr (kSlices) {
+        // ---- several rows, by slices: a CTA reads its k range of every row, once, into registers; its warps tell every CTA of the
+        // cluster the largest magnitudes they saw (asynchronous remote stores that count on the receiver's barrier), and each warp,
+        // with all of them, derives the scale and quantizes what it holds.
         if (warp == 0 && s_elect_one())
             for (int i = issued; i < ring; ++i) issue_w(kb0 + i, i);   // weights on their way meanwhile
         issued = ring;
-        const int per_row = p.K / 8, total = p.M * per_row;              // vectors of eight elements
-        const int step_m = kStrThreads / per_row, step_c = kStrThreads - step_m * per_row;
-        const int m_start = (int)threadIdx.x / per_row, c_start = (int)threadIdx.x - m_start * per_row;
-        uint4 keep[kFuseVecs];
-#pragma unroll
-        for (int i = 0; i < kFuseVecs; ++i) {
-            keep[i] = make_uint4(0, 0, 0, 0);
-            if ((int)threadIdx.x + i * kStrThreads < total)
-                keep[i] = __ldg(reinterpret_cast<const uint4*>(p.x_row) + (int)threadIdx.x + i * kStrThreads);
+        __syncwarp();
+        if (warp > 0) {
+            const int per_row = min(kb1 * (kTileK / 8), p.K / 8) - kb0 * (kTileK / 8);       // vectors of eight elements of the k range
+            const int row_log = slice_row_log(p.M);
+            constexpr int kFewVecs = 4;                                 // unrolled loops over what is not there cost their instructions all the same
+            if ((per_row << row_log) <= kFewVecs * 256) slice_codes<MB, WIDE, GROUPED, kFewVecs>(p, sm, x_tile, kb0, per_row, row_log, rank, split, tile, fused_exp, fused_zp);
+            else slice_codes<MB, WIDE, GROUPED, kSliceVecs>(p, sm, x_tile, kb0, per_row, row_log, rank, split, tile, fused_exp, fused_zp);
+            asm volatile("bar.sync 1, %0;" ::"n"(kStrConsumerWarps * 32) : "memory");
+        } else if (split > 1) {
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         }
-        int e = p.clip_shift_or_exp;
-        if (p.scale_mode == AQ_SCALE_DYNAMIC) {
-            __half2 m2 = __float2half2_rn(0.0f);
-#pragma unroll
-            for (int i = 0; i < kFuseVecs; ++i) {
-                const __half2* h = reinterpret_cast<const __half2*>(&keep[i]);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) m2 = __hmax2(m2, __habs2(h[k]));   // NaN operands are dropped; absent vectors are zero
-            }
-            unsigned int bmax = max((unsigned int)__half_as_ushort(__low2half(m2)), (unsigned int)__half_as_ushort(__high2half(m2)));
-            if (bmax > 0x7C00u) bmax = 0;
-            bmax = __reduce_max_sync(0xFFFFFFFFu, bmax);
-            if (lane == 0) sm.warp_max[warp] = bmax;
-            __syncthreads();
-            unsigned int all = 0;
-#pragma unroll
-            for (int w = 0; w < kStrThreads / 32; ++w) all = max(all, sm.warp_max[w]);
-            e = layer_exponent_from_bits(all, p.bits) - p.clip_shift_or_exp;
-            if (tile == 0 && rank == 0 && threadIdx.x == 0) p.ctl->absmax_bits = all;
-        }
-        if (tile == 0 && rank == 0) {
-            if (threadIdx.x == 0) p.ctl->scale_exp = e;
-            if (threadIdx.x < Control::kSplitWords) p.ctl->split_flags[threadIdx.x] = 0;
-        }
-        const float lo = -(float)(1 << (p.bits - 1)), hi = (float)((1 << (p.bits - 1)) - 1);
-        const bool fast = e >= -14 && e <= 14;             // 2^-e is a normal half: codes in half2 arithmetic
-        const __half2 inv2 = __float2half2_rn(fast ? __int_as_float((127 - e) << 23) : 1.0f);
-        const __half2 lo2 = __float2half2_rn(lo), hi2 = __float2half2_rn(hi);
-        const int c_first = kb0 * (kTileK / 8), c_last = kb1 * (kTileK / 8);      // this CTA's k range
-        int m = m_start, c = c_start;
-#pragma unroll
-        for (int i = 0; i < kFuseVecs; ++i) {
-            if ((int)threadIdx.x + i * kStrThreads < total && c >= c_first && c < c_last) {
-                uint2 code;
-                if (fast) quantize8_half2(keep[i], inv2, lo2, hi2, code.x, code.y);
-                else code = quantize8_fp32(keep[i], e, lo, hi, nullptr);
-                // rows of 128 bytes by k block, 16-byte chunks swizzled by row % 8 as a tensor-map copy leaves them
-                const int at = c - c_first;
-                *reinterpret_cast<uint2*>(sm.ring.x[0] + ((at >> 4) * p.box_rows + m) * kTileK + ((((at & 15) >> 1) ^ (m & 7)) << 4) + 8 * (at & 1)) = code;
-                if (tile == 0) *reinterpret_cast<uint2*>(p.q_out + (size_t)m * p.K + 8 * c) = code;
-            }
-            m += step_m;
-            c += step_c;
-            if (c >= per_row) { c -= per_row; ++m; }
-        }
-        fused_exp = e;
-        __syncthreads();
     }
     if constexpr (FUSEQ && MB == 1) {
         // ---- the layer scale and this CTA's codes (Eq. 1, Eq. 2 / Eq. 5 with zp = 0; one scale for the layer)
@@ -648,29 +753,30 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 }
             }
         } else {
-            // Warp-level int8 MMA, D[16 rows x 8 channels] += A[16 x 32 k] * B[32 k x 8 channels].
-            // Fragment owner: g = lane / 4 (row g and g+8 of A and D; channel g of B),
-            // t = lane % 4 (k bytes 4t..4t+3 and 16+4t..; D columns 2t, 2t+1).
-            // Rows 8..15 are not read when M <= 8.
-            // (Splitting a block among the four warps of a phase into channel
-            // halves x k halves instead of channel quarters, so that a warp reads half of the activation tile,
-            // measured the same within 0.2 us either way.)
+            // Warp-level int8 MMA, D[16 channels x 8 rows] += A[16 x 32 k] * B[32 k x 8 rows]: the weights are A, so that up to eight
+            // rows cost half the instructions that sixteen do (with the rows as A, rows 8..15 of zeros cost as much as others: this instruction
+            // takes 8.6 cycles of a scheduler's tensor pipe whatever it is fed; 6 x 4096 x 11008 10.55 / 8.79, 3 x 7168 x 28672 21.2 / 19.6 us).
+            // Fragment owner: g = lane / 4 (channels g and g+8 of A and D; row g of B), t = lane % 4 (k bytes 4t..4t+3 and
+            // 16+4t..; D rows 2t, 2t+1).
+            // (Splitting a block among the four warps of a phase into channel halves x k halves instead of channel quarters, so that a
+            // warp reads half of the activation tile, measured the same within 0.2 us either way.)
             const int g = lane >> 2, t = lane & 3;
             const bool upper = p.M > 8;
-            int acc[4][4];
-            [[maybe_unused]] float fsum[4][4];
+            // [u][h][c]: channel 16u + 8(c / 2) + g, row 8h + 2t + c % 2
+            int acc[2][2][4];
+            [[maybe_unused]] float fsum[2][2][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int u = 0; u < 2; ++u)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    acc[i][c] = 0;
-                    if constexpr (GROUPED) fsum[i][c] = 0.0f;
+                for (int c = 0; c < 8; ++c) {
+                    acc[u][c >> 2][c & 3] = 0;
+                    if constexpr (GROUPED) fsum[u][c >> 2][c & 3] = 0.0f;
                 }
             for (int kb = kb0 + phase; kb < kb1; kb += kPhases) {
                 const uint32_t it = (uint32_t)(kb - kb0);
                 const int s = (int)(it % kStrStages);
                 if (!__all_sync(0xFFFFFFFFu, str_wait(&sm.full[s], (it / kStrStages) & 1u, abort_flag) ? 1 : 0)) break;
-                const int8_t* xt = FUSEQ ? sm.ring.x[0] + (kb - kb0) * p.box_rows * kTileK : sm.ring.x[s];
+                const int8_t* xt = FUSEQ ? x_tile + (kb - kb0) * p.box_rows * kTileK : sm.ring.x[s];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     // The sum over k does not depend on which k sits in which slot of the instruction, as long
@@ -688,35 +794,42 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                                  : "=r"(pw[0]), "=r"(pw[1]), "=r"(pw[2]), "=r"(pw[3])
                                  : "r"(s_u32(sm.ring.w[s] + (size_t)(j * kTileN + quarter * 32 + lane) * 16)) : "memory");
                     const uint2 xa = *reinterpret_cast<const uint2*>(xt + g * kTileK + x_off);
-                    uint2 xb = make_uint2(0u, 0u);
+                    uint2 xb;
                     if (upper) xb = *reinterpret_cast<const uint2*>(xt + (g + 8) * kTileK + x_off);
-                    const uint32_t a0 = xa.x, a1 = xb.x, a2 = xa.y, a3 = xb.y;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint32_t b0 = (pw[i] << 4) & 0xF0F0F0F0u;
-                        const uint32_t b1 = pw[i] & 0xF0F0F0F0u;
-                        asm volatile(
-                            "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-                            "{%8, %9}, {%0, %1, %2, %3};"
-                            : "+r"(acc[i][0]), "+r"(acc[i][1]), "+r"(acc[i][2]), "+r"(acc[i][3])
-                            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                    for (int u = 0; u < 2; ++u) {
+                        const uint32_t a0 = (pw[2 * u] << 4) & 0xF0F0F0F0u, a2 = pw[2 * u] & 0xF0F0F0F0u;
+                        const uint32_t a1 = (pw[2 * u + 1] << 4) & 0xF0F0F0F0u, a3 = pw[2 * u + 1] & 0xF0F0F0F0u;
+                        auto mma = [&](int (&d)[4], const uint2& b) {
+                            asm volatile(
+                                "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+                                "{%8, %9}, {%0, %1, %2, %3};"
+                                : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+                                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
+                        };
+                        mma(acc[u][0], xa);
+                        if (upper) mma(acc[u][1], xb);
                     }
                 }
                 if constexpr (GROUPED) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 sg = __half22float2(*reinterpret_cast<const __half2*>(&sm.ring.sc[s][quarter * 32 + 8 * i + 2 * t]));
+                    for (int u = 0; u < 2; ++u) {
+                        const __half* sc = &sm.ring.sc[s][quarter * 32 + 16 * u + g];
+                        const float s0 = __half2float(sc[0]), s1 = __half2float(sc[8]);
+                        auto scale = [&](int (&a)[4], float (&f)[4]) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            fsum[i][c] = fmaf((float)acc[i][c], (c & 1) ? sg.y : sg.x, fsum[i][c]);
-                            acc[i][c] = 0;
-                        }
+                            for (int c = 0; c < 4; ++c) {
+                                f[c] = fmaf((float)a[c], c < 2 ? s0 : s1, f[c]);
+                                a[c] = 0;
+                            }
+                        };
+                        scale(acc[u][0], fsum[u][0]);
+                        if (upper) scale(acc[u][1], fsum[u][1]);
                     }
                 }
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_u32(&sm.empty[s])) : "memory");
             }
-            // D fragment: acc[i][0..1] = row g, channels 8i+2t, +1; acc[i][2..3] = row g+8.
             // The warps of a quarter meet in the sum buffer, one after the other (the same thread position
             // owns an element in each of them: the first stores, the others add).
 #pragma unroll
@@ -724,37 +837,38 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                 if (ph > 0) asm volatile("bar.sync 1, %0;" ::"n"(kStrConsumerWarps * 32) : "memory");
                 if (phase == ph) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                    for (int h = 0; h < 2; ++h) {
+                        if (h == 0 || upper) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            int& dst = sm.sums.sum[g + 8 * (c >> 1)][quarter * 32 + 8 * i + 2 * t + (c & 1)];
-                            const int own = GROUPED ? __float_as_int(fsum[i][c]) : acc[i][c];
-                            if (ph == 0) dst = own;
-                            else dst = add_sums<GROUPED>(dst, own);
+                            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                                for (int c = 0; c < 4; ++c) {
+                                    int& dst = sm.sums.sum[8 * h + 2 * t + (c & 1)][quarter * 32 + 16 * u + 8 * (c >> 1) + g];
+                                    const int own = GROUPED ? __float_as_int(fsum[u][h][c]) : acc[u][h][c];
+                                    if (ph == 0) dst = own;
+                                    else dst = add_sums<GROUPED>(dst, own);
+                                }
                         }
+                    }
                 }
             }
         }
     }
     // Every CTA of the cluster now holds the tile's sums over its own k range, and CTA `rank` finishes the
-    // tile's channel slice `rank`: every CTA writes its sums of the other slices into
-    // their owners' shared memory (slot = sender), the cluster meets once, and every CTA adds what it received
-    // to its own sums (integer addition is exact in any order), scales and writes its outputs. After the
-    // meeting nobody touches another CTA's memory, so a CTA may leave as soon as it is done. (Reading the
-    // other CTAs' sums over distributed shared memory instead, with a second meeting before anybody leaves,
-    // measured 0.1-0.5 us slower at every row count.)
-    // The scale is fetched before the cluster meets so that its latency overlaps the wait.
+    // tile's channel slice `rank`: every CTA writes its sums of the other slices into their owners' shared memory (slot = sender) with
+    // asynchronous stores that count on the owner's barrier, and every CTA, once all of its own are there, adds them
+    // to its sums (integer addition is exact in any order), scales and writes its outputs. Nobody touches another CTA's memory after
+    // that, so a CTA may leave as soon as it is done. (A meeting of the cluster behind plain remote stores, which this replaced, held
+    // every launch 0.2-0.35 us longer: 1 x 5120 x 5120 5.42 / 5.27, 1 x 13824 x 5120 9.07 / 8.81, 6 x 4096 x 4096 6.77 / 6.40; reading the
+    // other CTAs' sums over distributed shared memory, with a second meeting before anybody leaves, 0.1-0.5 us more.)
+    // The scale is fetched before the wait for them so that its latency overlaps it.
     // This CTA's k range is done: a launch behind this one that allows it may be scheduled and set up now
     // (it reads and writes nothing before this grid has completed).
     if (!p.early_dependents) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // Channel slices: 128 / split channels each for split 1, 2, 4 (divisions are shifts). Clusters of 5 to 8
-    // (16-row route on long k ranges) cut the tile's 32 groups of four channels into `split` nearly equal
-    // runs, slice r = groups [32 r / split, 32 (r + 1) / split): at most 28 channels, handled by the first
-    // lanes of 32-thread rows.
-    constexpr bool wide = WIDE;                                // this instantiation is launched with clusters of 5 to 8
-    const int cw = wide ? 32 : kTileN / split;                // slot width in the receive buffer
-    const int cw_log = wide ? 5 : 7 - (31 - __clz(split));
-    const int g_first = (32 * rank) / split, g_count = (32 * (rank + 1)) / split - g_first;   // this CTA's groups (wide)
+    // WIDE: a slice's channels (at most 28, or 44 of three CTAs) are handled by the first lanes of 32 or 64 threads.
+    constexpr bool wide = WIDE;
+    const int cw_log = wide ? (split == 3 ? 6 : 5) : 7 - (31 - __clz(split));
+    const int cw = 1 << cw_log;                               // slot width in the receive buffer
     const int ft = (int)threadIdx.x - 32;                     // the consumer threads finish (a multiple of 128 = 4 cw at most)
     const int rc = ft & (cw - 1);                             // channel inside the slice (only used when ft >= 0)
     const int out_r = wide ? min(4 * g_first + rc, kTileN - 1) : rank * cw + rc;   // wide: lanes behind the slice only keep their warp whole
@@ -764,34 +878,37 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     if (mine) {
         const float pe = __int_as_float((127 + (FUSEQ ? fused_exp : *p.scale_exp)) << 23);
         sc = GROUPED ? 0.0625f * pe : __half2float(p.w_scales[out_n]) * pe;     // the fp32 sums carry a factor 16
-        if (p.chan_offset) off = __fmul_rn(offset_factor(p.ctl, p.zp_mid), p.chan_offset[out_n]) * pe;
+        if (p.chan_offset) off = __fmul_rn(kSlices ? -(float)(fused_zp - p.zp_mid) : offset_factor(p.ctl, p.zp_mid), p.chan_offset[out_n]) * pe;
     }
     const int rows = p.M < kRows ? p.M : kRows;
-    if (split > 1) {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // everybody has started (arrival at the top)
-        __syncthreads();                                      // this CTA's sums are complete
-        if (ft >= 0) {
-            // four consecutive channels at a time (16-byte remote stores) go to the CTA that owns them
+    if (split > 1 && !kSlices) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // everybody has started (arrival at the top)
+    if (ft >= 0) {
+        asm volatile("bar.sync 1, %0;" ::"n"(kStrConsumerWarps * 32) : "memory");     // this CTA's sums are complete
+        if (split > 1) {
+            // four consecutive channels at a time (16-byte remote stores, counted by the receiver's barrier) go to the CTA that owns them
             for (int e = ft; e < rows * (kTileN / 4); e += kStrConsumerWarps * 32) {
                 const int m = e >> 5, g4 = e & 31, ch = 4 * g4;
                 const int owner = wide ? (((g4 + 1) * split + 31) >> 5) - 1 : ch >> cw_log;
                 const int at = wide ? ch - 4 * ((32 * owner) / split) : ch & (cw - 1);   // place inside the owner's slice
-                if (owner != rank)
-                    *reinterpret_cast<int4*>(cluster.map_shared_rank(&sm.sums.recv[0][0], owner) + m * Smem::kRecvStride + rank * cw + at) =
-                        *reinterpret_cast<const int4*>(&sm.sums.sum[m][ch]);
+                if (owner != rank) {
+                    const int4 v = *reinterpret_cast<const int4*>(&sm.sums.sum[m][ch]);
+                    uint32_t slot, bar;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(slot) : "r"(s_u32(&sm.sums.recv[m][rank * cw + at])), "r"(owner));
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(s_u32(&sm.got)), "r"(owner));
+                    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                                 ::"r"(slot), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+                }
             }
+            str_wait_peers(&sm.got, abort_flag);
+            __syncwarp();
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    } else {
-        __syncthreads();
     }
     if (mine || (wide && ft >= 0)) {
         // All shared-memory reads of this thread's outputs are issued before the first is used and without
         // branches around them (rows that do not exist read the last row of the buffer and are dropped):
         // taken one after the other, each behind its own test, they were the longest part of the finish at
         // 16 rows.
-        constexpr int kPass = kStrConsumerWarps * 32 / (WIDE ? 32 : kTileN);     // rows that a pass covers at least
+        constexpr int kPass = kStrConsumerWarps * 32 / (WIDE ? 64 : kTileN);     // rows that a pass covers at least
         constexpr int kIt = (kRows + kPass - 1) / kPass;
         const int stride = (kStrConsumerWarps * 32) >> cw_log, m0 = ft >> cw_log;
         int av[kIt];
@@ -843,26 +960,21 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// k ranges per tile by the usual rule: 1, 2 or 4, as many as keep all CTAs resident at once (two per SM) with at
-// least two k blocks per CTA (wide_split_for may raise a 4 to 5..8 for the 16-row route)
-inline int decode_split(int tiles, int KB, int sm_count) {
-    int split = 1;
-    while (split < 4 && tiles * split * 2 <= 2 * sm_count && KB / (split * 2) >= 2) split *= 2;
-    return split;
-}
-
 template <int MB, bool FUSEQ, bool WIDE, bool GROUPED>
-cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int wide_split = 0) {
+cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int split) {
     using Smem = StreamSmem<MB, WIDE, GROUPED, FUSEQ>;
+    const int tiles = round_up(a.N, kTileN) / kTileN;
     const size_t smem_bytes = sizeof(Smem) + 1024;
+    static_assert(2 * (sizeof(Smem) + 1024 + 1024) <= 228 * 1024, "two CTAs an SM");
     static SmemOptIn opt_in;
     if (const cudaError_t e = opt_in.ensure(gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED>, dev.device, smem_bytes); e != cudaSuccess)
         return e;
     CUtensorMap map = {};
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
     const cuuint64_t strides[1] = {(cuuint64_t)a.K};
-    // MMA route: 8 or 16 rows; rows 8..15 are neither copied nor read when M <= 8
-    const int box_rows = StreamCfg<MB>::kUseMma ? round_up(a.M, 8) : StreamCfg<MB>::kRows;
+    // MMA route: 8 or 16 rows; rows 8..15 are neither copied nor read when M <= 8. Quantized here: 1, 2 or 4 rows as well (what the
+    // instruction then reads as rows up to 7 is the next block's, or whatever follows in the ring, and its sums are dropped)
+    const int box_rows = !StreamCfg<MB>::kUseMma ? StreamCfg<MB>::kRows : FUSEQ ? 1 << slice_row_log(a.M) : round_up(a.M, 8);
     const cuuint32_t box[2] = {128u, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1u, 1u};
     const CUresult r = FUSEQ ? CUDA_SUCCESS : reinterpret_cast<EncodeTiledFn>(dev.encode_tiled)(      // (FUSEQ: nothing is fetched through it)
@@ -890,8 +1002,7 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     // everything before it has completed), or on the caller's promise that nothing in flight writes them.
     p.early_weights = (!p.clear_status || a.weights_stable) ? 1 : 0;
     p.early_dependents = a.weights_stable ? 1 : 0;
-    const int tiles = p.Npad / kTileN, KB = k_blocks(a.K);
-    const int split = WIDE ? wide_split : decode_split(tiles, KB, dev.sm_count);
+    p.alpha = a.fuse_alpha; p.k_max = a.fuse_k_max;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(StreamCfg<MB>::kThreads);
     cfg.dynamicSmemBytes = smem_bytes;
@@ -909,50 +1020,64 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     return cudaLaunchKernelEx(&cfg, gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED>, map, p);
 }
 
-// 16-row route: its consumers, not the memory, set a CTA's pace, so more CTAs per tile pay as long as each
-// keeps five k blocks and all clusters still run at once (a GPC holds only so many clusters of a size: the
-// occupancy query says how many the device does). Measured on the 13B shapes with N = 5120 (clusters of 7):
-// K = 13824 12.5 / 13.2 -> 9.8 / 10.4 us at M = 4 / 16, K = 5120 6.9 / 7.3 -> 6.0 / 6.5 us; a single row
-// loses with clusters of 8 (N = 4096, K = 5120: 5.1 -> 6.2 us). Plain and chained calls take the same cluster
-// (with per-group scales its size sets the order of the fp32 sums). Returns the cluster size (5 to 8), or 0 for the usual 1, 2 or 4.
+// Clusters of `split` CTAs that run at once, by the occupancy query (asked once per device and size).
 template <int MB, bool GROUPED>
-int wide_split_for(int K, int N, const DeviceInfo& dev) {
-    const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
-    if (decode_split(tiles, KB, dev.sm_count) != 4) return 0;
-    static std::atomic<int> fits[kMaxDevices][9];               // clusters of s that run at once, + 1 (0: not asked yet)
-    int s = (2 * dev.sm_count) / tiles;
-    if (s > 8) s = 8;
-    for (; s > 4; --s) {
-        if (KB / s < 5) continue;
-        int known = fits[dev.device][s].load(std::memory_order_relaxed);
-        if (known == 0) {
-            using Smem = StreamSmem<MB, true, GROUPED>;
-            const size_t smem_bytes = sizeof(Smem) + 1024;
-            static SmemOptIn opt_in;
-            int n = 0;
-            if (opt_in.ensure(gemm_decode_stream_kernel<MB, false, true, GROUPED>, dev.device, smem_bytes) == cudaSuccess) {
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(s, tiles, 1);
-                cfg.blockDim = dim3(StreamCfg<MB>::kThreads);
-                cfg.dynamicSmemBytes = smem_bytes;
-                cudaLaunchAttribute attr[1];
-                attr[0].id = cudaLaunchAttributeClusterDimension;
-                attr[0].val.clusterDim.x = s;
-                attr[0].val.clusterDim.y = 1;
-                attr[0].val.clusterDim.z = 1;
-                cfg.attrs = attr;
-                cfg.numAttrs = 1;
-                if (cudaOccupancyMaxActiveClusters(&n, gemm_decode_stream_kernel<MB, false, true, GROUPED>, &cfg) != cudaSuccess) {
-                    (void)cudaGetLastError();
-                    n = 0;
-                }
+int clusters_at_once(int split, const DeviceInfo& dev) {
+    static std::atomic<int> fits[kMaxDevices][9];               // + 1 (0: not asked yet)
+    int known = fits[dev.device][split].load(std::memory_order_relaxed);
+    if (known == 0) {
+        using Smem = StreamSmem<MB, true, GROUPED>;
+        const size_t smem_bytes = sizeof(Smem) + 1024;
+        static SmemOptIn opt_in;
+        int n = 0;
+        if (opt_in.ensure(gemm_decode_stream_kernel<MB, false, true, GROUPED>, dev.device, smem_bytes) == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(split, dev.sm_count, 1);
+            cfg.blockDim = dim3(StreamCfg<MB>::kThreads);
+            cfg.dynamicSmemBytes = smem_bytes;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = split;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&n, gemm_decode_stream_kernel<MB, false, true, GROUPED>, &cfg) != cudaSuccess) {
+                (void)cudaGetLastError();
+                n = 0;
             }
-            known = n + 1;
-            fits[dev.device][s].store(known, std::memory_order_relaxed);
         }
-        if (known - 1 >= tiles) return s;
+        known = n + 1;
+        fits[dev.device][split].store(known, std::memory_order_relaxed);
     }
-    return 0;
+    return known - 1;
+}
+
+// CTAs that share a tile of 128 channels, each with its range of k blocks: the number that leaves a warp the fewest blocks to go through
+// one after the other (two warps of a channel quarter take a CTA's blocks in turn), the smallest such. Only numbers whose clusters all run
+// at once, with some room: a grid's clusters find their places while the grid before it leaves, and what the query says fits just so often
+// has a cluster or two wait for the others to end (us, graph replay, stable weights, 6 rows; the query: 33 clusters of 8, 37 of 7, 45 of 6,
+// 56 of 5, 71 of 4, 93 of 3):
+//   K = 11008  32 tiles   8: 10.57  7: 8.71  6: 8.78  4: 10.88        K = 4096  56 tiles   5: 8.22  4: 6.48  3: 6.95
+//   K = 4096   36 tiles   7: 6.49   6: 5.66  5: 5.86  4: 5.96         K = 4096  72 tiles   4: 10.35  3: 7.34  2: 8.20
+//   K = 4096   48 tiles   5: 6.39   4: 6.03 (four turns each)         K = 4096  86 tiles   3: 8.25  2: 8.80
+// Short ranges are not worth the exchange: two blocks at least, four with 8 CTAs, five where the tile's channels divide unevenly. A single row takes
+// its blocks too fast for uneven slices on short ranges (K = 4096, 40 tiles: 6: 4.99  4: 4.44; K = 8192: 6: 6.31  4: 6.63), and three CTAs
+// win nothing over two there (86 tiles: 6.75 / 6.81, K = 8192 10.25 / 10.03).
+// Plain and chained calls take the same number (with per-group scales it sets the order of the fp32 sums).
+template <int MB, bool GROUPED>
+int stream_split(int K, int N, const DeviceInfo& dev) {
+    const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
+    int best = 1, least = 1 << 30;
+    for (int split = 1; split <= 8; ++split) {
+        const bool even = (split & (split - 1)) == 0;
+        const int blocks = split == 1 ? 1 : split == 8 ? 4 : even ? 2 : MB > 1 ? 5 : split == 3 ? 1 << 20 : 10;       // of a CTA, at least
+        if (tiles * split > 2 * dev.sm_count && split > 1) break;
+        if (KB < blocks * split || (split > 2 && 100 * tiles > 93 * clusters_at_once<MB, GROUPED>(split, dev))) continue;
+        const int turns = ((KB + split - 1) / split + StreamCfg<MB>::kPhases - 1) / StreamCfg<MB>::kPhases;
+        if (turns < least) { least = turns; best = split; }
+    }
+    return best;
 }
 
 template <int MB>
@@ -975,41 +1100,47 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
 }  // namespace
 
 // Whether the product kernel quantizes the rows itself (one launch for the layer). Dumps of per-group sums are left to the general
-// kernel. A single row: where a CTA's k range fits its code buffer. Several rows: up to kFuseElems elements of X. us with two
-// launches / one, graph replay and call by call, without the promise of stable weights and with it:
-//   16 x 768 x 768     5.26 / 4.55   6.20 / 5.01     5.63 / 4.49   6.37 / 4.93
-//   3 x 928 x 2048     4.93 / 3.72   5.78 / 4.20     5.15 / 3.95   5.80 / 4.39
-//   2 x 4096 x 2048 *  5.58 / 5.05   6.47 / 5.40     6.62 / 5.20   7.60 / 5.56      (* groups of 128)
-//   2 x 5120 x 5120         -             -          8.08 / 6.72   9.12 / 7.16
-// Beyond the line it would pay too, up to what more vectors a thread cost the calls below it (eight vectors, 18432 elements: 16 x 1024 x 1024
-// 5.14 / 4.04   5.90 / 4.58     5.56 / 4.14   6.14 / 4.48; 16 x 768 x 768 0.1 more); it lies where it was drawn before the kernel was that short.
-// Without the promise the weights' fetch starts only behind the kernel ahead, which a quantize kernel of the call would have
-// hidden: then small weights only (before the kernel was that short 4 x 2048 x 5504 took 6.40 / 6.83, 2 x 5120 x 5120 7.85 / 8.19).
-bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool weights_stable, const DeviceInfo& dev) {
+// kernel. A single row: where a CTA's k range fits its code buffer. Several rows, and any with a zero point or TRIP factors (plain: neither): while
+// a CTA's slice is kSliceVecs vectors a thread; beyond, every tile's CTAs quantizing the same slice cost more than a kernel that
+// does it once (16 x 11008 x 4096 in groups, 13 vectors, behind a quantize kernel / here: 12.6 / 13.3). us with two launches /
+// one, stable weights, graph replay and call by call, before and after (the number of CTAs a tile has and the order of the MMA's operands
+// changed with it):
+//   6 x 4096 x 4096 *   7.14 / 5.60   8.10 / 5.80     16 x 5120 x 5120    8.81 / 7.79   9.70 / 8.08     (* groups of 128)
+//   9 x 2048 x 2048 *   6.04 / 4.85   7.18 / 5.48      3 x 7168 x 7168   11.25 / 7.68   11.7 / 7.86
+//  16 x  768 x  768 zero point (three launches before)  7.09 / 4.00   8.07 / 4.52      1 x 4096 x 4096 * TRIP  6.73 / 5.6
+// 12289 to 16384 elements keep two launches, as their test asks. Without the promise of stable weights their fetch starts only behind the kernel
+// ahead, which a quantize kernel of the call would have hidden: then only up to four vectors a thread (16 x 5120 x 5120, eight of them:
+// 8.33 / 9.09; 6 x 4096 x 4096 * 7.17 / 6.15, 16 x 2048 x 2048 5.47 / 4.32), or few elements and small weights.
+bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool plain, bool weights_stable, const DeviceInfo& dev) {
     if (M > kFewRows || (group && dump)) return false;
     const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
-    int split = decode_split(tiles, KB, dev.sm_count);
-    if (M == 1) return (KB + split - 1) / split + 1 <= kFuseMaxBlocks;
-    if ((long)M * K > kFuseElems || (!weights_stable && (long)tiles * KB * kBlockBytes > kFuseWeightBytes)) return false;
-    if (const int ws = group ? wide_split_for<kFewRows, true>(K, N, dev) : wide_split_for<kFewRows, false>(K, N, dev)) split = ws;
-    return (KB + split - 1) / split * round_up(M, 8) * kTileK <= kFuseTileBytes;
+    if (M == 1 && plain) {
+        const int split = group ? stream_split<1, true>(K, N, dev) : stream_split<1, false>(K, N, dev);
+        return (KB + split - 1) / split + 1 <= kFuseMaxBlocks;
+    }
+    const int split = group ? stream_split<kFewRows, true>(K, N, dev) : stream_split<kFewRows, false>(K, N, dev);
+    const int vectors = ((((KB + split - 1) / split * (kTileK / 8)) << slice_row_log(M)) + 255) >> 8;      // a thread's
+    if (vectors > kSliceVecs) return false;
+    if (!plain) return weights_stable || vectors <= 4;
+    if ((long)M * K <= kFuseElems) return weights_stable || (long)tiles * KB * kBlockBytes <= kFuseWeightBytes;
+    return (long)M * K > kSliceElemsFrom && (weights_stable || vectors <= 4);
 }
 
 namespace {
 template <int MB, bool GROUPED>
-cudaError_t launch_stream_mma(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    if (const int ws = wide_split_for<MB, GROUPED>(a.K, a.N, dev))
-        return a.fuse_x ? launch_stream<MB, true, true, GROUPED>(a, dev, stream, ws) : launch_stream<MB, false, true, GROUPED>(a, dev, stream, ws);
-    return a.fuse_x ? launch_stream<MB, true, false, GROUPED>(a, dev, stream) : launch_stream<MB, false, false, GROUPED>(a, dev, stream);
+cudaError_t launch_stream_mb(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+    const int split = stream_split<MB, GROUPED>(a.K, a.N, dev);
+    const bool wide = split != 1 && split != 2 && split != 4;
+    if (a.fuse_x)
+        return wide ? launch_stream<MB, true, true, GROUPED>(a, dev, stream, split) : launch_stream<MB, true, false, GROUPED>(a, dev, stream, split);
+    return wide ? launch_stream<MB, false, true, GROUPED>(a, dev, stream, split) : launch_stream<MB, false, false, GROUPED>(a, dev, stream, split);
 }
+// one row: dp4a; from 2 rows on the warp MMA on 16-row tiles (fewer instructions per weight
+// chunk than dp4a from two rows on; measured faster at M = 4: 7.5 / 11.1 / 13.3 us against
+// 8.1 / 12.8 / 15.2 us on the three 13B shapes). A single row with a zero point or TRIP factors that is quantized here takes that route as well.
 template <bool GROUPED>
 cudaError_t launch_stream_rows(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    // one row: dp4a; from 2 rows on the warp MMA on 16-row tiles (fewer instructions per weight
-    // chunk than dp4a from two rows on; measured faster at M = 4: 7.5 / 11.1 / 13.3 us against
-    // 8.1 / 12.8 / 15.2 us on the three 13B shapes)
-    if (a.M <= 1 && a.fuse_x) return launch_stream<1, true, false, GROUPED>(a, dev, stream);
-    if (a.M <= 1) return launch_stream<1, false, false, GROUPED>(a, dev, stream);
-    return launch_stream_mma<16, GROUPED>(a, dev, stream);
+    return a.M <= 1 && !(a.fuse_x && (a.chan_offset || a.fuse_alpha)) ? launch_stream_mb<1, GROUPED>(a, dev, stream) : launch_stream_mb<kFewRows, GROUPED>(a, dev, stream);
 }
 }  // namespace
 

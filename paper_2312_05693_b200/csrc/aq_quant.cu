@@ -12,35 +12,6 @@ namespace aq {
 
 namespace {
 
-// The half2 route with TRIP factors (4-bit codes): lane k multiplies by 2^-(e + alpha_k), built from
-// the factor byte as a half bit pattern (exponent field 15 - e - alpha_k, which must be 1..30),
-// clamps to [-8, 7], rounds by adding and removing 1536, multiplies by 2^alpha_k (exact, |result|
-// <= 128) and adds 1536 again so that the value's two's-complement byte sits in the low 8 bits.
-__device__ __forceinline__ void quantize8_half2_trip(const uint4& d, int e, const uint2& al, uint32_t& w0, uint32_t& w1) {
-    const __half2* h = reinterpret_cast<const __half2*>(&d);
-    const __half2 bias = __floats2half2_rn(1536.0f, 1536.0f);
-    const __half2 lo2 = __floats2half2_rn(-8.0f, -8.0f), hi2 = __floats2half2_rn(7.0f, 7.0f);
-    const uint32_t inv_base = (uint32_t)(15 - e) * 0x04000400u;              // both lanes: (15 - e) << 10
-    const uint32_t one_base = 15u * 0x04000400u;                            // 1.0 in both lanes
-    uint32_t r[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t word = i < 2 ? al.x : al.y;
-        const uint32_t a0 = (word >> (16 * (i & 1))) & 0xFFu, a1 = (word >> (16 * (i & 1) + 8)) & 0xFFu;
-        const uint32_t apair = (a0 | (a1 << 16)) << 10;
-        uint32_t ib = inv_base - apair, sb = one_base + apair;
-        __half2 t = __hmul2(h[i], *reinterpret_cast<__half2*>(&ib));
-        const uint32_t ok = __heq2_mask(t, t);                              // clears NaN lanes
-        uint32_t tb = *reinterpret_cast<uint32_t*>(&t) & ok;
-        t = *reinterpret_cast<__half2*>(&tb);
-        t = __hsub2(__hadd2(__hmin2(__hmax2(t, lo2), hi2), bias), bias);    // the 4-bit code, rounded to nearest even
-        t = __hadd2(__hmul2(t, *reinterpret_cast<__half2*>(&sb)), bias);
-        r[i] = *reinterpret_cast<uint32_t*>(&t);
-    }
-    w0 = __byte_perm(r[0], r[1], 0x6420);
-    w1 = __byte_perm(r[2], r[3], 0x6420);
-}
-
 __device__ __forceinline__ uint4 quantize16_fp32(const uint4& d0, const uint4& d1, int e, float lo, float hi,
                                                  const uint4* al) {
     uint2 a0, a1;
@@ -315,64 +286,20 @@ quantize_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-elem
 }
 
 // ---- zero-point variant (Eq. 2, Eq. 5-7 with alpha = 0, power-of-two scale) ---------------
-// 8 halves -> 8 stored codes (q - 2^(b-1)) of the zero-point quantizer in half2 arithmetic, for
-// exponents whose 2^-e is a normal half. The product by 2^-e is exact (or saturates and is clamped);
-// NaN lanes are cleared to 0, which becomes the code zp; clamping rint(t) + zp to [0, qr] equals
-// clamping t to [-zp, qr - zp] before rounding (integer bounds); adding 1536 rounds to nearest even;
-// adding the integer zp - 2^(b-1) keeps the sum inside [1024, 2048), so the code's byte is the low
-// 8 bits of the half's bit pattern.
-__device__ __forceinline__ void quantize8_half2_asym(const uint4& d, __half2 inv2, __half2 lo2, __half2 hi2,
-                                                     __half2 shift2, uint32_t& w0, uint32_t& w1) {
-    const __half2* h = reinterpret_cast<const __half2*>(&d);
-    const __half2 bias = __floats2half2_rn(1536.0f, 1536.0f);
-    uint32_t r[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        __half2 t = __hmul2(h[i], inv2);
-        const uint32_t ok = __heq2_mask(t, t);
-        uint32_t tb = *reinterpret_cast<uint32_t*>(&t) & ok;
-        t = *reinterpret_cast<__half2*>(&tb);
-        t = __hadd2(__hadd2(__hmin2(__hmax2(t, lo2), hi2), bias), shift2);
-        r[i] = *reinterpret_cast<uint32_t*>(&t);
-    }
-    w0 = __byte_perm(r[0], r[1], 0x6420);
-    w1 = __byte_perm(r[2], r[3], 0x6420);
-}
-
 // Codes from the minimum and maximum that range_kernel left (`words` words), as quantize_kernel.
 __global__ void __launch_bounds__(kQuantThreads)
 quantize_asym_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-element units */,
                      const int32_t* __restrict__ row_idx, int bits, int words, Control* __restrict__ ctl,
                      uint4* __restrict__ q, int32_t* __restrict__ scale_exp_out, int32_t* __restrict__ zero_point_out) {
-    __shared__ int params[2];                          // e, zp
     asm volatile("griddepcontrol.wait;" ::: "memory");                 // see quantize_kernel
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t total = (size_t)M * units_per_row;
     const size_t u0 = (size_t)blockIdx.x * (kQuantThreads * kQuantUnits) + threadIdx.x;
     uint4 d[kQuantUnits][2];
     load_units(x, u0, total, units_per_row, row_idx, d);
-    if (threadIdx.x < 32) {
-        const unsigned int met = met_range(ctl, words);
-        if (threadIdx.x == 0) {
-            // +-Inf count as the largest half
-            const double dhi = (double)__half2float(__ushort_as_half((unsigned short)min(met & 0xFFFFu, 0x7BFFu)));
-            const double dlo = -(double)__half2float(__ushort_as_half((unsigned short)min(met >> 16, 0x7BFFu)));
-            const double qr = (double)((1 << bits) - 1);
-            const double range = dhi - dlo;
-            int ee = 0;
-            if (range > 0.0) {
-                int ex;
-                frexp(range / qr, &ex);              // a first guess within one of the answer
-                ee = ex;
-                while (ldexp(qr, ee) < range) ++ee;
-                while (ldexp(qr, ee - 1) >= range) --ee;
-            }
-            params[0] = ee;
-            params[1] = (int)fmin(fmax(rint(ldexp(-dlo, -ee)), 0.0), qr);
-        }
-    }
-    __syncthreads();
-    const int e = params[0], zp = params[1];
+    const unsigned int met = met_range(ctl, words);
+    int e, zp;
+    zero_point_scale(met & 0xFFFFu, met >> 16, bits, e, zp);
     publish_control(ctl, 0u, e, zp, scale_exp_out, zero_point_out);
     const int qr_i = (1 << bits) - 1, half_range = 1 << (bits - 1);
     const float inv = __int_as_float((127 - e) << 23);      // 2^-e
@@ -390,21 +317,8 @@ quantize_asym_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16
             quantize8_half2_asym(d[i][0], inv2, clo2, chi2, shift2, out[0], out[1]);
             quantize8_half2_asym(d[i][1], inv2, clo2, chi2, shift2, out[2], out[3]);
         } else {
-            const __half* h0 = reinterpret_cast<const __half*>(&d[i][0]);
-            const __half* h1 = reinterpret_cast<const __half*>(&d[i][1]);
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                uint32_t word = 0;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const int k = 4 * w + b;
-                    const float t = __half2float(k < 8 ? h0[k] : h1[k - 8]) * inv;    // exact
-                    int code = zp;                                                    // NaN: value 0
-                    if (t == t) code = (int)fminf(fmaxf(rintf(t) + fzp, 0.0f), fqr);
-                    word |= ((uint32_t)(code - half_range) & 0xFFu) << (8 * b);
-                }
-                out[w] = word;
-            }
+            const uint2 c0 = quantize8_fp32_asym(d[i][0], inv, zp, bits), c1 = quantize8_fp32_asym(d[i][1], inv, zp, bits);
+            out[0] = c0.x; out[1] = c0.y; out[2] = c1.x; out[3] = c1.y;
         }
         q[u] = make_uint4(out[0], out[1], out[2], out[3]);
     }

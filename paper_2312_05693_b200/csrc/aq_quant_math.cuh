@@ -63,6 +63,106 @@ __device__ __forceinline__ uint2 quantize8_fp32(const uint4& d, int e, float lo,
     return make_uint2(out[0], out[1]);
 }
 
+// The half2 route with TRIP factors (4-bit codes): lane k multiplies by 2^-(e + alpha_k), built from
+// the factor byte as a half bit pattern (exponent field 15 - e - alpha_k, which must be 1..30),
+// clamps to [-8, 7], rounds by adding and removing 1536, multiplies by 2^alpha_k (exact, |result|
+// <= 128) and adds 1536 again so that the value's two's-complement byte sits in the low 8 bits.
+__device__ __forceinline__ void quantize8_half2_trip(const uint4& d, int e, const uint2& al, uint32_t& w0, uint32_t& w1) {
+    const __half2* h = reinterpret_cast<const __half2*>(&d);
+    const __half2 bias = __floats2half2_rn(1536.0f, 1536.0f);
+    const __half2 lo2 = __floats2half2_rn(-8.0f, -8.0f), hi2 = __floats2half2_rn(7.0f, 7.0f);
+    const uint32_t inv_base = (uint32_t)(15 - e) * 0x04000400u;              // both lanes: (15 - e) << 10
+    const uint32_t one_base = 15u * 0x04000400u;                            // 1.0 in both lanes
+    uint32_t r[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t word = i < 2 ? al.x : al.y;
+        const uint32_t a0 = (word >> (16 * (i & 1))) & 0xFFu, a1 = (word >> (16 * (i & 1) + 8)) & 0xFFu;
+        const uint32_t apair = (a0 | (a1 << 16)) << 10;
+        uint32_t ib = inv_base - apair, sb = one_base + apair;
+        __half2 t = __hmul2(h[i], *reinterpret_cast<__half2*>(&ib));
+        const uint32_t ok = __heq2_mask(t, t);                              // clears NaN lanes
+        uint32_t tb = *reinterpret_cast<uint32_t*>(&t) & ok;
+        t = *reinterpret_cast<__half2*>(&tb);
+        t = __hsub2(__hadd2(__hmin2(__hmax2(t, lo2), hi2), bias), bias);    // the 4-bit code, rounded to nearest even
+        t = __hadd2(__hmul2(t, *reinterpret_cast<__half2*>(&sb)), bias);
+        r[i] = *reinterpret_cast<uint32_t*>(&t);
+    }
+    w0 = __byte_perm(r[0], r[1], 0x6420);
+    w1 = __byte_perm(r[2], r[3], 0x6420);
+}
+
+// 8 halves -> 8 stored codes (q - 2^(b-1)) of the zero-point quantizer in half2 arithmetic, for
+// exponents whose 2^-e is a normal half. The product by 2^-e is exact (or saturates and is clamped);
+// NaN lanes are cleared to 0, which becomes the code zp; clamping rint(t) + zp to [0, qr] equals
+// clamping t to [-zp, qr - zp] before rounding (integer bounds); adding 1536 rounds to nearest even;
+// adding the integer zp - 2^(b-1) keeps the sum inside [1024, 2048), so the code's byte is the low
+// 8 bits of the half's bit pattern.
+__device__ __forceinline__ void quantize8_half2_asym(const uint4& d, __half2 inv2, __half2 lo2, __half2 hi2,
+                                                     __half2 shift2, uint32_t& w0, uint32_t& w1) {
+    const __half2* h = reinterpret_cast<const __half2*>(&d);
+    const __half2 bias = __floats2half2_rn(1536.0f, 1536.0f);
+    uint32_t r[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        __half2 t = __hmul2(h[i], inv2);
+        const uint32_t ok = __heq2_mask(t, t);
+        uint32_t tb = *reinterpret_cast<uint32_t*>(&t) & ok;
+        t = *reinterpret_cast<__half2*>(&tb);
+        t = __hadd2(__hadd2(__hmin2(__hmax2(t, lo2), hi2), bias), shift2);
+        r[i] = *reinterpret_cast<uint32_t*>(&t);
+    }
+    w0 = __byte_perm(r[0], r[1], 0x6420);
+    w1 = __byte_perm(r[2], r[3], 0x6420);
+}
+// The same in fp32 arithmetic (inv = 2^-e), for the other exponents.
+__device__ __forceinline__ uint2 quantize8_fp32_asym(const uint4& d, float inv, int zp, int bits) {
+    const __half* h = reinterpret_cast<const __half*>(&d);
+    const float fzp = (float)zp, fqr = (float)((1 << bits) - 1);
+    uint32_t out[2];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+        uint32_t word = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const float t = __half2float(h[4 * w + b]) * inv;                          // exact
+            int code = zp;                                                             // NaN: value 0
+            if (t == t) code = (int)fminf(fmaxf(rintf(t) + fzp, 0.0f), fqr);
+            word |= ((uint32_t)(code - (1 << (bits - 1))) & 0xFFu) << (8 * b);
+        }
+        out[w] = word;
+    }
+    return make_uint2(out[0], out[1]);
+}
+
+// A finite half's magnitude (bit pattern) in units of 2^-24, of which every half is a whole number; Inf counts as 65504.
+__device__ __forceinline__ long long half_units(unsigned int bits) {
+    if (bits > 0x7BFFu) bits = 0x7BFFu;
+    const unsigned int ex = bits >> 10;
+    return ex ? (long long)(0x400u | (bits & 0x3FFu)) << (ex - 1) : (long long)bits;
+}
+// Exponent and zero point (Eq. 6, Eq. 7): e the smallest with (2^b - 1) 2^e >= max - min, zp = -min / 2^e rounded to nearest even,
+// clipped to the codes. hi, lo: bit patterns of the largest value and of the least one's magnitude, 0 where there is none.
+// Whole numbers: max - min has at most 41 bits in units of 2^-24.
+__device__ __forceinline__ void zero_point_scale(unsigned int hi, unsigned int lo, int bits, int& e, int& zp) {
+    const long long qr = (1 << bits) - 1, least = half_units(lo), range = half_units(hi) + least;
+    e = 0;
+    zp = 0;
+    if (range == 0) return;
+    int sh = (64 - __clzll(range)) - bits;               // e in units of 2^-24: qr 2^(sh + 1) >= range > qr 2^(sh - 1), for any sh
+    if (sh >= 0 ? (qr << sh) < range : qr < (range << -sh)) ++sh;
+    e = sh - 24;
+    long long z;
+    if (sh <= 0) {
+        z = least << -sh;
+    } else {
+        z = least >> sh;
+        const long long rest = least & ((1ll << sh) - 1), half = 1ll << (sh - 1);
+        if (rest > half || (rest == half && (z & 1))) ++z;
+    }
+    zp = (int)(z > qr ? qr : z);
+}
+
 // A CTA may write into another one's shared memory only once that one has started, which being scheduled together does
 // not promise: every thread arrives at its kernel's top and waits just before the kernel's first remote store (a CTA
 // whose share of X is empty gets there at once). Behind the loads the wait costs next to nothing: without it and with
