@@ -15,7 +15,7 @@
 // One persistent CTA per SM walks a static list of (channel tile, token tile) pairs.
 // Warp roles: 0 and 2 = TMA producers (activations / weights), 1 = MMA issuer (and owner of the TMEM
 // allocation), 3 = watches the accumulator barriers for the epilogue (per-group mode), 4-11 = weight unpack
-// (two groups of four taking alternate k blocks; only the first group works in per-group mode above 64 tokens),
+// (two groups of four taking alternate k blocks; the per-group kernel on 192-token tiles has one),
 // 12-19 = epilogue; registers are moved from
 // the first two roles to the epilogue with setmaxnreg. The issuing threads are chosen with elect.sync: then the
 // compiler knows that one thread is active, and a k block's four MMAs and three commits take about 100 cycles of
@@ -42,7 +42,9 @@ constexpr int kFirstUnpackWarp = 4;           // warps 0-3 (one warpgroup): two 
 constexpr int kWarps = 20;
 constexpr int kThreads = kWarps * 32;
 // Registers per thread after the roles split (setmaxnreg works on aligned groups of four warps):
-constexpr int kRegsControl = 40, kRegsUnpack = 48;
+// (Unpack warps with 40 instead of 48: 128 x 4096 x 11008 in groups 20.1 -> 19.0 us, 333 x 5120 x 5120 24.7 -> 23.4, 1000 x 1024 x 4096
+// 15.8 -> 15.2; the 64- and 192-token tiles within 1 %.)
+constexpr int kRegsControl = 40, kRegsUnpack = 40;
 // The warps behind the control warpgroup are unpack warps, then epilogue warps. Eight epilogue warps (two per
 // TMEM lane quarter, half of the token columns each) follow two groups of unpack warps; the per-group
 // kernels with 192-token tiles run twelve (three per quarter, a third of the columns each) behind
@@ -241,6 +243,11 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
     constexpr int kTmemCols = kTmemColsUsed <= 128 ? 128 : kTmemColsUsed <= 256 ? 256 : 512;
     static_assert(kTmemColsUsed <= 512, "tensor memory has 512 columns");
     static_assert(BM % 32 == 0 && BM >= 64 && BM <= 256, "token tile");
+    // Which epilogue warps share the watcher's barrier. Twelve: the four of a third of the columns, one on each scheduler, so that the
+    // three warps of a scheduler may be at different places of their blocks (with the three of a lane quarter, which share a scheduler,
+    // K, N = 4096, 4096 / 4096, 11008 / 11008, 4096 at M = 2048 take 61.3 / 125.8 / 131.9 us, so 60.5 / 123.3 / 129.6). Eight: the two of a lane
+    // quarter (by halves 509 x 4096 x 4096 with a zero point 22.3 -> 23.0).
+    constexpr int kMeetGroups = kEpiWarps == 12 ? 3 : 4;
     constexpr int kColsPerEpiWarp = R::kColsPerEpiWarp;   // each quarter's columns are split between two or three warps
     static_assert(kColsPerEpiWarp % 16 == 0 && (!GROUPED || kColsPerEpiWarp % 32 == 0), "epilogue chunking");
 
@@ -364,8 +371,8 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 tc_fence_after();
                 tc_fence_before();
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    asm volatile("bar.arrive %0, %1;" ::"r"(1 + q * kNumAcc + (int)a), "n"(32 + kEpiWarps * 8) : "memory");
+                for (int g = 0; g < kMeetGroups; ++g)
+                    asm volatile("bar.arrive %0, %1;" ::"r"(1 + g * kNumAcc + (int)a), "n"(32 + kEpiWarps * 32 / kMeetGroups) : "memory");
                 ph ^= 1u << a;
             };
             for (int tl = 0; tl < my_tiles && live; ++tl) {
@@ -465,10 +472,10 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const uint32_t total_iters = (uint32_t)my_tiles * (uint32_t)(kb_last - kb_first);
         int pending = -1;                             // slice whose store has been issued but not published
-        // With per-group rescaling and more than 64 tokens the epilogue sets the pace (about four times the MMA time per
-        // k block) and one group of unpack warps (about 500 cycles a block) keeps up; the second group would only poll barriers on the schedulers
-        // the epilogue warps issue from (measured: 1-2 % slower with it), so it leaves at once.
-        constexpr int kActiveGroups = GROUPED && BM > 64 ? 1 : kUnpackGroups;
+        // Per-group kernels on 192-token tiles have one group of unpack warps: the epilogue sets the pace there, and a second group
+        // (four warps more, 120 registers for the epilogue) wins 0.5 % at M = 2048. On 128-token tiles the second group shortens the
+        // block: 509 x 11008 x 4096 with a zero point 44.4 -> 43.0 us, 333 x 5120 x 5120 25.1 -> 24.7.
+        constexpr int kActiveGroups = GROUPED && BM > 128 ? 1 : kUnpackGroups;
         if (group >= kActiveGroups) goto role_done;
         uint32_t s = (uint32_t)group, s_ph = 0u, ai = (uint32_t)group, a_ph = 1u;
         for (uint32_t it = group; it < total_iters; it += kActiveGroups) {
@@ -516,6 +523,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         const int r = quarter * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const int col0 = half * kColsPerEpiWarp;
+        [[maybe_unused]] const int meet_group = kMeetGroups == 4 ? quarter : half;
         asm volatile("griddepcontrol.wait;" ::: "memory");               // see the activation producer
         const float pe = __int_as_float((127 + *p.scale_exp) << 23);     // 2^e
         [[maybe_unused]] const float off_factor = OFFSET ? offset_factor(p.ctl, p.zp_mid) : 0.0f;
@@ -672,7 +680,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 // cycles: the named barrier and the loop 100, the first load with the scale 130, the second with the release 150, and
                 // 460 of conversions and FMAs, which the three warps of a scheduler want at the same time.
                 auto block = [&](const uint32_t a, int kb) {
-                    asm volatile("bar.sync %0, %1;" ::"r"(1 + quarter * kNumAcc + (int)a), "n"(32 + kEpiWarps * 8) : "memory");   // the watcher's word
+                    asm volatile("bar.sync %0, %1;" ::"r"(1 + meet_group * kNumAcc + (int)a), "n"(32 + kEpiWarps * 32 / kMeetGroups) : "memory");   // the watcher's word
                     tc_fence_after();
                     // This block's MMAs are complete, so its stage (scales included) had landed: the
                     // issuer saw the unpack warps' signal, which they gave after seeing the TMA barrier.
