@@ -1,5 +1,6 @@
 // Log2 quantization of the softmax output (paper Eq. 3, Sec. 5.1) and the attention-times-value
 // product on its codes, where every product is a shift of the int8 value code.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "aq_attn_parts.cuh"
@@ -158,6 +159,235 @@ __device__ __forceinline__ __half2 log2_fast2(__half2 x2, const Log2Fast& f) {
     return __hmul2(r, valid);
 }
 
+// Byte factors of eight values where all bounds are normal halves: one mantissa, exponents one apart, so as integers B_j = B_1 - 1024 (j - 1)
+// and k = min((B_1 + 1023 - |x|) >> 10, 7) on the bit patterns, two to a register. Four k's select four bytes of the eight factors in one
+// byte permute; zeros, NaNs and negative inputs (recorded) give 0. cap: B_1 + 1023 in both halves. NEAR: the largest remainders (of 1024) of
+// the values with k < 7, the lanes apart: a B_1 larger by d, d < 1024, changes the factors where the remainder is 1024 - d or more, and no others;
+// least: the least distance from cap so far (0: a value of cap or more, negative or NaN).
+template <bool NEAR>
+__device__ __forceinline__ uint2 log2_factors8(const uint4& d, uint32_t cap, uint32_t& near, uint32_t& least, bool& bad) {
+    const uint32_t w[4] = {d.x, d.y, d.z, d.w};
+    uint32_t below[4], some[4], sel[2];
+    near = 0u;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        some[t] = __hgt2_mask(*reinterpret_cast<const __half2*>(&w[t]), __float2half2_rn(0.0f));
+        const uint32_t all = cap - __vminu2(w[t], cap);
+        if (NEAR) least = __vminu2(least, all);
+        below[t] = __vminu2(all, 0x1C001C00u);                // 7 * 1024: k = 7, remainder 0
+        if (NEAR) near = __vmaxu2(near, below[t] & 0x03FF03FFu);
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {                             // k of four values in four nibbles
+        const uint32_t k = ((below[2 * t] >> 10) & 0x00070007u) | ((below[2 * t + 1] >> 2) & 0x07000700u);
+        sel[t] = k | (k >> 12);
+    }
+    if ((w[0] | w[1] | w[2] | w[3]) & 0x80008000u) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            bad |= __hlt2_mask(*reinterpret_cast<const __half2*>(&w[t]), __float2half2_rn(0.0f)) != 0u;
+    }
+    return make_uint2(__byte_perm(0x10204080u, 0x01020408u, sel[0] & 0x7777u) & __byte_perm(some[0], some[1], 0x6420),
+                      __byte_perm(0x10204080u, 0x01020408u, sel[1] & 0x7777u) & __byte_perm(some[2], some[3], 0x6420));
+}
+// B_1 of a maximum, or 0 where not all bounds are normal halves (see log2_fast_bounds: the same, as a bit pattern).
+__device__ __forceinline__ unsigned int log2_first_bound(unsigned int max_bits) {
+    if (max_bits == 0u) return 0u;
+    int mb, eb, t_up, t_down;
+    half_parts(max_bits, mb, eb);
+    log2_thresholds(mb, t_up, t_down);
+    const int bits = t_down <= 2047 ? ((eb + 24) << 10) + t_down - 1024 : ((eb + 25) << 10) + max(t_up + 1, 1024) - 1024;
+    return bits >= 0x1C00 ? (unsigned int)bits : 0u;         // B_7 = B_1 / 64
+}
+__device__ __forceinline__ uint8_t log2_factor(unsigned int raw, unsigned int mb_bits, int eb, int t_up, int t_down, bool& bad) {
+    const int c = log2_code(raw, mb_bits, eb, t_up, t_down, 7);
+    bad |= c < 0;
+    return (uint8_t)(c > 0 ? 128u >> (c - 1) : 0u);
+}
+
+// ---- byte factors in one pass over x -----------------------------------------------------------
+// The maximum is known only when all of x has been read, but nearly all factors are settled before: by a maximum that is a little too small
+// a factor comes out wrong only where the value lies just under a bound, and values from 2^-6.5 of the maximum down have the
+// last factor whatever it is. So a cooperative grid reads x once, writes the factors by the largest maximum seen so far, and notes in shared
+// memory the vectors of eight that a maximum up to `kLead` steps further would change; when all is read the grid meets, and
+// the noted vectors are written again by the true maximum. So are all vectors of a warp's batches whose maximum was further off (the
+// first few), and of a warp whose notes did not fit: then x is read twice, as by the two kernels that this replaces for arrays larger
+// than the L2 keeps.
+// Bound by memory: 2 bytes in, 1 out per value, at 5.6 TB/s between the meetings (32 x 2048 x 2048).
+constexpr int kOnceThreads = 1024, kOnceNotes = 10240;
+constexpr unsigned int kLead = 320;                     // of 1024 steps to twice the bound
+constexpr unsigned int kBoundOfOne = 0x39A9u;           // B_1 where the maximum is 1: 1449 * 2^-11, 1449 the least whole number above 1024 sqrt(2)
+constexpr int kOnceChanges = 8;
+
+__global__ void __launch_bounds__(kOnceThreads, 1)
+log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control* __restrict__ ctl, uint8_t* __restrict__ factors,
+                         uint32_t* __restrict__ max_bits_out) {
+    __shared__ uint32_t notes[kOnceNotes];
+    __shared__ unsigned int noted, warp_max[kOnceThreads / 32];
+    // per warp: from which of its batches on its factors stood for which B_1 (a new entry where its maximum changed)
+    __shared__ unsigned short covers[kOnceThreads / 32][kOnceChanges];
+    __shared__ uint32_t from_batch[kOnceThreads / 32][kOnceChanges];
+    cg::grid_group grid = cg::this_grid();
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    const long long nvec = count / 8, stride = (long long)gridDim.x * kOnceThreads, at = (long long)blockIdx.x * kOnceThreads + threadIdx.x;
+    const uint4* const xv = reinterpret_cast<const uint4*>(x);
+    uint2* const out = reinterpret_cast<uint2*>(factors);
+    volatile unsigned int* const running = &ctl->absmax_bits;
+    __half2 m2 = __float2half2_rn(0.0f);                 // NaN operands are dropped
+    auto largest = [&](const uint4& d) {
+        const uint32_t w[4] = {d.x & 0x7FFF7FFFu, d.y & 0x7FFF7FFFu, d.z & 0x7FFF7FFFu, d.w & 0x7FFF7FFFu};
+#pragma unroll
+        for (int t = 0; t < 4; ++t) m2 = __hmax2(m2, *reinterpret_cast<const __half2*>(&w[t]));
+    };
+    // of this thread's values so far; Inf counts as the largest finite value
+    auto max_bits = [&] {
+        const unsigned int b = max((unsigned int)__half_as_ushort(__low2half(m2)), (unsigned int)__half_as_ushort(__high2half(m2)));
+        return min(b, 0x7BFFu);
+    };
+    // a first maximum: from the first batches of as many CTAs as the control block has words for
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctl->status = 0;
+        *running = 0u;
+    }
+    if (threadIdx.x == 0) noted = 0u;
+    if (blockIdx.x < Control::kRangeWords) {
+#pragma unroll
+        for (int k = 0; k < kLog2InFlight; ++k)
+            if (at + k * stride < nvec) largest(__ldg(xv + at + k * stride));
+        const unsigned int b = __reduce_max_sync(0xFFFFFFFFu, max_bits());
+        if (lane == 0) warp_max[warp] = b;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const unsigned int c = __reduce_max_sync(0xFFFFFFFFu, lane < kOnceThreads / 32 ? warp_max[lane] : 0u);
+            if (lane == 0) ctl->range[blockIdx.x] = c;
+        }
+    }
+    grid.sync();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const unsigned int words = min(gridDim.x, (unsigned int)Control::kRangeWords);
+    unsigned int known = __reduce_max_sync(0xFFFFFFFFu, lane < (int)words ? ((volatile unsigned int*)ctl->range)[lane] : 0u), used = ~0u;
+    uint32_t cap = 0u, edge = 0u;                        // edge: remainders from 1024 - lead on reach bit 15 when it is added
+    unsigned int bound = 0u;
+    int changes = 0;
+    uint32_t batch = 0;
+    bool bad = false, all_again = false;
+    const uint4* p = xv + at;
+    long long v = at;
+    for (long long left = nvec - (at - lane); left > 0; left -= kLog2InFlight * stride, p += kLog2InFlight * stride, v += kLog2InFlight * stride) {
+        uint4 d[kLog2InFlight];                          // left: vectors from the warp's first on
+        const bool whole = left > (kLog2InFlight - 1) * stride + 31;
+#pragma unroll
+        for (int k = 0; k < kLog2InFlight; ++k) {
+            d[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (whole || v + k * stride < nvec) d[k] = __ldg(p + k * stride);
+        }
+        const unsigned int next = *running;              // for the next batch
+        if (known != used) {
+            used = known;
+            bound = log2_first_bound(used);
+            cap = (bound + 1023u) * 0x00010001u;
+            // a softmax output is 1 at most
+            const unsigned int lead = used <= 0x3C00u ? min(kBoundOfOne - bound, kLead) : 64u;
+            edge = (0x8000u - 1024u + lead) * 0x00010001u;
+            // (with no place left the last entry stands for fewer batches than it could)
+            const int place = min(changes, kOnceChanges - 1);
+            if (lane == 0) {
+                covers[warp][place] = (unsigned short)(bound + lead);
+                from_batch[warp][place] = batch;
+            }
+            changes = place + 1;
+        }
+        ++batch;
+        if (bound == 0u) {
+            all_again = true;
+#pragma unroll
+            for (int k = 0; k < kLog2InFlight; ++k) largest(d[k]);
+        } else {
+            uint32_t least = cap;
+#pragma unroll
+            for (int k = 0; k < kLog2InFlight; ++k) {
+                uint32_t near;
+                const uint2 f = log2_factors8<true>(d[k], cap, near, least, bad);
+                if (whole || v + k * stride < nvec) {
+                    __stcs(out + v + k * stride, f);
+                    if ((near + edge) & 0x80008000u) {
+                        const unsigned int n = atomicAdd(&noted, 1u);
+                        if (n < (unsigned int)kOnceNotes) notes[n] = (uint32_t)(v + k * stride);
+                        else all_again = true;
+                    }
+                }
+            }
+            if (__vminu2(least, 0x00010001u) != 0x00010001u) {
+#pragma unroll
+                for (int k = 0; k < kLog2InFlight; ++k) largest(d[k]);
+            } else {
+                const uint32_t most = cap - least;
+                m2 = __hmax2(m2, *reinterpret_cast<const __half2*>(&most));
+            }
+        }
+        __syncwarp();
+        known = max(known, next);
+        const unsigned int own = __reduce_max_sync(0xFFFFFFFFu, max_bits());
+        if (own > known) {
+            if (lane == 0) atomicMax(&ctl->absmax_bits, own);
+            known = own;
+        }
+    }
+    // the ragged tail's maximum
+    for (long long i = nvec * 8 + at; i < count; i += stride) {
+        const unsigned int hb = __half_as_ushort(x[i]) & 0x7FFFu;
+        if (hb <= 0x7C00u) known = max(known, min(hb, 0x7BFFu));
+    }
+    __syncwarp();
+    {
+        const unsigned int b = __reduce_max_sync(0xFFFFFFFFu, max(known, max_bits()));
+        if (lane == 0) warp_max[warp] = b;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const unsigned int c = __reduce_max_sync(0xFFFFFFFFu, lane < kOnceThreads / 32 ? warp_max[lane] : 0u);
+            if (lane == 0 && c > *running) atomicMax(&ctl->absmax_bits, c);
+        }
+    }
+    grid.sync();
+    const unsigned int mb_bits = *running, final_bound = log2_first_bound(mb_bits);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && max_bits_out) *max_bits_out = mb_bits;
+    const uint32_t final_cap = (final_bound + 1023u) * 0x00010001u;
+    int mb = 1024, eb = 0, t_up = 0, t_down = 0;
+    if (mb_bits) half_parts(mb_bits, mb, eb);
+    log2_thresholds(mb, t_up, t_down);
+    uint32_t near, least = 0u;
+    // the batches up to the first change whose factors stand for the true bound
+    const bool again = __any_sync(0xFFFFFFFFu, all_again || final_bound == 0u);
+    long long redo = again ? nvec : 0;
+    if (!again && changes > 0) {
+        int c = 0;
+        while (c < changes && covers[warp][c] < final_bound) ++c;
+        redo = c == changes ? nvec : at + (long long)from_batch[warp][c] * kLog2InFlight * stride;
+    }
+    {
+        for (v = at; v < min(redo, nvec); v += stride) {
+            const uint4 d = __ldg(xv + v);
+            if (final_bound) {
+                out[v] = log2_factors8<false>(d, final_cap, near, least, bad);
+            } else {
+                const uint32_t w[4] = {d.x, d.y, d.z, d.w};
+                uint32_t o[2] = {0u, 0u};
+#pragma unroll
+                for (int t = 0; t < 8; ++t)
+                    o[t >> 2] |= (uint32_t)log2_factor((w[t >> 1] >> (16 * (t & 1))) & 0xFFFFu, mb_bits, eb, t_up, t_down, bad) << (8 * (t & 3));
+                out[v] = make_uint2(o[0], o[1]);
+            }
+        }
+    }
+    // (another warp's vectors may be among these, written by it above as well: the same factors)
+    if (final_bound)
+        for (unsigned int n = threadIdx.x; n < min(noted, (unsigned int)kOnceNotes); n += kOnceThreads)
+            out[notes[n]] = log2_factors8<false>(__ldg(xv + notes[n]), final_cap, near, least, bad);
+    for (long long i = nvec * 8 + at; i < count; i += stride)
+        factors[i] = log2_factor(__half_as_ushort(x[i]), mb_bits, eb, t_up, t_down, bad);
+    if (bad) atomicCAS(&ctl->status, 0u, 11u);
+}
+
 __global__ void __launch_bounds__(256, kLog2Ctas)
 log2_codes_kernel(const __half* __restrict__ x, long long count, int bits, int words, Control* __restrict__ ctl,
                   int8_t* __restrict__ codes, uint32_t* __restrict__ max_bits_out, int as_factors) {
@@ -182,33 +412,14 @@ log2_codes_kernel(const __half* __restrict__ x, long long count, int bits, int w
         const Log2Fast fast = log2_fast_bounds(mb, eb, t_up, t_down);
         const unsigned int b1 = __half_as_ushort(__low2half(fast.bound[0]));
         if (as_factors && (unsigned int)__half_as_ushort(__low2half(fast.bound[6])) >= 0x0400u) {
-            // All bounds are normal halves: one mantissa, exponents one apart, so as integers B_j = B_1 - 1024 (j - 1) and
-            // k = min((B_1 + 1023 - |x|) >> 10, 7) on the bit patterns, two to a register. Four k's select four bytes of
-            // the eight factors in one byte permute; zeros, NaNs and negative inputs (recorded) give 0. x is walked
-            // backwards, since its end is what the maximum's kernel has left in the L2 (57 MB of 268 MB hit there), with
+            // x is walked backwards, since its end is what the maximum's kernel has left in the L2 (57 MB of 268 MB hit there), with
             // stores marked as not used again (loads marked so cost 10 us). Both kernels on 32 x 2048 x 2048: 145.6 -> 107.3 us (45 us at
             // 5.9 TB/s and 66 us at 4.8 TB/s of HBM traffic, reads and writes mixed); on 4 heads, 33 MB, 28.8 -> 19.2 us.
             const uint32_t cap = (b1 + 1023u) * 0x00010001u;
             const long long stride = (long long)gridDim.x * blockDim.x;
             auto factors = [&](const uint4& d) {
-                const uint32_t w[4] = {d.x, d.y, d.z, d.w};
-                uint32_t sel[4], some[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    some[t] = __hgt2_mask(*reinterpret_cast<const __half2*>(&w[t]), __float2half2_rn(0.0f));
-                    const uint32_t steps = ((cap - __vminu2(w[t], cap)) >> 10) & 0x003F003Fu;
-                    const uint32_t k7 = __vminu2(steps, 0x00070007u);
-                    sel[t] = k7 | (k7 >> 12);
-                }
-                if ((w[0] | w[1] | w[2] | w[3]) & 0x80008000u) {
-#pragma unroll
-                    for (int t = 0; t < 4; ++t)
-                        bad |= __hlt2_mask(*reinterpret_cast<const __half2*>(&w[t]), __float2half2_rn(0.0f)) != 0u;
-                }
-                uint2 out;
-                out.x = __byte_perm(0x10204080u, 0x01020408u, __byte_perm(sel[0], sel[1], 0x0040)) & __byte_perm(some[0], some[1], 0x6420);
-                out.y = __byte_perm(0x10204080u, 0x01020408u, __byte_perm(sel[2], sel[3], 0x0040)) & __byte_perm(some[2], some[3], 0x6420);
-                return out;
+                uint32_t near, least = 0u;
+                return log2_factors8<false>(d, cap, near, least, bad);
             };
             long long v = nvec - 1 - ((long long)blockIdx.x * blockDim.x + threadIdx.x);       // this thread's vector, downwards
             const uint4* src = xv + v;
@@ -803,8 +1014,29 @@ cudaError_t launch_attn_qk_tc(const int8_t* qc, const int32_t* e_q, const int8_t
     return launch_attn_tc<128, true, 1, 8>(qc, kc, nullptr, e_q, e_k, 0, H, M, D, J, s_out, ctl, dev, stream, true);
 }
 
+// Values from which byte factors are made in one pass: 117 MB of them, about what the L2 holds. us in two kernels / one, graph replay,
+// softmax outputs of 56 x 2048 x 2048 values 191.6 / 134.2, 32 x 2048 x 2048 110.9 / 82.4, 40 x 1500 x 1024 53.7 / 49.3, 12 x 2048 x 2048
+// 44.9 / 43.8 (call by call 45.8 / 46.1), 16 x 1024 x 2048 31.8 / 33.9: the grid's two meetings and a launch that overlaps nothing cost some
+// 12 us, and below that size most of the second reading comes from the L2.
+constexpr long long kOnceCount = 7ll << 23;
+
 cudaError_t launch_log2_quantize(const __half* x, long long count, int bits, Control* ctl, int8_t* codes,
                                  uint32_t* max_bits_out, const DeviceInfo& dev, cudaStream_t stream, bool as_factors) {
+    if (as_factors && count >= kOnceCount && count < (1ll << 35) && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && (reinterpret_cast<uintptr_t>(codes) & 7u) == 0) {
+        // all CTAs at once: one an SM
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(dev.sm_count);
+        cfg.blockDim = dim3(kOnceThreads);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, log2_factors_once_kernel, x, count, ctl, reinterpret_cast<uint8_t*>(codes), max_bits_out);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+        (void)cudaGetLastError();                        // a part of the GPU only: in two kernels
+    }
     // as many clusters as the control block has words for (232 CTAs: two per SM of most), fewer for small arrays
     long long clusters = (count / 8 + kRangeCtas * kLog2MaxThreads - 1) / (kRangeCtas * kLog2MaxThreads);
     if (clusters > Control::kRangeWords) clusters = Control::kRangeWords;
