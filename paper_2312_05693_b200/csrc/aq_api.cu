@@ -154,7 +154,8 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     if (fuse) {
     } else if (w_offsets) {
         // zero-point variant: min / max, then e, zp and codes; the product adds the term -(zp - 2^(b-1)) * r[n]
-        e = launch_quantize_asym(xh, M, K, row_idx, bits, w.ctl, w.codes, nullptr, nullptr, stream);
+        e = quantize_small_fits(M, K) ? launch_quantize_small_asym(xh, M, K, row_idx, bits, w.ctl, w.codes, nullptr, nullptr, stream, h->weights_stable != 0)
+                                      : launch_quantize_asym(xh, M, K, row_idx, bits, w.ctl, w.codes, nullptr, nullptr, stream);
     } else {
         e = quantize_dispatch(h, xh, M, K, row_idx, bits, scale_mode, clip_shift_or_exp, w.ctl, w.codes, nullptr, alpha,
                               k_max, stream);
@@ -386,9 +387,10 @@ int aq_linear_w4a4(aq_handle_t h, const void* x_fp16, int M, int K, const void* 
                        row_idx, y_fp16, acc_dump, workspace, workspace_bytes_, stream);
 }
 
-int aq_gemm_w4(aq_handle_t h, const int8_t* q, int M, int K, const void* w_packed, const void* w_scales,
-               int N, int group_size, const int32_t* scale_exp, void* y_fp16, int32_t* acc_dump,
-               void* workspace, size_t workspace_bytes_, void* stream_) {
+// after_unpack: this call's own kernel ahead has set the control block up
+static int gemm_impl(aq_handle_t h, const int8_t* q, int M, int K, const void* w_packed, const void* w_scales,
+                     int N, int group_size, const int32_t* scale_exp, void* y_fp16, int32_t* acc_dump,
+                     void* workspace, size_t workspace_bytes_, void* stream_, bool after_unpack) {
     if (!h || !q || !w_packed || !w_scales || !scale_exp || !y_fp16) return AQ_ERR_INVALID_ARG;
     const int s = check_shape(M, K, N, group_size);
     if (s != AQ_OK) return s;
@@ -399,6 +401,7 @@ int aq_gemm_w4(aq_handle_t h, const int8_t* q, int M, int K, const void* w_packe
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const Workspace w = carve(workspace, M, K, N, workspace_bytes_);
     GemmArgs g;                    // the kernels clear the status word themselves
+    g.after_quantize = after_unpack;
     g.q = q; g.M = M; g.K = K; g.N = N; g.group = group_size;
     g.w_packed = static_cast<const uint8_t*>(w_packed);
     g.w_scales = static_cast<const __half*>(w_scales);
@@ -408,6 +411,12 @@ int aq_gemm_w4(aq_handle_t h, const int8_t* q, int M, int K, const void* w_packe
     g.ctl = w.ctl; g.scratch = w.scratch; g.scratch_bytes = w.scratch_bytes;
     g.split_scratch = w.split_scratch; g.split_bytes = w.split_bytes;
     return run_gemm(h, g, stream);
+}
+
+int aq_gemm_w4(aq_handle_t h, const int8_t* q, int M, int K, const void* w_packed, const void* w_scales,
+               int N, int group_size, const int32_t* scale_exp, void* y_fp16, int32_t* acc_dump,
+               void* workspace, size_t workspace_bytes_, void* stream_) {
+    return gemm_impl(h, q, M, K, w_packed, w_scales, N, group_size, scale_exp, y_fp16, acc_dump, workspace, workspace_bytes_, stream_, false);
 }
 
 size_t aq_act4_bytes(int M, int K) {
@@ -457,10 +466,9 @@ int aq_gemm_w4_act4(aq_handle_t h, const void* q4, int M, int K, const void* w_p
     if (!aligned(q4, 16) || !aligned(workspace, 256)) return AQ_ERR_ALIGNMENT;
     const Workspace w = carve(workspace, M, K, N, workspace_bytes_);
     const cudaError_t e = launch_act4_unpack(static_cast<const uint8_t*>(q4), (size_t)M * K, w.codes,
-                                             static_cast<cudaStream_t>(stream_));
+                                             static_cast<cudaStream_t>(stream_), w.ctl);
     if (e != cudaSuccess) return cuda_fail(h, e);
-    return aq_gemm_w4(h, w.codes, M, K, w_packed, w_scales, N, group_size, scale_exp, y_fp16, acc_dump, workspace,
-                      workspace_bytes_, stream_);
+    return gemm_impl(h, w.codes, M, K, w_packed, w_scales, N, group_size, scale_exp, y_fp16, acc_dump, workspace, workspace_bytes_, stream_, true);
 }
 
 int aq_token_select(aq_handle_t h, const float* scores, int M, int n_keep, int32_t* idx, void* workspace,
@@ -510,8 +518,10 @@ int aq_quantize_act_asym(aq_handle_t h, const void* x_fp16, int M, int K, int bi
         return AQ_ERR_ALIGNMENT;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     Control* ctl = static_cast<Control*>(workspace);
-    const cudaError_t e = launch_quantize_asym(static_cast<const __half*>(x_fp16), M, K, row_idx, bits, ctl, q, scale_exp_out,
-                                               zero_point_out, stream);
+    const __half* xh = static_cast<const __half*>(x_fp16);
+    const cudaError_t e =
+        quantize_small_fits(M, K) ? launch_quantize_small_asym(xh, M, K, row_idx, bits, ctl, q, scale_exp_out, zero_point_out, stream, h->weights_stable != 0)
+                                  : launch_quantize_asym(xh, M, K, row_idx, bits, ctl, q, scale_exp_out, zero_point_out, stream);
     return e == cudaSuccess ? AQ_OK : cuda_fail(h, e);
 }
 

@@ -129,7 +129,8 @@ cudaError_t launch_unpack_w4(const uint8_t* packed, int N, int K, int8_t* codes,
 // 4-bit activation codes, two per byte (code 2j in the low nibble of byte j); count = number of codes, a
 // multiple of 16, both buffers 16-byte (codes) / 8-byte (packed) aligned.
 cudaError_t launch_act4_pack(const int8_t* q, size_t count, uint8_t* out, cudaStream_t stream);
-cudaError_t launch_act4_unpack(const uint8_t* packed, size_t count, int8_t* q, cudaStream_t stream);
+// ctl: NULL, or the control block of the product that is launched next
+cudaError_t launch_act4_unpack(const uint8_t* packed, size_t count, int8_t* q, cudaStream_t stream, Control* ctl = nullptr);
 
 // Scale (unless given) and codes; fills the control block. alpha / k_max: TRIP factors, see below.
 cudaError_t launch_quantize(const __half* x, int M, int K, const int32_t* row_idx, int bits,
@@ -154,6 +155,9 @@ cudaError_t launch_trip_calibrate(const __half* x, int M, int K, const int32_t* 
 // codes, stored as q - 2^(b-1) in int8; fills the control block.
 cudaError_t launch_quantize_asym(const __half* x, int M, int K, const int32_t* row_idx, int bits, Control* ctl,
                                  int8_t* q, int32_t* scale_exp_out, int32_t* zero_point_out, cudaStream_t stream);
+// The same for activations that launch_quantize_small takes.
+cudaError_t launch_quantize_small_asym(const __half* x, int M, int K, const int32_t* row_idx, int bits, Control* ctl, int8_t* q, int32_t* scale_exp_out,
+                                       int32_t* zero_point_out, cudaStream_t stream, bool early_dependents);
 // r[n] = sum_g s_w[n,g] * sum_{k in g} c[n,k], from the packed weights (float [N]).
 cudaError_t launch_weight_offsets(const uint8_t* packed, const __half* scales, int N, int K, int group, float* r,
                                   cudaStream_t stream);

@@ -137,23 +137,41 @@ act4_pack_kernel(const uint4* __restrict__ q, size_t n16, uint2* __restrict__ ou
     out[i] = make_uint2(__byte_perm(r[0], r[1], 0x6420), __byte_perm(r[2], r[3], 0x6420));
 }
 
+// ctl (of a product call whose product kernel is the next launch): set up here, so that that kernel may be set up, and fetch its
+// weights, while this one runs; it may once everything ahead of this kernel has completed. Behind a plain launch, and as one, the pair
+// left 4 us between the kernel ahead and the product besides its own 4.
+constexpr int kUnpackUnits = 4;                     // of 16 codes, a thread
+
 __global__ void __launch_bounds__(256)
-act4_unpack_kernel(const uint2* __restrict__ p, size_t n16, uint4* __restrict__ q) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n16) return;
-    const uint2 b = p[i];
-    const uint32_t w[2] = {b.x, b.y};
-    uint32_t o[4];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        uint32_t lo = w[k] & 0x0F0F0F0Fu, hi = (w[k] >> 4) & 0x0F0F0F0Fu;
-        // sign extension inside each byte: bit 3 set -> bits 4-7 set (8 * 30 = 0xF0, no carry between bytes)
-        lo |= (lo & 0x08080808u) * 0x1Eu;
-        hi |= (hi & 0x08080808u) * 0x1Eu;
-        o[2 * k] = __byte_perm(lo, hi, 0x5140);      // codes 0..3 of this word's 8: lo0 hi0 lo1 hi1
-        o[2 * k + 1] = __byte_perm(lo, hi, 0x7362);  // codes 4..7: lo2 hi2 lo3 hi3
+act4_unpack_kernel(const uint2* __restrict__ p, size_t n16, uint4* __restrict__ q, Control* __restrict__ ctl) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (ctl && blockIdx.x == 0) {
+        if (threadIdx.x == 0) ctl->status = 0;
+        if (threadIdx.x < Control::kSplitWords) ctl->split_flags[threadIdx.x] = 0;
     }
-    q[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    const size_t first = (size_t)blockIdx.x * (256 * kUnpackUnits) + threadIdx.x;
+    uint2 b[kUnpackUnits];
+#pragma unroll
+    for (int u = 0; u < kUnpackUnits; ++u)
+        if (first + u * 256 < n16) b[u] = __ldg(p + first + u * 256);
+#pragma unroll
+    for (int u = 0; u < kUnpackUnits; ++u) {
+        const size_t i = first + u * 256;
+        if (i >= n16) break;
+        const uint32_t w[2] = {b[u].x, b[u].y};
+        uint32_t o[4];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            uint32_t lo = w[k] & 0x0F0F0F0Fu, hi = (w[k] >> 4) & 0x0F0F0F0Fu;
+            // sign extension inside each byte: bit 3 set -> bits 4-7 set (8 * 30 = 0xF0, no carry between bytes)
+            lo |= (lo & 0x08080808u) * 0x1Eu;
+            hi |= (hi & 0x08080808u) * 0x1Eu;
+            o[2 * k] = __byte_perm(lo, hi, 0x5140);      // codes 0..3 of this word's 8: lo0 hi0 lo1 hi1
+            o[2 * k + 1] = __byte_perm(lo, hi, 0x7362);  // codes 4..7: lo2 hi2 lo3 hi3
+        }
+        q[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
 }
 
 }  // namespace
@@ -166,12 +184,12 @@ cudaError_t launch_act4_pack(const int8_t* q, size_t count, uint8_t* out, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_act4_unpack(const uint8_t* packed, size_t count, int8_t* q, cudaStream_t stream) {
+cudaError_t launch_act4_unpack(const uint8_t* packed, size_t count, int8_t* q, cudaStream_t stream, Control* ctl) {
     const size_t n16 = count / 16;
     if (n16 == 0) return cudaSuccess;
-    act4_unpack_kernel<<<(unsigned int)((n16 + 255) / 256), 256, 0, stream>>>(reinterpret_cast<const uint2*>(packed), n16,
-                                                                            reinterpret_cast<uint4*>(q));
-    return cudaGetLastError();
+    const size_t per_cta = 256 * kUnpackUnits;
+    return launch_overlapped(act4_unpack_kernel, dim3((unsigned int)((n16 + per_cta - 1) / per_cta)), 256, stream, reinterpret_cast<const uint2*>(packed),
+                             n16, reinterpret_cast<uint4*>(q), ctl);
 }
 
 cudaError_t launch_weight_offsets(const uint8_t* packed, const __half* scales, int N, int K, int group, float* r,

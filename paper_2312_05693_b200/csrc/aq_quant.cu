@@ -25,18 +25,32 @@ __device__ __forceinline__ uint4 quantize16_fp32(const uint4& d0, const uint4& d
 // One cluster of 8 CTAs x 512 threads holds the whole activation in registers (up to 8 vectors of
 // 8 halves per thread), so x is read once; the CTAs' maxima are exchanged through distributed
 // shared memory. The kernel also initialises the control block, so no memset precedes it.
+// Latency is what it takes: one round trip for x, one for the exchange. us, graph replay, with two meetings, and a division per vector for
+// its place, and without: 2 x 768 1.76 / 1.50, 48 x 4096 3.46 / 2.28; layers of 48 rows 4096 x 4096 in groups 10.5 / 9.5. With a zero
+// point, which took the two kernels below before, 24 x 2048 x 2048 9.0 / 6.9.
 constexpr int kSmallCtas = 8, kSmallThreads = 512, kSmallVecs = 8;
 constexpr size_t kSmallMaxElems = (size_t)kSmallCtas * kSmallThreads * kSmallVecs * 8;   // 262144
 
+// ASYM: with a zero point (Eq. 2, Eq. 5-7): least and greatest value, no given exponent, no factors.
+template <bool ASYM>
 __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads)
 quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const int32_t* __restrict__ row_idx,
                       int bits, int scale_mode, int clip_shift_or_exp, Control* __restrict__ ctl,
                       uint2* __restrict__ q, int32_t* __restrict__ scale_exp_out, const uint2* __restrict__ alpha,
-                      int k_max, int early_dependents) {
-    cg::cluster_group cluster = cg::this_cluster();
-    __shared__ unsigned int warp_max[kSmallThreads / 32];
-    __shared__ unsigned int slots[kSmallCtas];
+                      int k_max, int early_dependents, int32_t* __restrict__ zero_point_out) {
+    constexpr int kWarps = kSmallThreads / 32;
+    __shared__ unsigned int seen[kSmallCtas * kWarps];      // what every warp of the cluster saw
+    __shared__ alignas(8) uint64_t met;                     // all of them are there
+    const int rank = (int)cg::this_cluster().block_rank(), warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    const uint32_t met_a = (uint32_t)__cvta_generic_to_shared(&met);
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(met_a) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(met_a), "r"((uint32_t)sizeof(seen)) : "memory");
+    }
+    __syncwarp();
     cluster_started_arrive();
+    __syncthreads();
     // The launch allows programmatic stream serialization, so this grid may be set up while the kernel
     // ahead of it drains; nothing is read or written before that kernel has completed. Only then is the
     // dependent launch allowed: a product kernel launched the same way behind this one may be set up on
@@ -47,10 +61,8 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
     if (early_dependents) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!early_dependents) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int rank = (int)cluster.block_rank();
     const int total = M * vec_per_row;
     uint4 buf[kSmallVecs];
-    __half2 m2 = __float2half2_rn(0.0f);
     // all loads first, then the maximum: the loads of a thread are in flight together (one memory round
     // trip for the whole activation instead of one per vector)
 #pragma unroll
@@ -58,52 +70,80 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
         const int v = (i * kSmallCtas + rank) * kSmallThreads + (int)threadIdx.x;
         buf[i] = make_uint4(0, 0, 0, 0);
         if (v < total) {
-            const int m = v / vec_per_row, c = v % vec_per_row;
-            buf[i] = __ldg(x + (size_t)(row_idx ? row_idx[m] : m) * vec_per_row + c);
+            if (row_idx) {
+                const int m = v / vec_per_row, c = v % vec_per_row;
+                buf[i] = __ldg(x + (size_t)row_idx[m] * vec_per_row + c);
+            } else {
+                buf[i] = __ldg(x + v);
+            }
         }
     }
+    __half2 hi2 = __float2half2_rn(0.0f), lo2 = hi2;
 #pragma unroll
     for (int i = 0; i < kSmallVecs; ++i) {
         const __half2* h = reinterpret_cast<const __half2*>(&buf[i]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) m2 = __hmax2(m2, __habs2(h[k]));   // NaN operands are dropped; absent vectors are zero
+        for (int k = 0; k < 4; ++k) {                                  // NaN operands are dropped; absent vectors are zero
+            if (ASYM) {
+                lo2 = __hmin2(lo2, h[k]);
+                hi2 = __hmax2(hi2, h[k]);
+            } else {
+                hi2 = __hmax2(hi2, __habs2(h[k]));
+            }
+        }
     }
-    unsigned int bits_max = max((unsigned int)__half_as_ushort(__low2half(m2)),
-                                (unsigned int)__half_as_ushort(__high2half(m2)));
-    if (bits_max > 0x7C00u) bits_max = 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) bits_max = max(bits_max, __shfl_xor_sync(0xFFFFFFFFu, bits_max, o));
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = bits_max;
+    lo2 = __habs2(lo2);
+    const unsigned int bmax = max((unsigned int)__half_as_ushort(__low2half(hi2)), (unsigned int)__half_as_ushort(__high2half(hi2)));
+    const unsigned int bmin = max((unsigned int)__half_as_ushort(__low2half(lo2)), (unsigned int)__half_as_ushort(__high2half(lo2)));
+    unsigned int all = __reduce_max_sync(0xFFFFFFFFu, bmax) | (ASYM ? __reduce_max_sync(0xFFFFFFFFu, bmin) << 16 : 0u);
     cluster_started_wait();
-    __syncthreads();
-    if (threadIdx.x < kSmallCtas) {
-        unsigned int b = 0;
-        for (int w = 0; w < kSmallThreads / 32; ++w) b = max(b, warp_max[w]);
-        *cluster.map_shared_rank(&slots[rank], (int)threadIdx.x) = b;   // my maximum into every CTA's table
+    // A warp's word goes to every CTA by an asynchronous remote store that counts on the receiver's barrier (a meeting inside each CTA and
+    // one of the cluster before: 48 x 4096 in a layer call 0.3 us more). A CTA waits for all words that are sent to it, and
+    // every warp sends its word whatever happens, so nobody writes to a CTA that has left.
+    if (lane < kSmallCtas) {
+        uint32_t slot, bar;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(slot) : "r"((uint32_t)__cvta_generic_to_shared(&seen[rank * kWarps + warp])), "r"(lane));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(met_a), "r"(lane));
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(slot), "r"(all), "r"(bar) : "memory");
     }
-    cluster.sync();
-    unsigned int all = 0;
+    __syncwarp();
+    bool came = false;
+    for (const long long t0 = clock64(); !came && (unsigned long long)(clock64() - t0) < 2 * kWaitCycles;) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(met_a) : "memory");
+        came = ok != 0;
+    }
+    __syncwarp();
+    all = 0;
 #pragma unroll
-    for (int r = 0; r < kSmallCtas; ++r) all = max(all, slots[r]);
-    const int e = scale_mode == AQ_SCALE_DYNAMIC ? layer_exponent_from_bits(all, bits) - clip_shift_or_exp - k_max
-                                                 : clip_shift_or_exp;
+    for (int i = 0; i < kSmallCtas * kWarps / 32; ++i) all = __vmaxu2(all, seen[i * 32 + lane]);
+    all = __reduce_max_sync(0xFFFFFFFFu, all & 0xFFFFu) | (ASYM ? __reduce_max_sync(0xFFFFFFFFu, all >> 16) << 16 : 0u);
+    int e, zp = 0;
+    if constexpr (ASYM) zero_point_scale(all & 0xFFFFu, all >> 16, bits, e, zp);
+    else e = scale_mode == AQ_SCALE_DYNAMIC ? layer_exponent_from_bits(all, bits) - clip_shift_or_exp - k_max : clip_shift_or_exp;
     if (rank == 0 && threadIdx.x == 0) {
-        ctl->absmax_bits = all;
+        ctl->absmax_bits = ASYM ? 0u : all;
         ctl->scale_exp = e;
-        ctl->status = 0;
+        ctl->status = came ? 0u : 13u;
         if (scale_exp_out) *scale_exp_out = e;
+        if constexpr (ASYM) {
+            ctl->zero_point = zp;
+            if (zero_point_out) *zero_point_out = zp;
+        }
     }
     if (rank == 0 && threadIdx.x < Control::kSplitWords) ctl->split_flags[threadIdx.x] = 0;    // the product kernel's shared-tile bits
     const float lo = -(float)(1 << (bits - 1)), hi = (float)((1 << (bits - 1)) - 1);
     if (alpha == nullptr && e >= -14 && e <= 14) {           // 2^-e is a normal half: codes in half2 arithmetic
         const __half2 inv2 = __float2half2_rn(__int_as_float((127 - e) << 23));
-        const __half2 lo2 = __float2half2_rn(lo), hi2 = __float2half2_rn(hi);
+        const __half2 clo2 = __float2half2_rn(ASYM ? -(float)zp : lo), chi2 = __float2half2_rn(ASYM ? (float)((1 << bits) - 1 - zp) : hi);
+        [[maybe_unused]] const __half2 shift2 = __float2half2_rn((float)(zp - (1 << (bits - 1))));
 #pragma unroll
         for (int i = 0; i < kSmallVecs; ++i) {
             const int v = (i * kSmallCtas + rank) * kSmallThreads + (int)threadIdx.x;
             if (v < total) {
                 uint2 w;
-                quantize8_half2(buf[i], inv2, lo2, hi2, w.x, w.y);
+                if (ASYM) quantize8_half2_asym(buf[i], inv2, clo2, chi2, shift2, w.x, w.y);
+                else quantize8_half2(buf[i], inv2, clo2, chi2, w.x, w.y);
                 q[v] = w;
             }
         }
@@ -115,7 +155,7 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
         if (v < total) {
             uint2 al;
             if (alpha) al = __ldg(alpha + v % vec_per_row);
-            q[v] = quantize8_fp32(buf[i], e, lo, hi, alpha ? &al : nullptr);
+            q[v] = ASYM ? quantize8_fp32_asym(buf[i], __int_as_float((127 - e) << 23), zp, bits) : quantize8_fp32(buf[i], e, lo, hi, alpha ? &al : nullptr);
         }
     }
 }
@@ -132,6 +172,10 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
 // 2048 x 11008 21.9 -> 18.0 us, 1024 x 5120 10.1 -> 6.6 us, 333 x 5120 8.3 -> 5.5 us.
 constexpr int kRangeThreads = 512;
 constexpr int kRangeInFlight = 8;
+constexpr size_t kRangeFewVecs = (size_t)Control::kRangeWords * kRangeThreads * kRangeInFlight * 2;      // 237568 vectors: two turns of all loads in flight
+// (Up to there 29 CTAs without a meeting beat clusters on all SMs: quantize calls, graph replay, 100 x 4096 4.12 / 3.69 us, 116 x 8192 4.71 / 3.94,
+// 333 x 5120 5.54 / 4.50, 230 x 8192 5.64 / 4.70; with four turns 509 x 4096 5.66 / 4.95, but 400 x 8192 5.85 / 6.13. Layer calls gain less,
+// 333 x 5120 x 5120 17.9 / 17.7, and 128 x 13824 x 5120 loses: 23.7 / 24.1.)
 
 // Place of element number v (per_row elements a row) in the gathered rows, carried along in steps: one division at the
 // start instead of one per element (a 64-bit one each cost 8 us on 2458 gathered rows of 7168).
@@ -157,11 +201,13 @@ struct RowWalk {
     }
 };
 
-template <bool ASYM>
-__global__ void __cluster_dims__(kRangeCtas, 1, 1) __launch_bounds__(kRangeThreads)
+// CLUSTERS: launched in clusters of kRangeCtas; otherwise every CTA leaves a word of its own (arrays small enough for as many CTAs as
+// there are words).
+template <bool ASYM, bool CLUSTERS>
+__global__ void __launch_bounds__(kRangeThreads)
 range_kernel(const uint4* __restrict__ x, size_t vecs /* of 8 halves */, int vec_per_row, const int32_t* __restrict__ row_idx,
              size_t vecs_per_cta, Control* __restrict__ ctl) {
-    cluster_started_arrive();
+    if constexpr (CLUSTERS) cluster_started_arrive();
     asm volatile("griddepcontrol.wait;" ::: "memory");      // the kernel ahead may have written X
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t v0 = (size_t)blockIdx.x * vecs_per_cta;
@@ -197,6 +243,18 @@ range_kernel(const uint4* __restrict__ x, size_t vecs /* of 8 halves */, int vec
     if (ASYM) {
         const __half2 n2 = __habs2(lo2);
         bmin = max((unsigned int)__half_as_ushort(__low2half(n2)), (unsigned int)__half_as_ushort(__high2half(n2)));
+    }
+    if constexpr (!CLUSTERS) {
+        __shared__ unsigned int warp_seen[kRangeThreads / 32];
+        const unsigned int seen = __reduce_max_sync(0xFFFFFFFFu, bmax) | (ASYM ? __reduce_max_sync(0xFFFFFFFFu, bmin) << 16 : 0u);
+        if ((threadIdx.x & 31) == 0) warp_seen[threadIdx.x >> 5] = seen;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const unsigned int w = threadIdx.x < kRangeThreads / 32 ? warp_seen[threadIdx.x] : 0u;
+            const unsigned int hi = __reduce_max_sync(0xFFFFFFFFu, w & 0xFFFFu), lo = __reduce_max_sync(0xFFFFFFFFu, w >> 16);
+            if (threadIdx.x == 0) ctl->range[blockIdx.x] = hi | (lo << 16);
+        }
+        return;
     }
     __shared__ unsigned int peers[kRangeCtas];
     cluster_started_wait();
@@ -523,6 +581,14 @@ namespace {
 template <bool ASYM>
 cudaError_t launch_range(const __half* x, int M, int K, const int32_t* row_idx, Control* ctl, cudaStream_t stream, int& words) {
     const size_t vecs = (size_t)M * (K / 8);
+    if (vecs <= kRangeFewVecs) {
+        // no meeting of clusters: as many CTAs as the control block has words for, fewer when one would have less than two vectors a thread
+        size_t ctas = (vecs + kRangeThreads * 2 - 1) / (kRangeThreads * 2);
+        if (ctas > Control::kRangeWords) ctas = Control::kRangeWords;
+        words = (int)ctas;
+        return launch_overlapped(range_kernel<ASYM, false>, dim3((unsigned int)ctas), kRangeThreads, stream, reinterpret_cast<const uint4*>(x), vecs, K / 8, row_idx,
+                                 (vecs + ctas - 1) / ctas, ctl);
+    }
     // as many clusters as the control block has words for (232 CTAs of 512 threads, all resident at once), fewer when
     // a CTA would have less than two vectors per thread
     const size_t per_cluster = (size_t)kRangeCtas * kRangeThreads * 2;
@@ -530,8 +596,20 @@ cudaError_t launch_range(const __half* x, int M, int K, const int32_t* row_idx, 
     if (clusters > Control::kRangeWords) clusters = Control::kRangeWords;
     words = (int)clusters;
     const size_t ctas = clusters * kRangeCtas;
-    return launch_overlapped(range_kernel<ASYM>, dim3((unsigned int)ctas), kRangeThreads, stream, reinterpret_cast<const uint4*>(x), vecs, K / 8, row_idx,
-                             (vecs + ctas - 1) / ctas, ctl);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned int)ctas);
+    cfg.blockDim = dim3(kRangeThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kRangeCtas;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, range_kernel<ASYM, true>, reinterpret_cast<const uint4*>(x), vecs, K / 8, row_idx, (vecs + ctas - 1) / ctas, ctl);
 }
 
 size_t quantize_grid(int M, int K) {
@@ -582,19 +660,16 @@ bool quantize_small_fits(int M, int K) { return (size_t)M * (size_t)K <= kSmallM
 cudaError_t launch_quantize_small(const __half* x, int M, int K, const int32_t* row_idx, int bits, int scale_mode,
                                   int clip_shift_or_exp, Control* ctl, int8_t* q, int32_t* scale_exp_out,
                                   cudaStream_t stream, const uint8_t* alpha, int k_max, bool early_dependents) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kSmallCtas);
-    cfg.blockDim = dim3(kSmallThreads);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;       // the kernel touches no memory before the kernel ahead of it has completed
-    return cudaLaunchKernelEx(&cfg, quantize_small_kernel, reinterpret_cast<const uint4*>(x), M, K / 8, row_idx, bits,
-                              scale_mode, clip_shift_or_exp, ctl, reinterpret_cast<uint2*>(q), scale_exp_out,
-                              reinterpret_cast<const uint2*>(alpha), k_max, early_dependents ? 1 : 0);
+    // the kernel touches no memory before the kernel ahead of it has completed
+    return launch_overlapped(quantize_small_kernel<false>, dim3(kSmallCtas), kSmallThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 8, row_idx, bits,
+                             scale_mode, clip_shift_or_exp, ctl, reinterpret_cast<uint2*>(q), scale_exp_out, reinterpret_cast<const uint2*>(alpha), k_max,
+                             early_dependents ? 1 : 0, nullptr);
+}
+
+cudaError_t launch_quantize_small_asym(const __half* x, int M, int K, const int32_t* row_idx, int bits, Control* ctl, int8_t* q, int32_t* scale_exp_out,
+                                       int32_t* zero_point_out, cudaStream_t stream, bool early_dependents) {
+    return launch_overlapped(quantize_small_kernel<true>, dim3(kSmallCtas), kSmallThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 8, row_idx, bits,
+                             AQ_SCALE_DYNAMIC, 0, ctl, reinterpret_cast<uint2*>(q), scale_exp_out, nullptr, 0, early_dependents ? 1 : 0, zero_point_out);
 }
 
 cudaError_t launch_token_select(const float* scores, int M, int n_keep, int32_t* idx, void* scratch,

@@ -44,6 +44,19 @@ def test_the_headers_map_no_peer_themselves():
     assert sorted(users) == ["log2_absmax_kernel", "range_kernel"]
 
 
+def test_asynchronous_remote_stores_come_behind_it_too():
+    """Kernels that send to a peer by st.async map its memory with mapa: behind a wait for the cluster in the same function, and
+    (the stores at the end of the few-row kernel) in the kernel's own text before them."""
+    found = 0
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        for at in (m.start() for m in re.finditer(r'"mapa\.', code)):
+            body = code[max(code.rfind("\n}\n", 0, at), 0):at]
+            assert WAIT.search(body), path
+            found += 1
+    assert found >= 6
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("M,K", [(1, 32), (1, 64), (3, 32), (3, 96), (16, 4096), (17, 16384)])
 def test_every_share_of_the_cluster_reaches_the_scale(M, K):
