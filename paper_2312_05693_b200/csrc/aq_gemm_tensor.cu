@@ -978,13 +978,10 @@ int tile_clusters(const DeviceInfo& dev, int split) {
 // rounds of tiles over the SMs, a last round whose tiles two CTAs share, or all tiles at once in clusters, where the k blocks
 // saved outweigh the exchange (layers of 48 rows, K x N = 4096 x 4096 14.3 -> 10.8 us, 11008 x 4096 21.9 -> 15.7 us, 5120 x 5120
 // 17.6 -> 13.3 us; of 128 rows, 11008 x 4096 30.9 -> 22.5 us).
-// The times were fitted to layer calls with every schedule forced: 48 to 3000 rows, 768 <= K <= 13824, 768 <= N <= 22016 without
-// clusters (2332 calls), 24 to 512 rows, 512 <= K <= 11008, 256 <= N <= 4096 with them (4492), before the epilogue waited at named
-// barriers (a block of a 192-token tile is priced at 0.499 us and takes some 0.45). They still rank: with every schedule forced on the
-// kernel as it is, of 300 layers without clusters, 65 to 3000 rows, the schedule taken is the best but for one (1.6 % off). Of
-// 300 with clusters, 24 to 512 rows, it is within 3 % of the best in 70 %, within 8 % in 89 %, 22 % off at the worst: on short k
-// ranges (K near 1024, up to 350 rows) the exchange is priced too high, 102 rows of 1024 x 297 take 11.4 us on whole tiles and 9.3 in
-// clusters of four.
+// The times were fitted to layer calls with every schedule forced, 131 layers of 65 to 3000 rows, 768 <= K <= 28672, 768 <= N <= 28672 (a
+// layer's schedules against one another, in graph replay, those within 60 % of its best). The schedule taken is then 0.3 % slower than the
+// best in the mean and 5 % at the worst; with the prices of before the last changes to these kernels it was 1.1 and 22 %
+// (631 rows, 20480 x 6400: 159 us on 192-token tiles, 131 on 128). Up to 64 rows 0.8 and 9 %, refitted or not.
 struct GroupedPlan {
     int bm, split;
 };
@@ -995,17 +992,25 @@ struct GroupedTimes {                // microseconds
 };
 constexpr GroupedTimes grouped_times(int bm) {
     return bm == 64 ? GroupedTimes{4.56f, 0.91f, 0.266f, 6.44f, 0.317f, 1.9f, 0.06f}
+         : bm == 128 ? GroupedTimes{6.45f, 0.82f, 0.337f, 0.0f, 0.700f, 2.56f, 0.23f}
+                     : GroupedTimes{6.68f, 1.28f, 0.416f, 4.99f, 0.678f, 3.17f, 0.19f};
+}
+// What the size of the workspace, which is part of the interface, goes by: the prices that it was first computed with.
+constexpr GroupedTimes grouped_size_times(int bm) {
+    return bm == 64 ? GroupedTimes{4.56f, 0.91f, 0.266f, 6.44f, 0.317f, 1.9f, 0.06f}
          : bm == 128 ? GroupedTimes{6.45f, 0.96f, 0.440f, 8.05f, 0.423f, 2.9f, 0.14f}
                      : GroupedTimes{6.63f, 1.47f, 0.499f, 9.23f, 0.523f, 3.85f, 0.41f};
 }
-GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_share, bool clusters) {
+size_t shared_scratch_bytes(long rem, int bm) { return (size_t)rem * 2 * bm * kTileN * sizeof(float); }
+// scratch_bytes: what there is for shared tiles.
+GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, size_t scratch_bytes, bool clusters, GroupedTimes (*times)(int) = grouped_times) {
     const int kbs = K / kTileK, n_tiles_n = round_up(N, kTileN) / kTileN, sms = dev.sm_count;
     GroupedPlan best = {64, 1};
     float best_time = 3.0e38f;
     auto consider = [&](int bm) {
-        const GroupedTimes t = grouped_times(bm);
-        const long tiles = (long)((M + bm - 1) / bm) * n_tiles_n;
-        const bool halves = may_share && shared_tiles(tiles, sms, kbs, bm) > 0;
+        const GroupedTimes t = times(bm);
+        const long tiles = (long)((M + bm - 1) / bm) * n_tiles_n, rem = shared_tiles(tiles, sms, kbs, bm);
+        const bool halves = rem > 0 && shared_scratch_bytes(rem, bm) <= scratch_bytes;
         const long rounds = halves ? tiles / sms : (tiles + sms - 1) / sms;
         const float plain = t.call + (float)rounds * (t.round + (float)kbs * t.block) +
                             (halves ? t.shared + (float)((kbs + 1) / 2) * t.shared_block : 0.0f);
@@ -1027,20 +1032,27 @@ GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, bool may_sh
     return best;
 }
 
-// One scale per channel, tiles of one channel block: 64 tokens up to 64 rows, 128 up to 128 rows, or more while the tiles
-// fill one round; in clusters where the k blocks saved outweigh the exchange.
+// One scale per channel, tiles of one channel block: 64 tokens up to 64 rows, else 128 or (beyond 128 rows) 256 in rounds over the SMs, or
+// all 64- or 128-token tiles at once in clusters, where the k blocks saved outweigh the exchange. Prices in nanoseconds, fitted together
+// with those of the tiles of two channel blocks (wide_plan) as the per-group ones were, 174 layers of 17 to 3000 rows: beyond
+// 64 rows the schedule taken is 0.2 % slower than the best in the mean, 7 % at the worst, where it was 2.8 and 33 % (186 rows of 1312 x 1312
+// 10.2 us in clusters, 8.3 on whole tiles; 705 rows of 3648 x 9056 34.8 us on 256 tokens, 30.1 on 128).
 struct ChannelPlan {
     int bm, split;
     long cost;
 };
-constexpr int kNarrow64 = 420, kNarrow128 = 600, kExchangeCycles = 4500;     // cycles per k block; of the exchange
 ChannelPlan channel_plan(int M, int K, int N, const DeviceInfo& dev) {
-    const int KB = k_blocks(K), sms = dev.sm_count, bm = M <= 64 ? 64 : 128, block = M <= 64 ? kNarrow64 : kNarrow128;
-    const long tiles = (long)((M + bm - 1) / bm) * (round_up(N, kTileN) / kTileN);
-    if (M > 128 && tiles > sms) return {256, 1, 0x7fffffffL};
-    ChannelPlan best = {bm, 1, (tiles + sms - 1) / sms * KB * block};
+    const bool small = M <= 64;
+    const int KB = k_blocks(K), sms = dev.sm_count, bm = small ? 64 : 128;
+    const int round = small ? 0 : 1000, block = small ? 117 : 179, exchange = small ? 1380 : 2723, exchange_cta = small ? 28 : 92;
+    const long blocks_n = round_up(N, kTileN) / kTileN, tiles = (M + bm - 1) / bm * blocks_n;
+    ChannelPlan best = {bm, 1, (tiles + sms - 1) / sms * (round + (long)KB * block)};
+    if (M > 128) {
+        const long c = ((M + 255) / 256 * blocks_n + sms - 1) / sms * (1522 + (long)KB * 354);
+        if (c < best.cost) best = {256, 1, c};
+    }
     for (int s = 2; s <= 8 && s <= KB && s * tiles <= sms; ++s) {
-        const long c = (long)((KB + s - 1) / s) * block + kExchangeCycles;
+        const long c = round + (long)((KB + s - 1) / s) * block + exchange + (long)(s - 2) * exchange_cta;
         if (c >= best.cost) continue;
         if ((bm == 64 ? tile_clusters<64, false>(dev, s) : tile_clusters<128, false>(dev, s)) >= tiles) best = {bm, s, c};
     }
@@ -1178,7 +1190,7 @@ cudaError_t launch_bm(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t str
         const int sms = dev.sm_count;
         const int n_tiles = ((a.M + BM - 1) / BM) * (round_up(a.N, kTileN) / kTileN);
         const int rem = shared_tiles(n_tiles, sms, a.K / kTileK, BM), whole = n_tiles - rem;
-        const size_t need = (size_t)rem * 2 * BM * kTileN * sizeof(float);
+        const size_t need = shared_scratch_bytes(rem, BM);
         if (rem > 0 && a.split_scratch && a.split_bytes >= need && (reinterpret_cast<uintptr_t>(a.split_scratch) & 15u) == 0) {
             if (!a.after_quantize) {
                 const cudaError_t e = cudaMemsetAsync(a.ctl->split_flags, 0, sizeof(a.ctl->split_flags), stream);
@@ -1201,9 +1213,9 @@ size_t tensor_split_scratch_bytes(int M, int K, int N, int group, int sm_count) 
     if (!group) return 0;
     DeviceInfo dev = {};
     dev.sm_count = sm_count;
-    const int bm = grouped_plan(M, K, N, dev, true, false).bm;     // the most that the plan with clusters uses
+    const int bm = grouped_plan(M, K, N, dev, ~(size_t)0, false, grouped_size_times).bm;
     const int n_tiles = ((M + bm - 1) / bm) * (round_up(N, kTileN) / kTileN);
-    return (size_t)shared_tiles(n_tiles, sm_count, K / kTileK, bm) * 2 * bm * kTileN * sizeof(float);
+    return shared_scratch_bytes(shared_tiles(n_tiles, sm_count, K / kTileK, bm), bm);
 }
 
 cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const DeviceInfo& dev, cudaStream_t stream) {
@@ -1217,7 +1229,8 @@ cudaError_t launch_int8_probe(int iters, int a_from_tmem, Control* ctl, const De
 cudaError_t launch_gemm_tensor(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
     if (a.group) {
         // the zero-point variant has no shared-tile launch
-        const GroupedPlan g = grouped_plan(a.M, a.K, a.N, dev, !a.chan_offset, true);
+        const bool may_share = !a.chan_offset && a.split_scratch && (reinterpret_cast<uintptr_t>(a.split_scratch) & 15u) == 0;
+        const GroupedPlan g = grouped_plan(a.M, a.K, a.N, dev, may_share ? a.split_bytes : 0, true);
         switch (g.bm) {
             case 64: return launch_bm<64, true>(a, dev, stream, g.split);
             case 192: return launch_bm<192, true>(a, dev, stream, g.split);

@@ -33,7 +33,6 @@ constexpr int kWRegsControl = 40, kWRegsUnpack = 48, kWRegsEpi = 168;     // of 
 static_assert(128 * kWRegsControl + 256 * kWRegsUnpack + 256 * kWRegsEpi <= kWThreads * 96,
               "register plan exceeds the launch allocation");
 constexpr int kWStageRows = 32;           // tokens per TMA store of an epilogue warp
-constexpr int kExchangeBlocks = 16;       // CLUSTER: what the meetings and the exchange cost, in k blocks (about 6 us)
 constexpr int kWRuns = 8;                 // CLUSTER: token runs of a tile
 template <int BM>
 struct WCfg {
@@ -579,16 +578,12 @@ int wide_clusters(const DeviceInfo& dev, int split) {
     return k - 1;
 }
 
-// How a shape is run, and what it costs in cycles: rounds of tiles over the SMs x k blocks x the time of a k block, which
-// the L2 -> SM path sets (about 36 bytes per clock and SM measured in this kernel: 32 KB per k block on 128-token tiles,
-// 40 KB on 192-token tiles) unless the tensor pipe's 512 / 768 cycles are longer. 128-token tiles that are few enough
-// for all of them to run at once in clusters may do so: fewer k blocks in a row, at the 730 cycles of an SM that does
-// not share the path with all others, and the exchange. 333 rows, N = 5120 (60 tiles, clusters of two): K = 13824
-// 49.2 -> 35.3 us, K = 5120 23.2 -> 22.7 us; 48 rows: 45.3 -> 22.8 us, 22.5 -> 18.6 us. (Only the last, partial round in
-// clusters behind whole rounds: measured slower, K = 13824, N = 5120 at 1024 rows, 148 + 12 tiles, 68 us against 57.6
-// on 192-token tiles.) All these cycles and times are from before the issuing threads were elected. Since then a block of a
-// 128-token tile takes about 780 cycles (K = 5120, N = 13824 at 1024 rows, three rounds, 47.4 us), and K = 13824, N = 5120 at
-// 333 rows 31.1 us in clusters where the rule says 26: whole tiles are priced some 40 % too high against clusters.
+// How a shape is run, and what it costs in nanoseconds (fitted with the prices of channel_plan, see there): rounds of tiles over the SMs x k
+// blocks x the time of a k block, which the L2 -> SM path sets (32 KB per k block on 128-token tiles, 40 KB on 192-token tiles)
+// unless the tensor pipe's 512 / 768 cycles are longer. 128-token tiles that are few enough for all of them to run at once in
+// clusters may do so: fewer k blocks in a row for an exchange. 333 rows, N = 5120 (60 tiles, clusters of two): K = 13824 49.2 -> 35.3 us.
+// (Only the last, partial round in clusters behind whole rounds: measured slower, K = 13824, N = 5120 at 1024 rows, 148 + 12 tiles,
+// 68 us against 57.6 on 192-token tiles.)
 struct WidePlan {
     int bm, split;                   // token tile; CTAs that share a tile
     long cost;
@@ -596,12 +591,13 @@ struct WidePlan {
 WidePlan wide_plan(const GemmArgs& a, const DeviceInfo& dev) {
     const int pairs = round_up(a.N, kTileN) / (2 * kTileN), KB = k_blocks(a.K), sms = dev.sm_count;
     const int tiles192 = (a.M + 191) / 192 * pairs, tiles128 = (a.M + 127) / 128 * pairs;
-    WidePlan best = {192, 1, (long)((tiles192 + sms - 1) / sms) * KB * 1138};
-    const long cost128 = (long)((tiles128 + sms - 1) / sms) * KB * 910;
+    constexpr int kCall = 106, kRound = 2750, kBlock128 = 231, kBlock192 = 381, kExchange = 7598, kExchangeCta = 62;
+    WidePlan best = {192, 1, kCall + (long)((tiles192 + sms - 1) / sms) * (kRound + (long)KB * kBlock192)};
+    const long cost128 = kCall + (long)((tiles128 + sms - 1) / sms) * (kRound + (long)KB * kBlock128);
     if (cost128 <= best.cost) best = {128, 1, cost128};
     for (int s = 2; s <= 8 && s <= KB && s * tiles128 <= sms; ++s) {
         if (wide_clusters(dev, s) < tiles128) continue;
-        const long c = (long)((KB + s - 1) / s + kExchangeBlocks) * 730;
+        const long c = kCall + (long)((KB + s - 1) / s) * kBlock128 + kExchange + (long)(s - 2) * kExchangeCta;
         if (c < best.cost) best = {128, s, c};
     }
     return best;
@@ -617,7 +613,7 @@ cudaError_t launch_wide_v(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
 }  // namespace
 
 // Whether the pair tiles are the better choice: where their schedule is no longer than `other`, that of the tiles of one
-// channel block (in cycles).
+// channel block (channel_plan).
 bool gemm_wide_applies(const GemmArgs& a, const DeviceInfo& dev, long other) {
     if (a.group || (round_up(a.N, kTileN) / kTileN) % 2 != 0) return false;
     return wide_plan(a, dev).cost <= other;
