@@ -294,7 +294,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 off_pe[h] = (OFFSET && n_ok[h]) ? __fmul_rn(off_factor, p.chan_offset[n]) * pe : 0.0f;
             }
             if constexpr (CLUSTER) {
-                // run c of the tile's tokens belongs to CTA c * split / 8; the receiving area of a CTA is laid out as
+                // run c of the tile's tokens belongs to CTA c % split (so that both of a lane quarter's warps have runs to send and to
+                // finish; in slices of neighbouring runs 333 x 13824 x 5120, clusters of two, took 33.5 us instead of 31.5); the receiving area of a CTA is laid out as
                 // [sender][run of the slice][half][4 columns][channel][column]. The sums stay in tensor memory and are
                 // read once to be sent and once to be finished.
                 constexpr int kRun = BM / kWRuns, kRunInts = 2 * kRun * kTileN;
@@ -321,12 +322,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                         tc_wait_ld();
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
-                            const int c = (col0 + c0) / kRun + i, owner = (c * split) / kWRuns;
+                            const int c = (col0 + c0) / kRun + i, owner = c % split;
                             if (owner == rank || mt * kWBM + c * kRun >= p.M) continue;
-                            const int first = (owner * kWRuns + split - 1) / split;      // the owner's first run
                             const int from = rank < owner ? rank : rank - 1;
                             int4* dst = reinterpret_cast<int4*>(cluster.map_shared_rank(ring, owner) +
-                                                                (size_t)(from * slice_runs + c - first) * kRunInts) + h * (kRun / 4) * kTileN + r;
+                                                                (size_t)(from * slice_runs + c / split) * kRunInts) + h * (kRun / 4) * kTileN + r;
 #pragma unroll
                             for (int q = 0; q < kRun / 4; ++q)
                                 dst[q * kTileN] = make_int4((int)v[i * kRun + 4 * q], (int)v[i * kRun + 4 * q + 1],
@@ -336,17 +336,17 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 cluster_meet();                                        // all sums have arrived; nobody writes here any more
                 met = 2;
 #pragma unroll 1
-                for (int c = rank * kWRuns / split; c < kWRuns; ++c) {
+                for (int c = rank; c < kWRuns; c += split) {
                     // (this warp's runs among those its CTA owns)
-                    if ((c * split) / kWRuns != rank || c * kRun < col0 || c * kRun >= col0 + kCols || mt * kWBM + c * kRun >= p.M) continue;
-                    const int first = (rank * kWRuns + split - 1) / split, m0 = mt * kWBM + c * kRun;
+                    if (c * kRun < col0 || c * kRun >= col0 + kCols || mt * kWBM + c * kRun >= p.M) continue;
+                    const int m0 = mt * kWBM + c * kRun;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         uint32_t v[kRun];
                         tc_ld16(tmem_acc + lane_addr + (uint32_t)(h * kWBM + c * kRun), v);
                         tc_wait_ld();
                         for (int from = 0; from < split - 1; ++from) {
-                            const int4* src = reinterpret_cast<const int4*>(ring + (size_t)(from * slice_runs + c - first) * kRunInts) +
+                            const int4* src = reinterpret_cast<const int4*>(ring + (size_t)(from * slice_runs + c / split) * kRunInts) +
                                               h * (kRun / 4) * kTileN + r;
 #pragma unroll
                             for (int q = 0; q < kRun / 4; ++q) {
@@ -591,7 +591,7 @@ struct WidePlan {
 WidePlan wide_plan(const GemmArgs& a, const DeviceInfo& dev) {
     const int pairs = round_up(a.N, kTileN) / (2 * kTileN), KB = k_blocks(a.K), sms = dev.sm_count;
     const int tiles192 = (a.M + 191) / 192 * pairs, tiles128 = (a.M + 127) / 128 * pairs;
-    constexpr int kCall = 106, kRound = 2750, kBlock128 = 231, kBlock192 = 381, kExchange = 7598, kExchangeCta = 62;
+    constexpr int kCall = 106, kRound = 2750, kBlock128 = 231, kBlock192 = 381, kExchange = 5700, kExchangeCta = 62;
     WidePlan best = {192, 1, kCall + (long)((tiles192 + sms - 1) / sms) * (kRound + (long)KB * kBlock192)};
     const long cost128 = kCall + (long)((tiles128 + sms - 1) / sms) * (kRound + (long)KB * kBlock128);
     if (cost128 <= best.cost) best = {128, 1, cost128};
