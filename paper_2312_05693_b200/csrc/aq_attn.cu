@@ -211,19 +211,65 @@ __device__ __forceinline__ uint8_t log2_factor(unsigned int raw, unsigned int mb
 // last factor whatever it is. So a cooperative grid reads x once, writes the factors by the largest maximum seen so far, and notes in shared
 // memory the vectors of eight that a maximum up to `kLead` steps further would change; when all is read the grid meets, and
 // the noted vectors are written again by the true maximum. So are all vectors of a warp's batches whose maximum was further off (the
-// first few), and of a warp whose notes did not fit: then x is read twice, as by the two kernels that this replaces for arrays larger
-// than the L2 keeps.
+// first few). Where notes come too fast to fit (many values near the maximum, as in a softmax of small differences) a warp stops writing
+// and only looks for the maximum: x is then read twice, from its end, as by the two kernels that this replaces for arrays larger than
+// the L2 keeps.
 // Bound by memory: 2 bytes in, 1 out per value, at 5.6 TB/s between the meetings (32 x 2048 x 2048).
 constexpr int kOnceThreads = 1024, kOnceNotes = 10240;
 constexpr unsigned int kLead = 320;                     // of 1024 steps to twice the bound
 constexpr unsigned int kBoundOfOne = 0x39A9u;           // B_1 where the maximum is 1: 1449 * 2^-11, 1449 the least whole number above 1024 sqrt(2)
 constexpr int kOnceChanges = 8;
 
+// The factors of a thread's vectors from v downwards (see log2_codes_kernel); whether a negative value was met.
+__device__ __forceinline__ bool log2_write_again(const uint4* xv, uint2* out, long long v, long long stride, uint32_t cap) {
+    bool bad = false;
+    uint32_t near, least = 0u;
+    const uint4* src = xv + v;
+    uint2* dst = out + v;
+    for (; v >= (kLog2InFlight - 1) * stride; v -= kLog2InFlight * stride, src -= kLog2InFlight * stride, dst -= kLog2InFlight * stride) {
+        uint4 d[kLog2InFlight];
+#pragma unroll
+        for (int k = 0; k < kLog2InFlight; ++k) d[k] = __ldg(src - k * stride);
+#pragma unroll
+        for (int k = 0; k < kLog2InFlight; ++k) __stcs(dst - k * stride, log2_factors8<false>(d[k], cap, near, least, bad));
+    }
+    for (; v >= 0; v -= stride, src -= stride, dst -= stride) __stcs(dst, log2_factors8<false>(__ldg(src), cap, near, least, bad));
+    return bad;
+}
+
+// The same where not all bounds are normal halves, by comparisons with each (see log2_codes_kernel).
+__device__ __forceinline__ bool log2_write_by_bounds(const uint4* xv, uint2* out, long long v, long long nvec, long long stride, unsigned int mb_bits, int mb, int eb,
+                                                     int t_up, int t_down) {
+    if (mb_bits == 0u) {
+        for (; v < nvec; v += stride) __stcs(out + v, make_uint2(0u, 0u));
+        return false;
+    }
+    const Log2Fast fast = log2_fast_bounds(mb, eb, t_up, t_down);
+    bool bad = false;
+#pragma unroll 4
+    for (; v < nvec; v += stride) {
+        const uint4 d = __ldg(xv + v);
+        const uint32_t w[4] = {d.x, d.y, d.z, d.w};
+        uint32_t m[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const __half2 x2 = *reinterpret_cast<const __half2*>(&w[t]);
+            __half2 r = log2_fast2<true>(x2, fast);
+            const __half2 neg = __hlt2(x2, __float2half2_rn(0.0f));
+            bad |= (*reinterpret_cast<const uint32_t*>(&neg) != 0u);
+            r = __hadd2(__hfma2(neg, __hneg2(r), r), __float2half2_rn(1024.0f));
+            m[t] = *reinterpret_cast<uint32_t*>(&r);
+        }
+        __stcs(out + v, make_uint2(__byte_perm(m[0], m[1], 0x6420), __byte_perm(m[2], m[3], 0x6420)));
+    }
+    return bad;
+}
+
 __global__ void __launch_bounds__(kOnceThreads, 1)
 log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control* __restrict__ ctl, uint8_t* __restrict__ factors,
                          uint32_t* __restrict__ max_bits_out) {
     __shared__ uint32_t notes[kOnceNotes];
-    __shared__ unsigned int noted, warp_max[kOnceThreads / 32];
+    __shared__ unsigned int noted, note_rate, warp_max[kOnceThreads / 32];
     // per warp: from which of its batches on its factors stood for which B_1 (a new entry where its maximum changed)
     __shared__ unsigned short covers[kOnceThreads / 32][kOnceChanges];
     __shared__ uint32_t from_batch[kOnceThreads / 32][kOnceChanges];
@@ -249,7 +295,12 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
         ctl->status = 0;
         *running = 0u;
     }
-    if (threadIdx.x == 0) noted = 0u;
+    // of each warp; the vectors of all but its last one are all there
+    const uint32_t batches = (uint32_t)((nvec + kLog2InFlight * stride - 1) / (kLog2InFlight * stride));
+    if (threadIdx.x == 0) {
+        noted = 0u;
+        note_rate = 2 * kOnceNotes / batches;            // twice the notes that would fit at an even rate, per batch
+    }
     if (blockIdx.x < Control::kRangeWords) {
 #pragma unroll
         for (int k = 0; k < kLog2InFlight; ++k)
@@ -269,17 +320,16 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
     uint32_t cap = 0u, edge = 0u;                        // edge: remainders from 1024 - lead on reach bit 15 when it is added
     unsigned int bound = 0u;
     int changes = 0;
-    uint32_t batch = 0;
     bool bad = false, all_again = false;
     const uint4* p = xv + at;
-    long long v = at;
-    for (long long left = nvec - (at - lane); left > 0; left -= kLog2InFlight * stride, p += kLog2InFlight * stride, v += kLog2InFlight * stride) {
-        uint4 d[kLog2InFlight];                          // left: vectors from the warp's first on
-        const bool whole = left > (kLog2InFlight - 1) * stride + 31;
+    uint2* dst = out + at;
+    for (uint32_t batch = 0; batch < batches; ++batch, p += kLog2InFlight * stride, dst += kLog2InFlight * stride) {
+        uint4 d[kLog2InFlight];
+        const bool whole = batch + 1 < batches;
 #pragma unroll
         for (int k = 0; k < kLog2InFlight; ++k) {
             d[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (whole || v + k * stride < nvec) d[k] = __ldg(p + k * stride);
+            if (whole || p + k * stride < xv + nvec) d[k] = __ldg(p + k * stride);
         }
         const unsigned int next = *running;              // for the next batch
         if (known != used) {
@@ -297,9 +347,8 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
             }
             changes = place + 1;
         }
-        ++batch;
-        if (bound == 0u) {
-            all_again = true;
+        if (bound == 0u) all_again = true;
+        if (all_again) {
 #pragma unroll
             for (int k = 0; k < kLog2InFlight; ++k) largest(d[k]);
         } else {
@@ -308,12 +357,12 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
             for (int k = 0; k < kLog2InFlight; ++k) {
                 uint32_t near;
                 const uint2 f = log2_factors8<true>(d[k], cap, near, least, bad);
-                if (whole || v + k * stride < nvec) {
-                    __stcs(out + v + k * stride, f);
+                if (whole || p + k * stride < xv + nvec) {
+                    __stcs(dst + k * stride, f);
                     if ((near + edge) & 0x80008000u) {
                         const unsigned int n = atomicAdd(&noted, 1u);
-                        if (n < (unsigned int)kOnceNotes) notes[n] = (uint32_t)(v + k * stride);
-                        else all_again = true;
+                        if (n < (unsigned int)kOnceNotes) notes[n] = (uint32_t)(p - xv + k * stride);
+                        all_again |= n >= min((unsigned int)kOnceNotes, note_rate * (batch + 1));
                     }
                 }
             }
@@ -325,7 +374,7 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
                 m2 = __hmax2(m2, *reinterpret_cast<const __half2*>(&most));
             }
         }
-        __syncwarp();
+        all_again = __any_sync(0xFFFFFFFFu, all_again);
         known = max(known, next);
         const unsigned int own = __reduce_max_sync(0xFFFFFFFFu, max_bits());
         if (own > known) {
@@ -358,26 +407,17 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
     uint32_t near, least = 0u;
     // the batches up to the first change whose factors stand for the true bound
     const bool again = __any_sync(0xFFFFFFFFu, all_again || final_bound == 0u);
-    long long redo = again ? nvec : 0;
+    long long redo = again ? batches : 0;
     if (!again && changes > 0) {
         int c = 0;
         while (c < changes && covers[warp][c] < final_bound) ++c;
-        redo = c == changes ? nvec : at + (long long)from_batch[warp][c] * kLog2InFlight * stride;
+        redo = c == changes ? batches : from_batch[warp][c];
     }
-    {
-        for (v = at; v < min(redo, nvec); v += stride) {
-            const uint4 d = __ldg(xv + v);
-            if (final_bound) {
-                out[v] = log2_factors8<false>(d, final_cap, near, least, bad);
-            } else {
-                const uint32_t w[4] = {d.x, d.y, d.z, d.w};
-                uint32_t o[2] = {0u, 0u};
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    o[t >> 2] |= (uint32_t)log2_factor((w[t >> 1] >> (16 * (t & 1))) & 0xFFFFu, mb_bits, eb, t_up, t_down, bad) << (8 * (t & 3));
-                out[v] = make_uint2(o[0], o[1]);
-            }
-        }
+    if (final_bound) {
+        const long long end = min(nvec, redo * kLog2InFlight * stride + at);
+        if (end > at) bad |= log2_write_again(xv, out, at + (end - 1 - at) / stride * stride, stride, final_cap);
+    } else {
+        bad |= log2_write_by_bounds(xv, out, at, nvec, stride, mb_bits, mb, eb, t_up, t_down);
     }
     // (another warp's vectors may be among these, written by it above as well: the same factors)
     if (final_bound)
@@ -1014,11 +1054,13 @@ cudaError_t launch_attn_qk_tc(const int8_t* qc, const int32_t* e_q, const int8_t
     return launch_attn_tc<128, true, 1, 8>(qc, kc, nullptr, e_q, e_k, 0, H, M, D, J, s_out, ctl, dev, stream, true);
 }
 
-// Values from which byte factors are made in one pass: 117 MB of them, about what the L2 holds. us in two kernels / one, graph replay,
-// softmax outputs of 56 x 2048 x 2048 values 191.6 / 134.2, 32 x 2048 x 2048 110.9 / 82.4, 40 x 1500 x 1024 53.7 / 49.3, 12 x 2048 x 2048
-// 44.9 / 43.8 (call by call 45.8 / 46.1), 16 x 1024 x 2048 31.8 / 33.9: the grid's two meetings and a launch that overlaps nothing cost some
-// 12 us, and below that size most of the second reading comes from the L2.
-constexpr long long kOnceCount = 7ll << 23;
+// Values from which byte factors are made in one pass: 235 MB of them, nearly twice what the L2 holds. us in two kernels / one, graph replay,
+// softmax outputs of normal scores with a deviation of 3: 56 x 2048 x 2048 values 191.4 / 134.0, 32 x 2048 x 2048 110.9 / 83.5, 24 x 2048 x
+// 2048 84.0 / 69.9, 40 x 1500 x 1024 53.7 / 50.5, 16 x 1024 x 2048 31.8 / 33.9: the grid's two meetings and a launch that overlaps nothing
+// cost some 12 us, and in smaller arrays more of the second reading comes from the L2. Flatter outputs, many of whose values lie
+// near the maximum, gain less or lose: 32 x 2048 x 2048, deviation 2, 111.0 / 103.2, deviation 1 110.8 / 133.7; 24 x 2048 x 2048,
+// deviation 2, 84.0 / 97.2, 40 x 1500 x 1024 53.8 / 62.1. The line lies where the first kind gains more than the second loses.
+constexpr long long kOnceCount = 14ll << 23;
 
 cudaError_t launch_log2_quantize(const __half* x, long long count, int bits, Control* ctl, int8_t* codes,
                                  uint32_t* max_bits_out, const DeviceInfo& dev, cudaStream_t stream, bool as_factors) {

@@ -10,14 +10,14 @@ from paper_2312_05693_b200 import binding
 
 pytestmark = pytest.mark.gpu
 
-COUNT = 7 << 23                                                  # the first size that takes it
+COUNT = 14 << 23                                                 # the first size that takes it
 
 
-def softmax_rows(n, j, seed):
+def softmax_rows(n, j, seed, deviation=3.0):
     g = torch.Generator(device="cuda").manual_seed(seed)
     x = torch.empty((n // j + 1, j), dtype=torch.float16, device="cuda")
     for part in x.split(16384):
-        part.copy_(torch.softmax(3.0 * torch.randn(part.shape, generator=g, device="cuda"), dim=-1))
+        part.copy_(torch.softmax(deviation * torch.randn(part.shape, generator=g, device="cuda"), dim=-1))
     return x.flatten()[:n]
 
 
@@ -48,6 +48,11 @@ def check(x):
 @pytest.mark.parametrize("extra", [-1, 0, 7, 12345, COUNT // 2 + 40])
 def test_softmax_outputs(extra):
     check(softmax_rows(COUNT + extra, 2048, 3))
+
+
+@pytest.mark.parametrize("deviation", [2.0, 1.0, 0.3, 0.01])     # flatter: ever earlier too many values near the maximum
+def test_flat_softmax_outputs(deviation):
+    check(softmax_rows(COUNT + 4099, 2048, 6, deviation))
 
 
 @pytest.mark.parametrize("case", ["first", "last", "tail", "rising", "falling", "dense", "above one", "subnormal", "zeros", "infinite", "negative"])
