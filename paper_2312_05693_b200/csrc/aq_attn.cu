@@ -366,7 +366,8 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
                     }
                 }
             }
-            if (__vminu2(least, 0x00010001u) != 0x00010001u) {
+            // (where cap lies above infinity a NaN may be what comes nearest to it: the values themselves then)
+            if (__vminu2(least, 0x00010001u) != 0x00010001u || cap > 0x7C007C00u) {
 #pragma unroll
                 for (int k = 0; k < kLog2InFlight; ++k) largest(d[k]);
             } else {

@@ -73,6 +73,17 @@ def test_maxima_and_values(case):
     check(x)
 
 
+@pytest.mark.parametrize("nan", [0x7C01, 0x7C4F, 0x7DA7, 0x7E00, 0xFC01])
+def test_each_nan_alone_is_dropped(nan):
+    """A running maximum from 46400 on: B_1 + 1023 is then above the pattern of infinity, so that NaN patterns lie below it too."""
+    x = (uniform(COUNT + 8 * 4096) * 10000 + 40000).half()       # none near the bounds of the running maximum: factors are written
+    bits = x.view(torch.int16)
+    at = COUNT - 8 * 5000                                        # beside the maximum, in the same half of a register and in the other
+    x[at] = 65504.0
+    bits[at + 1:at + 8] = nan - 0x10000 if nan > 0x7FFF else nan
+    check(x)
+
+
 def test_in_a_graph_and_again():
     """The same control block call after call, larger and smaller maxima in turn."""
     from gpu_util import handle
