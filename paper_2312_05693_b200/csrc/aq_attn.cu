@@ -331,7 +331,8 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
             d[k] = make_uint4(0u, 0u, 0u, 0u);
             if (whole || p + k * stride < xv + nvec) d[k] = __ldg(p + k * stride);
         }
-        const unsigned int next = *running;              // for the next batch
+        // for the next batch, one lane's for all: others write it meanwhile, and the warp's bound and notes have to agree
+        const unsigned int next = __shfl_sync(0xFFFFFFFFu, *running, 0);
         if (known != used) {
             used = known;
             bound = log2_first_bound(used);

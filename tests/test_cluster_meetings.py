@@ -57,6 +57,16 @@ def test_asynchronous_remote_stores_come_behind_it_too():
     assert found >= 6
 
 
+def test_a_running_maximum_is_one_value_for_a_warp():
+    """What a warp reads of a word that others raise meanwhile is one lane's reading for all: its lanes would otherwise go by bounds
+    of their own while one of them notes which batches a bound stands for."""
+    code = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "aq_attn.cu")).read())
+    readings = re.findall(r"unsigned int (?:next|hint) = ([^;]*);", code)
+    assert readings
+    for r in readings:
+        assert re.fullmatch(r"__shfl_sync\(0xFFFFFFFFu, .*, 0\)", r), r
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("M,K", [(1, 32), (1, 64), (3, 32), (3, 96), (16, 4096), (17, 16384)])
 def test_every_share_of_the_cluster_reaches_the_scale(M, K):
