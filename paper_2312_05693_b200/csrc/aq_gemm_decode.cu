@@ -218,10 +218,20 @@ __device__ __forceinline__ bool str_wait(uint64_t* bar, uint32_t parity, volatil
 }
 
 // Bounded wait for what the cluster's other CTAs send, also after this CTA has given up elsewhere: it must be there when it comes.
+// Their stores count at the scope of the cluster, so this waits at that scope (a wait without it is one at the scope of the CTA).
+__device__ __forceinline__ bool str_try_wait_peers(uint64_t* bar) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(s_u32(bar)) : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ void str_wait_peers(uint64_t* bar, volatile uint32_t* abort_flag) {
-    if (str_try_wait(bar, 0u)) return;
+    if (str_try_wait_peers(bar)) return;
     const long long t0 = clock64();
-    while (!str_try_wait(bar, 0u))
+    while (!str_try_wait_peers(bar))
         if ((unsigned long long)(clock64() - t0) > kStrPeerCycles) { *abort_flag = 1; return; }
 }
 

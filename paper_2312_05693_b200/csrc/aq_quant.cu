@@ -110,7 +110,7 @@ quantize_small_kernel(const uint4* __restrict__ x, int M, int vec_per_row, const
     bool came = false;
     for (const long long t0 = clock64(); !came && (unsigned long long)(clock64() - t0) < 2 * kWaitCycles;) {
         uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(met_a) : "memory");
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(met_a) : "memory");
         came = ok != 0;
     }
     __syncwarp();

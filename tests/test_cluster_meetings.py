@@ -57,6 +57,27 @@ def test_asynchronous_remote_stores_come_behind_it_too():
     assert found >= 6
 
 
+def test_waits_for_what_peers_send_are_at_their_scope():
+    """A barrier that other CTAs' st.async count on (its address goes through mapa) is waited for at the scope of the cluster:
+    without a scope the wait orders nothing that another CTA wrote."""
+    found = 0
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        mapped = set(re.findall(r'"mapa\.[^;]*;" : "=r"\(bar\) : "r"\((?:s_u32\(&sm\.)?(\w+)\)', code))
+        for name in mapped:
+            waits = re.findall(r"str_(?:wait|wait_peers|try_wait)\(&sm\.%s\b" % name, code)
+            if waits:                                           # by a helper: the one whose instruction has the scope
+                assert all(w.startswith("str_wait_peers") for w in waits), (path, name)
+                body = code[code.index("bool str_try_wait_peers"):]
+                assert "try_wait.parity.acquire.cluster" in body[:body.index("\n}\n")]
+                assert "str_try_wait(" not in code[code.index("void str_wait_peers"):].split("\n}\n")[0]
+            else:
+                direct = re.findall(r'mbarrier\.try_wait\.([\w.:]*) p, \[%%1\][^"]*"[^;]*"r"\(%s\)' % name, code)
+                assert direct and all("acquire.cluster" in d for d in direct), (path, name, direct)
+            found += 1
+    assert found >= 3
+
+
 def test_a_running_maximum_is_one_value_for_a_warp():
     """What a warp reads of a word that others raise meanwhile is one lane's reading for all: its lanes would otherwise go by bounds
     of their own while one of them notes which batches a bound stands for."""
