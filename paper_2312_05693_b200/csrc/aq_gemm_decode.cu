@@ -312,13 +312,13 @@ struct StreamParams {
     int early_dependents;          // the launch behind this one may be set up from this kernel's start
     int next_packed;
     int box_rows;                  // MMA route: rows of a k block's codes in shared memory
-    // FUSEQ: the activations themselves; the kernel finds the layer scale (several rows: or scale and zero point), writes the codes of
+    // FUSEQ: the activations themselves; the kernel finds the layer scale (and zero point), writes the codes of
     // its k range to shared memory (and, from the first channel tile, to q_out) and fills the control block
     const __half* x_row;           // the rows, K halves each
     const int32_t* row_idx;        // one row: NULL or its index, the row is x_row + row_idx[0] * K
     int8_t* q_out;                 // [M][K] codes
     int bits, scale_mode, clip_shift_or_exp;
-    const uint8_t* alpha;          // several rows: NULL or the TRIP factors, K bytes, none above k_max
+    const uint8_t* alpha;          // NULL or the TRIP factors, K bytes, none above k_max
     int k_max;
 };
 
@@ -470,7 +470,9 @@ __device__ __forceinline__ void slice_codes(const StreamParams& p, StreamSmem<MB
     }
 }
 
-template <int MB, bool FUSEQ = false, bool WIDE = false, bool GROUPED = false>
+// PLAIN: neither a zero point nor TRIP factors where one row is quantized here. (A parameter, so that the kernel of plain rows has none of the other
+// quantizers in it; slices of several rows choose at run time.)
+template <int MB, bool FUSEQ = false, bool WIDE = false, bool GROUPED = false, bool PLAIN = true>
 __global__ void __launch_bounds__(StreamCfg<MB>::kThreads, 2)
 gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const StreamParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -603,15 +605,28 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
             for (int i = issued; i < ring; ++i) issue_w(kb0 + i, i);   // weights on their way meanwhile
         issued = ring;
         const uint4* xv = reinterpret_cast<const uint4*>(p.x_row + (p.row_idx ? (size_t)p.row_idx[0] * p.K : 0));
-        int e = p.clip_shift_or_exp;
+        int e = p.clip_shift_or_exp, zp = 0;
+        const bool asym = !PLAIN && p.chan_offset != nullptr;
+        const int v0 = kb0 * (kTileK / 8), v1 = min(kb1 * (kTileK / 8), p.K / 8);       // 8-element vectors of this k range
+        [[maybe_unused]] uint2 alpha_first = make_uint2(0u, 0u);                        // of this thread's first one, on its way meanwhile
+        if constexpr (!PLAIN)
+            if (p.alpha && v0 + (int)threadIdx.x < v1) alpha_first = __ldg(reinterpret_cast<const uint2*>(p.alpha) + v0 + threadIdx.x);
         // up to kKeep vectors per thread stay in registers between the two passes (K <= 18432); longer rows
         // are read again (from L2) for the codes
         constexpr int kKeep = 8;
         uint4 keep[kKeep];
         const int n_vec = p.K / 8;
         const bool kept = n_vec <= kKeep * kStrThreads;
-        if (p.scale_mode == AQ_SCALE_DYNAMIC || kept) {
-            __half2 m2 = __float2half2_rn(0.0f);
+        if (asym || p.scale_mode == AQ_SCALE_DYNAMIC || kept) {
+            __half2 m2 = __float2half2_rn(0.0f), least2 = m2;
+            auto take = [&](const uint4& d) {                              // NaN operands are dropped
+                const __half2* h = reinterpret_cast<const __half2*>(&d);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (asym) least2 = __hmin2(least2, h[k]);
+                    m2 = __hmax2(m2, asym ? h[k] : __habs2(h[k]));
+                }
+            };
             if (kept) {
 #pragma unroll
                 for (int i = 0; i < kKeep; ++i) {
@@ -619,59 +634,79 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
                     keep[i] = v < n_vec ? __ldg(xv + v) : make_uint4(0, 0, 0, 0);
                 }
 #pragma unroll
-                for (int i = 0; i < kKeep; ++i) {
-                    const __half2* h = reinterpret_cast<const __half2*>(&keep[i]);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) m2 = __hmax2(m2, __habs2(h[k]));   // NaN operands are dropped
-                }
+                for (int i = 0; i < kKeep; ++i) take(keep[i]);
             } else {
-                for (int v = (int)threadIdx.x; v < n_vec; v += kStrThreads) {
-                    const uint4 d = __ldg(xv + v);
-                    const __half2* h = reinterpret_cast<const __half2*>(&d);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) m2 = __hmax2(m2, __habs2(h[k]));
-                }
+                for (int v = (int)threadIdx.x; v < n_vec; v += kStrThreads) take(__ldg(xv + v));
             }
             unsigned int bmax = max((unsigned int)__half_as_ushort(__low2half(m2)), (unsigned int)__half_as_ushort(__high2half(m2)));
             if (bmax > 0x7C00u) bmax = 0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) bmax = max(bmax, __shfl_xor_sync(0xFFFFFFFFu, bmax, o));
+            if (asym) {                                                    // the least value's magnitude in the upper half
+                const __half2 n2 = __habs2(least2);
+                bmax |= __reduce_max_sync(0xFFFFFFFFu, max((unsigned int)__half_as_ushort(__low2half(n2)), (unsigned int)__half_as_ushort(__high2half(n2)))) << 16;
+            }
             if (lane == 0) sm.warp_max[warp] = bmax;
             __syncthreads();
             unsigned int all = 0;
 #pragma unroll
-            for (int w = 0; w < kStrThreads / 32; ++w) all = max(all, sm.warp_max[w]);
-            if (p.scale_mode == AQ_SCALE_DYNAMIC) {
-                e = layer_exponent_from_bits(all, p.bits) - p.clip_shift_or_exp;
-                if (tile == 0 && rank == 0 && threadIdx.x == 0) p.ctl->absmax_bits = all;
+            for (int w = 0; w < kStrThreads / 32; ++w) all = PLAIN ? max(all, sm.warp_max[w]) : __vmaxu2(all, sm.warp_max[w]);
+            if (asym) {
+                zero_point_scale(all & 0xFFFFu, all >> 16, p.bits, e, zp);
+                all = 0u;
+            } else if (p.scale_mode == AQ_SCALE_DYNAMIC) {
+                e = layer_exponent_from_bits(all, p.bits) - p.clip_shift_or_exp - (PLAIN ? 0 : p.k_max);
             }
+            if ((asym || p.scale_mode == AQ_SCALE_DYNAMIC) && tile == 0 && rank == 0 && threadIdx.x == 0) p.ctl->absmax_bits = all;
         }
         if (tile == 0 && rank == 0) {
-            if (threadIdx.x == 0) { p.ctl->scale_exp = e; p.ctl->status = 0; }
+            if (threadIdx.x == 0) {
+                p.ctl->scale_exp = e;
+                p.ctl->status = 0;
+                if (!PLAIN) p.ctl->zero_point = zp;
+            }
             if (threadIdx.x < Control::kSplitWords) p.ctl->split_flags[threadIdx.x] = 0;
         }
         const float lo = -(float)(1 << (p.bits - 1)), hi = (float)((1 << (p.bits - 1)) - 1);
-        const int v0 = kb0 * (kTileK / 8), v1 = min(kb1 * (kTileK / 8), p.K / 8);       // 8-element vectors of this k range
         const bool fast = e >= -14 && e <= 14;             // 2^-e is a normal half: codes in half2 arithmetic
         const __half2 inv2 = __float2half2_rn(fast ? __int_as_float((127 - e) << 23) : 1.0f);
         const __half2 lo2 = __float2half2_rn(lo), hi2 = __float2half2_rn(hi);
         auto code8 = [&](const uint4& d, int v) {
             uint2 c;
-            if (fast) quantize8_half2(d, inv2, lo2, hi2, c.x, c.y);
-            else c = quantize8_fp32(d, e, lo, hi, nullptr);
+            if constexpr (!PLAIN) {
+                if (asym) {
+                    if (fast) {
+                        const __half2 clo2 = __float2half2_rn(-(float)zp), chi2 = __float2half2_rn((float)((1 << p.bits) - 1 - zp));
+                        quantize8_half2_asym(d, inv2, clo2, chi2, __float2half2_rn((float)(zp - (1 << (p.bits - 1)))), c.x, c.y);
+                    } else {
+                        c = quantize8_fp32_asym(d, __int_as_float((127 - e) << 23), zp, p.bits);
+                    }
+                } else {
+                    const uint2 al = v == v0 + (int)threadIdx.x ? alpha_first : __ldg(reinterpret_cast<const uint2*>(p.alpha) + v);
+                    if (p.bits == 4 && e >= -14 && e <= 10) quantize8_half2_trip(d, e, al, c.x, c.y);      // 2^-(e + alpha) is a normal half, alpha <= 4
+                    else c = quantize8_fp32(d, e, lo, hi, &al);
+                }
+            } else if (fast) {
+                quantize8_half2(d, inv2, lo2, hi2, c.x, c.y);
+            } else {
+                c = quantize8_fp32(d, e, lo, hi, nullptr);
+            }
             reinterpret_cast<uint2*>(sm.xq)[v - v0] = c;
             if (tile == 0) reinterpret_cast<uint2*>(p.q_out)[v] = c;
         };
-        if (kept) {
+        if (PLAIN && kept) {
 #pragma unroll
             for (int i = 0; i < kKeep; ++i) {
                 const int v = (int)threadIdx.x + i * kStrThreads;
                 if (v >= v0 && v < v1) code8(keep[i], v);
             }
         } else {
+            // (not PLAIN: once or a few times for a thread, unrolled eight times the quantizers' code would be the longer part)
+#pragma unroll 1
             for (int v = v0 + (int)threadIdx.x; v < v1; v += kStrThreads) code8(__ldg(xv + v), v);
         }
         fused_exp = e;
+        fused_zp = zp;
         __syncthreads();
     }
     if (warp == 0) {
@@ -888,7 +923,7 @@ gemm_decode_stream_kernel(const __grid_constant__ CUtensorMap x_map, const Strea
     if (mine) {
         const float pe = __int_as_float((127 + (FUSEQ ? fused_exp : *p.scale_exp)) << 23);
         sc = GROUPED ? 0.0625f * pe : __half2float(p.w_scales[out_n]) * pe;     // the fp32 sums carry a factor 16
-        if (p.chan_offset) off = __fmul_rn(kSlices ? -(float)(fused_zp - p.zp_mid) : offset_factor(p.ctl, p.zp_mid), p.chan_offset[out_n]) * pe;
+        if (p.chan_offset) off = __fmul_rn(FUSEQ ? -(float)(fused_zp - p.zp_mid) : offset_factor(p.ctl, p.zp_mid), p.chan_offset[out_n]) * pe;
     }
     const int rows = p.M < kRows ? p.M : kRows;
     if (split > 1 && !kSlices) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // everybody has started (arrival at the top)
@@ -970,14 +1005,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-template <int MB, bool FUSEQ, bool WIDE, bool GROUPED>
+template <int MB, bool FUSEQ, bool WIDE, bool GROUPED, bool PLAIN = true>
 cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream, int split) {
     using Smem = StreamSmem<MB, WIDE, GROUPED, FUSEQ>;
     const int tiles = round_up(a.N, kTileN) / kTileN;
     const size_t smem_bytes = sizeof(Smem) + 1024;
     static_assert(2 * (sizeof(Smem) + 1024 + 1024) <= 228 * 1024, "two CTAs an SM");
     static SmemOptIn opt_in;
-    if (const cudaError_t e = opt_in.ensure(gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED>, dev.device, smem_bytes); e != cudaSuccess)
+    if (const cudaError_t e = opt_in.ensure(gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED, PLAIN>, dev.device, smem_bytes); e != cudaSuccess)
         return e;
     CUtensorMap map = {};
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
@@ -1027,7 +1062,7 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;       // the kernel reads and writes nothing before the kernel ahead of it has completed
-    return cudaLaunchKernelEx(&cfg, gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED>, map, p);
+    return cudaLaunchKernelEx(&cfg, gemm_decode_stream_kernel<MB, FUSEQ, WIDE, GROUPED, PLAIN>, map, p);
 }
 
 // Clusters of `split` CTAs that run at once, by the occupancy query (asked once per device and size).
@@ -1110,7 +1145,7 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
 }  // namespace
 
 // Whether the product kernel quantizes the rows itself (one launch for the layer). Dumps of per-group sums are left to the general
-// kernel. A single row: where a CTA's k range fits its code buffer. Several rows, and any with a zero point or TRIP factors (plain: neither): while
+// kernel. A single row: where a CTA's k range fits its code buffer. Several rows: while
 // a CTA's slice is kSliceVecs vectors a thread; beyond, every tile's CTAs quantizing the same slice cost more than a kernel that
 // does it once (16 x 11008 x 4096 in groups, 13 vectors, behind a quantize kernel / here: 12.6 / 13.3). us with two launches /
 // one, stable weights, graph replay and call by call, before and after (the number of CTAs a tile has and the order of the MMA's operands
@@ -1124,7 +1159,7 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
 bool decode_can_fuse_quantize(int M, int K, int N, int group, bool dump, bool plain, bool weights_stable, const DeviceInfo& dev) {
     if (M > kFewRows || (group && dump)) return false;
     const int tiles = round_up(N, kTileN) / kTileN, KB = k_blocks(K);
-    if (M == 1 && plain) {
+    if (M == 1) {
         const int split = group ? stream_split<1, true>(K, N, dev) : stream_split<1, false>(K, N, dev);
         return (KB + split - 1) / split + 1 <= kFuseMaxBlocks;
     }
@@ -1141,16 +1176,20 @@ template <int MB, bool GROUPED>
 cudaError_t launch_stream_mb(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
     const int split = stream_split<MB, GROUPED>(a.K, a.N, dev);
     const bool wide = split != 1 && split != 2 && split != 4;
+    if constexpr (MB == 1)
+        if (a.fuse_x && (a.chan_offset || a.fuse_alpha))
+            return wide ? launch_stream<MB, true, true, GROUPED, false>(a, dev, stream, split) : launch_stream<MB, true, false, GROUPED, false>(a, dev, stream, split);
     if (a.fuse_x)
         return wide ? launch_stream<MB, true, true, GROUPED>(a, dev, stream, split) : launch_stream<MB, true, false, GROUPED>(a, dev, stream, split);
     return wide ? launch_stream<MB, false, true, GROUPED>(a, dev, stream, split) : launch_stream<MB, false, false, GROUPED>(a, dev, stream, split);
 }
 // one row: dp4a; from 2 rows on the warp MMA on 16-row tiles (fewer instructions per weight
 // chunk than dp4a from two rows on; measured faster at M = 4: 7.5 / 11.1 / 13.3 us against
-// 8.1 / 12.8 / 15.2 us on the three 13B shapes). A single row with a zero point or TRIP factors that is quantized here takes that route as well.
+// 8.1 / 12.8 / 15.2 us on the three 13B shapes). By the rows alone, whoever quantizes them: with per-group scales the routes round their fp32
+// sums differently, and calls that differ in what they name (a row by its index, an output over the input, the codes themselves) agree in every bit.
 template <bool GROUPED>
 cudaError_t launch_stream_rows(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
-    return a.M <= 1 && !(a.fuse_x && (a.chan_offset || a.fuse_alpha)) ? launch_stream_mb<1, GROUPED>(a, dev, stream) : launch_stream_mb<kFewRows, GROUPED>(a, dev, stream);
+    return a.M <= 1 ? launch_stream_mb<1, GROUPED>(a, dev, stream) : launch_stream_mb<kFewRows, GROUPED>(a, dev, stream);
 }
 }  // namespace
 
