@@ -209,14 +209,22 @@ __device__ __forceinline__ uint8_t log2_factor(unsigned int raw, unsigned int mb
 // The maximum is known only when all of x has been read, but nearly all factors are settled before: by a maximum that is a little too small
 // a factor comes out wrong only where the value lies just under a bound, and values from 2^-6.5 of the maximum down have the
 // last factor whatever it is. So a cooperative grid reads x once, writes the factors by the largest maximum seen so far, and notes in shared
-// memory the vectors of eight that a maximum up to `kLead` steps further would change; when all is read the grid meets, and
-// the noted vectors are written again by the true maximum. So are all vectors of a warp's batches whose maximum was further off (the
-// first few). Where notes come too fast to fit (many values near the maximum, as in a softmax of small differences) a warp stops writing
-// and only looks for the maximum: x is then read twice, from its end, as by the two kernels that this replaces for arrays larger than
-// the L2 keeps.
+// memory the vectors of eight that a maximum up to the lead further would change; when all is read the grid meets, and
+// the noted vectors are written again by the true maximum. The lead reaches to a maximum of 1, so that no softmax output goes
+// beyond it; were a maximum beyond it to come all the same, the batches that it found written are written again.
+// That pays where a sample, taken before, shows that 1 is near and that few vectors will be noted; elsewhere (softmax of small differences)
+// the grid reads x for its maximum alone and again, from its end, for the factors, as the two kernels do that this replaces for arrays
+// larger than the L2 keeps. Rules of kLead, kOnceShare: a noted vector costs a scattered read and a partial write, 28 heads of 2048 x 2048 some
+// 20 us for every hundredth of the vectors while the maximum stays where it is (117 us with half an octave to 1 and 15 notes in 1000 vectors, 92.3 in two
+// kernels, 77 without notes); one that rises soon costs less (2.5 standard deviations of scores, 278 steps and 14 in 1000: 83). The
+// decision is one for the grid: where some CTAs read twice and others wrote, all waited for the slower ones (126 us).
 // Bound by memory: 2 bytes in, 1 out per value, at 5.6 TB/s between the meetings (32 x 2048 x 2048).
 constexpr int kOnceThreads = 1024, kOnceNotes = 10240;
-constexpr unsigned int kLead = 320;                     // of 1024 steps to twice the bound
+constexpr unsigned int kLead = 300;                     // of 1024 steps to twice the bound
+constexpr int kOnceShare = 64;                          // one vector in so many may be noted
+// Bytes of x, read last, that the L2 is to keep for the second reading: what comes before is marked as first to go (28 / 32 / 56 heads read
+// twice without the marks 96.7 / 111.1 / -, with them and 116 MB 92.0 / 104.6 / 181.9, 97 MB 91.9 / 104.5 / 180.9, 78 MB 91.1 / 104.1 / 179.9).
+constexpr long long kOnceKeep = 78ll << 20;
 constexpr unsigned int kBoundOfOne = 0x39A9u;           // B_1 where the maximum is 1: 1449 * 2^-11, 1449 the least whole number above 1024 sqrt(2)
 constexpr int kOnceChanges = 8;
 
@@ -285,12 +293,19 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
 #pragma unroll
         for (int t = 0; t < 4; ++t) m2 = __hmax2(m2, *reinterpret_cast<const __half2*>(&w[t]));
     };
+    auto load = [&](uint4 (&d)[kLog2InFlight], const uint4* src, bool whole) {
+#pragma unroll
+        for (int k = 0; k < kLog2InFlight; ++k) {
+            d[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (whole || src + k * stride < xv + nvec) d[k] = __ldg(src + k * stride);
+        }
+    };
     // of this thread's values so far; Inf counts as the largest finite value
     auto max_bits = [&] {
         const unsigned int b = max((unsigned int)__half_as_ushort(__low2half(m2)), (unsigned int)__half_as_ushort(__high2half(m2)));
         return min(b, 0x7BFFu);
     };
-    // a first maximum: from the first batches of as many CTAs as the control block has words for
+    // a first maximum: from the first batches of as many CTAs as the control block has words for, and from vectors spread over all of x
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->status = 0;
         *running = 0u;
@@ -301,54 +316,84 @@ log2_factors_once_kernel(const __half* __restrict__ x, long long count, Control*
         noted = 0u;
         note_rate = 2 * kOnceNotes / batches;            // twice the notes that would fit at an even rate, per batch
     }
-    if (blockIdx.x < Control::kRangeWords) {
+    const unsigned int words = min(gridDim.x, (unsigned int)Control::kRangeWords);
+    if (blockIdx.x < words) {
+        // (a warp's side by side; they also tell how many vectors have values in the range of the factors below 1)
+        const uint4 probe = __ldg(xv + (long long)(blockIdx.x * (kOnceThreads / 32) + warp) * (nvec / (words * (kOnceThreads / 32))) + lane);
 #pragma unroll
         for (int k = 0; k < kLog2InFlight; ++k)
             if (at + k * stride < nvec) largest(__ldg(xv + at + k * stride));
+        largest(probe);
         const unsigned int b = __reduce_max_sync(0xFFFFFFFFu, max_bits());
         if (lane == 0) warp_max[warp] = b;
-        __syncthreads();
+        uint32_t near, least = 0u;
+        bool negative = false;
+        (void)log2_factors8<true>(probe, (kBoundOfOne + 1023u) * 0x00010001u, near, least, negative);
+        const unsigned int hits = (unsigned int)__syncthreads_count(near != 0u);
         if (threadIdx.x < 32) {
             const unsigned int c = __reduce_max_sync(0xFFFFFFFFu, lane < kOnceThreads / 32 ? warp_max[lane] : 0u);
-            if (lane == 0) ctl->range[blockIdx.x] = c;
+            if (lane == 0) ctl->range[blockIdx.x] = c | (hits << 16);
         }
     }
     grid.sync();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const unsigned int words = min(gridDim.x, (unsigned int)Control::kRangeWords);
-    unsigned int known = __reduce_max_sync(0xFFFFFFFFu, lane < (int)words ? ((volatile unsigned int*)ctl->range)[lane] : 0u), used = ~0u;
+    const unsigned int word = lane < (int)words ? ((volatile unsigned int*)ctl->range)[lane] : 0u;
+    unsigned int known = __reduce_max_sync(0xFFFFFFFFu, word & 0xFFFFu), used = ~0u;
     uint32_t cap = 0u, edge = 0u;                        // edge: remainders from 1024 - lead on reach bit 15 when it is added
     unsigned int bound = 0u;
     int changes = 0;
     bool bad = false, all_again = false;
+    auto take_bound = [&](uint32_t batch) {
+        used = known;
+        bound = log2_first_bound(used);
+        cap = (bound + 1023u) * 0x00010001u;
+        // a softmax output is 1 at most
+        const unsigned int lead = used <= 0x3C00u ? min(kBoundOfOne - bound, kLead) : 64u;
+        edge = (0x8000u - 1024u + lead) * 0x00010001u;
+        // (with no place left the last entry stands for fewer batches than it could)
+        const int place = min(changes, kOnceChanges - 1);
+        if (lane == 0) {
+            covers[warp][place] = (unsigned short)(bound + lead);
+            from_batch[warp][place] = batch;
+        }
+        changes = place + 1;
+    };
+    take_bound(0u);
+    const long long hits = __reduce_add_sync(0xFFFFFFFFu, word >> 16), to_one = (long long)kBoundOfOne - bound;
+    // of the vectors in that range to_one / 1024 are noted, remainders being as good as even; half the room for notes is to spare
+    const bool twice = bound == 0u || to_one < 0 || to_one > kLead || hits * to_one * kOnceShare > (long long)words * kOnceThreads * 1024 ||
+                       hits * to_one * nvec > (long long)words * kOnceThreads * 1024 * (kOnceNotes / 2) * gridDim.x;
     const uint4* p = xv + at;
     uint2* dst = out + at;
-    for (uint32_t batch = 0; batch < batches; ++batch, p += kLog2InFlight * stride, dst += kLog2InFlight * stride) {
+    if (twice) {
+        all_again = true;
+        uint64_t pass;
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pass));
+        const long long keep = kOnceKeep / (long long)(kLog2InFlight * stride * sizeof(uint4));
+        uint32_t batch = 0;
+        for (; batch + 1 + keep < batches; ++batch, p += kLog2InFlight * stride) {
+            uint4 d[kLog2InFlight];
+#pragma unroll
+            for (int k = 0; k < kLog2InFlight; ++k)
+                asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+                             : "=r"(d[k].x), "=r"(d[k].y), "=r"(d[k].z), "=r"(d[k].w) : "l"(p + k * stride), "l"(pass));
+#pragma unroll
+            for (int k = 0; k < kLog2InFlight; ++k) largest(d[k]);
+        }
+        for (; batch < batches; ++batch, p += kLog2InFlight * stride) {
+            uint4 d[kLog2InFlight];
+            load(d, p, batch + 1 < batches);
+#pragma unroll
+            for (int k = 0; k < kLog2InFlight; ++k) largest(d[k]);
+        }
+    }
+    for (uint32_t batch = twice ? batches : 0; batch < batches; ++batch, p += kLog2InFlight * stride, dst += kLog2InFlight * stride) {
         uint4 d[kLog2InFlight];
         const bool whole = batch + 1 < batches;
-#pragma unroll
-        for (int k = 0; k < kLog2InFlight; ++k) {
-            d[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (whole || p + k * stride < xv + nvec) d[k] = __ldg(p + k * stride);
-        }
+        load(d, p, whole);
         // for the next batch, one lane's for all: others write it meanwhile, and the warp's bound and notes have to agree
         const unsigned int next = __shfl_sync(0xFFFFFFFFu, *running, 0);
-        if (known != used) {
-            used = known;
-            bound = log2_first_bound(used);
-            cap = (bound + 1023u) * 0x00010001u;
-            // a softmax output is 1 at most
-            const unsigned int lead = used <= 0x3C00u ? min(kBoundOfOne - bound, kLead) : 64u;
-            edge = (0x8000u - 1024u + lead) * 0x00010001u;
-            // (with no place left the last entry stands for fewer batches than it could)
-            const int place = min(changes, kOnceChanges - 1);
-            if (lane == 0) {
-                covers[warp][place] = (unsigned short)(bound + lead);
-                from_batch[warp][place] = batch;
-            }
-            changes = place + 1;
-        }
-        if (bound == 0u) all_again = true;
+        if (known != used) take_bound(batch);
         if (all_again) {
 #pragma unroll
             for (int k = 0; k < kLog2InFlight; ++k) largest(d[k]);
@@ -1056,12 +1101,11 @@ cudaError_t launch_attn_qk_tc(const int8_t* qc, const int32_t* e_q, const int8_t
     return launch_attn_tc<128, true, 1, 8>(qc, kc, nullptr, e_q, e_k, 0, H, M, D, J, s_out, ctl, dev, stream, true);
 }
 
-// Values from which byte factors are made in one pass: 235 MB of them, nearly twice what the L2 holds. us in two kernels / one, graph replay,
-// softmax outputs of normal scores with a deviation of 3: 56 x 2048 x 2048 values 191.4 / 134.0, 32 x 2048 x 2048 110.9 / 83.5, 24 x 2048 x
-// 2048 84.0 / 69.9, 40 x 1500 x 1024 53.7 / 50.5, 16 x 1024 x 2048 31.8 / 33.9: the grid's two meetings and a launch that overlaps nothing
-// cost some 12 us, and in smaller arrays more of the second reading comes from the L2. Flatter outputs, many of whose values lie
-// near the maximum, gain less or lose: 32 x 2048 x 2048, deviation 2, 111.0 / 103.2, deviation 1 110.8 / 133.7; 24 x 2048 x 2048,
-// deviation 2, 84.0 / 97.2, 40 x 1500 x 1024 53.8 / 62.1. The line lies where the first kind gains more than the second loses.
+// Values from which one kernel makes the byte factors: 235 MB of them, nearly twice what the L2 holds. us in two kernels / one, graph replay, softmax
+// outputs of normal scores with a deviation of 3 (x read once): 56 x 2048 x 2048 values 188.8 / 133.0, 32 x 2048 x 2048 106.2 / 82.6, 28 x 2048 x 2048
+// 92.4 / 76.4, 24 x 2048 x 2048 77.3 / 67.6, 40 x 1500 x 1024 47.1 / 49.4, 16 x 1024 x 2048 24.0 / 32.6; of 1 (read twice): 188.6 / 183.5, 106.3 /
+// 104.1, 92.2 / 91.4, 77.3 / 78.3, 47.0 / 49.3, 23.9 / 28.1. The grid's two meetings and a launch that overlaps nothing cost some 10 us, and in smaller
+// arrays more of the second reading comes from the L2: the line lies where neither kind loses.
 constexpr long long kOnceCount = 14ll << 23;
 
 cudaError_t launch_log2_quantize(const __half* x, long long count, int bits, Control* ctl, int8_t* codes,
