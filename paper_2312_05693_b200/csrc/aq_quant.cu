@@ -280,13 +280,14 @@ __device__ __forceinline__ void publish_control(Control* ctl, unsigned int absma
 constexpr int kQuantThreads = 256;
 constexpr int kQuantUnits = 4;                               // units of 16 elements per thread, all loads in flight
 
-// Loads of a thread's units: unit i is u0 + i * kQuantThreads.
+// Loads of a thread's units: unit i is u0 + i * THREADS.
+template <int THREADS>
 __device__ __forceinline__ void load_units(const uint4* __restrict__ x, size_t u0, size_t total, int units_per_row,
                                            const int32_t* __restrict__ row_idx, uint4 (&d)[kQuantUnits][2]) {
-    RowWalk at(row_idx ? u0 : 0, units_per_row, kQuantThreads);
+    RowWalk at(row_idx ? u0 : 0, units_per_row, THREADS);
 #pragma unroll
     for (int i = 0; i < kQuantUnits; ++i) {
-        const size_t u = u0 + (size_t)i * kQuantThreads;
+        const size_t u = u0 + (size_t)i * THREADS;
         if (u < total) {
             const size_t src = 2 * (row_idx ? at.source(row_idx) : u);
             d[i][0] = __ldg(x + src);
@@ -309,7 +310,7 @@ quantize_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-elem
     const size_t total = (size_t)M * units_per_row;
     const size_t u0 = (size_t)blockIdx.x * (kQuantThreads * kQuantUnits) + threadIdx.x;
     uint4 d[kQuantUnits][2];
-    load_units(x, u0, total, units_per_row, row_idx, d);
+    load_units<kQuantThreads>(x, u0, total, units_per_row, row_idx, d);
     unsigned int absmax = 0;
     int e = clip_shift_or_exp;
     if (words) {
@@ -346,16 +347,17 @@ quantize_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-elem
 
 // ---- zero-point variant (Eq. 2, Eq. 5-7 with alpha = 0, power-of-two scale) ---------------
 // Codes from the minimum and maximum that range_kernel left (`words` words), as quantize_kernel.
-__global__ void __launch_bounds__(kQuantThreads)
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
 quantize_asym_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16-element units */,
                      const int32_t* __restrict__ row_idx, int bits, int words, Control* __restrict__ ctl,
                      uint4* __restrict__ q, int32_t* __restrict__ scale_exp_out, int32_t* __restrict__ zero_point_out) {
     asm volatile("griddepcontrol.wait;" ::: "memory");                 // see quantize_kernel
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t total = (size_t)M * units_per_row;
-    const size_t u0 = (size_t)blockIdx.x * (kQuantThreads * kQuantUnits) + threadIdx.x;
+    const size_t u0 = (size_t)blockIdx.x * (THREADS * kQuantUnits) + threadIdx.x;
     uint4 d[kQuantUnits][2];
-    load_units(x, u0, total, units_per_row, row_idx, d);
+    load_units<THREADS>(x, u0, total, units_per_row, row_idx, d);
     const unsigned int met = met_range(ctl, words);
     int e, zp;
     zero_point_scale(met & 0xFFFFu, met >> 16, bits, e, zp);
@@ -369,7 +371,7 @@ quantize_asym_kernel(const uint4* __restrict__ x, int M, int units_per_row /* 16
     const __half2 shift2 = __float2half2_rn((float)(zp - half_range));
 #pragma unroll
     for (int i = 0; i < kQuantUnits; ++i) {
-        const size_t u = u0 + (size_t)i * kQuantThreads;
+        const size_t u = u0 + (size_t)i * THREADS;
         if (u >= total) break;
         uint32_t out[4];
         if (fast) {
@@ -627,8 +629,8 @@ cudaError_t launch_range(const __half* x, int M, int K, const int32_t* row_idx, 
     return cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const uint4*>(x), vecs, K / 8, row_idx, per_cta, ctl);
 }
 
-size_t quantize_grid(int M, int K) {
-    const size_t per_cta = (size_t)kQuantThreads * kQuantUnits;
+size_t quantize_grid(int M, int K, int threads) {
+    const size_t per_cta = (size_t)threads * kQuantUnits;
     return ((size_t)M * (K / 16) + per_cta - 1) / per_cta;
 }
 }  // namespace
@@ -641,7 +643,7 @@ cudaError_t launch_quantize(const __half* x, int M, int K, const int32_t* row_id
         const cudaError_t e = launch_range<false>(x, M, K, row_idx, ctl, stream, words);
         if (e != cudaSuccess) return e;
     }
-    return launch_overlapped(quantize_kernel, dim3((unsigned int)quantize_grid(M, K)), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
+    return launch_overlapped(quantize_kernel, dim3((unsigned int)quantize_grid(M, K, kQuantThreads)), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
                              row_idx, bits, words, clip_shift_or_exp, ctl, reinterpret_cast<uint4*>(q), scale_exp_out,
                              reinterpret_cast<const uint4*>(alpha), k_max);
 }
@@ -666,8 +668,15 @@ cudaError_t launch_quantize_asym(const __half* x, int M, int K, const int32_t* r
     int words = 0;
     const cudaError_t e = launch_range<true>(x, M, K, row_idx, ctl, stream, words);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(quantize_asym_kernel, dim3((unsigned int)quantize_grid(M, K)), kQuantThreads, stream, reinterpret_cast<const uint4*>(x), M, K / 16,
-                             row_idx, bits, words, ctl, reinterpret_cast<uint4*>(q), scale_exp_out, zero_point_out);
+    // 256 threads a CTA, or 512 where that makes one to four CTAs an SM. The kernel is set up while range_kernel's CTAs, one or two an SM, still run,
+    // and takes few registers (48): up to three of its small CTAs then crowd the SMs with room while others get none. us a quantize call, 256 / 512
+    // threads: 504 x 8064 6.84 / 6.74, 1199 x 5504 7.25 / 6.84, 2048 x 4096 7.38 / 7.03; but 333 x 5120 4.59 / 5.20, 2048 x 11008 12.5 / 13.7.
+    const size_t ctas = quantize_grid(M, K, kQuantThreads);
+    const bool large = ctas > 148 && ctas <= 4 * 148;
+    const int threads = large ? 2 * kQuantThreads : kQuantThreads;
+    return launch_overlapped(large ? quantize_asym_kernel<2 * kQuantThreads> : quantize_asym_kernel<kQuantThreads>, dim3((unsigned int)quantize_grid(M, K, threads)),
+                             threads, stream, reinterpret_cast<const uint4*>(x), M, K / 16, row_idx, bits, words, ctl, reinterpret_cast<uint4*>(q), scale_exp_out,
+                             zero_point_out);
 }
 
 bool quantize_small_fits(int M, int K) { return (size_t)M * (size_t)K <= kSmallMaxElems; }

@@ -135,32 +135,17 @@ __device__ __forceinline__ uint2 quantize8_fp32_asym(const uint4& d, float inv, 
     return make_uint2(out[0], out[1]);
 }
 
-// A finite half's magnitude (bit pattern) in units of 2^-24, of which every half is a whole number; Inf counts as 65504.
-__device__ __forceinline__ long long half_units(unsigned int bits) {
-    if (bits > 0x7BFFu) bits = 0x7BFFu;
-    const unsigned int ex = bits >> 10;
-    return ex ? (long long)(0x400u | (bits & 0x3FFu)) << (ex - 1) : (long long)bits;
-}
 // Exponent and zero point (Eq. 6, Eq. 7): e the smallest with (2^b - 1) 2^e >= max - min, zp = -min / 2^e rounded to nearest even,
-// clipped to the codes. hi, lo: bit patterns of the largest value and of the least one's magnitude, 0 where there is none.
-// Whole numbers: max - min has at most 41 bits in units of 2^-24.
+// clipped to the codes. hi, lo: bit patterns of the largest value and of the least one's magnitude, 0 where there is none; Inf counts as 65504.
+// In single precision: 2^b - 1 times a power of two is a float, so that it is no less than max - min just when it is no less than the float
+// next above that sum, and min / 2^e is exact. (Every thread does this behind the meeting of the maxima: in 64-bit integers, shifted by
+// variables, 504 x 8064 took 7.17 us a quantize call instead of 6.84, 24 x 2048 2.28 instead of 2.17.)
 __device__ __forceinline__ void zero_point_scale(unsigned int hi, unsigned int lo, int bits, int& e, int& zp) {
-    const long long qr = (1 << bits) - 1, least = half_units(lo), range = half_units(hi) + least;
-    e = 0;
-    zp = 0;
-    if (range == 0) return;
-    int sh = (64 - __clzll(range)) - bits;               // e in units of 2^-24: qr 2^(sh + 1) >= range > qr 2^(sh - 1), for any sh
-    if (sh >= 0 ? (qr << sh) < range : qr < (range << -sh)) ++sh;
-    e = sh - 24;
-    long long z;
-    if (sh <= 0) {
-        z = least << -sh;
-    } else {
-        z = least >> sh;
-        const long long rest = least & ((1ll << sh) - 1), half = 1ll << (sh - 1);
-        if (rest > half || (rest == half && (z & 1))) ++z;
-    }
-    zp = (int)(z > qr ? qr : z);
+    const float least = __half2float(__ushort_as_half((unsigned short)min(lo, 0x7BFFu)));
+    const int range = __float_as_int(__fadd_ru(__half2float(__ushort_as_half((unsigned short)min(hi, 0x7BFFu))), least));
+    const int full = ((1 << (bits - 1)) - 1) << (24 - bits);            // the fraction of 2^b - 1: b - 1 ones
+    e = range ? (range >> 23) - 127 - (bits - 1) + ((range & 0x7FFFFF) > full ? 1 : 0) : 0;
+    zp = min(__float2int_rn(least * __int_as_float((127 - e) << 23)), (1 << bits) - 1);
 }
 
 // A CTA may write into another one's shared memory only once that one has started, which being scheduled together does
