@@ -175,7 +175,8 @@ constexpr int kRangeInFlight = 8;
 constexpr size_t kRangeFewVecs = (size_t)Control::kRangeWords * kRangeThreads * kRangeInFlight * 2;      // 237568 vectors: two turns of all loads in flight
 // (Up to there 29 CTAs without a meeting beat clusters on all SMs: quantize calls, graph replay, 100 x 4096 4.12 / 3.69 us, 116 x 8192 4.71 / 3.94,
 // 333 x 5120 5.54 / 4.50, 230 x 8192 5.64 / 4.70; with four turns 509 x 4096 5.66 / 4.95, but 400 x 8192 5.85 / 6.13. Layer calls gain less,
-// 333 x 5120 x 5120 17.9 / 17.7, and 128 x 13824 x 5120 loses: 23.7 / 24.1.)
+// 333 x 5120 x 5120 17.9 / 17.7, and 128 x 13824 x 5120 loses: 23.7 / 24.1. Gathered rows shorter than a CTA's step, every vector behind an index
+// of its own: one turn. 2075 of 512 6.07 / 6.68, 1600 of 1152 6.48 / 6.84, but 333 of 5120 6.52 / 6.06, and with a zero point 1600 of 1152 7.20 / 6.77.)
 
 // Place of element number v (per_row elements a row) in the gathered rows, carried along in steps: one division at the
 // start instead of one per element (a 64-bit one each cost 8 us on 2458 gathered rows of 7168).
@@ -594,7 +595,7 @@ namespace {
 template <bool ASYM>
 cudaError_t launch_range(const __half* x, int M, int K, const int32_t* row_idx, Control* ctl, cudaStream_t stream, int& words) {
     const size_t vecs = (size_t)M * (K / 8);
-    if (vecs <= kRangeFewVecs) {
+    if (vecs <= (!ASYM && row_idx && K / 8 < kRangeThreads ? kRangeFewVecs / 2 : kRangeFewVecs)) {
         // no meeting of clusters: as many CTAs as the control block has words for, fewer when one would have less than two vectors a thread
         size_t ctas = (vecs + kRangeThreads * 2 - 1) / (kRangeThreads * 2);
         if (ctas > Control::kRangeWords) ctas = Control::kRangeWords;
