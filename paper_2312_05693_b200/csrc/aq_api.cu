@@ -135,9 +135,9 @@ int linear_impl(aq_handle_t h, int bits, const void* x, int M, int K, const void
     const __half* xh = static_cast<const __half*>(x);
     if (alpha && !aligned(alpha, 16)) return AQ_ERR_ALIGNMENT;
     cudaError_t e = cudaSuccess;
-    // A single row, or a few short ones, on the few-row kernel: that kernel finds the scale and makes the codes itself. Every CTA
-    // then reads all of X, and writes its outputs when others may not have read yet, so nothing that the call writes may
-    // lie over what it reads: those calls quantize in a launch ahead, as calls with more rows do. Which rows an index names
+    // A single row, or several within the limits of decode_can_fuse_quantize, on the few-row kernel: that kernel finds the scale and makes the codes
+    // itself. Every cluster then reads all of X (of a single row every CTA), and writes its outputs when others may not have read yet, so nothing
+    // that the call writes may lie over what it reads: those calls quantize in a launch ahead, as calls with more rows do. Which rows an index names
     // is not known here: several indexed rows are quantized ahead too (a single one is not: see the header).
     const size_t x_bytes = (size_t)M * K * sizeof(__half), outs = (size_t)M * N;
     const bool apart = row_idx ? M == 1

@@ -220,7 +220,7 @@ struct GemmArgs {
     size_t split_bytes = 0;
     // Limit of the waits of gemm_tensor_kernel.
     unsigned long long wait_cycles = kWaitCycles;
-    // One row, or a few short ones: the few-row streaming kernel quantizes the activations itself (no quantize kernel runs
+    // Few rows (decode_can_fuse_quantize): the few-row streaming kernel quantizes the activations itself (no quantize kernel runs
     // ahead); q then receives the codes, the control block the exponent.
     const __half* fuse_x = nullptr;
     const int32_t* fuse_row_idx = nullptr;

@@ -9,7 +9,7 @@
 //  * a streaming one for M <= 16: a thread-block cluster shares a
 //    128-channel tile and splits K; in each CTA a producer thread streams 8 KB packed blocks
 //    and their activation codes into a shared-memory ring with TMA, eight consumer warps
-//    multiply (dp4a for one row, the warp-level int8 MMA on a 16-row tile above). Every CTA keeps the sums over
+//    multiply (dp4a for one row, the warp-level int8 MMA, weights by eight or twice eight rows, above). Every CTA keeps the sums over
 //    its k range in its own shared memory and writes those of the channels it does not finish into the shared
 //    memory of the CTA that does, whose barrier counts them, and every CTA finishes its slice of the tile's channels
 //    (integer sums are exact in any order, fp32 ones are added in an order that does not depend on timing). No
@@ -235,9 +235,8 @@ __device__ __forceinline__ void str_wait_peers(uint64_t* bar, volatile uint32_t*
         if ((unsigned long long)(clock64() - t0) > kStrPeerCycles) { *abort_flag = 1; return; }
 }
 
-// One row uses dp4a with one lane per channel; more rows use the warp-level int8 MMA
-// (m16n8k32) on 16 rows, with the activation tile stored 128-byte swizzled so that fragment
-// loads are free of bank conflicts.
+// One row uses dp4a; more rows use the warp-level int8 MMA (m16n8k32: 16 channels by eight rows, once or twice),
+// with the activation tile stored 128-byte swizzled so that fragment loads are free of bank conflicts.
 // Ring depth 8 (64 KB of weights in flight per CTA, two CTAs per SM): 9 stages for 16 rows and 12 for one
 // row, which shared memory would allow, measured no faster.
 template <int MB> struct StreamCfg {
@@ -1017,7 +1016,7 @@ cudaError_t launch_stream(const GemmArgs& a, const DeviceInfo& dev, cudaStream_t
     CUtensorMap map = {};
     const cuuint64_t dims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
     const cuuint64_t strides[1] = {(cuuint64_t)a.K};
-    // MMA route: 8 or 16 rows; rows 8..15 are neither copied nor read when M <= 8. Quantized here: 1, 2 or 4 rows as well (what the
+    // MMA route: 8 or 16 rows; rows 8..15 are neither copied nor read when M <= 8. Quantized here: 2 or 4 rows as well (what the
     // instruction then reads as rows up to 7 is the next block's, or whatever follows in the ring, and its sums are dropped)
     const int box_rows = !StreamCfg<MB>::kUseMma ? StreamCfg<MB>::kRows : FUSEQ ? 1 << slice_row_log(a.M) : round_up(a.M, 8);
     const cuuint32_t box[2] = {128u, (cuuint32_t)box_rows};
@@ -1152,7 +1151,7 @@ cudaError_t launch_mb(const GemmArgs& a, cudaStream_t stream) {
 // changed with it):
 //   6 x 4096 x 4096 *   7.14 / 5.60   8.10 / 5.80     16 x 5120 x 5120    8.81 / 7.79   9.70 / 8.08     (* groups of 128)
 //   9 x 2048 x 2048 *   6.04 / 4.85   7.18 / 5.48      3 x 7168 x 7168   11.25 / 7.68   11.7 / 7.86
-//  16 x  768 x  768 zero point (three launches before)  7.09 / 4.00   8.07 / 4.52      1 x 4096 x 4096 * TRIP  6.73 / 5.6
+//  16 x  768 x  768 zero point (three launches before)  7.09 / 4.00   8.07 / 4.52      1 x 4096 x 4096 * TRIP  6.68 / 4.48, zero point 6.96 / 4.94
 // 12289 to 16384 elements keep two launches, as their test asks. Without the promise of stable weights their fetch starts only behind the kernel
 // ahead, which a quantize kernel of the call would have hidden: then only up to four vectors a thread (16 x 5120 x 5120, eight of them:
 // 8.33 / 9.09; 6 x 4096 x 4096 * 7.17 / 6.15, 16 x 2048 x 2048 5.47 / 4.32), or few elements and small weights.

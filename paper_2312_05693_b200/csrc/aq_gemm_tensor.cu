@@ -349,7 +349,7 @@ gemm_tensor_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
         }
       } else {
         if (GROUPED && warp == 3) {
-            // ------------- watcher: tells the epilogue warps, through a named barrier per lane quarter and accumulator stage,
+            // ------------- watcher: tells the epilogue warps, through named barriers of an accumulator stage (one a column third or lane quarter: kMeetGroups),
             // that an accumulation is complete. A look at an mbarrier costs a warp some 200 cycles in this kernel even where
             // the phase is long over, a named barrier some 30, and the epilogue's chain per block sets the pace (K, N = 4096,
             // 11008 at M = 2048: 124 -> 120 us).
@@ -981,7 +981,8 @@ int tile_clusters(const DeviceInfo& dev, int split) {
 // The times were fitted to layer calls with every schedule forced, 131 layers of 65 to 3000 rows, 768 <= K <= 28672, 768 <= N <= 28672 (a
 // layer's schedules against one another, in graph replay, those within 60 % of its best). The schedule taken is then 0.3 % slower than the
 // best in the mean and 5 % at the worst; with the prices of before the last changes to these kernels it was 1.1 and 22 %
-// (631 rows, 20480 x 6400: 159 us on 192-token tiles, 131 on 128). Up to 64 rows 0.8 and 9 %, refitted or not.
+// (631 rows, 20480 x 6400: 159 us on 192-token tiles, 131 on 128). Up to 64 rows 0.8 and 9 %, refitted or not. On 126 other products of
+// 65 to 3000 rows 0.4 and 7 %.
 struct GroupedPlan {
     int bm, split;
 };
@@ -1036,7 +1037,8 @@ GroupedPlan grouped_plan(int M, int K, int N, const DeviceInfo& dev, size_t scra
 // all 64- or 128-token tiles at once in clusters, where the k blocks saved outweigh the exchange. Prices in nanoseconds, fitted together
 // with those of the tiles of two channel blocks (wide_plan) as the per-group ones were, 174 layers of 17 to 3000 rows: beyond
 // 64 rows the schedule taken is 0.2 % slower than the best in the mean, 7 % at the worst, where it was 2.8 and 33 % (186 rows of 1312 x 1312
-// 10.2 us in clusters, 8.3 on whole tiles; 705 rows of 3648 x 9056 34.8 us on 256 tokens, 30.1 on 128).
+// 10.2 us in clusters, 8.3 on whole tiles; 705 rows of 3648 x 9056 34.8 us on 256 tokens, 30.1 on 128). On 294 other products, 65 to 3000 rows,
+// K and N from 512 to 14000 to the 32: 0.8 % in the mean, 15 % at the worst (946 rows of 6944 x 704 14.6 us, 12.6 on 128-token tiles in pairs).
 struct ChannelPlan {
     int bm, split;
     long cost;
